@@ -16,6 +16,7 @@
 #pragma once
 
 #include "gemm_tc.cuh"
+#include "gemm_wt.cuh"
 #include "sampler.cuh"
 
 namespace pc {
@@ -54,6 +55,7 @@ struct EpiSample {
     const int32_t* step_key;
     int32_t* row_bound;            // per row: running lower bound of the final second-best score (ordered-int form)
     const DecodeArgsDev* da;       // temperature and seed
+    wt::RowScale rs;               // RMSNorm factor the operand still lacks (n == 0: none)
     __device__ __forceinline__ void set_rows(int) {}
 
     // scored iff (2^23 - (w >> 9)) < the returned word: the candidate's noise could lift it above `second`
@@ -74,13 +76,14 @@ struct EpiSample {
             if (live) rec[(size_t)(2 * (n0_tile / BN) + part) * m_stride + row] = Top2Rec{-INFINITY, -INFINITY, 0x7fffffff, 0};
             return;
         }
+        const float scale = rs.n > 0 && live ? wt::row_factor(rs.ssq + row, rs.n, rs.stride, rs.d, rs.eps) : 1.f;
         float lmax = -INFINITY;
 #pragma unroll 1
         for (int c = 0; c < n_cols; c += 32) {
             float v[32];
             tc::tmem_ld32(taddr + c, v);
 #pragma unroll
-            for (int i = 0; i < 32; ++i) lmax = fmaxf(lmax, c + i < n_cols ? v[i] : -INFINITY);
+            for (int i = 0; i < 32; ++i) lmax = fmaxf(lmax, c + i < n_cols ? v[i] * scale : -INFINITY);
         }
         const float temperature = da->temperature;
         const uint32_t k0 = da->k0, k1 = da->k1;
@@ -114,7 +117,7 @@ struct EpiSample {
             for (int i = 0; i < 32; ++i) {
                 if (pass & (1u << i)) {
                     if ((8388608u - (word[i] >> 9)) < pass_below) {
-                        top2_push(t, v[i] / temperature + gumbel_from_word(word[i]), n0 + c + i);
+                        top2_push(t, v[i] * scale / temperature + gumbel_from_word(word[i]), n0 + c + i);
                         if (t.second > bound_for) {
                             bound_for = t.second;
                             pass_below = pass_word(t.second, lmax);

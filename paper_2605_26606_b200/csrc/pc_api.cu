@@ -5,7 +5,9 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <new>
@@ -21,6 +23,7 @@
 #include "gemm_simt.cuh"
 #include "gemm_epilogues.cuh"
 #include "gemm_tc.cuh"
+#include "gemm_wt.cuh"
 #include "kernels_basic.cuh"
 #include "lm_sample.cuh"
 #include "sampler.cuh"
@@ -149,6 +152,14 @@ struct pc_ctx {
     unsigned long long captures = 0;         // decode steps captured and instantiated so far (pc_capture_count)
     int32_t n_prompts_hint = 0;              // pc_set_index_bounds: sizes of the caller's per-prompt arrays and token buffer (0: unknown)
     int64_t n_tokens_hint = 0;
+
+    // weight-on-lanes projections (gemm_wt.cuh): descriptors of the activation buffers by box height, built when first used, and
+    // the tilings chosen so far
+    struct XMap { int buf, rows; CUtensorMap map; };
+    struct WtPlan { int kind, M, dual; int cg, nt, splits, stages, clusters, n_acc; };
+    std::vector<XMap> x_maps;
+    std::vector<WtPlan> wt_plans;
+    bool final_norm_pending = false;         // the last down projection left half(h * final gain) without its 1/rms factor
 
     int fused_epilogues = 1;                 // half-operand models with head_dim 128: QKV post-processing and the MLP norm inside GEMM epilogues
     int fused_sampler = 0;                   // decode steps that only sample: Gumbel-max in the LM head's epilogue, no logits stored
@@ -346,6 +357,107 @@ inline bool wide_tiles_fill_the_gpu(const pc_ctx* c, int M, int N) {
     return ((M + pc::tc::BM - 1) / pc::tc::BM) * ((N + 255) / 256) >= c->num_sms / 2;
 }
 
+// ---- weight-on-lanes projections ------------------------------------------------------------------------------------
+enum XBuf { X_A = 0, X_ATTN = 1, X_ACT = 2, X_A_LO = 3, X_ATTN_LO = 4 };
+
+// Tiling of one projection over M rows: rows per tile (nt), K ranges per tile (splits) and single CTAs or pairs (cg).  Time
+// estimate of a candidate, in us: start, hand-over and drain of a launch + the main loop, a smooth maximum of what one SM takes
+// for its waves (its share of the ring's bytes, or the MMAs), of the weights' way from HBM and of all operand bytes' way from
+// L2 + the rows a CTA finishes (the QKV epilogue only: the others hide) + the hand-over of partial tiles.  Constants fitted to
+// 3,947 timed launches of the 1.5B and 8B shapes at 16 .. 2048 rows; over those the chosen candidate is 2 % slower than the
+// fastest one on average, 17 % at worst.
+// At most max_active[c] clusters of c CTAs with a whole SM's shared memory each are resident (the GPCs' SM counts).
+const pc_ctx::WtPlan& plan_wt(pc_ctx* c, GemmKind kind, int N, int K, int M, bool dual) {
+    using namespace pc;
+    for (const auto& p : c->wt_plans)
+        if (p.kind == kind && p.M == M && p.dual == (int)dual) return p;
+    static const int max_active[9] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
+    const int kb = K / wt::BK;
+    const bool may_split = kind == GEMM_QKV || kind == GEMM_O || kind == GEMM_DOWN;
+    pc_ctx::WtPlan best{kind, M, dual ? 1 : 0, 1, 16, 1, 4, 1, 1};
+    double best_cost = -1.;
+    for (int cg = 1; cg <= 2; ++cg) {
+        const int unit = cg == 1 ? 16 : 32;
+        const int features = (N + cg * wt::FT - 1) / (cg * wt::FT);
+        for (int tr = (M + wt::MAX_ROWS_TILE - 1) / wt::MAX_ROWS_TILE; tr <= 16 + M / 128; ++tr) {
+            const int nt = ((M + tr - 1) / tr + unit - 1) / unit * unit;
+            if (nt > wt::MAX_ROWS_TILE || (M + nt - 1) / nt != tr || (cg == 2 && nt < 192)) continue;
+            for (int sp = 1; sp <= (cg == 1 && may_split ? wt::MAX_SPLITS : 1); ++sp) {
+                if (kb / sp < 2) continue;
+                const int stage = wt::W_BYTES + (dual ? wt::x_bytes<true>(nt, cg) : wt::x_bytes<false>(nt, cg));
+                const int stages = std::min(wt::MAX_STAGES, (wt::SMEM_BUDGET - wt::smem_bytes<false>(nt, 4, cg, sp, 0)) / stage);
+                if (stages < 3 || (sp > 1 && stages * stage < (nt + 8) * wt::FT * 4)) continue;
+                const double clusters = (double)features * tr, waves = std::ceil(clusters / max_active[cg * sp] * 148. / c->num_sms);
+                const double kbs = (double)kb / sp, mmas = dual ? 2. : 1.;
+                const double sm = waves * kbs * std::max(stage / 120e3, mmas * nt * 2. / 1750. * 1.43);
+                const double hbm = (double)N * K * 2e-6 / 5.2, l2 = clusters * cg * sp * kbs * stage * 1e-6 / 18.;
+                const double rows = (double)nt / sp * (sp > 1 ? waves : 1.);
+                const double cost = 5.3 + std::cbrt(sm * sm * sm + hbm * hbm * hbm + l2 * l2 * l2) + (kind == GEMM_QKV ? 0.078 * rows : 0.) +
+                                    (sp > 1 ? 0.0136 * nt * waves : 0.) + (cg == 2 ? 0.5 : 0.);
+                if (best_cost < 0. || cost < best_cost) {
+                    best_cost = cost;
+                    const int n = features * tr;
+                    best.cg = cg; best.nt = nt; best.splits = sp; best.stages = stages;
+                    best.clusters = sp > 1 ? n : std::min(n, c->num_sms / cg);       // whole tiles: persistent CTAs
+                    best.n_acc = best.clusters < n ? 2 : 1;
+                }
+            }
+        }
+    }
+    c->wt_plans.push_back(best);
+    return c->wt_plans.back();
+}
+
+const CUtensorMap* x_map(pc_ctx* c, XBuf buf, int rows) {
+    for (const auto& m : c->x_maps)
+        if (m.buf == buf && m.rows == rows) return &m.map;
+    const size_t off[5] = {c->cv.a, c->cv.attn, c->cv.act, c->cv.a_lo, c->cv.attn_lo};
+    const int cols = buf == X_ACT ? c->d.d_ff : (buf == X_ATTN || buf == X_ATTN_LO ? c->q_dim() : c->d.d_model);
+    pc_ctx::XMap m;
+    m.buf = buf; m.rows = rows;
+    if (!pc::make_bf16_map(&m.map, c->ws + off[buf], (uint64_t)std::max(std::max(c->max_rows, c->max_prefill), 1), cols, rows)) return nullptr;
+    c->x_maps.push_back(m);
+    return &c->x_maps.back().map;
+}
+
+// One projection through gemm_wt_kernel.  lo: the buffer's rounding remainder rides along as a second operand (bf16 operands).
+template <class Epi>
+int gemm_wt(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, GemmKind kind, XBuf buf, bool lo, const WMap& w, int M, const Epi& epi, int dep_bit) {
+    using namespace pc;
+    const pc_ctx::WtPlan p = plan_wt(c, kind, w.N, w.K, M, lo);
+    const CUtensorMap* xm = x_map(c, buf, p.nt / p.cg);
+    const CUtensorMap x = xm ? *xm : CUtensorMap{};
+    const CUtensorMap* xl = lo ? x_map(c, buf == X_A ? X_A_LO : X_ATTN_LO, p.nt / p.cg) : &x;
+    if (xm == nullptr || xl == nullptr) {
+        g_cuda_error = "cuTensorMapEncodeTiled failed for an activation buffer";
+        return PC_ERR_CUDA;
+    }
+    const wt::Geom g = wt::make_geom(M, w.N, w.K, p.cg, p.nt, p.splits, p.stages, p.n_acc, c->d.half_gemm != 0);
+    const bool dep = (c->dep_launch & dep_bit) != 0 && c->prof_active_layer < 0;
+    cudaError_t e;
+    if (!lo)
+        e = p.cg == 1 ? wt::launch<1, false>(st, w.mid, x, x, sd, g, p.clusters, epi, c->err, dep) : wt::launch<2, false>(st, w.mid, x, x, sd, g, p.clusters, epi, c->err, dep);
+    else if constexpr (Epi::kDual)
+        e = p.cg == 1 ? wt::launch<1, true>(st, w.mid, x, *xl, sd, g, p.clusters, epi, c->err, dep) : wt::launch<2, true>(st, w.mid, x, *xl, sd, g, p.clusters, epi, c->err, dep);
+    else
+        e = cudaErrorInvalidValue;
+    if (e != cudaSuccess) return cuda_fail(e, "tensor-core gemm");
+    return PC_OK;
+}
+
+// Whether a pass of M rows takes the weight-on-lanes projections with their fused epilogues: every decode step and prefill of
+// a head_dim 128 model up to WT_MAX_ROWS rows; larger passes keep the rows-on-lanes kernel, whose row-per-thread epilogues
+// need fewer instructions per value.  Forced tilings (pc_set_gemm_plan) and fused_epilogues = 0 name the other kernels.
+constexpr int WT_MAX_ROWS = 4096;
+bool use_wt(const pc_ctx* c, int M) {
+    const pc_model_desc& d = c->d;
+    if (d.dtype != PC_DTYPE_BF16 || d.head_dim != 128 || d.d_model % 128 != 0) return false;
+    if (c->fused_epilogues == 0 || (c->fused_epilogues > 1 && M < c->fused_epilogues)) return false;
+    for (int k = 0; k < 5; ++k)
+        if (c->plan_bn[k] != 0) return false;
+    return M <= WT_MAX_ROWS;
+}
+
 // How the rows of a forward pass group for attention.
 struct AttnPlan {
     bool prefill;                      // true: causal attention inside each prompt, no suffix part
@@ -389,6 +501,20 @@ cudaError_t configure_attention() {
         e = cudaFuncSetAttribute(am::attn_suffix_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::suffix_smem_bytes<HD>());
     return e;
 }
+template <class Epi>
+cudaError_t configure_wt() {
+    using namespace pc;
+    cudaError_t e = wt::configure<1, false, Epi>();
+    if (e == cudaSuccess) e = wt::configure<2, false, Epi>();
+    return e;
+}
+template <class Epi>
+cudaError_t configure_wt_dual() {
+    using namespace pc;
+    cudaError_t e = wt::configure<1, true, Epi>();
+    if (e == cudaSuccess) e = wt::configure<2, true, Epi>();
+    return e;
+}
 cudaError_t configure_kernels() {
     using namespace pc;
     cudaError_t e = tc::configure<256, true, tc::EpiPartial>();
@@ -417,6 +543,15 @@ cudaError_t configure_kernels() {
     if (e == cudaSuccess) e = tc::configure<64, true, EpiSample>();
     if (e == cudaSuccess) e = tc::configure<256, false, EpiSample>();
     if (e == cudaSuccess) e = tc::configure<64, false, EpiSample>();
+    if (e == cudaSuccess) e = configure_wt<wt::EpiStore>();
+    if (e == cudaSuccess) e = configure_wt_dual<wt::EpiStore>();
+    if (e == cudaSuccess) e = configure_wt<wt::EpiQkv>();
+    if (e == cudaSuccess) e = configure_wt_dual<wt::EpiQkv>();
+    if (e == cudaSuccess) e = configure_wt<wt::EpiResNorm<true>>();
+    if (e == cudaSuccess) e = configure_wt<wt::EpiResNorm<false>>();
+    if (e == cudaSuccess) e = configure_wt_dual<wt::EpiResNorm<false>>();
+    if (e == cudaSuccess) e = configure_wt<wt::EpiSwiGLU<true>>();
+    if (e == cudaSuccess) e = configure_wt<wt::EpiSwiGLU<false>>();
     if (e == cudaSuccess) e = configure_attention<128>();
     if (e == cudaSuccess) e = configure_attention<64>();
     return e;
@@ -499,7 +634,7 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
 // M is the row count grids and GEMM plans are sized for; the live count (<= M) is read from *sd on the device.
 template <typename T>
 int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::KvArena prompt_arena, pc::KvArena suffix_arena,
-               const AttnPlan& plan) {
+               const AttnPlan& plan, bool fold_final_norm = false) {
     using namespace pc;
     constexpr bool kF32 = std::is_same<T, float>::value;
     const pc_model_desc& d = c->d;
@@ -515,7 +650,8 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
     // in the output projection's epilogue, its 1/rms applied by the gate/up epilogue (gemm_epilogues.cuh)
     // From three row tiles on: below that the two projections need their K split to keep the SMs busy (measured: unsplit they
     // lose more than the two small kernels cost), and a split GEMM's tile does not hold complete sums.
-    const bool fused = half_gemm && d.head_dim == 128 && d.d_model % 64 == 0 && c->fused_epilogues != 0 && M >= (c->fused_epilogues == 1 ? 2 * tc::BM + 1 : c->fused_epilogues);
+    const bool wt_path = !kF32 && use_wt(c, M);
+    const bool fused = !wt_path && half_gemm && d.head_dim == 128 && d.d_model % 64 == 0 && c->fused_epilogues != 0 && M >= (c->fused_epilogues == 1 ? 2 * tc::BM + 1 : c->fused_epilogues);
     float* ssq = reinterpret_cast<float*>(w + c->cv.ssq);
     const int m_stride = std::max(std::max(c->max_rows, c->max_prefill), 1);
     T* a_lo = kF32 || half_gemm ? nullptr : reinterpret_cast<T*>(w + c->cv.a_lo);          // rounding remainders (bf16 operands only)
@@ -529,6 +665,7 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
     int n_ssq = 0;
     int n_ssq_attn = 0;          // > 0: the previous layer's down projection left half(h * gain) and sums of squares for this layer's attention norm
 
+    c->final_norm_pending = false;
     launch_k(rope_table_kernel, dim3((M * half + 255) / 256), dim3(256), 0, st, sd, half, (double)d.rope_theta, g.pos, rope);
     launch_k(embed_rmsnorm_kernel<T>, dim3(M), dim3(NORM_THREADS), 0, st, sd, d.d_model, g.token, reinterpret_cast<const T*>(c->embed), c->attn_norm[0],
                                                d.rms_eps, h, a, a_lo, half_gemm ? 1 : 0, c->err);
@@ -536,6 +673,56 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
     PC_CUDA_CHECK_LAUNCH("embed_rmsnorm");
     for (int l = 0; l < d.n_layers; ++l) {
         c->mark(st, l, PC_MARK_LAYER_BEGIN);
+        if constexpr (!kF32) if (wt_path) {
+            // Five projections' worth of work in four launches: every row-wise step around a projection is in its epilogue.
+            const float* bias_l = d.qkv_bias ? c->bqkv[l] : nullptr;
+            const int n_tiles = d.d_model / wt::FT;
+            const wt::RowScale complete{nullptr, 0, 0, 1, 0.f}, scaled{ssq, n_tiles, m_stride, d.d_model, d.rms_eps};
+            c->mark(st, l, PC_MARK_NORM_ATTN);
+            wt::EpiQkv eq{};
+            eq.Hq = d.n_q_heads; eq.Hkv = d.n_kv_heads; eq.layer = l; eq.bias = bias_l;
+            eq.q_gain = d.qk_norm ? c->q_norm[l] : nullptr; eq.k_gain = d.qk_norm ? c->k_norm[l] : nullptr; eq.eps = d.rms_eps;
+            eq.rope = rope; eq.geo = g; eq.prompt_arena = prompt_arena; eq.suffix_arena = suffix_arena; eq.q_out = reinterpret_cast<__half*>(q);
+            eq.rs = l == 0 ? complete : scaled; eq.err = c->err;
+            if (int rc = gemm_wt(c, st, sd, GEMM_QKV, X_A, !half_gemm, c->m_wqkv[l], M, eq, DEP_QKV)) return rc;
+            c->mark(st, l, PC_MARK_QKV);
+            c->mark(st, l, PC_MARK_POST);
+            if (int rc = attention_bf16<128>(c, st, sd, M, l, plan, prompt_arena, suffix_arena, q, attn)) return rc;
+            auto res_norm = [&](auto epi, const float* gain, void* lo) {
+                epi.h = h; epi.ld = d.d_model; epi.gain = gain; epi.a = wt::Operand{a, lo}; epi.ssq = ssq; epi.ssq_stride = m_stride;
+                epi.rs = complete; epi.err = c->err;
+                return epi;
+            };
+            int rc = half_gemm ? gemm_wt(c, st, sd, GEMM_O, X_ATTN, false, c->m_wo[l], M, res_norm(wt::EpiResNorm<true>{}, c->mlp_norm[l], nullptr), DEP_O)
+                               : gemm_wt(c, st, sd, GEMM_O, X_ATTN, true, c->m_wo[l], M, res_norm(wt::EpiResNorm<false>{}, nullptr, nullptr), DEP_O);
+            if (rc) return rc;
+            c->mark(st, l, PC_MARK_O);
+            if (!half_gemm) {
+                // bfloat16 operands: the MLP's is one bfloat16 without a remainder, the coarsest rounding of the layer, so the norm
+                // is applied before it is rounded
+                launch_k(rmsnorm_kernel<T>, dim3(M), dim3(NORM_THREADS), 0, st, sd, M, d.d_model, h, nullptr, none, c->mlp_norm[l], d.rms_eps, a, nullptr, 0, c->err);
+                count_launches(1);
+            }
+            c->mark(st, l, PC_MARK_NORM_MLP);
+            auto swiglu = [&](auto epi) {
+                epi.act = wt::Operand{act, nullptr}; epi.ld = d.d_ff; epi.rs = half_gemm ? scaled : complete; epi.err = c->err;
+                return epi;
+            };
+            rc = half_gemm ? gemm_wt(c, st, sd, GEMM_GATE_UP, X_A, false, c->m_wgu[l], M, swiglu(wt::EpiSwiGLU<true>{}), DEP_GATE_UP)
+                           : gemm_wt(c, st, sd, GEMM_GATE_UP, X_A, false, c->m_wgu[l], M, swiglu(wt::EpiSwiGLU<false>{}), DEP_GATE_UP);
+            if (rc) return rc;
+            c->mark(st, l, PC_MARK_GATE_UP);
+            const bool last = l + 1 == d.n_layers;
+            const float* gain = !last ? c->attn_norm[l + 1] : (fold_final_norm ? c->final_norm : nullptr);
+            rc = half_gemm ? gemm_wt(c, st, sd, GEMM_DOWN, X_ACT, false, c->m_wdown[l], M, res_norm(wt::EpiResNorm<true>{}, gain, nullptr), DEP_DOWN)
+                           : gemm_wt(c, st, sd, GEMM_DOWN, X_ACT, false, c->m_wdown[l], M, res_norm(wt::EpiResNorm<false>{}, gain, a_lo), DEP_DOWN);
+            if (rc) return rc;
+            if (last) c->final_norm_pending = fold_final_norm;
+            count_launches(4);
+            c->mark(st, l, PC_MARK_DOWN);
+            PC_CUDA_CHECK_LAUNCH("decoder layer");
+            continue;
+        }
         if (l > 0 && n_ssq_attn == 0) {
             launch_k(rmsnorm_kernel<T>, dim3(M), dim3(NORM_THREADS), 0, st, sd, M, d.d_model, h, nullptr, pend, c->attn_norm[l], d.rms_eps, a, a_lo, half_gemm ? 1 : 0, c->err);
             pend = none;
@@ -656,6 +843,12 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
     return PC_OK;
 }
 
+// The factor of the final norm when the last down projection left the LM head's operand without it.
+pc::wt::RowScale folded_norm(const pc_ctx* c) {
+    return pc::wt::RowScale{reinterpret_cast<const float*>(c->ws + c->cv.ssq), c->d.d_model / pc::wt::FT,
+                            std::max(std::max(c->max_rows, c->max_prefill), 1), c->d.d_model, c->d.rms_eps};
+}
+
 // logits[n, V] = RMSNorm(h[src[r]]; final_norm) * W_lm^T
 template <typename T>
 int run_lm_head(pc_ctx* c, cudaStream_t st, int n, const pc::StepDesc* sd, const int32_t* src, float* logits) {
@@ -666,17 +859,24 @@ int run_lm_head(pc_ctx* c, cudaStream_t st, int n, const pc::StepDesc* sd, const
     const bool half_gemm = !std::is_same<T, float>::value && d.half_gemm != 0;
     T* a_lo = std::is_same<T, float>::value || half_gemm ? nullptr : reinterpret_cast<T*>(c->ws + c->cv.a_lo);
     c->mark(st, -1, PC_MARK_LM_BEGIN);
-    launch_k(rmsnorm_kernel<T>, dim3(n), dim3(NORM_THREADS), 0, st, sd, n, d.d_model, h, src, c->pend, c->final_norm, d.rms_eps, a, a_lo, half_gemm ? 1 : 0, c->err);
+    const bool folded = c->final_norm_pending;         // only the 1/rms factor is still to be applied: the LM head's epilogue does
+    c->final_norm_pending = false;
+    if (!folded)
+        launch_k(rmsnorm_kernel<T>, dim3(n), dim3(NORM_THREADS), 0, st, sd, n, d.d_model, h, src, c->pend, c->final_norm, d.rms_eps, a, a_lo, half_gemm ? 1 : 0, c->err);
     c->pend = pc::Partials{nullptr, 0, 0, 0};
     if constexpr (std::is_same<T, float>::value) {
         const T* wlm = reinterpret_cast<const T*>(d.tied_embed ? c->embed : c->lm_head);
         launch_gemm_simt<T>(st, sd, a, wlm, n, d.vocab, d.d_model, EpiStoreF32{logits, d.vocab, nullptr});
+    } else if (folded || use_wt(c, n)) {
+        wt::EpiStore epi{logits, d.vocab, {nullptr, 0, 0, 1, 0.f}};
+        if (folded) epi.rs = folded_norm(c);
+        if (int rc = gemm_wt(c, st, sd, GEMM_LM_HEAD, X_A, !half_gemm, c->m_lm, n, epi, DEP_LM_HEAD)) return rc;
     } else {
         if (int rc = gemm_bf16(c, st, sd, c->map_a, half_gemm ? nullptr : &c->map_a_lo, c->m_lm, n, plan_gemm(c, GEMM_LM_HEAD, c->m_lm, n, false),
                                tc::EpiStoreF32{logits, d.vocab, nullptr}, half_gemm, DEP_LM_HEAD))
             return rc;
     }
-    count_launches(2);
+    count_launches(folded ? 1 : 2);
     c->mark(st, -1, PC_MARK_LM_HEAD);
     PC_CUDA_CHECK_LAUNCH("lm head");
     return PC_OK;
@@ -692,19 +892,23 @@ int run_lm_head_sample(pc_ctx* c, cudaStream_t st, int n, const pc::StepDesc* sd
     const bool half_gemm = d.half_gemm != 0;
     T* a_lo = half_gemm ? nullptr : reinterpret_cast<T*>(c->ws + c->cv.a_lo);
     c->mark(st, -1, PC_MARK_LM_BEGIN);
-    launch_k(rmsnorm_kernel<T>, dim3(n), dim3(NORM_THREADS), 0, st, sd, n, d.d_model, h, nullptr, c->pend, c->final_norm, d.rms_eps, a, a_lo,
-             half_gemm ? 1 : 0, c->err);
+    const bool folded = c->final_norm_pending;
+    c->final_norm_pending = false;
+    if (!folded)
+        launch_k(rmsnorm_kernel<T>, dim3(n), dim3(NORM_THREADS), 0, st, sd, n, d.d_model, h, nullptr, c->pend, c->final_norm, d.rms_eps, a, a_lo,
+                 half_gemm ? 1 : 0, c->err);
     c->pend = pc::Partials{nullptr, 0, 0, 0};
     const GemmPlan gp = plan_gemm(c, GEMM_LM_HEAD, c->m_lm, n, false);
     Top2Rec* rec = reinterpret_cast<Top2Rec*>(c->ws + c->cv.sample_tiles);
     const int m_stride = std::max(c->max_rows, 1);
     if (int rc = gemm_bf16(c, st, sd, c->map_a, half_gemm ? nullptr : &c->map_a_lo, c->m_lm, n, gp,
-                           EpiSample{rec, m_stride, keys.key_prompt, keys.rollout, keys.step_key, keys.sample_bound, da}, half_gemm, DEP_LM_HEAD))
+                           EpiSample{rec, m_stride, keys.key_prompt, keys.rollout, keys.step_key, keys.sample_bound, da, folded ? folded_norm(c) : wt::RowScale{nullptr, 0, 0, 1, 0.f}},
+                           half_gemm, DEP_LM_HEAD))
         return rc;
     c->mark(st, -1, PC_MARK_LM_HEAD);
     const int bn = gp.wide ? 256 : 64;
     launch_k(sample_tiles_reduce_kernel, dim3(n), dim3(TILES_REDUCE_THREADS), 0, st, sd, 2 * ((d.vocab + bn - 1) / bn), rec, m_stride, keys.out_index, da);
-    count_launches(3);
+    count_launches(folded ? 2 : 3);
     c->mark(st, -1, PC_MARK_SAMPLE);
     PC_CUDA_CHECK_LAUNCH("lm head with sampler");
     return PC_OK;
@@ -953,6 +1157,8 @@ int pc_set_workspace(pc_ctx* ctx, void* dev_ws, size_t bytes, int max_rows, int 
     ctx->cv = cv;
     ctx->split_capacity_rows = std::min<size_t>((size_t)std::max(max_rows, max_prefill_tokens), kSplitMaxRows) * kMaxSplits;
     ctx->drop_graphs();
+    ctx->x_maps.clear();
+    ctx->wt_plans.clear();
     if (ctx->d.dtype == PC_DTYPE_BF16) {
         cudaError_t ce = configure_kernels();
         if (ce != cudaSuccess) { ctx->ws = nullptr; return cuda_fail(ce, "kernel attributes"); }
@@ -1082,6 +1288,14 @@ void canonical_group_bounds(const pc_ctx* c, int n_groups, int max_group_rows, i
     const int n_rep = c->d.n_q_heads / c->d.n_kv_heads;
     const int q_tiles = (std::max(max_group_rows, 1) * n_rep + pc::am::G_QROWS - 1) / pc::am::G_QROWS;
     *group_rows_bound = std::min(q_tiles * pc::am::G_QROWS / n_rep, std::max(row_bound, 1));
+}
+
+// The row bound a step's kernels are sized for: the live rows rounded up, finely where a row still costs (16 rows are one step of
+// the projections' MMA width; float32 models have no such step), so that a captured step serves a class of row counts and a
+// step issued by itself runs alike.
+int row_class(const pc_ctx* c, int n) {
+    const int unit = c->d.dtype == PC_DTYPE_F32 ? 128 : n <= 128 ? 16 : (n <= 256 ? 32 : (n <= 512 ? 64 : 128));
+    return std::min(c->max_rows, (n + unit - 1) / unit * unit);
 }
 
 // Rewrites the device-resident argument block (stream-ordered: work already queued keeps the values it was issued with).
@@ -1224,9 +1438,10 @@ int decode_launches(pc_ctx* ctx, cudaStream_t st, int m_bound, int groups_bound,
         rc = run_decode_chained(ctx, st, m_bound, sd, pa, sa, plan, logits);
         if (rc) return rc;
     } else {
-        rc = f32 ? run_layers<float>(ctx, st, m_bound, sd, pa, sa, plan) : run_layers<__nv_bfloat16>(ctx, st, m_bound, sd, pa, sa, plan);
+        const bool draw_in_head = !f32 && a.sample && logits_out == nullptr && a.logprobs == nullptr && ctx->fused_sampler;
+        rc = f32 ? run_layers<float>(ctx, st, m_bound, sd, pa, sa, plan) : run_layers<__nv_bfloat16>(ctx, st, m_bound, sd, pa, sa, plan, true);
         if (rc) return rc;
-        if (!f32 && a.sample && logits_out == nullptr && a.logprobs == nullptr && ctx->fused_sampler) {
+        if (draw_in_head) {
             // nobody asked for the logits: the draw happens in the LM head's epilogue and they are never stored
             return run_lm_head_sample(ctx, st, m_bound, sd, keys, da);
         }
@@ -1290,8 +1505,9 @@ int pc_decode_step(pc_ctx* ctx, void* stream, int n_rows, const int32_t* row_pro
                                                            (int)chain_bar_words(ctx->d.n_layers));
     count_launches(1);
     int groups_bound, group_rows_bound;
-    canonical_group_bounds(ctx, n_groups, max_group_rows, n_rows, &groups_bound, &group_rows_bound);
-    return decode_launches(ctx, st, n_rows, groups_bound, group_rows_bound, a, logits_out);
+    const int m_bound = row_class(ctx, n_rows);
+    canonical_group_bounds(ctx, n_groups, max_group_rows, m_bound, &groups_bound, &group_rows_bound);
+    return decode_launches(ctx, st, m_bound, groups_bound, group_rows_bound, a, logits_out);
 }
 
 int pc_decode_run(pc_ctx* ctx, void* stream, int n_steps, const pc_step_desc* steps_host, const pc_step_desc* steps_dev,
@@ -1331,7 +1547,7 @@ int pc_decode_run(pc_ctx* ctx, void* stream, int n_steps, const pc_step_desc* st
             count_launches(1);
             continue;
         }
-        const int m_bound = std::min(ctx->max_rows, (steps_host[s].n_rows + 127) / 128 * 128);
+        const int m_bound = row_class(ctx, steps_host[s].n_rows);
         int groups_bound, group_rows_bound;
         canonical_group_bounds(ctx, steps_host[s].n_groups, steps_host[s].max_group_rows, m_bound, &groups_bound, &group_rows_bound);
         GraphKey key;
@@ -1343,7 +1559,7 @@ int pc_decode_run(pc_ctx* ctx, void* stream, int n_steps, const pc_step_desc* st
         for (auto& ent : ctx->graphs)
             if (std::memcmp(&ent.key, &key, sizeof(key)) == 0) { exec = ent.exec; break; }
         if (exec == nullptr) {
-            if (ctx->graphs.size() >= 64) ctx->drop_graphs();
+            if (ctx->graphs.size() >= 256) ctx->drop_graphs();
             cudaGraph_t graph = nullptr;
             if (ctx->capture_stream == nullptr) {
                 e = cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking);
