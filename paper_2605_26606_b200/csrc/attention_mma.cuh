@@ -639,6 +639,7 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
         for (int i = 0; i < 2000; ++i) __nanosleep(1000);
     }
     __syncthreads();
+    grid_dep_wait();          // decode steps start this kernel when the shared-prefix kernel's CTAs leave: that one ends first
 }
 
 // ---------------------------------------------------------------------------------------------

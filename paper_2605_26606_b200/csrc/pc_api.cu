@@ -18,6 +18,7 @@
 
 #include "attention_mma.cuh"
 #include "attention_simt.cuh"
+#include "attention_tc.cuh"
 #include "common.cuh"
 #include "decode_chain.cuh"
 #include "gemm_simt.cuh"
@@ -492,11 +493,15 @@ int arena_maps(pc_ctx* c, const void* prompt_kv, int64_t prompt_slots, const voi
 template <int HD>
 cudaError_t configure_attention() {
     using namespace pc;
-    cudaError_t e = cudaFuncSetAttribute(am::attn_group_kernel<HD, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         am::group_smem_bytes<HD>());
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(am::attn_group_kernel<HD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 am::group_smem_bytes<HD>());
+    cudaError_t e = cudaSuccess;
+    if constexpr (HD == 128) {
+        e = cudaFuncSetAttribute(at::attn_prefix_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, at::SMEM_BYTES);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(at::attn_prefix_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, at::SMEM_BYTES);
+    } else {
+        e = cudaFuncSetAttribute(am::attn_group_kernel<HD, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::group_smem_bytes<HD>());
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(am::attn_group_kernel<HD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::group_smem_bytes<HD>());
+    }
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(am::attn_suffix_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::suffix_smem_bytes<HD>());
     return e;
@@ -557,6 +562,9 @@ cudaError_t configure_kernels() {
     return e;
 }
 
+// Query rows one CTA of the shared-prefix / causal-prefill attention takes.
+constexpr int prefix_q_rows(int head_dim) { return head_dim == 128 ? pc::at::QROWS : pc::am::G_QROWS; }
+
 // part_out != nullptr: the records are left unmerged and described there (the caller merges them).
 template <int HD>
 int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, int layer, const AttnPlan& plan, pc::KvArena prompt_arena,
@@ -570,7 +578,7 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
     const float scale_log2 = 1.4426950408889634f / sqrtf((float)d.head_dim);
     const int n_rep = d.n_q_heads / d.n_kv_heads;
     // a group with few query rows keeps few CTAs busy: cut its prompt into ranges so that about one CTA per SM runs
-    const int q_tiles = (plan.max_group_rows * n_rep + am::G_QROWS - 1) / am::G_QROWS;
+    const int q_tiles = (plan.max_group_rows * n_rep + prefix_q_rows(HD) - 1) / prefix_q_rows(HD);
     const int base_ctas = std::max(1, q_tiles * d.n_kv_heads * plan.n_groups);
     // (two of these CTAs fit on an SM)
     const int n_parts = plan.prefill ? 1 : std::max(1, std::min(am::MAX_PREFIX_PARTS, 2 * c->num_sms / base_ctas));
@@ -581,11 +589,16 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
     am::PrefixPartial part{reinterpret_cast<float*>(c->ws + c->cv.part_m), reinterpret_cast<float*>(c->ws + c->cv.part_l),
                            reinterpret_cast<float*>(c->ws + c->cv.part_o), n_parts, (size_t)std::max(c->max_rows, 1) * d.n_q_heads,
                            d.n_kv_heads, sgrid * am::S_WARPS};
-    const dim3 ggrid(q_tiles * n_parts, d.n_kv_heads, plan.n_groups);
+    const dim3 ggrid = HD == 128 ? dim3(q_tiles * n_parts * d.n_kv_heads * plan.n_groups) : dim3(q_tiles * n_parts, d.n_kv_heads, plan.n_groups);
     if (plan.prefill) {
-        launch_k(am::attn_group_kernel<HD, true>, dim3(ggrid), dim3(am::G_THREADS), am::group_smem_bytes<HD>(), st, 
-            c->map_prompt_kv, sd, prompt_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, plan.group_row_start, g, scale_log2,
-            part, attn, attn_lo, c->err);
+        if constexpr (HD == 128)
+            launch_k(at::attn_prefix_kernel<true>, ggrid, dim3(at::THREADS), at::SMEM_BYTES, st,
+                c->map_prompt_kv, sd, prompt_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, plan.group_row_start, g, scale_log2,
+                part, q_tiles, attn, attn_lo, c->err);
+        else
+            launch_k(am::attn_group_kernel<HD, true>, ggrid, dim3(am::G_THREADS), am::group_smem_bytes<HD>(), st,
+                c->map_prompt_kv, sd, prompt_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, plan.group_row_start, g, scale_log2,
+                part, attn, attn_lo, c->err);
         count_launches(1);
         return PC_OK;
     }
@@ -607,12 +620,17 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
     // after the QKV post-processing kernel or the QKV projection (both signal their dependents early); not on the side stream
     // of the fork and not after the persistent kernel
     const bool group_dep = !overlap && part_out == nullptr && dependent_launch(c, DEP_GROUP, M);
-    launch_k_dep(group_dep, am::attn_group_kernel<HD, false>, dim3(ggrid), dim3(am::G_THREADS), am::group_smem_bytes<HD>(), gst, 
-        c->map_prompt_kv, sd, prompt_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, plan.group_row_start, g, scale_log2, part,
-        attn, attn_lo, c->err);
+    if constexpr (HD == 128)
+        launch_k_dep(group_dep, at::attn_prefix_kernel<false>, ggrid, dim3(at::THREADS), at::SMEM_BYTES, gst,
+            c->map_prompt_kv, sd, prompt_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, plan.group_row_start, g, scale_log2, part, q_tiles,
+            attn, attn_lo, c->err);
+    else
+        launch_k_dep(group_dep, am::attn_group_kernel<HD, false>, ggrid, dim3(am::G_THREADS), am::group_smem_bytes<HD>(), gst,
+            c->map_prompt_kv, sd, prompt_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, plan.group_row_start, g, scale_log2, part,
+            attn, attn_lo, c->err);
     if (overlap) cudaEventRecord(c->ev_join, gst);
     c->mark(st, layer, PC_MARK_GROUP);
-    launch_k(am::attn_suffix_kernel<HD>, dim3(sgrid), dim3(am::S_WARPS * 32), am::suffix_smem_bytes<HD>(), st, 
+    launch_k_dep(group_dep, am::attn_suffix_kernel<HD>, dim3(sgrid), dim3(am::S_WARPS * 32), am::suffix_smem_bytes<HD>(), st,
         c->map_suffix_kv, sd, suffix_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, g, scale_log2, part, c->err);
     if (overlap) cudaStreamWaitEvent(st, c->ev_join, 0);
     c->mark(st, layer, PC_MARK_SUFFIX);
@@ -1286,8 +1304,8 @@ void canonical_group_bounds(const pc_ctx* c, int n_groups, int max_group_rows, i
     while (gb < n_groups) gb <<= 1;
     *groups_bound = std::min(gb, std::max(row_bound, 1));
     const int n_rep = c->d.n_q_heads / c->d.n_kv_heads;
-    const int q_tiles = (std::max(max_group_rows, 1) * n_rep + pc::am::G_QROWS - 1) / pc::am::G_QROWS;
-    *group_rows_bound = std::min(q_tiles * pc::am::G_QROWS / n_rep, std::max(row_bound, 1));
+    const int q_rows = prefix_q_rows(c->d.head_dim), q_tiles = (std::max(max_group_rows, 1) * n_rep + q_rows - 1) / q_rows;
+    *group_rows_bound = std::min(q_tiles * q_rows / n_rep, std::max(row_bound, 1));
 }
 
 // The row bound a step's kernels are sized for: the live rows rounded up, finely where a row still costs (16 rows are one step of
