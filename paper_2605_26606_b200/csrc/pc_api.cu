@@ -520,6 +520,12 @@ cudaError_t configure_wt_dual() {
     if (e == cudaSuccess) e = wt::configure<2, true, Epi>();
     return e;
 }
+cudaError_t configure_simt() {
+    cudaError_t e = pc::configure_gemm_simt<pc::EpiStoreF32>();
+    if (e == cudaSuccess) e = pc::configure_gemm_simt<pc::EpiResidual>();
+    if (e == cudaSuccess) e = pc::configure_gemm_simt<pc::EpiSwiGLU>();
+    return e;
+}
 cudaError_t configure_kernels() {
     using namespace pc;
     cudaError_t e = tc::configure<256, true, tc::EpiPartial>();
@@ -750,7 +756,7 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
         const float* bias = d.qkv_bias ? c->bqkv[l] : nullptr;
         Partials qkv_parts{qkv, 1, (size_t)M * c->n_qkv(), c->n_qkv()};
         if constexpr (kF32) {
-            launch_gemm_simt<T>(st, sd, a, reinterpret_cast<const T*>(c->wqkv[l]), M, c->n_qkv(), d.d_model,
+            launch_gemm_simt(st, sd, a, reinterpret_cast<const T*>(c->wqkv[l]), M, c->n_qkv(), d.d_model,
                                 EpiStoreF32{qkv, c->n_qkv(), nullptr});
         } else if (fused) {
             const EpiQkvPost epi{d.n_q_heads, d.n_kv_heads, l, bias, d.qk_norm ? c->q_norm[l] : nullptr, d.qk_norm ? c->k_norm[l] : nullptr,
@@ -776,16 +782,12 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
         c->mark(st, l, PC_MARK_POST);
         if constexpr (kF32) {
             c->mark(st, l, PC_MARK_GROUP);
-            if (d.head_dim == 128)
-                attn_row_simt_kernel<T, 128><<<dim3(M, d.n_kv_heads), 128, 0, st>>>(sd, d.n_q_heads, d.n_kv_heads, l, q, g,
-                                                                                   prompt_arena, suffix_arena, scale, attn);
-            else
-                attn_row_simt_kernel<T, 64><<<dim3(M, d.n_kv_heads), 128, 0, st>>>(sd, d.n_q_heads, d.n_kv_heads, l, q, g,
-                                                                                  prompt_arena, suffix_arena, scale, attn);
+            if (d.head_dim == 128) launch_attn_row_simt<128>(st, sd, M, d.n_q_heads, d.n_kv_heads, l, q, g, prompt_arena, suffix_arena, scale, attn);
+            else launch_attn_row_simt<64>(st, sd, M, d.n_q_heads, d.n_kv_heads, l, q, g, prompt_arena, suffix_arena, scale, attn);
             c->mark(st, l, PC_MARK_SUFFIX);
             c->mark(st, l, PC_MARK_MERGE);
             count_launches(1);
-            launch_gemm_simt<T>(st, sd, attn, reinterpret_cast<const T*>(c->wo[l]), M, d.d_model, c->q_dim(), EpiResidual{h, d.d_model});
+            launch_gemm_simt(st, sd, attn, reinterpret_cast<const T*>(c->wo[l]), M, d.d_model, c->q_dim(), EpiResidual{h, d.d_model});
         } else {
             int rc = d.head_dim == 128
                          ? attention_bf16<128>(c, st, sd, M, l, plan, prompt_arena, suffix_arena, q, attn)
@@ -816,10 +818,10 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
         count_launches(fused ? 1 : 2);
         c->mark(st, l, PC_MARK_NORM_MLP);
         if constexpr (kF32) {
-            launch_gemm_simt<T>(st, sd, a, reinterpret_cast<const T*>(c->w_gate_up[l]), M, 2 * d.d_ff, d.d_model,
-                                EpiSwiGLU<T>{act, d.d_ff});
+            launch_gemm_simt(st, sd, a, reinterpret_cast<const T*>(c->w_gate_up[l]), M, 2 * d.d_ff, d.d_model,
+                                EpiSwiGLU{act, d.d_ff});
             c->mark(st, l, PC_MARK_GATE_UP);
-            launch_gemm_simt<T>(st, sd, act, reinterpret_cast<const T*>(c->w_down[l]), M, d.d_model, d.d_ff, EpiResidual{h, d.d_model});
+            launch_gemm_simt(st, sd, act, reinterpret_cast<const T*>(c->w_down[l]), M, d.d_model, d.d_ff, EpiResidual{h, d.d_model});
         } else if (fused) {
             const EpiSwiGLUNorm epi{reinterpret_cast<__half*>(act), d.d_ff, ssq, n_ssq, m_stride, d.d_model, d.rms_eps, c->err};
             const int rc = plan_gemm(c, GEMM_GATE_UP, c->m_wgu[l], M, false).wide ? gemm_half_bn<256>(c, st, sd, c->map_a, c->m_wgu[l], M, epi, DEP_GATE_UP)
@@ -884,7 +886,7 @@ int run_lm_head(pc_ctx* c, cudaStream_t st, int n, const pc::StepDesc* sd, const
     c->pend = pc::Partials{nullptr, 0, 0, 0};
     if constexpr (std::is_same<T, float>::value) {
         const T* wlm = reinterpret_cast<const T*>(d.tied_embed ? c->embed : c->lm_head);
-        launch_gemm_simt<T>(st, sd, a, wlm, n, d.vocab, d.d_model, EpiStoreF32{logits, d.vocab, nullptr});
+        launch_gemm_simt(st, sd, a, wlm, n, d.vocab, d.d_model, EpiStoreF32{logits, d.vocab, nullptr});
     } else if (folded || use_wt(c, n)) {
         wt::EpiStore epi{logits, d.vocab, {nullptr, 0, 0, 1, 0.f}};
         if (folded) epi.rs = folded_norm(c);
@@ -1177,6 +1179,10 @@ int pc_set_workspace(pc_ctx* ctx, void* dev_ws, size_t bytes, int max_rows, int 
     ctx->drop_graphs();
     ctx->x_maps.clear();
     ctx->wt_plans.clear();
+    if (ctx->d.dtype == PC_DTYPE_F32) {
+        const cudaError_t ce = configure_simt();
+        if (ce != cudaSuccess) { ctx->ws = nullptr; return cuda_fail(ce, "kernel attributes"); }
+    }
     if (ctx->d.dtype == PC_DTYPE_BF16) {
         cudaError_t ce = configure_kernels();
         if (ce != cudaSuccess) { ctx->ws = nullptr; return cuda_fail(ce, "kernel attributes"); }
