@@ -40,6 +40,33 @@ def _dev_matrix(w: Weights, names: List[str], model: ModelShape, device, interle
     return t.view(torch.bfloat16) if model.dtype == DTYPE_BF16 else t
 
 
+def upload(arrays, device) -> List[torch.Tensor]:
+    """Host arrays to the device in ONE asynchronous copy (through a pinned buffer of torch's caching host allocator): the
+    returned tensors are views of one device buffer.  A copy per array, from pageable memory, was 30 us of host time each
+    and waited for the stream."""
+    arrays = [np.ascontiguousarray(a) for a in arrays]
+    at, end = [], 0
+    for a in arrays:
+        at.append(end)
+        end += (a.nbytes + 15) // 16 * 16
+    host = torch.empty(max(end, 16), dtype=torch.uint8, pin_memory=True)
+    flat = host.numpy()
+    for a, o in zip(arrays, at):
+        flat[o:o + a.nbytes] = a.reshape(-1).view(np.uint8)
+    dev = host.to(device, non_blocking=True)
+    return [dev[o:o + a.nbytes].view(torch.from_numpy(a.reshape(-1)[:0]).dtype) for a, o in zip(arrays, at)]
+
+
+def download(tensors) -> List[np.ndarray]:
+    """Device tensors to host arrays behind one synchronisation.  The arrays live in pinned buffers that the next call may be
+    given again: copy what is kept."""
+    host = [torch.empty(t.shape, dtype=t.dtype, pin_memory=True) for t in tensors]
+    for h, t in zip(host, tensors):
+        h.copy_(t, non_blocking=True)
+    torch.cuda.current_stream().synchronize()
+    return [h.numpy() for h in host]
+
+
 STEP_DESC_DTYPE = np.dtype([("n_rows", np.int32), ("n_groups", np.int32), ("max_group_rows", np.int32), ("reserved", np.int32),
                             ("row_offset", np.int64), ("group_offset", np.int64)])
 
@@ -117,10 +144,12 @@ class RolloutEngine:
 
     # ------------------------------------------------------------------------------------------
     def kv_arena(self, n_slots: int, which: str) -> torch.Tensor:
-        """An arena of n_slots slots; the previous arena of the same role is reused when it has the same size
-        (two 75 GB arenas must never be alive together)."""
+        """An arena of at least n_slots slots; the previous arena of the same role is reused when it has the size this one would
+        get (two 75 GB arenas must never be alive together).  Sizes are rounded up by at most 1/16, so that batches of similar size
+        meet the same arena, and with it the captured decode steps, again."""
         m = self.model
-        shape = (m.n_layers, 2, m.n_kv_heads, max(n_slots, 1), m.head_dim)
+        unit = 1 << max(max(n_slots, 1).bit_length() - 5, 0)
+        shape = (m.n_layers, 2, m.n_kv_heads, max(-(-n_slots // unit) * unit, 1), m.head_dim)
         old = self._arenas.get(which)
         if old is not None and tuple(old.shape) == shape:
             return old
@@ -140,26 +169,27 @@ class RolloutEngine:
         """Uploads the batch and allocates the KV arenas and every output buffer of the step."""
         dev, P, G = self.device, wl.n_prompts, wl.group_size
         self.wl, self.batch = wl, batch
-        up = lambda a, dt: torch.from_numpy(np.ascontiguousarray(a)).to(dev, dtype=dt, non_blocking=True)
+        caps = batch.caps.astype(np.int64)
+        small = [batch.prompt_lens.astype(np.int32), batch.prompt_offsets[:-1].astype(np.int64),
+                 np.repeat(batch.reward_threshold, G).astype(np.int32),
+                 np.arange(P * G, dtype=np.int64) * wl.max_new + caps.reshape(-1) - 1, np.arange(P, dtype=np.int32) * G,
+                 np.full(P, wl.n_pilot, dtype=np.int32)]
+        if host_inputs is None:
+            small += [batch.prompt_tokens.astype(np.int32), batch.prompt_offsets.astype(np.int32)]
+        self.prompt_len, self.prompt_kv_start, self.thresholds, self.last_index, self.group_start, self.pilot_count, *rest = upload(small, dev)
         if host_inputs is not None:           # pinned host buffers prepared by the caller (end-to-end timing)
             self.prompt_tokens = host_inputs["prompt_tokens"].to(dev, non_blocking=True)
             self.prompt_offsets = host_inputs["prompt_offsets"].to(dev, non_blocking=True)
         else:
-            self.prompt_tokens = up(batch.prompt_tokens, torch.int32)
-            self.prompt_offsets = up(batch.prompt_offsets, torch.int32)
-        self.prompt_len = up(batch.prompt_lens, torch.int32)
-        self.prompt_kv_start = up(batch.prompt_offsets[:-1].astype(np.int64), torch.int64)
+            self.prompt_tokens, self.prompt_offsets = rest
         self.total_prompt_tokens = int(batch.prompt_offsets[-1])
         self.prompt_kv = self.kv_arena(self.total_prompt_tokens, "prompt")
         # every rollout (p, i) owns caps[p, i] suffix slots and max_new token cells
-        caps = batch.caps.astype(np.int64)
         kv_start = np.zeros(P * G, dtype=np.int64)
         kv_start[1:] = np.cumsum(caps.reshape(-1))[:-1]
         self.kv_start_host = kv_start.reshape(P, G)
-        self.suffix_slots = int(caps.sum())
-        self.prompt_kv = self.prompt_kv
         self.suffix_kv = None
-        self.suffix_kv = self.kv_arena(self.suffix_slots, "suffix")
+        self.suffix_kv = self.kv_arena(int(caps.sum()), "suffix")
         self.tokens = torch.full((P * G * wl.max_new,), -1, dtype=torch.int32, device=dev)
         self.logprobs = torch.zeros(P * G * wl.max_new, dtype=torch.float32, device=dev) if self.collect_logprobs else None
         B.pc_set_logprob_buffer(self.ctx, self.logprobs)
@@ -168,23 +198,21 @@ class RolloutEngine:
         self.prompt_key_dev = None
         B.pc_set_prompt_keys(self.ctx, None)
         self.last_logits = torch.empty((P, self.model.vocab), dtype=torch.float32, device=dev)
-        self.rewards = torch.zeros(P * G, dtype=torch.float32, device=dev)
-        self.adv = torch.zeros(P * G, dtype=torch.float32, device=dev)
-        self.thresholds = up(np.repeat(batch.reward_threshold, G), torch.int32)
-        self.last_index = up((np.arange(P * G, dtype=np.int64) * wl.max_new + caps.reshape(-1) - 1), torch.int64)
-        self.group_start = up(np.arange(P, dtype=np.int32) * G, torch.int32)
-        i32 = lambda: torch.zeros(P, dtype=torch.int32, device=dev)
-        f32 = lambda: torch.zeros(P, dtype=torch.float32, device=dev)
-        self.pilot_n, self.pilot_success, self.pilot_mean, self.pilot_var = i32(), i32(), f32(), f32()
-        self.union_n, self.union_success, self.union_mean, self.union_var = i32(), i32(), f32(), f32()
-        self.status, self.extra, self.evict = i32(), i32(), i32()
-        self.n_selected = torch.zeros(1, dtype=torch.int32, device=dev)
-        self.total_rollouts = torch.zeros(1, dtype=torch.int64, device=dev)
+        # the step's small outputs: one zeroed buffer, read back in one copy
+        sizes = [2, P * G, P * G] + [P] * 11 + [1]
+        ends = np.cumsum([-(-n // 4) * 4 for n in sizes])
+        self._small = torch.zeros(int(ends[-1]), dtype=torch.int32, device=dev)
+        cut = [self._small[int(e) - -(-n // 4) * 4:int(e) - -(-n // 4) * 4 + n] for n, e in zip(sizes, ends)]
+        self._small_cut = [(int(e) - -(-n // 4) * 4, n) for n, e in zip(sizes, ends)]
+        f32 = lambda k: cut[k].view(torch.float32)
+        self.total_rollouts = cut[0].view(torch.int64)
+        self.rewards, self.adv, self.pilot_mean, self.pilot_var, self.union_mean, self.union_var = (f32(k) for k in range(1, 7))
+        self.pilot_n, self.pilot_success, self.union_n, self.union_success, self.status, self.extra, self.evict, self.n_selected = cut[7:]
 
     def prefill(self) -> None:
         b = self.batch
         B.pc_prefill_shared(self.ctx, self.wl.n_prompts, self.prompt_tokens, self.prompt_offsets, self.total_prompt_tokens,
-                            int(b.prompt_lens.max()), self.prompt_kv, self.total_prompt_tokens, self.prompt_kv_start,
+                            int(b.prompt_lens.max()), self.prompt_kv, self.prompt_kv.shape[3], self.prompt_kv_start,
                             self.last_logits)
 
     # ------------------------------------------------------------------------------------------
@@ -192,36 +220,41 @@ class RolloutEngine:
         """Rollouts (prompts[j], rollouts[j]), sorted by (prompt, rollout), all starting together.
 
         A rollout with cap c takes part in decode steps 0 .. c-2 (its c-th token needs no further forward)."""
-        wl, dev = self.wl, self.device
+        return self._build_schedule(prompts, rollouts, [])[0]
+
+    def _build_schedule(self, prompts: np.ndarray, rollouts: np.ndarray, more: List[np.ndarray]):
+        """The schedule, and the arrays `more` on the device: everything travels in one copy."""
+        wl = self.wl
         caps = self.batch.caps[prompts, rollouts].astype(np.int64)
         rid = prompts.astype(np.int64) * wl.group_size + rollouts
         kv0 = self.kv_start_host[prompts, rollouts]
         n_steps = int(max(caps.max() - 1, 0)) if len(caps) else 0
-        rp, rr, rs, rk, rt, gs = [], [], [], [], [], []
-        rows_per_step = np.zeros(n_steps, dtype=np.int64)
-        groups_per_step = np.zeros(n_steps, dtype=np.int64)
+        # (step, rollout) pairs in schedule order: rollout j is live at steps 0 .. caps[j] - 2
+        step, who = np.nonzero(np.arange(1, n_steps + 1)[:, None] < caps[None, :])
+        p = prompts[who]
+        rows_per_step = np.bincount(step, minlength=n_steps).astype(np.int64)
+        row_off = np.cumsum(rows_per_step) - rows_per_step
+        # groups: runs of one prompt inside a step; a step's boundaries are its groups' first rows and its row count
+        new = np.ones(len(p), dtype=bool)
+        new[1:] = (p[1:] != p[:-1]) | (step[1:] != step[:-1])
+        first = np.flatnonzero(new)
+        g_step = step[first]
+        groups_per_step = np.bincount(g_step, minlength=n_steps).astype(np.int64)
+        group_off = np.cumsum(groups_per_step + 1) - (groups_per_step + 1)
+        bounds = np.zeros(len(first) + n_steps, dtype=np.int32)
+        bounds[np.arange(len(first)) + g_step] = first - row_off[g_step]
+        bounds[group_off + groups_per_step] = rows_per_step
         max_group = np.zeros(n_steps, dtype=np.int64)
-        for s in range(n_steps):
-            live = caps > s + 1
-            p = prompts[live]
-            rows_per_step[s] = p.shape[0]
-            rp.append(p); rr.append(rollouts[live]); rk.append(kv0[live]); rt.append(rid[live] * wl.max_new + s)
-            rs.append(np.full(p.shape[0], s, dtype=np.int32))
-            starts = np.flatnonzero(np.r_[True, p[1:] != p[:-1]])
-            bounds = np.r_[starts, p.shape[0]]
-            groups_per_step[s] = starts.shape[0]
-            max_group[s] = int(np.max(np.diff(bounds)))
-            gs.append(bounds.astype(np.int32))
-        cat = lambda xs, dt: torch.from_numpy(np.concatenate(xs).astype(dt) if xs else np.zeros(0, dt)).to(dev)
-        row_off = np.r_[0, np.cumsum(rows_per_step)[:-1]] if n_steps else np.zeros(0, np.int64)
-        group_off = np.r_[0, np.cumsum(groups_per_step + 1)[:-1]] if n_steps else np.zeros(0, np.int64)
+        np.maximum.at(max_group, g_step, np.diff(np.append(first, len(p))))
         steps = np.zeros(n_steps, dtype=STEP_DESC_DTYPE)
         steps["n_rows"], steps["n_groups"], steps["max_group_rows"] = rows_per_step, groups_per_step, max_group
         steps["row_offset"], steps["group_offset"] = row_off, group_off
-        steps_dev = torch.from_numpy(steps.view(np.uint8).reshape(-1).copy()).to(dev) if n_steps else torch.zeros(1, dtype=torch.uint8, device=dev)
-        return StageSchedule(n_steps, rows_per_step, row_off, groups_per_step, group_off, max_group,
-                             cat(rp, np.int32), cat(rr, np.int32), cat(rs, np.int32), cat(rk, np.int64), cat(rt, np.int64),
-                             cat(gs, np.int32), int(rows_per_step.sum()), steps, steps_dev)
+        raw = steps.view(np.uint8).reshape(-1) if n_steps else np.zeros(1, np.uint8)
+        rk, rt, rp, rr, rs, gs, steps_dev, *extra = upload(
+            [kv0[who], rid[who] * wl.max_new + step, p.astype(np.int32), rollouts[who].astype(np.int32), step.astype(np.int32), bounds, raw] + more,
+            self.device)
+        return StageSchedule(n_steps, rows_per_step, row_off, groups_per_step, group_off, max_group, rp, rr, rs, rk, rt, gs,
+                             int(rows_per_step.sum()), steps, steps_dev), extra
 
     def run_stage(self, prompts: np.ndarray, rollouts: np.ndarray, record_logits: Optional[dict] = None,
                   teacher_forced: bool = False, step_range: Optional[tuple] = None) -> int:
@@ -237,19 +270,16 @@ class RolloutEngine:
         if n == 0:
             return 0
         sp = B.SampleParams(wl.temperature, wl.sample_seed)
-        d_p = torch.from_numpy(prompts.astype(np.int32)).to(dev)
-        d_r = torch.from_numpy(rollouts.astype(np.int32)).to(dev)
-        d_key = d_p if self.prompt_key_host is None else torch.from_numpy(self.prompt_key_host[prompts].astype(np.int32)).to(dev)
-        d_zero = torch.zeros(n, dtype=torch.int32, device=dev)
         rid = prompts.astype(np.int64) * wl.group_size + rollouts
-        d_first = torch.from_numpy(rid * wl.max_new).to(dev)
+        key = prompts if self.prompt_key_host is None else self.prompt_key_host[prompts]
+        sch, (d_first, d_p, d_r, d_key, d_zero) = self._build_schedule(
+            prompts, rollouts, [rid * wl.max_new, prompts.astype(np.int32), rollouts.astype(np.int32), key.astype(np.int32), np.zeros(n, np.int32)])
         if not teacher_forced and step_range is None:
             B.pc_sample(n, self.model.vocab, self.last_logits, d_p, wl.temperature, wl.sample_seed, d_key, d_r, d_zero,
                         self.tokens, out_index=d_first)
             if self.logprobs is not None:
                 B.pc_token_logprob(n, self.model.vocab, self.last_logits, d_p, wl.temperature, self.tokens, d_first, self.logprobs,
                                    d_first)
-        sch = self.build_schedule(prompts, rollouts)
         pr, rr, rs = sch.row_prompt.data_ptr(), sch.row_rollout.data_ptr(), sch.row_step.data_ptr()
         rk, rt, gs = sch.row_kv_start.data_ptr(), sch.row_tok_index.data_ptr(), sch.group_row_start.data_ptr()
         first, last = (0, sch.n_steps) if step_range is None else (step_range[0], min(step_range[1], sch.n_steps))
@@ -268,8 +298,8 @@ class RolloutEngine:
                 self.profile_samples.append((evs, nr, s + 1))
             B.pc_decode_step(self.ctx, nr, pr + 4 * o, rr + 4 * o, rs + 4 * o, rk + 8 * o, self.tokens, rt + 8 * o,
                              int(sch.groups_per_step[s]), gs + 4 * go, int(sch.max_group_rows[s]), self.prompt_len,
-                             self.prompt_kv, self.total_prompt_tokens, self.prompt_kv_start, self.suffix_kv,
-                             self.suffix_slots, logits_out, None if teacher_forced else sp)
+                             self.prompt_kv, self.prompt_kv.shape[3], self.prompt_kv_start, self.suffix_kv,
+                             self.suffix_kv.shape[3], logits_out, None if teacher_forced else sp)
             if logits_out is not None and self.record_rows is not None:
                 _, rec_p, rec_r = record_logits[s]
                 keep = np.flatnonzero([(int(a), int(b)) in self.record_rows for a, b in zip(rec_p, rec_r)])
@@ -293,8 +323,8 @@ class RolloutEngine:
             # steps s .. e-1 natively: one graph launch per step, issued by the library
             item = STEP_DESC_DTYPE.itemsize
             B.pc_decode_run(self.ctx, e - s, sch.steps_host.ctypes.data + s * item, sch.steps_dev.data_ptr() + s * item,
-                            pr, rr, rs, rk, self.tokens, rt, gs, self.prompt_len, self.prompt_kv, self.total_prompt_tokens,
-                            self.prompt_kv_start, self.suffix_kv, self.suffix_slots, sp)
+                            pr, rr, rs, rk, self.tokens, rt, gs, self.prompt_len, self.prompt_kv, self.prompt_kv.shape[3],
+                            self.prompt_kv_start, self.suffix_kv, self.suffix_kv.shape[3], sp)
             s = e
         self._keep_schedule = sch
         self.stage_rows_per_step.append(sch.rows_per_step.copy())
@@ -322,19 +352,18 @@ class RolloutEngine:
         self.prefill_events[1].record()
         pp, rr = np.repeat(np.arange(P), k), np.tile(np.arange(k), P)
         n_tok = self.run_stage(pp, rr, record_logits=self.record_pilot_logits)
-        pilot_count = torch.full((P,), k, dtype=torch.int32, device=self.device)
         B.pc_reward_last_token(P * G, self.tokens, self.last_index, self.thresholds, self.rewards)
-        B.pc_group_stats(P, self.rewards, self.group_start, pilot_count, self.pilot_n, self.pilot_success, self.pilot_mean,
+        B.pc_group_stats(P, self.rewards, self.group_start, self.pilot_count, self.pilot_n, self.pilot_success, self.pilot_mean,
                          self.pilot_var)
         B.pc_allocate(P, self.pilot_success, self.pilot_n, B.AllocParams(wl.p_lower, wl.p_upper, wl.p_solve, G - k, b_t),
                       self.status, self.extra, self.evict, self.n_selected, self.total_rollouts)
-        status = self.status.cpu().numpy()            # the commit stage's row set depends on it
+        status = download([self.status])[0].copy()    # the commit stage's row set depends on it
         commit = np.flatnonzero(status == B.PC_STATUS_COMMIT)
         if G > k and commit.size:
             n_tok += self.run_stage(np.repeat(commit, G - k), np.tile(np.arange(k, G), commit.size),
                                     record_logits=self.record_commit_logits)
         B.pc_reward_last_token(P * G, self.tokens, self.last_index, self.thresholds, self.rewards)
-        union_count = torch.from_numpy(np.where(status == B.PC_STATUS_COMMIT, G, k).astype(np.int32)).to(self.device)
+        union_count, = upload([np.where(status == B.PC_STATUS_COMMIT, G, k).astype(np.int32)], self.device)
         B.pc_group_stats(P, self.rewards, self.group_start, union_count, self.union_n, self.union_success, self.union_mean,
                          self.union_var)
         B.pc_grpo_advantage(P, self.rewards, self.group_start, union_count, self.status, self.adv)
@@ -371,7 +400,7 @@ class RolloutEngine:
             off0 = int(offsets[nA])
             offs_b = torch.from_numpy((offsets[nA:] - off0).astype(np.int32)).to(dev)
             B.pc_prefill_shared(self.ctx, PB, self.prompt_tokens[off0:], offs_b, int(offsets[-1]) - off0,
-                                int(batch_b.prompt_lens.max()), self.prompt_kv, self.total_prompt_tokens,
+                                int(batch_b.prompt_lens.max()), self.prompt_kv, self.prompt_kv.shape[3],
                                 self.prompt_kv_start[nA:], self.last_logits[nA:])
         self.prompt_key_host = np.concatenate([commit_a, np.arange(PB)]).astype(np.int32)
         self.prompt_key_dev = torch.from_numpy(self.prompt_key_host).to(dev)
@@ -392,19 +421,23 @@ class RolloutEngine:
 
     def collect(self, status: np.ndarray) -> dict:
         wl, P, G, k = self.wl, self.wl.n_prompts, self.wl.group_size, self.wl.n_pilot
-        self.check_error_flag()
-        toks = self.tokens.cpu().numpy().reshape(P, G, wl.max_new)
+        flag, toks, small, *lp = download([self.err_flag, self.tokens, self._small] + ([] if self.logprobs is None else [self.logprobs]))
+        if int(flag[0]) != 0:
+            raise RuntimeError(f"device error flag = {int(flag[0])}")
+        toks = toks.reshape(P, G, wl.max_new)
         generated = np.zeros((P, G), dtype=bool)
         generated[:, :k] = True
         generated[status == B.PC_STATUS_COMMIT, :] = True
         tokens = [[toks[p, i, :self.batch.caps[p, i]].copy() if generated[p, i] else None for i in range(G)] for p in range(P)]
-        rewards = self.rewards.cpu().numpy().reshape(P, G).copy()
+        total, rewards, adv, pilot_mean, pilot_var, union_mean, union_var, pilot_n, pilot_success, union_n, union_success, _, extra, evict, n_sel = (
+            small[o:o + n].copy() for o, n in self._small_cut)
+        f32 = lambda a: a.view(np.float32)
+        rewards = f32(rewards).reshape(P, G)
         rewards[~generated] = 0.0          # cells of rollouts that were never generated hold no reward
-        h = lambda t: t.cpu().numpy()
         return dict(tokens=tokens, rewards=rewards, generated=generated,
-                    pilot_n=h(self.pilot_n), pilot_success=h(self.pilot_success), pilot_mean=h(self.pilot_mean),
-                    pilot_var=h(self.pilot_var), status=status, extra=h(self.extra), evict=h(self.evict),
-                    n_selected=int(self.n_selected.item()), total_rollouts=int(self.total_rollouts.item()),
-                    union_n=h(self.union_n), union_success=h(self.union_success), union_mean=h(self.union_mean),
-                    union_var=h(self.union_var), advantages=h(self.adv).reshape(P, G),
-                    logprobs=None if self.logprobs is None else h(self.logprobs).reshape(P, G, wl.max_new))
+                    pilot_n=pilot_n, pilot_success=pilot_success, pilot_mean=f32(pilot_mean),
+                    pilot_var=f32(pilot_var), status=status, extra=extra, evict=evict,
+                    n_selected=int(n_sel[0]), total_rollouts=int(total.view(np.int64)[0]),
+                    union_n=union_n, union_success=union_success, union_mean=f32(union_mean),
+                    union_var=f32(union_var), advantages=f32(adv).reshape(P, G),
+                    logprobs=lp[0].reshape(P, G, wl.max_new).copy() if lp else None)

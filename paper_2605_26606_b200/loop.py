@@ -86,7 +86,6 @@ class RolloutLoop:
         eng.batch = Batch(np.zeros(R, np.int32), np.zeros(R + 1, np.int32), np.zeros(0, np.int32), np.zeros(R), np.zeros(R, np.int32),
                           np.ones((R, G), np.int32))
         eng.prompt_kv = eng.kv_arena(self.capacity_slots, "prompt")
-        eng.total_prompt_tokens = self.capacity_slots
         eng.tokens = torch.full((R * G * wl.max_new,), -1, dtype=torch.int32, device=dev)
         eng.logprobs = None
         B.pc_set_logprob_buffer(eng.ctx, None)
@@ -120,7 +119,7 @@ class RolloutLoop:
         offsets[1:] = np.cumsum(lens)
         logits = torch.empty((len(ids), eng.model.vocab), dtype=torch.float32, device=dev)
         B.pc_prefill_shared(eng.ctx, len(ids), torch.from_numpy(np.concatenate(toks).astype(np.int32)).to(dev),
-                            torch.from_numpy(offsets).to(dev), int(offsets[-1]), int(max(lens)), eng.prompt_kv, self.capacity_slots,
+                            torch.from_numpy(offsets).to(dev), int(offsets[-1]), int(max(lens)), eng.prompt_kv, eng.prompt_kv.shape[3],
                             torch.tensor(starts, dtype=torch.int64, device=dev), logits)
         eng.last_logits[torch.tensor(rows, device=dev)] = logits
         self._upload_prompt_tables()
@@ -158,8 +157,7 @@ class RolloutLoop:
         start = np.zeros(len(items), np.int64)
         start[1:] = np.cumsum(caps)[:-1]
         eng.kv_start_host[rows, rolls] = start
-        eng.suffix_slots = int(caps.sum())
-        eng.suffix_kv = eng.kv_arena(eng.suffix_slots, "suffix")
+        eng.suffix_kv = eng.kv_arena(int(caps.sum()), "suffix")
         eng.run_stage(rows, rolls)
         self.passes += 1
 
