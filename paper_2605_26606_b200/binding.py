@@ -118,6 +118,25 @@ def _lib():
     return _LIB
 
 
+_CALLS = None
+
+
+def _calls():
+    """The native wrappers of the calls that are shorter than their own marshalling (csrc/py_calls.cpp), bound to the library."""
+    global _CALLS
+    if _CALLS is None:
+        lib = _lib()
+        try:
+            from . import _pc_calls
+        except ImportError as e:
+            raise RuntimeError("_pc_calls.so is missing or does not load: build it with `python -m paper_2605_26606_b200.build` "
+                               "(there is no fallback path)") from e
+        _pc_calls.bind(*(C.cast(getattr(lib, n), C.c_void_p).value for n in
+                         ("pc_reward_last_token", "pc_group_stats", "pc_allocate", "pc_allocate_variance", "pc_grpo_advantage")))
+        _CALLS = _pc_calls
+    return _CALLS
+
+
 def _check(status: int, where: str) -> None:
     if status != PC_OK:
         raise PcError(status, where)
@@ -139,6 +158,8 @@ def _ptr(t: Optional[torch.Tensor], dtype: Optional[torch.dtype] = None) -> Opti
 
 
 def _stream() -> int:
+    if torch.cuda.is_initialized():          # torch's own accessor without the Stream object around it
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return torch.cuda.current_stream().cuda_stream
 
 
@@ -328,32 +349,33 @@ def pc_set_prompt_keys(ctx: Context, prompt_key: Optional[torch.Tensor]) -> None
 
 
 def pc_reward_last_token(n, tokens, last_index, threshold, reward) -> None:
-    _check(_lib().pc_reward_last_token(_stream(), n, _ptr(tokens, torch.int32), _ptr(last_index, torch.int64),
-                                       _ptr(threshold, torch.int32), _ptr(reward, torch.float32)), "pc_reward_last_token")
+    status = (_CALLS or _calls()).reward_last_token(n, tokens, last_index, threshold, reward)
+    if status:
+        raise PcError(status, "pc_reward_last_token")
 
 
 def pc_group_stats(n_groups, rewards, group_start, group_count, n, n_success, mean, var) -> None:
-    _check(_lib().pc_group_stats(_stream(), n_groups, _ptr(rewards, torch.float32), _ptr(group_start, torch.int32),
-                                 _ptr(group_count, torch.int32), _ptr(n, torch.int32), _ptr(n_success, torch.int32),
-                                 _ptr(mean, torch.float32), _ptr(var, torch.float32)), "pc_group_stats")
+    status = (_CALLS or _calls()).group_stats(n_groups, rewards, group_start, group_count, n, n_success, mean, var)
+    if status:
+        raise PcError(status, "pc_group_stats")
 
 
 def pc_allocate(n_prompts, pilot_success, pilot_n, params: AllocParams, status, extra_rollouts, evict, n_selected,
                 total_rollouts) -> None:
-    _check(_lib().pc_allocate(_stream(), n_prompts, _ptr(pilot_success, torch.int32), _ptr(pilot_n, torch.int32),
-                              C.byref(params), _ptr(status, torch.int32), _ptr(extra_rollouts, torch.int32),
-                              _ptr(evict, torch.int32), _ptr(n_selected, torch.int32), _ptr(total_rollouts, torch.int64)),
-           "pc_allocate")
+    rc = (_CALLS or _calls()).allocate(n_prompts, pilot_success, pilot_n, params, status, extra_rollouts, evict, n_selected, total_rollouts)
+    if rc:
+        raise PcError(rc, "pc_allocate")
 
 
 def pc_allocate_variance(n_prompts, pilot_var, pilot_n, var_min: float, n_commit: int, b_t: int, status, extra_rollouts, n_selected,
                          total_rollouts) -> None:
-    _check(_lib().pc_allocate_variance(_stream(), n_prompts, _ptr(pilot_var, torch.float32), _ptr(pilot_n, torch.int32), var_min,
-                                       n_commit, b_t, _ptr(status, torch.int32), _ptr(extra_rollouts, torch.int32),
-                                       _ptr(n_selected, torch.int32), _ptr(total_rollouts, torch.int64)), "pc_allocate_variance")
+    rc = (_CALLS or _calls()).allocate_variance(n_prompts, pilot_var, pilot_n, var_min, n_commit, b_t, status, extra_rollouts, n_selected,
+                                                total_rollouts)
+    if rc:
+        raise PcError(rc, "pc_allocate_variance")
 
 
 def pc_grpo_advantage(n_groups, rewards, group_start, group_count, status, adv) -> None:
-    _check(_lib().pc_grpo_advantage(_stream(), n_groups, _ptr(rewards, torch.float32), _ptr(group_start, torch.int32),
-                                    _ptr(group_count, torch.int32), _ptr(status), _ptr(adv, torch.float32)),
-           "pc_grpo_advantage")
+    rc = (_CALLS or _calls()).grpo_advantage(n_groups, rewards, group_start, group_count, status, adv)
+    if rc:
+        raise PcError(rc, "pc_grpo_advantage")

@@ -1,15 +1,18 @@
-"""Builds the CUDA library in-tree: paper_2605_26606_b200/libpc.so (sm_100a only)."""
+"""Builds the CUDA library (libpc.so, sm_100a only) and the native call wrappers (_pc_calls.so) in-tree."""
 from __future__ import annotations
 
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libpc.so")
 SOURCES = ["pc_api.cu"]
+CALLS = os.path.join(HERE, "_pc_calls.so")
+CALLS_SOURCE = os.path.join(CSRC, "py_calls.cpp")
 
 
 def _nvcc() -> str:
@@ -23,11 +26,31 @@ def _stale() -> bool:
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(HERE, "..", "include", "pc.h"), __file__]
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if not f.endswith(".cpp")] + [os.path.join(HERE, "..", "include", "pc.h"), __file__]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_calls(force: bool = False) -> str:
+    """The CPython extension of csrc/py_calls.cpp (host code only)."""
+    deps = [CALLS_SOURCE, os.path.join(HERE, "..", "include", "pc.h"), __file__]
+    if not force and os.path.exists(CALLS) and all(os.path.getmtime(d) <= os.path.getmtime(CALLS) for d in deps):
+        return CALLS
+    import torch
+    from torch.utils import cpp_extension
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_nvcc()))), "include")
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    for inc in cpp_extension.include_paths() + [sysconfig.get_paths()["include"], cuda]:
+        cmd += ["-isystem", inc]
+    cmd += [CALLS_SOURCE, "-o", CALLS, "-L" + lib, "-ltorch_python", "-lc10", "-lc10_cuda", "-Wl,-rpath," + lib]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("g++ failed:\n" + res.stdout + res.stderr)
+    return CALLS
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_calls(force)
     if not force and not _stale():
         return LIB
     cmd = [_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
