@@ -311,8 +311,8 @@ typedef struct pc_step_desc {
 /* n_steps consecutive decode steps (each exactly a pc_decode_step with sampling and no logits output) over a
  * schedule that already lives on the device: the row_* arrays and group_row_start hold every step's entries back to
  * back and step s uses the slices named by steps[s].  steps_host and steps_dev are the same n_steps descriptors in
- * host and in device memory.  The kernels of a step are captured once per shape class (rows rounded up to 128, groups
- * to a power of two, largest group to a query-tile boundary; per pair of KV arenas) into a CUDA graph and replayed, so
+ * host and in device memory.  The kernels of a step are captured once per shape class (rows rounded up to 16 .. 128, groups
+ * to an eighth of a power of two, largest group to a query-tile boundary; per pair of KV arenas) into a CUDA graph and replayed, so
  * the host issues one launch per step; the caller's arrays and sampling parameters are read through a device-resident
  * argument block, so a new schedule, token buffer or seed needs no new capture.  The first call creates a CUDA stream
  * owned by the context (captures run there) and every capture instantiates a graph; pc_destroy, pc_set_workspace,

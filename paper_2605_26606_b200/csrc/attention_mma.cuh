@@ -11,8 +11,8 @@
 //                       query row carries its own number of visible prompt slots, which also makes this
 //                       the causal prefill kernel.  Decode: leaves (m, l, unnormalised O) per query row
 //                       in scratch.  Prefill: writes the normalised output.
-//   attn_suffix_kernel  one warp per (rollout, KV head) streams the rollout's own suffix K/V through a
-//                       3-stage TMA ring at full HBM rate.  Positions sit on the MMA M axis (S^T = K Q^T,
+//   attn_suffix_kernel  one warp per (rollout, KV head, range of the suffix) streams the rollout's own suffix K/V
+//                       through a 3-stage TMA ring.  Positions sit on the MMA M axis (S^T = K Q^T,
 //                       O^T = V^T P^T), so the 6-8 query heads fill the N = 8 axis and no MMA work is
 //                       padded; P is transposed between the two MMAs with movmatrix.  It leaves its
 //                       (m, l, unnormalised O) record next to the prefix records.
@@ -80,6 +80,14 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // exp2 that maps -inf to 0 without producing NaN when both operands are -inf
 __device__ __forceinline__ float exp2_safe(float x, float m) { return m == -INFINITY ? 0.f : exp2f(x - m); }
 
+// K and V of one tile of consecutive slots in one request: the arena as [K|V][64-dim half][row][64], row counted from plane 0
+// (make_kv_tile_map).
+__device__ __forceinline__ void tma_load_kv(uint32_t dst, const CUtensorMap* map, uint32_t bar, int row) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %3, %3}], [%2];"
+        ::"r"(dst), "l"(map), "r"(bar), "r"(0), "r"(row)
+        : "memory");
+}
 // Byte offset of (row r, dim d) (d a multiple of 8) in a swizzled tile of ROWS rows: boxes of 64 dims,
 // rows of 128 bytes, 16-byte chunk index XORed with (r mod 8).
 template <int ROWS>
@@ -99,9 +107,9 @@ struct PrefixPartial {
     int n_kv_heads;
     int n_suffix_warps;     // warps of the suffix kernel's grid: how suffixes are cut into ranges is planned for this many
 };
-constexpr int MAX_PREFIX_PARTS = 8;
-constexpr int MAX_SUFFIX_CHUNKS = 8;
-constexpr int MAX_RECORDS = MAX_PREFIX_PARTS + MAX_SUFFIX_CHUNKS;
+constexpr int MAX_PREFIX_PARTS = 8, MAX_MERGED_PARTS = 4;      // (the second where the suffix kernel merges)
+constexpr int MAX_SUFFIX_CHUNKS = 12;
+constexpr int MAX_RECORDS = MAX_PREFIX_PARTS + MAX_SUFFIX_CHUNKS, MAX_MERGED_RECORDS = MAX_MERGED_PARTS + 3;
 
 // ---------------------------------------------------------------------------------------------
 // Group (shared-prefix / causal-prefill) kernel
@@ -366,8 +374,11 @@ attn_group_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* __
 // ---------------------------------------------------------------------------------------------
 // Suffix kernel
 // ---------------------------------------------------------------------------------------------
-constexpr int S_WARPS = 4;
-constexpr int S_TP = 32;            // positions per stage
+// A warp's tile -- ldmatrix, two rounds of MMAs, the softmax between them -- is one chain of about 900 clocks for 8 KB, so a warp
+// of its own per scheduler cannot keep up with HBM (4 warps, 32 positions at a time: 4.35 TB/s at 237 rows x 512); two per
+// scheduler can.  192 KB of tiles are in flight per SM.
+constexpr int S_WARPS = 8;
+constexpr int S_TP = 16;            // positions per stage: one MMA tile
 constexpr int S_STAGES = 3;
 template <int HD> constexpr int suffix_smem_bytes() {
     return S_WARPS * (S_STAGES * 2 * S_TP * HD * 2 + 8 * HD * 4) + 1024 + 256;
@@ -377,18 +388,18 @@ template <int HD> constexpr int suffix_smem_bytes() {
 // warps doubles the kernel's time.  The suffix of a rollout is therefore cut into ranges of tiles ("chunks") that
 // are spread over the warps; every chunk leaves its own record.  Tiles per chunk (ct) and chunk slots per (row, KV
 // head) item (cpi) for a step whose longest suffix has max_slen slots: among 1..MAX_SUFFIX_CHUNKS chunks per item, the
-// choice that minimises (units the busiest warp gets) x (tiles per unit + 2), the + 2 standing for the fixed cost of a
+// choice that minimises (units the busiest warp gets) x (tiles per unit + 4), the + 4 standing for the fixed cost of a
 // unit (length lookup, first TMA round trip, record) in tile times.  The same value serves every row of the step, and
 // the merge kernel recomputes it from the same inputs.
 struct SuffixPlan { int ct, cpi; };
-__device__ __forceinline__ SuffixPlan suffix_plan(int max_slen, int n_items, int n_warps) {
+__device__ __forceinline__ SuffixPlan suffix_plan(int max_slen, int n_items, int n_warps, int max_chunks = MAX_SUFFIX_CHUNKS) {
     const int ntiles = max(1, (max_slen + S_TP - 1) / S_TP);
     SuffixPlan best{ntiles, 1};
     long long best_cost = -1;
-    for (int c = 1; c <= MAX_SUFFIX_CHUNKS; ++c) {
+    for (int c = 1; c <= max_chunks; ++c) {
         const int ct = (ntiles + c - 1) / c;
         const int cc = (ntiles + ct - 1) / ct;
-        const long long cost = (long long)((n_items * cc + n_warps - 1) / max(n_warps, 1)) * (ct + 2);
+        const long long cost = (long long)((n_items * cc + n_warps - 1) / max(n_warps, 1)) * (ct + 4);
         if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = SuffixPlan{ct, cc}; }
     }
     return best;
@@ -398,10 +409,131 @@ __device__ __forceinline__ int suffix_chunks(int n, int ct) {             // rec
     return (ntiles + ct - 1) / ct;
 }
 
+// Normalises and stores one (row, query head): IEEE half, or bf16 with its rounding remainder (second operand of the O projection).
+// A lane holds dims lane * HD/32 ...
 template <int HD>
+__device__ __forceinline__ void store_attention(int lane, size_t rh, float* acc, float denom, __nv_bfloat16* __restrict__ out,
+                                                __nv_bfloat16* __restrict__ out_lo, int32_t* err) {
+    constexpr int EPL = HD / 32;
+    const float inv = denom > 0.f ? 1.f / denom : 0.f;
+    float lo[EPL];
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) {
+        acc[e] *= inv;
+        lo[e] = acc[e] - __bfloat162float(__float2bfloat16_rn(acc[e]));
+    }
+    __nv_bfloat16* dst = out + rh * HD + lane * EPL;
+    if (out_lo == nullptr) {                 // the output projection takes IEEE half operands: no remainder needed
+        if (EPL == 4) *reinterpret_cast<uint2*>(dst) = make_uint2(pack_f16_guard(acc[0], acc[1], err), pack_f16_guard(acc[EPL - 2], acc[EPL - 1], err));
+        else *reinterpret_cast<uint32_t*>(dst) = pack_f16_guard(acc[0], acc[1], err);
+        return;
+    }
+    __nv_bfloat16* dst_lo = out_lo + rh * HD + lane * EPL;
+    if (EPL == 4) {
+        *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16(acc[0], acc[1]), pack_bf16(acc[EPL - 2], acc[EPL - 1]));
+        *reinterpret_cast<uint2*>(dst_lo) = make_uint2(pack_bf16(lo[0], lo[1]), pack_bf16(lo[EPL - 2], lo[EPL - 1]));
+    } else {
+        *reinterpret_cast<uint32_t*>(dst) = pack_bf16(acc[0], acc[1]);
+        *reinterpret_cast<uint32_t*>(dst_lo) = pack_bf16(lo[0], lo[1]);
+    }
+}
+
+// Merge of records 0 .. n-1 of all n_rep (<= 8) query heads of one row and KV head by a warp, in index order, by their
+// log-sum-exp:  M = max m_i,  out = sum_i O_i 2^(m_i - M) / sum_i l_i 2^(m_i - M).  m and l of all (record, head) pairs come in one
+// round trip, the outputs of two records in another each.  own_*: one more record, the last, that is still in shared memory ([8]
+// values, [8][HD] outputs), or nullptr.
+template <int HD>
+__device__ __forceinline__ void merge_heads_warp(int lane, size_t rh0, int n_rep, const PrefixPartial& part, int n, const float* own_m,
+                                                 const float* own_l, const float* own_o, __nv_bfloat16* __restrict__ out,
+                                                 __nv_bfloat16* __restrict__ out_lo, int32_t* err) {
+    constexpr int EPL = HD / 32, NH = 8, B = 2, MR = (MAX_MERGED_RECORDS + 3) / 4;
+    const int hj = lane & 7, pi = lane >> 3;        // lane 8 p + j holds records p, p + 4, ... of head j
+    float m[MR], l[MR], M = own_m != nullptr && hj < n_rep ? own_m[hj] : -INFINITY;
+#pragma unroll
+    for (int k = 0; k < MR; ++k) {
+        const int i = pi + 4 * k;
+        const bool on = i < n && hj < n_rep;
+        m[k] = on ? __ldcg(part.m + (size_t)i * part.stride + rh0 + hj) : -INFINITY;
+        l[k] = on ? __ldcg(part.l + (size_t)i * part.stride + rh0 + hj) : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < MR; ++k) M = fmaxf(M, m[k]);
+    M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 8));
+    M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 16));
+#pragma unroll
+    for (int k = 0; k < MR; ++k) m[k] = exp2_safe(m[k], M);        // weights
+    float acc[NH][EPL], denom = 0.f;
+#pragma unroll
+    for (int j = 0; j < NH; ++j)
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) acc[j][e] = 0.f;
+#pragma unroll
+    for (int k = 0; k < MR; ++k) {
+#pragma unroll
+        for (int p0 = 0; p0 < 4; p0 += B) {
+            if (4 * k + p0 >= n) break;
+            float v[B][NH][EPL];
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                const float* src = part.o + ((size_t)(4 * k + p0 + b) * part.stride + rh0) * HD + lane * EPL;
+#pragma unroll
+                for (int j = 0; j < NH; ++j) {
+                    // a record with m = -inf was left by an empty range: its output is not defined
+                    const bool have = j < n_rep && __shfl_sync(0xffffffffu, m[k], 8 * (p0 + b) + j) > 0.f;
+                    if (EPL == 4) {
+                        const float4 x = have ? __ldcg(reinterpret_cast<const float4*>(src + j * HD)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        v[b][j][0] = x.x; v[b][j][1] = x.y; v[b][j][EPL - 2] = x.z; v[b][j][EPL - 1] = x.w;
+                    } else {
+                        const float2 x = have ? __ldcg(reinterpret_cast<const float2*>(src + j * HD)) : make_float2(0.f, 0.f);
+                        v[b][j][0] = x.x; v[b][j][1] = x.y;
+                    }
+                }
+            }
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                denom = __fmaf_rn(__shfl_sync(0xffffffffu, l[k], 8 * (p0 + b) + hj), __shfl_sync(0xffffffffu, m[k], 8 * (p0 + b) + hj), denom);
+#pragma unroll
+                for (int j = 0; j < NH; ++j) {
+                    const float wj = __shfl_sync(0xffffffffu, m[k], 8 * (p0 + b) + j);
+#pragma unroll
+                    for (int e = 0; e < EPL; ++e) acc[j][e] = __fmaf_rn(v[b][j][e], wj, acc[j][e]);
+                }
+            }
+        }
+    }
+    float wo = 0.f;
+    if (own_m != nullptr && hj < n_rep) {
+        wo = exp2_safe(own_m[hj], M);
+        denom = __fmaf_rn(own_l[hj], wo, denom);
+    }
+#pragma unroll
+    for (int j = 0; j < NH; ++j) {
+        const float wj = __shfl_sync(0xffffffffu, wo, j), dj = __shfl_sync(0xffffffffu, denom, j);
+        if (j < n_rep) {
+            if (own_o != nullptr) {
+#pragma unroll
+                for (int e = 0; e < EPL; ++e) acc[j][e] = __fmaf_rn(own_o[j * HD + lane * EPL + e], wj, acc[j][e]);
+            }
+            store_attention<HD>(lane, rh0 + j, acc[j], dj, out, out_lo, err);
+        }
+    }
+}
+
+// MERGE: no merge kernel follows.  A warp that holds an item's whole suffix merges it with the prefix records from shared memory;
+// of the few warps that share an item (at most MERGE_CHUNKS) each leaves its record and the last one merges.  For batches with
+// enough items to occupy the warps with few chunks: with many chunks per item one warp's merge is a longer chain than the merge
+// kernel's (one warp per head, every record in flight).
+constexpr int MERGE_CHUNKS = 3;
+struct SuffixMerge {
+    int32_t* arrived;           // [rows capacity * Hkv]: warps that have left their record of an item; 0 between launches
+    __nv_bfloat16* out;
+    __nv_bfloat16* out_lo;
+};
+
+template <int HD, bool MERGE>
 __global__ void __launch_bounds__(S_WARPS * 32, 1)
 attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* __restrict__ sd, int64_t n_slots, int Hq, int Hkv,
-                   int layer, const __nv_bfloat16* __restrict__ q, RowGeom g, float scale_log2, PrefixPartial part, int32_t* err) {
+                   int layer, const __nv_bfloat16* __restrict__ q, RowGeom g, float scale_log2, PrefixPartial part, SuffixMerge mg, int32_t* err) {
     constexpr int KS = HD / 16;                   // k-steps of K Q^T
     constexpr int DT = HD / 16;                   // 16-dim m-tiles of O^T
     constexpr int TILE_BYTES = S_TP * HD * 2;
@@ -425,13 +557,15 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
     }
     __syncthreads();
 
+    if (!MERGE) grid_dep_launch_dependents();      // the merge may start when this grid's CTAs leave; it waits for all of them
+    bool waited = false;                   // the prefix records are there
     // work unit u = (item, chunk), item = (row, kv head); units of one item are consecutive, so they land on different warps
     const int max_slen = *g.max_slen;
-    const SuffixPlan sp = suffix_plan(max_slen, sd->n_rows * Hkv, part.n_suffix_warps);
+    const SuffixPlan sp = suffix_plan(max_slen, sd->n_rows * Hkv, part.n_suffix_warps, MERGE ? MERGE_CHUNKS : MAX_SUFFIX_CHUNKS);
     const int ct = sp.ct, cpi = sp.cpi;                                                            // tiles per chunk, unit slots per item
     const int n_items = sd->n_rows * Hkv * cpi;
     const int item_stride = gridDim.x * S_WARPS;
-    const int first_item = blockIdx.x * S_WARPS + warp;
+    const int first_item = warp * gridDim.x + blockIdx.x;          // few units: one per SM before a second one
     // tile range [t0, t1) of unit u for a row with n suffix slots; empty when the row has fewer chunks
     auto unit_range = [&](int u, int n, int& t0, int& t1) {
         const int ntiles = (n + S_TP - 1) / S_TP;
@@ -441,7 +575,7 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
 
     // producer cursor (tracked identically by every lane; lane 0 issues)
     int p_item = first_item, p_tile = 0, p_ntiles = 0;
-    int64_t p_krow = 0, p_vrow = 0;
+    int64_t p_krow = 0;
     auto p_load_item = [&]() {
         while (p_item < n_items) {
             const int it = p_item / cpi;
@@ -450,9 +584,7 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
             unit_range(p_item, g.s_len[row], t0, t1);
             if (t1 > t0) {
                 p_ntiles = t1;
-                const int64_t st = g.s_start[row];
-                p_krow = (((int64_t)layer * 2 + 0) * Hkv + kvh) * n_slots + st;
-                p_vrow = (((int64_t)layer * 2 + 1) * Hkv + kvh) * n_slots + st;
+                p_krow = ((int64_t)layer * 2 * Hkv + kvh) * n_slots + g.s_start[row];
                 p_tile = t0;
                 return;
             }
@@ -464,14 +596,9 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
     auto p_issue = [&]() {          // loads the producer cursor's tile into the next ring slot and advances the cursor
         const int stage = issued % S_STAGES;
         if (lane == 0) {
-            const uint32_t kb = tiles_u32 + stage * 2 * TILE_BYTES, vb = kb + TILE_BYTES;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             mbar_arrive_expect_tx(full0 + 8 * stage, 2 * TILE_BYTES);
-#pragma unroll
-            for (int b = 0; b < HD / 64; ++b) {
-                tma_load_2d(kb + b * (S_TP * 128), &kv_map, full0 + 8 * stage, b * 64, (int)(p_krow + (int64_t)p_tile * S_TP));
-                tma_load_2d(vb + b * (S_TP * 128), &kv_map, full0 + 8 * stage, b * 64, (int)(p_vrow + (int64_t)p_tile * S_TP));
-            }
+            tma_load_kv(tiles_u32 + stage * 2 * TILE_BYTES, &kv_map, full0 + 8 * stage, (int)(p_krow + (int64_t)p_tile * S_TP));
         }
         ++issued;
         if (++p_tile == p_ntiles) { p_item += item_stride; p_load_item(); }
@@ -521,33 +648,34 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
             if (!mbar_wait(full0 + 8 * stage, phase, &s_abort)) { ok = false; break; }
             const uint32_t kb = tiles_u32 + stage * 2 * TILE_BYTES, vb = kb + TILE_BYTES;
             const int valid = min(S_TP, n - tile * S_TP);
-            // S^T = K Q^T : positions on M (two 16-row tiles), heads on N
-            float s[2][4];
+            const int mat = lane >> 3;
+            // All fragments of the tile first: the loads are in flight together, and the ring slot is free again before any
+            // arithmetic.  (Interleaved, every MMA waits for its own ldmatrix.)
+            uint32_t ka[KS][4], va[DT][4];
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
-                s[mt][0] = s[mt][1] = s[mt][2] = s[mt][3] = 0.f;
-                if (mt * 16 < valid) {
-#pragma unroll
-                    for (int ks = 0; ks < KS; ++ks) {
-                        const int mat = lane >> 3;
-                        const int r = mt * 16 + (lane & 7) + ((mat & 1) << 3), d = ks * 16 + ((mat >> 1) << 3);
-                        uint32_t a0, a1, a2, a3;
-                        ldsm_x4(kb + tile_off<S_TP>(r, d), a0, a1, a2, a3);
-                        mma_f16(s[mt], a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
-                    }
-                }
+            for (int ks = 0; ks < KS; ++ks) {
+                const int r = (lane & 7) + ((mat & 1) << 3), d = ks * 16 + ((mat >> 1) << 3);
+                ldsm_x4(kb + tile_off<S_TP>(r, d), ka[ks][0], ka[ks][1], ka[ks][2], ka[ks][3]);
             }
-            // mask + per-head block max (a head's column is spread over the 8 lanes sharing lane % 4)
+#pragma unroll
+            for (int dt = 0; dt < DT; ++dt) {
+                const int r = (lane & 7) + ((mat >> 1) << 3), d = dt * 16 + ((mat & 1) << 3);
+                ldsm_x4_t(vb + tile_off<S_TP>(r, d), va[dt][0], va[dt][1], va[dt][2], va[dt][3]);
+            }
+            ++consumed;
+            __syncwarp();
+            if (p_item < n_items) p_issue();      // refill the slot just drained
+            // S^T = K Q^T : 16 positions on M, heads on N; two chains so that consecutive MMAs do not wait for one another
+            float s[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int ks = 0; ks < KS; ++ks) mma_f16((ks & 1) ? s2 : s, ka[ks][0], ka[ks][1], ka[ks][2], ka[ks][3], qb[ks][0], qb[ks][1]);
+            // mask + per-head tile max (a head's column is spread over the 8 lanes sharing lane % 4)
             float bmax[2] = {-INFINITY, -INFINITY};
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const int pos = mt * 16 + (lane >> 2) + ((c >> 1) << 3);
-                    const float v = pos < valid ? s[mt][c] * scale_log2 : -INFINITY;
-                    s[mt][c] = v;
-                    bmax[c & 1] = fmaxf(bmax[c & 1], v);
-                }
+            for (int c = 0; c < 4; ++c) {
+                const int pos = (lane >> 2) + ((c >> 1) << 3);
+                s[c] = pos < valid ? (s[c] + s2[c]) * scale_log2 : -INFINITY;
+                bmax[c & 1] = fmaxf(bmax[c & 1], s[c]);
             }
             float corr[2];
 #pragma unroll
@@ -555,43 +683,29 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
                 bmax[i] = fmaxf(bmax[i], __shfl_xor_sync(0xffffffffu, bmax[i], 4));
                 bmax[i] = fmaxf(bmax[i], __shfl_xor_sync(0xffffffffu, bmax[i], 8));
                 bmax[i] = fmaxf(bmax[i], __shfl_xor_sync(0xffffffffu, bmax[i], 16));
-                const float mnew = fmaxf(mh[i], bmax[i]);
-                corr[i] = exp2_safe(mh[i], mnew);
+                const float mnew = fmaxf(mh[i], bmax[i]);          // finite: a tile has a position
+                corr[i] = exp2f(mh[i] - mnew);
                 mh[i] = mnew;
                 lh[i] *= corr[i];
             }
 #pragma unroll
             for (int t = 0; t < DT; ++t) { o[t][0] *= corr[0]; o[t][1] *= corr[1]; o[t][2] *= corr[0]; o[t][3] *= corr[1]; }
-            // O^T += V^T P^T, 16 positions per k-step; P^T fragments come from S^T through movmatrix
+            // O^T += V^T P^T; P^T fragments come from S^T through movmatrix
+            float p[4];
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
-                if (mt * 16 >= valid) break;
-                float p[4];
+            for (int c = 0; c < 4; ++c) { p[c] = exp2f(s[c] - mh[c & 1]); lh[c & 1] += p[c]; }
+            const uint32_t b0 = movmatrix_t(pack_f16(p[0], p[1])), b1 = movmatrix_t(pack_f16(p[2], p[3]));
+            if (valid < S_TP) {
+                // slots past the rollout's last token may be uninitialised: zero them (0 * NaN = NaN).  After the transposing
+                // load a thread holds positions (lane%4)*2 + {0,1} in registers 0 and 1, + 8 in 2 and 3.
+                const int pp = (lane & 3) * 2;
+                const uint32_t m_lo = (pp < valid ? 0x0000ffffu : 0u) | (pp + 1 < valid ? 0xffff0000u : 0u);
+                const uint32_t m_hi = (pp + 8 < valid ? 0x0000ffffu : 0u) | (pp + 9 < valid ? 0xffff0000u : 0u);
 #pragma unroll
-                for (int c = 0; c < 4; ++c) { p[c] = exp2_safe(s[mt][c], mh[c & 1]); lh[c & 1] += p[c]; }
-                const uint32_t b0 = movmatrix_t(pack_f16(p[0], p[1]));
-                const uint32_t b1 = movmatrix_t(pack_f16(p[2], p[3]));
-                const bool ragged = mt * 16 + 16 > valid;              // warp-uniform
-#pragma unroll
-                for (int dt = 0; dt < DT; ++dt) {
-                    const int mat = lane >> 3;
-                    const int r = mt * 16 + (lane & 7) + ((mat >> 1) << 3), d = dt * 16 + ((mat & 1) << 3);
-                    uint32_t a0, a1, a2, a3;
-                    ldsm_x4_t(vb + tile_off<S_TP>(r, d), a0, a1, a2, a3);
-                    if (ragged) {
-                        // slots past the rollout's last token may be uninitialised: zero them (0 * NaN = NaN).
-                        // After the transposing load a thread holds positions mt*16 + (lane%4)*2 + {0,1} in a0/a1, + 8 in a2/a3.
-                        const int pp = mt * 16 + (lane & 3) * 2;
-                        const uint32_t m_lo = (pp < valid ? 0x0000ffffu : 0u) | (pp + 1 < valid ? 0xffff0000u : 0u);
-                        const uint32_t m_hi = (pp + 8 < valid ? 0x0000ffffu : 0u) | (pp + 9 < valid ? 0xffff0000u : 0u);
-                        a0 &= m_lo; a1 &= m_lo; a2 &= m_hi; a3 &= m_hi;
-                    }
-                    mma_f16(o[dt], a0, a1, a2, a3, b0, b1);
-                }
+                for (int dt = 0; dt < DT; ++dt) { va[dt][0] &= m_lo; va[dt][1] &= m_lo; va[dt][2] &= m_hi; va[dt][3] &= m_hi; }
             }
-            ++consumed;
-            __syncwarp();
-            if (p_item < n_items) p_issue();      // refill the slot just drained
+#pragma unroll
+            for (int dt = 0; dt < DT; ++dt) mma_f16(o[dt], va[dt][0], va[dt][1], va[dt][2], va[dt][3], b0, b1);
         }
         if (!ok) break;
 
@@ -616,15 +730,38 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
             obuf[(hh + 1) * HD + d + 8] = o[dt][3];
         }
         __syncwarp();
-        // leave this chunk as record number part.n_parts + chunk, next to the prefix records; attn_merge_kernel combines them
         constexpr int EPL = HD / 32;
-        const size_t base = (size_t)(part.n_parts + chunk) * part.stride + (size_t)row * Hq + (size_t)kvh * n_rep;
-        if (lane < n_rep) { part.m[base + lane] = s_ml[warp][lane]; part.l[base + lane] = s_ml[warp][8 + lane]; }
-        for (int j = 0; j < n_rep; ++j) {
-            float* dst = part.o + (base + j) * HD + lane * EPL;
-            const float* src = obuf + j * HD + lane * EPL;
-            if (EPL == 4) *reinterpret_cast<float4*>(dst) = *reinterpret_cast<const float4*>(src);
-            else *reinterpret_cast<float2*>(dst) = *reinterpret_cast<const float2*>(src);
+        const size_t rh0 = (size_t)row * Hq + (size_t)kvh * n_rep;
+        const int n_own = MERGE ? suffix_chunks(n, ct) : 0;
+        if (MERGE && !waited) {
+            grid_dep_wait();
+            grid_dep_launch_dependents();          // the output projection may request its weights once there is room for it
+            waited = true;
+        }
+        if (MERGE && n_own == 1) {
+            merge_heads_warp<HD>(lane, rh0, n_rep, part, part.n_parts, s_ml[warp], s_ml[warp] + 8, obuf, mg.out, mg.out_lo, err);
+        } else {
+            // leave this chunk as record number part.n_parts + chunk, next to the prefix records
+            const size_t base = (size_t)(part.n_parts + chunk) * part.stride + rh0;
+            if (lane < n_rep) { part.m[base + lane] = s_ml[warp][lane]; part.l[base + lane] = s_ml[warp][8 + lane]; }
+            for (int j = 0; j < n_rep; ++j) {
+                float* dst = part.o + (base + j) * HD + lane * EPL;
+                const float* src = obuf + j * HD + lane * EPL;
+                if (EPL == 4) *reinterpret_cast<float4*>(dst) = *reinterpret_cast<const float4*>(src);
+                else *reinterpret_cast<float2*>(dst) = *reinterpret_cast<const float2*>(src);
+            }
+            if (MERGE) {
+                __threadfence();                   // the record is visible before this warp counts as arrived
+                __syncwarp();
+                int last = 0;
+                if (lane == 0) {
+                    last = atomicAdd(mg.arrived + it, 1) == n_own - 1;
+                    if (last) mg.arrived[it] = 0;  // for the next layer
+                    __threadfence();
+                }
+                if (__shfl_sync(0xffffffffu, last, 0))
+                    merge_heads_warp<HD>(lane, rh0, n_rep, part, part.n_parts + n_own, nullptr, nullptr, nullptr, mg.out, mg.out_lo, err);
+            }
         }
         __syncwarp();
     }
@@ -639,7 +776,7 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
         for (int i = 0; i < 2000; ++i) __nanosleep(1000);
     }
     __syncthreads();
-    grid_dep_wait();          // decode steps start this kernel when the shared-prefix kernel's CTAs leave: that one ends first
+    if (!waited) grid_dep_wait();          // decode steps start this kernel when the shared-prefix kernel's CTAs leave: that one ends first
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -650,8 +787,7 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
 // rh = row * Hq + head (the caller keeps it below n_live * Hq).  ct = tiles per suffix chunk of this step (suffix_plan);
 // n_load > 0 = how many records to request: every record index the step can have produced (part.n_parts + chunk slots per
 // item), so that the loads do not wait for the row's suffix length; records past the row's own count are ignored.
-// STREAM: wait for the suffix length and request the row's own records only, one after the other (n_load is not used).
-template <int HD, bool STREAM = false>
+template <int HD>
 __device__ __forceinline__ void merge_item_warp(int lane, size_t rh, int Hq, const RowGeom& g, const PrefixPartial& part, int ct, int n_load,
                                                 __nv_bfloat16* __restrict__ out, __nv_bfloat16* __restrict__ out_lo, int32_t* err) {
     constexpr int EPL = HD / 32;
@@ -662,27 +798,6 @@ __device__ __forceinline__ void merge_item_warp(int lane, size_t rh, int Hq, con
 #pragma unroll
     for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
     float denom = 0.f;
-    if constexpr (STREAM) {
-        // Large batches: the row's own records only, streamed (few registers, so many warps are resident): first the
-        // largest m, then the weighted sums in index order -- the same operations in the same order as below.
-        const int n_own = part.n_parts + suffix_chunks(slen, ct);
-        for (int i = 0; i < n_own; ++i) M = fmaxf(M, part.m[(size_t)i * part.stride + rh]);
-#pragma unroll 2
-        for (int i = 0; i < n_own; ++i) {
-            const float w = exp2_safe(part.m[(size_t)i * part.stride + rh], M);
-            if (w > 0.f) {
-                denom += part.l[(size_t)i * part.stride + rh] * w;
-                const float* src = part.o + ((size_t)i * part.stride + rh) * HD + lane * EPL;
-                if (EPL == 4) {
-                    const float4 v = *reinterpret_cast<const float4*>(src);
-                    acc[0] += v.x * w; acc[1] += v.y * w; acc[2] += v.z * w; acc[3] += v.w * w;
-                } else {
-                    const float2 v = *reinterpret_cast<const float2*>(src);
-                    acc[0] += v.x * w; acc[1] += v.y * w;
-                }
-            }
-        }
-    } else {
     float mi[MAX_RECORDS], li[MAX_RECORDS];
     float ov[MAX_RECORDS][EPL];
 #pragma unroll
@@ -714,42 +829,20 @@ __device__ __forceinline__ void merge_item_warp(int lane, size_t rh, int Hq, con
             for (int e = 0; e < EPL; ++e) acc[e] += ov[i][e] * w;
         }
     }
-    }
-    const float inv = denom > 0.f ? 1.f / denom : 0.f;
-    float lo[EPL];
-#pragma unroll
-    for (int e = 0; e < EPL; ++e) {
-        acc[e] *= inv;
-        lo[e] = acc[e] - __bfloat162float(__float2bfloat16_rn(acc[e]));     // rounding remainder: second operand of the O projection
-    }
-    __nv_bfloat16* dst = out + rh * HD + lane * EPL;
-    if (out_lo == nullptr) {                 // the output projection takes IEEE half operands: no remainder needed
-        if (EPL == 4) *reinterpret_cast<uint2*>(dst) = make_uint2(pack_f16_guard(acc[0], acc[1], err), pack_f16_guard(acc[2], acc[3], err));
-        else *reinterpret_cast<uint32_t*>(dst) = pack_f16_guard(acc[0], acc[1], err);
-        return;
-    }
-    __nv_bfloat16* dst_lo = out_lo + rh * HD + lane * EPL;
-    if (EPL == 4) {
-        *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]));
-        *reinterpret_cast<uint2*>(dst_lo) = make_uint2(pack_bf16(lo[0], lo[1]), pack_bf16(lo[2], lo[3]));
-    } else {
-        *reinterpret_cast<uint32_t*>(dst) = pack_bf16(acc[0], acc[1]);
-        *reinterpret_cast<uint32_t*>(dst_lo) = pack_bf16(lo[0], lo[1]);
-    }
+    store_attention<HD>(lane, rh, acc, denom, out, out_lo, err);
 }
 
 // Stand-alone form: the grid covers the row bound of the step.
-template <int HD, bool STREAM>
+template <int HD>
 __global__ void __launch_bounds__(256) attn_merge_kernel(const StepDesc* __restrict__ sd, int Hq, RowGeom g, PrefixPartial part,
                                                          __nv_bfloat16* __restrict__ out, __nv_bfloat16* __restrict__ out_lo, int32_t* err) {
     const size_t rh = (size_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    grid_dep_wait();                       // the suffix records, and with them the prefix records: that kernel waits for its own
     grid_dep_launch_dependents();          // the output projection may set itself up and request its first weight tiles
     const int n_live = sd->n_rows;
     if (rh >= (size_t)n_live * Hq) return;
     const SuffixPlan sp = suffix_plan(*g.max_slen, n_live * part.n_kv_heads, part.n_suffix_warps);
-    // few items (host: STREAM = false): request every record slot of the step at once (latency); many items: only the row's
-    // own records, with few registers (occupancy)
-    merge_item_warp<HD, STREAM>(threadIdx.x & 31, rh, Hq, g, part, sp.ct, part.n_parts + sp.cpi, out, out_lo, err);
+    merge_item_warp<HD>(threadIdx.x & 31, rh, Hq, g, part, sp.ct, part.n_parts + sp.cpi, out, out_lo, err);
 }
 
 }  // namespace am

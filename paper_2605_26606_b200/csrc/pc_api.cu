@@ -84,7 +84,7 @@ constexpr int kMaxSplits = pc::PARTIALS_MAX;
 
 struct Carve {
     size_t h, a, qkv, q, attn, act, logits, rope, pos, wslot, warena, p_start, p_len, s_start, s_len, token, last_row,
-        part_m, part_l, part_o, res_part, step_desc, step_counter, max_slen, sample_scratch, a_lo, attn_lo, chain_layers, chain_glob,
+        part_m, part_l, part_o, arrived, res_part, step_desc, step_counter, max_slen, sample_scratch, a_lo, attn_lo, chain_layers, chain_glob,
         chain_bar, dargs, key_prompt, key_rollout, key_step, out_index, group_start, sample_tiles, sample_bound, ssq, total;
 };
 
@@ -241,6 +241,7 @@ Carve carve(const pc_ctx* c, int max_rows, int max_prefill) {
     v.part_m = take(pc::am::MAX_RECORDS * R * d.n_q_heads * 4);
     v.part_l = take(pc::am::MAX_RECORDS * R * d.n_q_heads * 4);
     v.part_o = take(pc::am::MAX_RECORDS * R * d.n_q_heads * d.head_dim * 4);
+    v.arrived = take(R * d.n_kv_heads * 4);
     v.total = off;
     return v;
 }
@@ -480,7 +481,7 @@ int arena_maps(pc_ctx* c, const void* prompt_kv, int64_t prompt_slots, const voi
     }
     if (suffix_kv != nullptr && (suffix_kv != c->suffix_arena_ptr || suffix_slots != c->suffix_arena_slots)) {
         if (planes * (uint64_t)suffix_slots >= (1ull << 31)) return PC_ERR_CAPACITY;
-        if (!pc::make_bf16_map(&c->map_suffix_kv, suffix_kv, planes * suffix_slots, d.head_dim, pc::am::S_TP)) {
+        if (!pc::make_kv_tile_map(&c->map_suffix_kv, suffix_kv, planes, suffix_slots, d.n_kv_heads, d.head_dim, pc::am::S_TP)) {
             g_cuda_error = "cuTensorMapEncodeTiled failed for the suffix KV arena";
             return PC_ERR_CUDA;
         }
@@ -503,7 +504,9 @@ cudaError_t configure_attention() {
             e = cudaFuncSetAttribute(am::attn_group_kernel<HD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::group_smem_bytes<HD>());
     }
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(am::attn_suffix_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::suffix_smem_bytes<HD>());
+        e = cudaFuncSetAttribute(am::attn_suffix_kernel<HD, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::suffix_smem_bytes<HD>());
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(am::attn_suffix_kernel<HD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::suffix_smem_bytes<HD>());
     return e;
 }
 template <class Epi>
@@ -586,12 +589,13 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
     // a group with few query rows keeps few CTAs busy: cut its prompt into ranges so that about one CTA per SM runs
     const int q_tiles = (plan.max_group_rows * n_rep + prefix_q_rows(HD) - 1) / prefix_q_rows(HD);
     const int base_ctas = std::max(1, q_tiles * d.n_kv_heads * plan.n_groups);
-    // (two of these CTAs fit on an SM)
-    const int n_parts = plan.prefill ? 1 : std::max(1, std::min(am::MAX_PREFIX_PARTS, 2 * c->num_sms / base_ctas));
+    const bool overlap = !plan.prefill && c->attn_overlap != 0 && c->prof_active_layer < 0;
+    // batches whose items occupy the suffix kernel's warps with few chunks each: it merges by itself
+    const bool merge_inside = part_out == nullptr && !overlap && (long long)M * d.n_kv_heads * am::MERGE_CHUNKS >= (long long)c->num_sms * am::S_WARPS;
+    const int n_parts = plan.prefill ? 1 : std::max(1, std::min(merge_inside ? am::MAX_MERGED_PARTS : am::MAX_PREFIX_PARTS, c->num_sms / base_ctas));
     // the suffix kernel takes one warp per (rollout, KV head, range of the suffix); how the suffixes are cut into ranges
     // is decided on the device for the warps of this grid (the longest suffix of the step is only known there)
-    const int items = M * d.n_kv_heads * am::MAX_SUFFIX_CHUNKS;
-    const int sgrid = std::min(c->num_sms, (items + am::S_WARPS - 1) / am::S_WARPS);
+    const int sgrid = std::min(c->num_sms, M * d.n_kv_heads * am::MAX_SUFFIX_CHUNKS);      // units go round the CTAs first
     am::PrefixPartial part{reinterpret_cast<float*>(c->ws + c->cv.part_m), reinterpret_cast<float*>(c->ws + c->cv.part_l),
                            reinterpret_cast<float*>(c->ws + c->cv.part_o), n_parts, (size_t)std::max(c->max_rows, 1) * d.n_q_heads,
                            d.n_kv_heads, sgrid * am::S_WARPS};
@@ -610,7 +614,6 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
     }
     // The two kernels are independent (both read q, each leaves its own records), so outside profiled steps they are issued
     // on two streams -- a fork and a join inside the captured step -- and share the GPU.
-    const bool overlap = c->attn_overlap != 0 && c->prof_active_layer < 0;
     cudaStream_t gst = st;
     if (overlap) {
         if (c->side_stream == nullptr) {
@@ -636,8 +639,13 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
             attn, attn_lo, c->err);
     if (overlap) cudaEventRecord(c->ev_join, gst);
     c->mark(st, layer, PC_MARK_GROUP);
-    launch_k_dep(group_dep, am::attn_suffix_kernel<HD>, dim3(sgrid), dim3(am::S_WARPS * 32), am::suffix_smem_bytes<HD>(), st,
-        c->map_suffix_kv, sd, suffix_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, g, scale_log2, part, c->err);
+    const am::SuffixMerge mg{reinterpret_cast<int32_t*>(c->ws + c->cv.arrived), attn, attn_lo};
+    if (merge_inside)
+        launch_k_dep(group_dep, am::attn_suffix_kernel<HD, true>, dim3(sgrid), dim3(am::S_WARPS * 32), am::suffix_smem_bytes<HD>(), st,
+            c->map_suffix_kv, sd, suffix_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, g, scale_log2, part, mg, c->err);
+    else
+        launch_k_dep(group_dep, am::attn_suffix_kernel<HD, false>, dim3(sgrid), dim3(am::S_WARPS * 32), am::suffix_smem_bytes<HD>(), st,
+            c->map_suffix_kv, sd, suffix_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, g, scale_log2, part, mg, c->err);
     if (overlap) cudaStreamWaitEvent(st, c->ev_join, 0);
     c->mark(st, layer, PC_MARK_SUFFIX);
     if (part_out != nullptr) {
@@ -645,10 +653,12 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
         count_launches(2);
         return PC_OK;
     }
-    if ((long long)M * d.n_q_heads > 8192)
-        launch_k(am::attn_merge_kernel<HD, true>, dim3((M * d.n_q_heads + 7) / 8), dim3(256), 0, st, sd, d.n_q_heads, g, part, attn, attn_lo, c->err);
-    else
-        launch_k(am::attn_merge_kernel<HD, false>, dim3((M * d.n_q_heads + 7) / 8), dim3(256), 0, st, sd, d.n_q_heads, g, part, attn, attn_lo, c->err);
+    if (merge_inside) {
+        c->mark(st, layer, PC_MARK_MERGE);
+        count_launches(2);
+        return PC_OK;
+    }
+    launch_k(am::attn_merge_kernel<HD>, dim3((M * d.n_q_heads + 7) / 8), dim3(256), 0, st, sd, d.n_q_heads, g, part, attn, attn_lo, c->err);
     c->mark(st, layer, PC_MARK_MERGE);
     count_launches(3);
     return PC_OK;
@@ -1303,12 +1313,12 @@ pc::RowKeys row_keys(const pc_ctx* c) {
 }
 
 // Upper bounds of a step's group geometry, rounded up to classes so that steps of similar shape share a captured graph
-// and a step-by-step call picks the same attention plan as a captured one: the number of groups to the next power of
-// two, the largest group to the most rows that need the same number of query tiles (neither beyond the row bound).
+// and a step-by-step call picks the same attention plan as a captured one: the number of groups to the next eighth of a power of
+// two (how often a group's prompt is cut depends on it), the largest group to the most rows that need the same number of query tiles (neither beyond the row bound).
 void canonical_group_bounds(const pc_ctx* c, int n_groups, int max_group_rows, int row_bound, int* groups_bound, int* group_rows_bound) {
-    int gb = 1;
-    while (gb < n_groups) gb <<= 1;
-    *groups_bound = std::min(gb, std::max(row_bound, 1));
+    int unit = 1;
+    while (unit * 16 <= n_groups) unit <<= 1;
+    *groups_bound = std::min((n_groups + unit - 1) / unit * unit, std::max(row_bound, 1));
     const int n_rep = c->d.n_q_heads / c->d.n_kv_heads;
     const int q_rows = prefix_q_rows(c->d.head_dim), q_tiles = (std::max(max_group_rows, 1) * n_rep + q_rows - 1) / q_rows;
     *group_rows_bound = std::min(q_tiles * q_rows / n_rep, std::max(row_bound, 1));
@@ -1450,7 +1460,8 @@ int decode_launches(pc_ctx* ctx, cudaStream_t st, int m_bound, int groups_bound,
     ctx->prof_active_layer = -1;
     if (cap == cudaStreamCaptureStatusNone && ctx->prof_layer >= 0) { ctx->prof_active_layer = ctx->prof_layer; ctx->prof_layer = -1; }
     struct Disarm { pc_ctx* c; ~Disarm() { c->prof_active_layer = -1; } } disarm{ctx};
-    launch_k(pc::prep_decode_rows, dim3((m_bound + 128) / 128), dim3(128), 0, st, sd, da, a.prompt_slots, a.suffix_slots, ctx->d.vocab, g, keys, ctx->err);
+    launch_k(pc::prep_decode_rows, dim3((m_bound + 128) / 128), dim3(128), 0, st, sd, da, a.prompt_slots, a.suffix_slots, ctx->d.vocab, g, keys,
+             reinterpret_cast<int32_t*>(ctx->ws + ctx->cv.arrived), ctx->d.n_kv_heads, ctx->err);
     count_launches(1);
     PC_CUDA_CHECK_LAUNCH("prep_decode_rows");
     const pc::KvArena pa{const_cast<void*>(a.prompt_kv), a.prompt_slots}, sa{a.suffix_kv, a.suffix_slots};
