@@ -226,10 +226,8 @@ PC_API int pc_set_dependent_launch(pc_ctx* ctx, int mask);
  * buffer.  Drops captured steps. */
 PC_API int pc_set_fused_sampler(pc_ctx* ctx, int on);
 
-/* bf16 models, decode steps: 1 issues the shared-prefix attention kernel and the per-rollout suffix attention
- * kernel of a layer on two streams (the second one is created by the context on first use and released by pc_destroy), so
- * that they can overlap; 0 (the default: measured no faster, both kernels fill the SMs) issues them one after the other.
- * Results are identical.  Drops captured decode steps. */
+/* Accepted for callers that set it; it changes nothing.  The shared-prefix attention kernel and the per-rollout suffix attention
+ * kernel of a decode step run side by side by themselves (the second is launched as a programmatic dependent of the first). */
 PC_API int pc_set_attention_overlap(pc_ctx* ctx, int on);
 
 /* How the decode steps of a bf16 model with half_gemm = 1 are issued.  mode 1: everything between two

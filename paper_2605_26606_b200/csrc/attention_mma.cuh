@@ -16,8 +16,6 @@
 //                       O^T = V^T P^T), so the 6-8 query heads fill the N = 8 axis and no MMA work is
 //                       padded; P is transposed between the two MMAs with movmatrix.  It leaves its
 //                       (m, l, unnormalised O) record next to the prefix records.
-//   attn_merge_kernel   combines the prefix records and the suffix record of every (row, head) by their
-//                       log-sum-exp and writes the bf16 attention output.
 //
 // Scores are kept in the log2 domain (scaled by log2(e) / sqrt(head_dim)) so that exp2f is the only
 // transcendental.  Waits on mbarriers are bounded (see gemm_tc.cuh).
@@ -108,8 +106,9 @@ struct PrefixPartial {
     int n_suffix_warps;     // warps of the suffix kernel's grid: how suffixes are cut into ranges is planned for this many
 };
 constexpr int MAX_PREFIX_PARTS = 8, MAX_MERGED_PARTS = 4;      // (the second where the suffix kernel merges)
-constexpr int MAX_SUFFIX_CHUNKS = 12;
-constexpr int MAX_RECORDS = MAX_PREFIX_PARTS + MAX_SUFFIX_CHUNKS, MAX_MERGED_RECORDS = MAX_MERGED_PARTS + 3;
+constexpr int MERGE_CHUNKS = 3;
+constexpr int MAX_MERGED_RECORDS = MAX_MERGED_PARTS + MERGE_CHUNKS;
+constexpr int MAX_RECORDS = MAX_PREFIX_PARTS > MAX_MERGED_RECORDS ? MAX_PREFIX_PARTS : MAX_MERGED_RECORDS;
 
 // ---------------------------------------------------------------------------------------------
 // Group (shared-prefix / causal-prefill) kernel
@@ -387,16 +386,16 @@ template <int HD> constexpr int suffix_smem_bytes() {
 // With few rollouts there are about as many (rollout, KV head) streams as warps on the GPU, and one stream more than
 // warps doubles the kernel's time.  The suffix of a rollout is therefore cut into ranges of tiles ("chunks") that
 // are spread over the warps; every chunk leaves its own record.  Tiles per chunk (ct) and chunk slots per (row, KV
-// head) item (cpi) for a step whose longest suffix has max_slen slots: among 1..MAX_SUFFIX_CHUNKS chunks per item, the
+// head) item (cpi) for a step whose longest suffix has max_slen slots: among 1..MERGE_CHUNKS chunks per item, the
 // choice that minimises (units the busiest warp gets) x (tiles per unit + 4), the + 4 standing for the fixed cost of a
 // unit (length lookup, first TMA round trip, record) in tile times.  The same value serves every row of the step, and
 // the merge kernel recomputes it from the same inputs.
 struct SuffixPlan { int ct, cpi; };
-__device__ __forceinline__ SuffixPlan suffix_plan(int max_slen, int n_items, int n_warps, int max_chunks = MAX_SUFFIX_CHUNKS) {
+__device__ __forceinline__ SuffixPlan suffix_plan(int max_slen, int n_items, int n_warps) {
     const int ntiles = max(1, (max_slen + S_TP - 1) / S_TP);
     SuffixPlan best{ntiles, 1};
     long long best_cost = -1;
-    for (int c = 1; c <= max_chunks; ++c) {
+    for (int c = 1; c <= MERGE_CHUNKS; ++c) {
         const int ct = (ntiles + c - 1) / c;
         const int cc = (ntiles + ct - 1) / ct;
         const long long cost = (long long)((n_items * cc + n_warps - 1) / max(n_warps, 1)) * (ct + 4);
@@ -407,6 +406,95 @@ __device__ __forceinline__ SuffixPlan suffix_plan(int max_slen, int n_items, int
 __device__ __forceinline__ int suffix_chunks(int n, int ct) {             // records a row with n suffix slots leaves
     const int ntiles = (n + S_TP - 1) / S_TP;
     return (ntiles + ct - 1) / ct;
+}
+
+// One tile of 16 positions: K fragments against the heads' queries, online softmax, V.  loaded() is called once the tile is in
+// registers (its ring slot is free).
+template <int HD, class Loaded>
+__device__ __forceinline__ void suffix_tile(uint32_t kb, uint32_t vb, int lane, int valid, float scale_log2, const uint32_t (&qb)[HD / 16][2],
+                                            float (&o)[HD / 16][4], float (&mh)[2], float (&lh)[2], Loaded loaded) {
+    constexpr int KS = HD / 16, DT = HD / 16;
+    const int mat = lane >> 3;
+    // All fragments of the tile first: the loads are in flight together, and the ring slot is free again before any
+    // arithmetic.  (Interleaved, every MMA waits for its own ldmatrix.)
+    uint32_t ka[KS][4], va[DT][4];
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks) {
+        const int r = (lane & 7) + ((mat & 1) << 3), d = ks * 16 + ((mat >> 1) << 3);
+        ldsm_x4(kb + tile_off<S_TP>(r, d), ka[ks][0], ka[ks][1], ka[ks][2], ka[ks][3]);
+    }
+#pragma unroll
+    for (int dt = 0; dt < DT; ++dt) {
+        const int r = (lane & 7) + ((mat >> 1) << 3), d = dt * 16 + ((mat & 1) << 3);
+        ldsm_x4_t(vb + tile_off<S_TP>(r, d), va[dt][0], va[dt][1], va[dt][2], va[dt][3]);
+    }
+    loaded();
+    // S^T = K Q^T : 16 positions on M, heads on N; two chains so that consecutive MMAs do not wait for one another
+    float s[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks) mma_f16((ks & 1) ? s2 : s, ka[ks][0], ka[ks][1], ka[ks][2], ka[ks][3], qb[ks][0], qb[ks][1]);
+    // mask + per-head tile max (a head's column is spread over the 8 lanes sharing lane % 4)
+    float bmax[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const int pos = (lane >> 2) + ((c >> 1) << 3);
+        s[c] = pos < valid ? (s[c] + s2[c]) * scale_log2 : -INFINITY;
+        bmax[c & 1] = fmaxf(bmax[c & 1], s[c]);
+    }
+    float corr[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        bmax[i] = fmaxf(bmax[i], __shfl_xor_sync(0xffffffffu, bmax[i], 4));
+        bmax[i] = fmaxf(bmax[i], __shfl_xor_sync(0xffffffffu, bmax[i], 8));
+        bmax[i] = fmaxf(bmax[i], __shfl_xor_sync(0xffffffffu, bmax[i], 16));
+        const float mnew = fmaxf(mh[i], bmax[i]);          // finite: a tile has a position
+        corr[i] = exp2f(mh[i] - mnew);
+        mh[i] = mnew;
+        lh[i] *= corr[i];
+    }
+#pragma unroll
+    for (int t = 0; t < DT; ++t) { o[t][0] *= corr[0]; o[t][1] *= corr[1]; o[t][2] *= corr[0]; o[t][3] *= corr[1]; }
+    // O^T += V^T P^T; P^T fragments come from S^T through movmatrix
+    float p[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) { p[c] = exp2f(s[c] - mh[c & 1]); lh[c & 1] += p[c]; }
+    const uint32_t b0 = movmatrix_t(pack_f16(p[0], p[1])), b1 = movmatrix_t(pack_f16(p[2], p[3]));
+    if (valid < S_TP) {
+        // slots past the rollout's last token may be uninitialised: zero them (0 * NaN = NaN).  After the transposing
+        // load a thread holds positions (lane%4)*2 + {0,1} in registers 0 and 1, + 8 in 2 and 3.
+        const int pp = (lane & 3) * 2;
+        const uint32_t m_lo = (pp < valid ? 0x0000ffffu : 0u) | (pp + 1 < valid ? 0xffff0000u : 0u);
+        const uint32_t m_hi = (pp + 8 < valid ? 0x0000ffffu : 0u) | (pp + 9 < valid ? 0xffff0000u : 0u);
+#pragma unroll
+        for (int dt = 0; dt < DT; ++dt) { va[dt][0] &= m_lo; va[dt][1] &= m_lo; va[dt][2] &= m_hi; va[dt][3] &= m_hi; }
+    }
+#pragma unroll
+    for (int dt = 0; dt < DT; ++dt) mma_f16(o[dt], va[dt][0], va[dt][1], va[dt][2], va[dt][3], b0, b1);
+}
+// A warp's share of an item: m8 / l8 [8 heads], obuf [8 heads][HD] unnormalised.
+template <int HD>
+__device__ __forceinline__ void suffix_finish(int lane, const float (&o)[HD / 16][4], const float (&mh)[2], float (&lh)[2], float* m8, float* l8, float* obuf) {
+    constexpr int DT = HD / 16;
+    // reduce the per-thread partial sums of each head over the 8 lanes sharing lane % 4
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        lh[i] += __shfl_xor_sync(0xffffffffu, lh[i], 4);
+        lh[i] += __shfl_xor_sync(0xffffffffu, lh[i], 8);
+        lh[i] += __shfl_xor_sync(0xffffffffu, lh[i], 16);
+    }
+    if (lane < 4) {
+        m8[lane * 2] = mh[0]; m8[lane * 2 + 1] = mh[1];
+        l8[lane * 2] = lh[0]; l8[lane * 2 + 1] = lh[1];
+    }
+    // O^T fragment (dims dt*16 + lane/4 (+8), heads (lane%4)*2 + {0,1}) -> obuf[head][dim]
+#pragma unroll
+    for (int dt = 0; dt < DT; ++dt) {
+        const int d = dt * 16 + (lane >> 2), hh = (lane & 3) * 2;
+        obuf[hh * HD + d] = o[dt][0];
+        obuf[(hh + 1) * HD + d] = o[dt][1];
+        obuf[hh * HD + d + 8] = o[dt][2];
+        obuf[(hh + 1) * HD + d + 8] = o[dt][3];
+    }
 }
 
 // Normalises and stores one (row, query head): IEEE half, or bf16 with its rounding remainder (second operand of the O projection).
@@ -519,18 +607,16 @@ __device__ __forceinline__ void merge_heads_warp(int lane, size_t rh0, int n_rep
     }
 }
 
-// MERGE: no merge kernel follows.  A warp that holds an item's whole suffix merges it with the prefix records from shared memory;
-// of the few warps that share an item (at most MERGE_CHUNKS) each leaves its record and the last one merges.  For batches with
-// enough items to occupy the warps with few chunks: with many chunks per item one warp's merge is a longer chain than the merge
-// kernel's (one warp per head, every record in flight).
-constexpr int MERGE_CHUNKS = 3;
+// A warp that holds an item's whole suffix merges it with the prefix records from shared memory; of the few warps that share an
+// item (at most MERGE_CHUNKS) each leaves its record and the last one merges.  For batches with enough items to occupy the warps
+// that way; smaller ones take attn_suffix_team_kernel.
 struct SuffixMerge {
     int32_t* arrived;           // [rows capacity * Hkv]: warps that have left their record of an item; 0 between launches
     __nv_bfloat16* out;
     __nv_bfloat16* out_lo;
 };
 
-template <int HD, bool MERGE>
+template <int HD>
 __global__ void __launch_bounds__(S_WARPS * 32, 1)
 attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* __restrict__ sd, int64_t n_slots, int Hq, int Hkv,
                    int layer, const __nv_bfloat16* __restrict__ q, RowGeom g, float scale_log2, PrefixPartial part, SuffixMerge mg, int32_t* err) {
@@ -557,11 +643,10 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
     }
     __syncthreads();
 
-    if (!MERGE) grid_dep_launch_dependents();      // the merge may start when this grid's CTAs leave; it waits for all of them
     bool waited = false;                   // the prefix records are there
     // work unit u = (item, chunk), item = (row, kv head); units of one item are consecutive, so they land on different warps
     const int max_slen = *g.max_slen;
-    const SuffixPlan sp = suffix_plan(max_slen, sd->n_rows * Hkv, part.n_suffix_warps, MERGE ? MERGE_CHUNKS : MAX_SUFFIX_CHUNKS);
+    const SuffixPlan sp = suffix_plan(max_slen, sd->n_rows * Hkv, part.n_suffix_warps);
     const int ct = sp.ct, cpi = sp.cpi;                                                            // tiles per chunk, unit slots per item
     const int n_items = sd->n_rows * Hkv * cpi;
     const int item_stride = gridDim.x * S_WARPS;
@@ -647,98 +732,25 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
             const uint32_t phase = (uint32_t)(consumed / S_STAGES) & 1u;
             if (!mbar_wait(full0 + 8 * stage, phase, &s_abort)) { ok = false; break; }
             const uint32_t kb = tiles_u32 + stage * 2 * TILE_BYTES, vb = kb + TILE_BYTES;
-            const int valid = min(S_TP, n - tile * S_TP);
-            const int mat = lane >> 3;
-            // All fragments of the tile first: the loads are in flight together, and the ring slot is free again before any
-            // arithmetic.  (Interleaved, every MMA waits for its own ldmatrix.)
-            uint32_t ka[KS][4], va[DT][4];
-#pragma unroll
-            for (int ks = 0; ks < KS; ++ks) {
-                const int r = (lane & 7) + ((mat & 1) << 3), d = ks * 16 + ((mat >> 1) << 3);
-                ldsm_x4(kb + tile_off<S_TP>(r, d), ka[ks][0], ka[ks][1], ka[ks][2], ka[ks][3]);
-            }
-#pragma unroll
-            for (int dt = 0; dt < DT; ++dt) {
-                const int r = (lane & 7) + ((mat >> 1) << 3), d = dt * 16 + ((mat & 1) << 3);
-                ldsm_x4_t(vb + tile_off<S_TP>(r, d), va[dt][0], va[dt][1], va[dt][2], va[dt][3]);
-            }
-            ++consumed;
-            __syncwarp();
-            if (p_item < n_items) p_issue();      // refill the slot just drained
-            // S^T = K Q^T : 16 positions on M, heads on N; two chains so that consecutive MMAs do not wait for one another
-            float s[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int ks = 0; ks < KS; ++ks) mma_f16((ks & 1) ? s2 : s, ka[ks][0], ka[ks][1], ka[ks][2], ka[ks][3], qb[ks][0], qb[ks][1]);
-            // mask + per-head tile max (a head's column is spread over the 8 lanes sharing lane % 4)
-            float bmax[2] = {-INFINITY, -INFINITY};
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int pos = (lane >> 2) + ((c >> 1) << 3);
-                s[c] = pos < valid ? (s[c] + s2[c]) * scale_log2 : -INFINITY;
-                bmax[c & 1] = fmaxf(bmax[c & 1], s[c]);
-            }
-            float corr[2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                bmax[i] = fmaxf(bmax[i], __shfl_xor_sync(0xffffffffu, bmax[i], 4));
-                bmax[i] = fmaxf(bmax[i], __shfl_xor_sync(0xffffffffu, bmax[i], 8));
-                bmax[i] = fmaxf(bmax[i], __shfl_xor_sync(0xffffffffu, bmax[i], 16));
-                const float mnew = fmaxf(mh[i], bmax[i]);          // finite: a tile has a position
-                corr[i] = exp2f(mh[i] - mnew);
-                mh[i] = mnew;
-                lh[i] *= corr[i];
-            }
-#pragma unroll
-            for (int t = 0; t < DT; ++t) { o[t][0] *= corr[0]; o[t][1] *= corr[1]; o[t][2] *= corr[0]; o[t][3] *= corr[1]; }
-            // O^T += V^T P^T; P^T fragments come from S^T through movmatrix
-            float p[4];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) { p[c] = exp2f(s[c] - mh[c & 1]); lh[c & 1] += p[c]; }
-            const uint32_t b0 = movmatrix_t(pack_f16(p[0], p[1])), b1 = movmatrix_t(pack_f16(p[2], p[3]));
-            if (valid < S_TP) {
-                // slots past the rollout's last token may be uninitialised: zero them (0 * NaN = NaN).  After the transposing
-                // load a thread holds positions (lane%4)*2 + {0,1} in registers 0 and 1, + 8 in 2 and 3.
-                const int pp = (lane & 3) * 2;
-                const uint32_t m_lo = (pp < valid ? 0x0000ffffu : 0u) | (pp + 1 < valid ? 0xffff0000u : 0u);
-                const uint32_t m_hi = (pp + 8 < valid ? 0x0000ffffu : 0u) | (pp + 9 < valid ? 0xffff0000u : 0u);
-#pragma unroll
-                for (int dt = 0; dt < DT; ++dt) { va[dt][0] &= m_lo; va[dt][1] &= m_lo; va[dt][2] &= m_hi; va[dt][3] &= m_hi; }
-            }
-#pragma unroll
-            for (int dt = 0; dt < DT; ++dt) mma_f16(o[dt], va[dt][0], va[dt][1], va[dt][2], va[dt][3], b0, b1);
+            suffix_tile<HD>(kb, vb, lane, min(S_TP, n - tile * S_TP), scale_log2, qb, o, mh, lh, [&]() {
+                ++consumed;
+                __syncwarp();
+                if (p_item < n_items) p_issue();      // refill the slot just drained
+            });
         }
         if (!ok) break;
 
-        // reduce the per-thread partial sums of each head over the 8 lanes sharing lane % 4
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            lh[i] += __shfl_xor_sync(0xffffffffu, lh[i], 4);
-            lh[i] += __shfl_xor_sync(0xffffffffu, lh[i], 8);
-            lh[i] += __shfl_xor_sync(0xffffffffu, lh[i], 16);
-        }
-        if (lane < 4) {
-            s_ml[warp][lane * 2] = mh[0]; s_ml[warp][lane * 2 + 1] = mh[1];
-            s_ml[warp][8 + lane * 2] = lh[0]; s_ml[warp][8 + lane * 2 + 1] = lh[1];
-        }
-        // O^T fragment (dims dt*16 + lane/4 (+8), heads (lane%4)*2 + {0,1}) -> obuf[head][dim]
-#pragma unroll
-        for (int dt = 0; dt < DT; ++dt) {
-            const int d = dt * 16 + (lane >> 2), hh = (lane & 3) * 2;
-            obuf[hh * HD + d] = o[dt][0];
-            obuf[(hh + 1) * HD + d] = o[dt][1];
-            obuf[hh * HD + d + 8] = o[dt][2];
-            obuf[(hh + 1) * HD + d + 8] = o[dt][3];
-        }
+        suffix_finish<HD>(lane, o, mh, lh, s_ml[warp], s_ml[warp] + 8, obuf);
         __syncwarp();
         constexpr int EPL = HD / 32;
         const size_t rh0 = (size_t)row * Hq + (size_t)kvh * n_rep;
-        const int n_own = MERGE ? suffix_chunks(n, ct) : 0;
-        if (MERGE && !waited) {
+        const int n_own = suffix_chunks(n, ct);
+        if (!waited) {
             grid_dep_wait();
             grid_dep_launch_dependents();          // the output projection may request its weights once there is room for it
             waited = true;
         }
-        if (MERGE && n_own == 1) {
+        if (n_own == 1) {
             merge_heads_warp<HD>(lane, rh0, n_rep, part, part.n_parts, s_ml[warp], s_ml[warp] + 8, obuf, mg.out, mg.out_lo, err);
         } else {
             // leave this chunk as record number part.n_parts + chunk, next to the prefix records
@@ -750,18 +762,16 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
                 if (EPL == 4) *reinterpret_cast<float4*>(dst) = *reinterpret_cast<const float4*>(src);
                 else *reinterpret_cast<float2*>(dst) = *reinterpret_cast<const float2*>(src);
             }
-            if (MERGE) {
-                __threadfence();                   // the record is visible before this warp counts as arrived
-                __syncwarp();
-                int last = 0;
-                if (lane == 0) {
-                    last = atomicAdd(mg.arrived + it, 1) == n_own - 1;
-                    if (last) mg.arrived[it] = 0;  // for the next layer
-                    __threadfence();
-                }
-                if (__shfl_sync(0xffffffffu, last, 0))
-                    merge_heads_warp<HD>(lane, rh0, n_rep, part, part.n_parts + n_own, nullptr, nullptr, nullptr, mg.out, mg.out_lo, err);
+            __threadfence();                   // the record is visible before this warp counts as arrived
+            __syncwarp();
+            int last = 0;
+            if (lane == 0) {
+                last = atomicAdd(mg.arrived + it, 1) == n_own - 1;
+                if (last) mg.arrived[it] = 0;  // for the next layer
+                __threadfence();
             }
+            if (__shfl_sync(0xffffffffu, last, 0))
+                merge_heads_warp<HD>(lane, rh0, n_rep, part, part.n_parts + n_own, nullptr, nullptr, nullptr, mg.out, mg.out_lo, err);
         }
         __syncwarp();
     }
@@ -777,72 +787,6 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
     }
     __syncthreads();
     if (!waited) grid_dep_wait();          // decode steps start this kernel when the shared-prefix kernel's CTAs leave: that one ends first
-}
-
-// ---------------------------------------------------------------------------------------------
-// Merge of the prefix records 0 .. n_parts-1 and the suffix record n_parts of every (row, query head) by their
-// log-sum-exp:  M = max m_i,  out = sum_i O_i 2^(m_i - M) / sum_i l_i 2^(m_i - M).  Records are added in index order.
-// One warp per (row, head); a lane owns HD/32 consecutive dims.
-// ---------------------------------------------------------------------------------------------
-// rh = row * Hq + head (the caller keeps it below n_live * Hq).  ct = tiles per suffix chunk of this step (suffix_plan);
-// n_load > 0 = how many records to request: every record index the step can have produced (part.n_parts + chunk slots per
-// item), so that the loads do not wait for the row's suffix length; records past the row's own count are ignored.
-template <int HD>
-__device__ __forceinline__ void merge_item_warp(int lane, size_t rh, int Hq, const RowGeom& g, const PrefixPartial& part, int ct, int n_load,
-                                                __nv_bfloat16* __restrict__ out, __nv_bfloat16* __restrict__ out_lo, int32_t* err) {
-    constexpr int EPL = HD / 32;
-    const int row = (int)(rh / Hq);
-    const int slen = g.s_len[row];
-    float M = -INFINITY;
-    float acc[EPL];
-#pragma unroll
-    for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
-    float denom = 0.f;
-    float mi[MAX_RECORDS], li[MAX_RECORDS];
-    float ov[MAX_RECORDS][EPL];
-#pragma unroll
-    for (int i = 0; i < MAX_RECORDS; ++i) {
-        const bool ld = i < n_load;
-        mi[i] = ld ? part.m[(size_t)i * part.stride + rh] : -INFINITY;
-        li[i] = ld ? part.l[(size_t)i * part.stride + rh] : 0.f;
-        const float* src = part.o + ((size_t)i * part.stride + rh) * HD + lane * EPL;
-        if (EPL == 4) {
-            const float4 v = ld ? *reinterpret_cast<const float4*>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
-            ov[i][0] = v.x; ov[i][1] = v.y; ov[i][2] = v.z; ov[i][3] = v.w;
-        } else {
-            const float2 v = ld ? *reinterpret_cast<const float2*>(src) : make_float2(0.f, 0.f);
-            ov[i][0] = v.x; ov[i][1] = v.y;
-        }
-    }
-    const int n_rec = part.n_parts + suffix_chunks(slen, ct);
-#pragma unroll
-    for (int i = 0; i < MAX_RECORDS; ++i)
-        if (i >= n_rec) mi[i] = -INFINITY;           // not a record of this row (stale memory)
-#pragma unroll
-    for (int i = 0; i < MAX_RECORDS; ++i) M = fmaxf(M, mi[i]);
-#pragma unroll
-    for (int i = 0; i < MAX_RECORDS; ++i) {
-        const float w = exp2_safe(mi[i], M);
-        if (i < n_rec && w > 0.f) {          // a record with m = -inf was left by an empty range: its output slice is not defined
-            denom += li[i] * w;
-#pragma unroll
-            for (int e = 0; e < EPL; ++e) acc[e] += ov[i][e] * w;
-        }
-    }
-    store_attention<HD>(lane, rh, acc, denom, out, out_lo, err);
-}
-
-// Stand-alone form: the grid covers the row bound of the step.
-template <int HD>
-__global__ void __launch_bounds__(256) attn_merge_kernel(const StepDesc* __restrict__ sd, int Hq, RowGeom g, PrefixPartial part,
-                                                         __nv_bfloat16* __restrict__ out, __nv_bfloat16* __restrict__ out_lo, int32_t* err) {
-    const size_t rh = (size_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    grid_dep_wait();                       // the suffix records, and with them the prefix records: that kernel waits for its own
-    grid_dep_launch_dependents();          // the output projection may set itself up and request its first weight tiles
-    const int n_live = sd->n_rows;
-    if (rh >= (size_t)n_live * Hq) return;
-    const SuffixPlan sp = suffix_plan(*g.max_slen, n_live * part.n_kv_heads, part.n_suffix_warps);
-    merge_item_warp<HD>(threadIdx.x & 31, rh, Hq, g, part, sp.ct, part.n_parts + sp.cpi, out, out_lo, err);
 }
 
 }  // namespace am

@@ -2,7 +2,7 @@
 // PHASES of one cooperative kernel (one CTA per SM) separated by grid-wide barriers, instead of one launch each.
 //
 //   segment -1 :  embedding + RMSNorm  |  QKV GEMM of layer 0  |  bias / QK-norm / RoPE / KV append
-//   segment  l :  [merge of the attention records]  |  output projection  |  residual + RMSNorm  |  gate/up GEMM + SwiGLU  |
+//   segment  l :  output projection  |  residual + RMSNorm  |  gate/up GEMM + SwiGLU  |
 //                 down projection  |  residual + RMSNorm (gains of layer l+1, or the final norm)  |
 //                 QKV GEMM of layer l+1  |  its post-processing          (last layer: LM head instead of the last two)
 //
@@ -55,7 +55,7 @@ constexpr int BAR_WORDS_PER_SEG = 16;
 constexpr int SMEM_BYTES = RING_BYTES + 1024 /*align*/ + 512 /*barriers, flags*/;
 constexpr uint32_t GRID_WAIT_LIMIT = 1u << 22;
 
-enum Phase : int { PH_END = 0, PH_EMBED, PH_MERGE, PH_O, PH_NORM_MLP, PH_GU, PH_DOWN, PH_NORM_NEXT, PH_QKV, PH_POST, PH_LM };
+enum Phase : int { PH_END = 0, PH_EMBED, PH_O, PH_NORM_MLP, PH_GU, PH_DOWN, PH_NORM_NEXT, PH_QKV, PH_POST, PH_LM };
 enum GemmKindId : int { GK_QKV = 0, GK_O = 1, GK_GU = 2, GK_DOWN = 3, GK_LM = 4 };
 
 __host__ __device__ constexpr int bn_index(int bn) { return bn == 64 ? 0 : (bn == 128 ? 1 : 2); }
@@ -83,7 +83,6 @@ struct ChainParams {
     const StepDesc* sd;
     int M;                       // row bound the tiles and the partial-sum layout are sized for
     int seg;                     // -1: embedding .. QKV of layer 0;  l >= 0: output projection of layer l .. QKV of layer l + 1
-    int with_merge;              // segment l starts with the merge of the attention records
     int n_layers, d_model, n_qkv, q_dim, d_ff, vocab, Hq, Hkv, hd;
     float eps;
     int bn[5], splits[5];        // tile width and K-slices per GEMM kind
@@ -102,7 +101,6 @@ struct ChainParams {
     const float2* rope;
     RowGeom g;
     KvArena prompt_arena, suffix_arena;
-    am::PrefixPartial part;
     int32_t* bar;                // BAR_WORDS_PER_SEG words per segment, zero when the step starts
     int32_t* err;
     long long* trace;            // optional: SM clock stamps of the first TRACE_CTAS CTAs, [segment][phase][cta][TRACE_EVENTS]
@@ -121,16 +119,14 @@ __device__ __forceinline__ bool is_gemm(int ph) { return ph == PH_O || ph == PH_
 __device__ __forceinline__ int phase_at(const ChainParams& p, int j) {
     if (p.seg < 0) return j == 0 ? PH_EMBED : (j == 1 ? PH_QKV : (j == 2 ? PH_POST : PH_END));
     const bool last = p.seg == p.n_layers - 1;
-    if (!p.with_merge) ++j;
     switch (j) {
-        case 0: return PH_MERGE;
-        case 1: return PH_O;
-        case 2: return PH_NORM_MLP;
-        case 3: return PH_GU;
-        case 4: return PH_DOWN;
-        case 5: return PH_NORM_NEXT;
-        case 6: return last ? PH_LM : PH_QKV;
-        case 7: return last ? PH_END : PH_POST;
+        case 0: return PH_O;
+        case 1: return PH_NORM_MLP;
+        case 2: return PH_GU;
+        case 3: return PH_DOWN;
+        case 4: return PH_NORM_NEXT;
+        case 5: return last ? PH_LM : PH_QKV;
+        case 6: return last ? PH_END : PH_POST;
         default: return PH_END;
     }
 }
@@ -475,14 +471,6 @@ __global__ void __launch_bounds__(THREADS, 1) decode_chain_kernel(const __grid_c
                         else if (nb == 3) qkv_post_items_warp<__nv_bfloat16, 3>(lane, A, rows, heads, 3);
                         else if (nb == 2) qkv_post_items_warp<__nv_bfloat16, 2>(lane, A, rows, heads, 2);
                         else qkv_post_items_warp<__nv_bfloat16, 1>(lane, A, rows, heads, 1);
-                    }
-                } else if (ph == PH_MERGE) {
-                    const int items = m_live * p.Hq;
-                    const am::SuffixPlan sp = am::suffix_plan(*p.g.max_slen, p.sd->n_rows * p.part.n_kv_heads, p.part.n_suffix_warps);
-                    const int n_load = p.part.n_parts + sp.cpi;
-                    for (int it = gw; it < items; it += n_gw) {
-                        if (p.hd == 128) am::merge_item_warp<128>(lane, it, p.Hq, p.g, p.part, sp.ct, n_load, p.attn, nullptr, p.err);
-                        else am::merge_item_warp<64>(lane, it, p.Hq, p.g, p.part, sp.ct, n_load, p.attn, nullptr, p.err);
                     }
                 }
             }

@@ -19,6 +19,7 @@
 #include "attention_mma.cuh"
 #include "attention_simt.cuh"
 #include "attention_tc.cuh"
+#include "attention_team.cuh"
 #include "common.cuh"
 #include "decode_chain.cuh"
 #include "gemm_simt.cuh"
@@ -165,10 +166,6 @@ struct pc_ctx {
     int fused_epilogues = 1;                 // half-operand models with head_dim 128: QKV post-processing and the MLP norm inside GEMM epilogues
     int fused_sampler = 0;                   // decode steps that only sample: Gumbel-max in the LM head's epilogue, no logits stored
     int dep_launch = 63;                     // bit per kernel (1 QKV, 2 output, 4 gate/up, 8 down projection, 16 LM head, 32 shared-prefix attention): launched as a programmatic dependent of the kernel before it
-    int attn_overlap = 0;                    // decode: shared-prefix and suffix attention kernels of a layer on two streams
-    cudaStream_t side_stream = nullptr;      // second branch of that fork (created on first use)
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-
     std::vector<GraphEntry> graphs;
     cudaStream_t capture_stream = nullptr;      // decode steps are captured here (the caller's stream may be the default one)
     void drop_graphs() {
@@ -178,9 +175,6 @@ struct pc_ctx {
     ~pc_ctx() {
         drop_graphs();
         if (capture_stream) cudaStreamDestroy(capture_stream);
-        if (side_stream) cudaStreamDestroy(side_stream);
-        if (ev_fork) cudaEventDestroy(ev_fork);
-        if (ev_join) cudaEventDestroy(ev_join);
     }
 
     int n_qkv() const { return (d.n_q_heads + 2 * d.n_kv_heads) * d.head_dim; }
@@ -327,7 +321,7 @@ template <class Epi>
 int gemm_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, const CUtensorMap& map_a, const CUtensorMap* map_a_lo, const WMap& w,
               int M, GemmPlan p, Epi epi, bool half_operands = false, int dep_bit = 0) {
     // dep: launched as a programmatic dependent.  Every projection of a pass follows a kernel that signals its dependents
-    // early (a row norm, the attention merge, another projection), so this launch may set itself up and request its first
+    // early (a row norm, the suffix attention, another projection), so this launch may set itself up and request its first
     // weight tiles while that kernel is still running; after any other kernel it simply starts when that one has ended.
     const bool dep = dependent_launch(c, dep_bit, M);
     cudaError_t e;
@@ -504,9 +498,9 @@ cudaError_t configure_attention() {
             e = cudaFuncSetAttribute(am::attn_group_kernel<HD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::group_smem_bytes<HD>());
     }
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(am::attn_suffix_kernel<HD, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::suffix_smem_bytes<HD>());
+        e = cudaFuncSetAttribute(am::attn_suffix_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::suffix_smem_bytes<HD>());
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(am::attn_suffix_kernel<HD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::suffix_smem_bytes<HD>());
+        e = cudaFuncSetAttribute(am::attn_suffix_team_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::TEAM_SMEM_BYTES);
     return e;
 }
 template <class Epi>
@@ -574,11 +568,10 @@ cudaError_t configure_kernels() {
 // Query rows one CTA of the shared-prefix / causal-prefill attention takes.
 constexpr int prefix_q_rows(int head_dim) { return head_dim == 128 ? pc::at::QROWS : pc::am::G_QROWS; }
 
-// part_out != nullptr: the records are left unmerged and described there (the caller merges them).
+// after_chain: the kernel before this one is the persistent one (plain stream order).
 template <int HD>
 int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, int layer, const AttnPlan& plan, pc::KvArena prompt_arena,
-                   pc::KvArena suffix_arena, const __nv_bfloat16* q, __nv_bfloat16* attn,
-                   pc::am::PrefixPartial* part_out = nullptr) {
+                   pc::KvArena suffix_arena, const __nv_bfloat16* q, __nv_bfloat16* attn, bool after_chain = false) {
     using namespace pc;
     const pc_model_desc& d = c->d;
     // half_gemm: the attention output is written once, as IEEE half; else as bf16 plus its bf16 rounding remainder
@@ -589,16 +582,13 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
     // a group with few query rows keeps few CTAs busy: cut its prompt into ranges so that about one CTA per SM runs
     const int q_tiles = (plan.max_group_rows * n_rep + prefix_q_rows(HD) - 1) / prefix_q_rows(HD);
     const int base_ctas = std::max(1, q_tiles * d.n_kv_heads * plan.n_groups);
-    const bool overlap = !plan.prefill && c->attn_overlap != 0 && c->prof_active_layer < 0;
-    // batches whose items occupy the suffix kernel's warps with few chunks each: it merges by itself
-    const bool merge_inside = part_out == nullptr && !overlap && (long long)M * d.n_kv_heads * am::MERGE_CHUNKS >= (long long)c->num_sms * am::S_WARPS;
-    const int n_parts = plan.prefill ? 1 : std::max(1, std::min(merge_inside ? am::MAX_MERGED_PARTS : am::MAX_PREFIX_PARTS, c->num_sms / base_ctas));
-    // the suffix kernel takes one warp per (rollout, KV head, range of the suffix); how the suffixes are cut into ranges
-    // is decided on the device for the warps of this grid (the longest suffix of the step is only known there)
-    const int sgrid = std::min(c->num_sms, M * d.n_kv_heads * am::MAX_SUFFIX_CHUNKS);      // units go round the CTAs first
+    // batches whose items occupy the suffix kernel's warps with few ranges each; smaller ones take a team of CTAs per item
+    const int items = M * d.n_kv_heads;
+    const bool teams = items <= 2 * c->num_sms;
+    const int n_parts = plan.prefill ? 1 : std::max(1, std::min(teams ? am::MAX_PREFIX_PARTS : am::MAX_MERGED_PARTS, c->num_sms / base_ctas));
     am::PrefixPartial part{reinterpret_cast<float*>(c->ws + c->cv.part_m), reinterpret_cast<float*>(c->ws + c->cv.part_l),
                            reinterpret_cast<float*>(c->ws + c->cv.part_o), n_parts, (size_t)std::max(c->max_rows, 1) * d.n_q_heads,
-                           d.n_kv_heads, sgrid * am::S_WARPS};
+                           d.n_kv_heads, c->num_sms * am::S_WARPS};
     const dim3 ggrid = HD == 128 ? dim3(q_tiles * n_parts * d.n_kv_heads * plan.n_groups) : dim3(q_tiles * n_parts, d.n_kv_heads, plan.n_groups);
     if (plan.prefill) {
         if constexpr (HD == 128)
@@ -612,55 +602,52 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
         count_launches(1);
         return PC_OK;
     }
-    // The two kernels are independent (both read q, each leaves its own records), so outside profiled steps they are issued
-    // on two streams -- a fork and a join inside the captured step -- and share the GPU.
-    cudaStream_t gst = st;
-    if (overlap) {
-        if (c->side_stream == nullptr) {
-            cudaError_t e = cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking);
-            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
-            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming);
-            if (e != cudaSuccess) return cuda_fail(e, "side stream of the attention fork");
-        }
-        cudaEventRecord(c->ev_fork, st);
-        cudaStreamWaitEvent(c->side_stream, c->ev_fork, 0);
-        gst = c->side_stream;
-    }
-    // after the QKV post-processing kernel or the QKV projection (both signal their dependents early); not on the side stream
-    // of the fork and not after the persistent kernel
-    const bool group_dep = !overlap && part_out == nullptr && dependent_launch(c, DEP_GROUP, M);
+    // The shared-prefix kernel depends on the QKV projection (or its post-processing), the suffix kernel on the shared-prefix
+    // kernel; each may start when the one before it has begun, and reads what it needs of it after its wait.
+    const bool group_dep = !after_chain && dependent_launch(c, DEP_GROUP, M);
     if constexpr (HD == 128)
-        launch_k_dep(group_dep, at::attn_prefix_kernel<false>, ggrid, dim3(at::THREADS), at::SMEM_BYTES, gst,
+        launch_k_dep(group_dep, at::attn_prefix_kernel<false>, ggrid, dim3(at::THREADS), at::SMEM_BYTES, st,
             c->map_prompt_kv, sd, prompt_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, plan.group_row_start, g, scale_log2, part, q_tiles,
             attn, attn_lo, c->err);
     else
-        launch_k_dep(group_dep, am::attn_group_kernel<HD, false>, ggrid, dim3(am::G_THREADS), am::group_smem_bytes<HD>(), gst,
+        launch_k_dep(group_dep, am::attn_group_kernel<HD, false>, ggrid, dim3(am::G_THREADS), am::group_smem_bytes<HD>(), st,
             c->map_prompt_kv, sd, prompt_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, plan.group_row_start, g, scale_log2, part,
             attn, attn_lo, c->err);
-    if (overlap) cudaEventRecord(c->ev_join, gst);
     c->mark(st, layer, PC_MARK_GROUP);
-    const am::SuffixMerge mg{reinterpret_cast<int32_t*>(c->ws + c->cv.arrived), attn, attn_lo};
-    if (merge_inside)
-        launch_k_dep(group_dep, am::attn_suffix_kernel<HD, true>, dim3(sgrid), dim3(am::S_WARPS * 32), am::suffix_smem_bytes<HD>(), st,
+    if (teams) {
+        // a cluster of CTAs per (row, KV head): as many as fit beside the shared-prefix kernel, one CTA of each per SM
+        int team = 8;
+        while (team > 1 && items * team > c->num_sms) team >>= 1;
+        cudaLaunchConfig_t cfg;
+        std::memset(&cfg, 0, sizeof(cfg));
+        cfg.gridDim = dim3((unsigned)(items * team)); cfg.blockDim = dim3(am::T_WARPS * 32);
+        cfg.dynamicSmemBytes = am::TEAM_SMEM_BYTES; cfg.stream = st;
+        cudaLaunchAttribute attr[2];
+        int n_attr = 0;
+        if (team > 1) {
+            attr[n_attr].id = cudaLaunchAttributeClusterDimension;
+            attr[n_attr].val.clusterDim.x = team; attr[n_attr].val.clusterDim.y = 1; attr[n_attr].val.clusterDim.z = 1;
+            ++n_attr;
+        }
+        if (group_dep) {
+            attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[n_attr].val.programmaticStreamSerializationAllowed = 1;
+            ++n_attr;
+        }
+        cfg.attrs = attr; cfg.numAttrs = n_attr;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, am::attn_suffix_team_kernel<HD>, c->map_suffix_kv, sd, suffix_arena.n_slots, d.n_q_heads,
+                                                 d.n_kv_heads, layer, q, g, scale_log2, part, team, attn, attn_lo, c->err);
+        if (e != cudaSuccess) return cuda_fail(e, "suffix attention");
+    } else {
+        // one warp per (rollout, KV head, range of the suffix); how the suffixes are cut into ranges is decided on the device for
+        // the warps of this grid (the longest suffix of the step is only known there)
+        const am::SuffixMerge mg{reinterpret_cast<int32_t*>(c->ws + c->cv.arrived), attn, attn_lo};
+        launch_k_dep(group_dep, am::attn_suffix_kernel<HD>, dim3(c->num_sms), dim3(am::S_WARPS * 32), am::suffix_smem_bytes<HD>(), st,
             c->map_suffix_kv, sd, suffix_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, g, scale_log2, part, mg, c->err);
-    else
-        launch_k_dep(group_dep, am::attn_suffix_kernel<HD, false>, dim3(sgrid), dim3(am::S_WARPS * 32), am::suffix_smem_bytes<HD>(), st,
-            c->map_suffix_kv, sd, suffix_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, g, scale_log2, part, mg, c->err);
-    if (overlap) cudaStreamWaitEvent(st, c->ev_join, 0);
+    }
     c->mark(st, layer, PC_MARK_SUFFIX);
-    if (part_out != nullptr) {
-        *part_out = part;
-        count_launches(2);
-        return PC_OK;
-    }
-    if (merge_inside) {
-        c->mark(st, layer, PC_MARK_MERGE);
-        count_launches(2);
-        return PC_OK;
-    }
-    launch_k(am::attn_merge_kernel<HD>, dim3((M * d.n_q_heads + 7) / 8), dim3(256), 0, st, sd, d.n_q_heads, g, part, attn, attn_lo, c->err);
     c->mark(st, layer, PC_MARK_MERGE);
-    count_launches(3);
+    count_launches(2);
     return PC_OK;
 }
 
@@ -1027,8 +1014,6 @@ int pc_set_dependent_launch(pc_ctx* ctx, int mask) {
 
 int pc_set_attention_overlap(pc_ctx* ctx, int on) {
     if (ctx == nullptr || (on != 0 && on != 1)) return PC_ERR_INVALID_ARG;
-    if (on != ctx->attn_overlap) ctx->drop_graphs();
-    ctx->attn_overlap = on;
     return PC_OK;
 }
 
@@ -1362,13 +1347,13 @@ int check_decode_args(const pc_ctx* ctx, const DecodeArgs& a) {
 
 // One segment of the persistent decode kernel (decode_chain.cuh) over the rows described by *sd.
 int launch_chain(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, int seg, pc::KvArena prompt_arena, pc::KvArena suffix_arena,
-                 const pc::am::PrefixPartial* part, float* logits) {
+                 float* logits) {
     using namespace pc;
     const pc_model_desc& d = c->d;
     char* w = c->ws;
     chain::ChainParams p;
     std::memset(&p, 0, sizeof(p));
-    p.sd = sd; p.M = M; p.seg = seg; p.with_merge = part != nullptr ? 1 : 0;
+    p.sd = sd; p.M = M; p.seg = seg;
     p.n_layers = d.n_layers; p.d_model = d.d_model; p.n_qkv = c->n_qkv(); p.q_dim = c->q_dim(); p.d_ff = d.d_ff; p.vocab = d.vocab;
     p.Hq = d.n_q_heads; p.Hkv = d.n_kv_heads; p.hd = d.head_dim; p.eps = d.rms_eps;
     const WMap* maps[5] = {&c->m_wqkv[0], &c->m_wo[0], &c->m_wgu[0], &c->m_wdown[0], &c->m_lm};
@@ -1404,7 +1389,6 @@ int launch_chain(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, int 
     p.rope = reinterpret_cast<const float2*>(w + c->cv.rope);
     p.g = geom(c);
     p.prompt_arena = prompt_arena; p.suffix_arena = suffix_arena;
-    if (part != nullptr) p.part = *part;
     p.bar = reinterpret_cast<int32_t*>(w + c->cv.chain_bar);
     p.err = c->err;
     p.trace = c->chain_trace;
@@ -1432,15 +1416,14 @@ int run_decode_chained(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd
     launch_k(rope_table_kernel, dim3((M * half + 255) / 256), dim3(256), 0, st, sd, half, (double)d.rope_theta, g.pos, reinterpret_cast<float2*>(w + c->cv.rope));
     count_launches(1);
     PC_CUDA_CHECK_LAUNCH("rope table");
-    if (int rc = launch_chain(c, st, M, sd, -1, prompt_arena, suffix_arena, nullptr, logits)) return rc;
+    if (int rc = launch_chain(c, st, M, sd, -1, prompt_arena, suffix_arena, logits)) return rc;
     const __nv_bfloat16* q = reinterpret_cast<const __nv_bfloat16*>(w + c->cv.q);
     __nv_bfloat16* attn = reinterpret_cast<__nv_bfloat16*>(w + c->cv.attn);
     for (int l = 0; l < d.n_layers; ++l) {
-        am::PrefixPartial part;
-        int rc = d.head_dim == 128 ? attention_bf16<128>(c, st, sd, M, l, plan, prompt_arena, suffix_arena, q, attn, &part)
-                                   : attention_bf16<64>(c, st, sd, M, l, plan, prompt_arena, suffix_arena, q, attn, &part);
+        int rc = d.head_dim == 128 ? attention_bf16<128>(c, st, sd, M, l, plan, prompt_arena, suffix_arena, q, attn, true)
+                                   : attention_bf16<64>(c, st, sd, M, l, plan, prompt_arena, suffix_arena, q, attn, true);
         if (rc) return rc;
-        if ((rc = launch_chain(c, st, M, sd, l, prompt_arena, suffix_arena, &part, logits))) return rc;
+        if ((rc = launch_chain(c, st, M, sd, l, prompt_arena, suffix_arena, logits))) return rc;
     }
     PC_CUDA_CHECK_LAUNCH("chained decode step");
     return PC_OK;
