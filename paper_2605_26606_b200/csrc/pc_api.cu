@@ -23,7 +23,6 @@
 #include "common.cuh"
 #include "decode_chain.cuh"
 #include "gemm_simt.cuh"
-#include "gemm_epilogues.cuh"
 #include "gemm_tc.cuh"
 #include "gemm_wt.cuh"
 #include "kernels_basic.cuh"
@@ -340,19 +339,6 @@ int gemm_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, const CUtensor
     return PC_OK;
 }
 
-// Unsplit GEMM with an explicit tile width (the fused epilogues need complete sums in a tile).
-template <int BN, class Epi>
-int gemm_half_bn(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, const CUtensorMap& map_a, const WMap& w, int M, Epi epi, int dep_bit = 0) {
-    const CUtensorMap& mw = BN == 256 ? w.wide : (BN == 128 ? w.mid : w.narrow);
-    const bool dep = dependent_launch(c, dep_bit, M);
-    const cudaError_t e = pc::tc::launch<BN, false>(st, map_a, map_a, mw, sd, M, w.N, w.K, 1, epi, c->err, c->num_sms, true, dep);
-    if (e != cudaSuccess) return cuda_fail(e, "tensor-core gemm (fused epilogue)");
-    return PC_OK;
-}
-inline bool wide_tiles_fill_the_gpu(const pc_ctx* c, int M, int N) {
-    return ((M + pc::tc::BM - 1) / pc::tc::BM) * ((N + 255) / 256) >= c->num_sms / 2;
-}
-
 // ---- weight-on-lanes projections ------------------------------------------------------------------------------------
 enum XBuf { X_A = 0, X_ATTN = 1, X_ACT = 2, X_A_LO = 3, X_ATTN_LO = 4 };
 
@@ -379,7 +365,7 @@ const pc_ctx::WtPlan& plan_wt(pc_ctx* c, GemmKind kind, int N, int K, int M, boo
             const int nt = ((M + tr - 1) / tr + unit - 1) / unit * unit;
             if (nt > wt::MAX_ROWS_TILE || (M + nt - 1) / nt != tr || (cg == 2 && nt < 192)) continue;
             for (int sp = 1; sp <= (cg == 1 && may_split ? wt::MAX_SPLITS : 1); ++sp) {
-                if (kb / sp < 2) continue;
+                if (kb / sp < 2 || (sp > 1 && features * tr >= c->num_sms)) break;      // enough whole tiles for every SM
                 const int stage = wt::W_BYTES + (dual ? wt::x_bytes<true>(nt, cg) : wt::x_bytes<false>(nt, cg));
                 const int stages = std::min(wt::MAX_STAGES, (wt::SMEM_BUDGET - wt::smem_bytes<false>(nt, 4, cg, sp, 0)) / stage);
                 if (stages < 3 || (sp > 1 && stages * stage < (nt + 8) * wt::FT * 4)) continue;
@@ -400,6 +386,7 @@ const pc_ctx::WtPlan& plan_wt(pc_ctx* c, GemmKind kind, int N, int K, int M, boo
             }
         }
     }
+    if (c->wt_plans.size() >= 512) c->wt_plans.clear();       // prefill passes come in any number of rows
     c->wt_plans.push_back(best);
     return c->wt_plans.back();
 }
@@ -441,13 +428,14 @@ int gemm_wt(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, GemmKind kind, X
     return PC_OK;
 }
 
-// Whether a pass of M rows takes the weight-on-lanes projections with their fused epilogues: every decode step and prefill of
-// a head_dim 128 model up to WT_MAX_ROWS rows; larger passes keep the rows-on-lanes kernel, whose row-per-thread epilogues
-// need fewer instructions per value.  Forced tilings (pc_set_gemm_plan) and fused_epilogues = 0 name the other kernels.
-constexpr int WT_MAX_ROWS = 4096;
+// Whether a pass of M rows takes the weight-on-lanes projections with their fused epilogues: every pass of a head_dim 128 model.
+// (16 prompts, 10,184 rows: 32.2 ms with rows on the lanes and the row-wise steps fused there, 27.1 ms this way -- CTA pairs move a
+// third less from L2 per MMA and the vector epilogues hide behind the next tile.)  Above WT_MAX_ROWS the tile arithmetic is no
+// longer exact.  Forced tilings (pc_set_gemm_plan) and fused_epilogues = 0 name the other kernels.
+constexpr int WT_MAX_ROWS = 1 << 20;
 bool use_wt(const pc_ctx* c, int M) {
     const pc_model_desc& d = c->d;
-    if (d.dtype != PC_DTYPE_BF16 || d.head_dim != 128 || d.d_model % 128 != 0) return false;
+    if (d.dtype != PC_DTYPE_BF16 || d.head_dim != 128 || d.d_model % 64 != 0) return false;
     if (c->fused_epilogues == 0 || (c->fused_epilogues > 1 && M < c->fused_epilogues)) return false;
     for (int k = 0; k < 5; ++k)
         if (c->plan_bn[k] != 0) return false;
@@ -541,12 +529,6 @@ cudaError_t configure_kernels() {
     if (e == cudaSuccess) e = tc::configure<64, true, tc::EpiStoreF32>();
     if (e == cudaSuccess) e = tc::configure<256, false, tc::EpiStoreF32>();
     if (e == cudaSuccess) e = tc::configure<64, false, tc::EpiStoreF32>();
-    if (e == cudaSuccess) e = tc::configure<128, false, EpiQkvPost>();
-    if (e == cudaSuccess) e = tc::configure<256, false, EpiQkvPost>();
-    if (e == cudaSuccess) e = tc::configure<64, false, EpiResNorm>();
-    if (e == cudaSuccess) e = tc::configure<256, false, EpiResNorm>();
-    if (e == cudaSuccess) e = tc::configure<64, false, EpiSwiGLUNorm>();
-    if (e == cudaSuccess) e = tc::configure<256, false, EpiSwiGLUNorm>();
     if (e == cudaSuccess) e = tc::configure<256, true, EpiSample>();
     if (e == cudaSuccess) e = tc::configure<64, true, EpiSample>();
     if (e == cudaSuccess) e = tc::configure<256, false, EpiSample>();
@@ -667,12 +649,7 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
     T* attn = reinterpret_cast<T*>(w + c->cv.attn);
     T* act = reinterpret_cast<T*>(w + c->cv.act);
     const bool half_gemm = !kF32 && d.half_gemm != 0;      // every GEMM operand in IEEE half
-    // QKV post-processing in the QKV GEMM's epilogue; residual add, operand of the gate/up GEMM and the norm's sum of squares
-    // in the output projection's epilogue, its 1/rms applied by the gate/up epilogue (gemm_epilogues.cuh)
-    // From three row tiles on: below that the two projections need their K split to keep the SMs busy (measured: unsplit they
-    // lose more than the two small kernels cost), and a split GEMM's tile does not hold complete sums.
     const bool wt_path = !kF32 && use_wt(c, M);
-    const bool fused = !wt_path && half_gemm && d.head_dim == 128 && d.d_model % 64 == 0 && c->fused_epilogues != 0 && M >= (c->fused_epilogues == 1 ? 2 * tc::BM + 1 : c->fused_epilogues);
     float* ssq = reinterpret_cast<float*>(w + c->cv.ssq);
     const int m_stride = std::max(std::max(c->max_rows, c->max_prefill), 1);
     T* a_lo = kF32 || half_gemm ? nullptr : reinterpret_cast<T*>(w + c->cv.a_lo);          // rounding remainders (bf16 operands only)
@@ -683,8 +660,6 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
     float* res_part = reinterpret_cast<float*>(w + c->cv.res_part);
     const Partials none{nullptr, 0, 0, 0};
     Partials pend = none;
-    int n_ssq = 0;
-    int n_ssq_attn = 0;          // > 0: the previous layer's down projection left half(h * gain) and sums of squares for this layer's attention norm
 
     c->final_norm_pending = false;
     launch_k(rope_table_kernel, dim3((M * half + 255) / 256), dim3(256), 0, st, sd, half, (double)d.rope_theta, g.pos, rope);
@@ -697,7 +672,7 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
         if constexpr (!kF32) if (wt_path) {
             // Five projections' worth of work in four launches: every row-wise step around a projection is in its epilogue.
             const float* bias_l = d.qkv_bias ? c->bqkv[l] : nullptr;
-            const int n_tiles = d.d_model / wt::FT;
+            const int n_tiles = (d.d_model + wt::FT - 1) / wt::FT;
             const wt::RowScale complete{nullptr, 0, 0, 1, 0.f}, scaled{ssq, n_tiles, m_stride, d.d_model, d.rms_eps};
             c->mark(st, l, PC_MARK_NORM_ATTN);
             wt::EpiQkv eq{};
@@ -744,7 +719,7 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
             PC_CUDA_CHECK_LAUNCH("decoder layer");
             continue;
         }
-        if (l > 0 && n_ssq_attn == 0) {
+        if (l > 0) {
             launch_k(rmsnorm_kernel<T>, dim3(M), dim3(NORM_THREADS), 0, st, sd, M, d.d_model, h, nullptr, pend, c->attn_norm[l], d.rms_eps, a, a_lo, half_gemm ? 1 : 0, c->err);
             pend = none;
             count_launches(1);
@@ -755,14 +730,6 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
         if constexpr (kF32) {
             launch_gemm_simt(st, sd, a, reinterpret_cast<const T*>(c->wqkv[l]), M, c->n_qkv(), d.d_model,
                                 EpiStoreF32{qkv, c->n_qkv(), nullptr});
-        } else if (fused) {
-            const EpiQkvPost epi{d.n_q_heads, d.n_kv_heads, l, bias, d.qk_norm ? c->q_norm[l] : nullptr, d.qk_norm ? c->k_norm[l] : nullptr,
-                                 d.rms_eps, rope, g, prompt_arena, suffix_arena, reinterpret_cast<__half*>(q), c->err, ssq, n_ssq_attn, m_stride, d.d_model};
-            n_ssq_attn = 0;
-            const bool wide_qkv = c->plan_bn[GEMM_QKV] != 0 ? c->plan_bn[GEMM_QKV] == 256 : wide_tiles_fill_the_gpu(c, M, c->n_qkv());
-            const int rc = wide_qkv ? gemm_half_bn<256>(c, st, sd, c->map_a, c->m_wqkv[l], M, epi, DEP_QKV)
-                                    : gemm_half_bn<128>(c, st, sd, c->map_a, c->m_wqkv[l], M, epi, DEP_QKV);
-            if (rc) return rc;
         } else {
             const GemmPlan gp = plan_gemm(c, GEMM_QKV, c->m_wqkv[l], M, true);
             qkv_parts.n = gp.splits;
@@ -772,10 +739,10 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
         }
         c->mark(st, l, PC_MARK_QKV);
         const int post_items = M * (d.n_q_heads + 2 * d.n_kv_heads);
-        if (!fused) launch_k(qkv_post_kernel<T>, dim3((post_items + ROW_WARPS - 1) / ROW_WARPS), dim3(ROW_WARPS * 32), 0, st, 
+        launch_k(qkv_post_kernel<T>, dim3((post_items + ROW_WARPS - 1) / ROW_WARPS), dim3(ROW_WARPS * 32), 0, st,
             sd, QkvPostArgs<T>{d.n_q_heads, d.n_kv_heads, d.head_dim, l, qkv_parts, bias, d.qk_norm ? c->q_norm[l] : nullptr,
                                d.qk_norm ? c->k_norm[l] : nullptr, d.rms_eps, rope, g, prompt_arena, suffix_arena, q, c->err});
-        count_launches(fused ? 1 : 2);
+        count_launches(2);
         c->mark(st, l, PC_MARK_POST);
         if constexpr (kF32) {
             c->mark(st, l, PC_MARK_GROUP);
@@ -791,14 +758,7 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
                          : attention_bf16<64>(c, st, sd, M, l, plan, prompt_arena, suffix_arena, q, attn);
             if (rc) return rc;
             const GemmPlan gp = plan_gemm(c, GEMM_O, c->m_wo[l], M, true);
-            if (fused) {
-                const bool wide = c->plan_bn[GEMM_O] != 0 ? c->plan_bn[GEMM_O] == 256 : wide_tiles_fill_the_gpu(c, M, d.d_model);
-                n_ssq = (d.d_model + (wide ? 256 : 64) - 1) / (wide ? 256 : 64);
-                const EpiResNorm epi{h, d.d_model, c->mlp_norm[l], reinterpret_cast<__half*>(a), ssq, m_stride, c->err};
-                const int rc2 = wide ? gemm_half_bn<256>(c, st, sd, c->map_attn, c->m_wo[l], M, epi, DEP_O)
-                                     : gemm_half_bn<64>(c, st, sd, c->map_attn, c->m_wo[l], M, epi, DEP_O);
-                if (rc2) return rc2;
-            } else if (gp.splits == 1) {
+            if (gp.splits == 1) {
                 if (int rc2 = gemm_bf16(c, st, sd, c->map_attn, half_gemm ? nullptr : &c->map_attn_lo, c->m_wo[l], M, gp,
                                         tc::EpiResidual{h, d.d_model}, half_gemm, DEP_O))
                     return rc2;
@@ -810,36 +770,15 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
             }
         }
         c->mark(st, l, PC_MARK_O);
-        if (!fused) launch_k(rmsnorm_kernel<T>, dim3(M), dim3(NORM_THREADS), 0, st, sd, M, d.d_model, h, nullptr, pend, c->mlp_norm[l], d.rms_eps, a, nullptr, half_gemm ? 1 : 0, c->err);
+        launch_k(rmsnorm_kernel<T>, dim3(M), dim3(NORM_THREADS), 0, st, sd, M, d.d_model, h, nullptr, pend, c->mlp_norm[l], d.rms_eps, a, nullptr, half_gemm ? 1 : 0, c->err);
         pend = none;
-        count_launches(fused ? 1 : 2);
+        count_launches(2);
         c->mark(st, l, PC_MARK_NORM_MLP);
         if constexpr (kF32) {
             launch_gemm_simt(st, sd, a, reinterpret_cast<const T*>(c->w_gate_up[l]), M, 2 * d.d_ff, d.d_model,
                                 EpiSwiGLU{act, d.d_ff});
             c->mark(st, l, PC_MARK_GATE_UP);
             launch_gemm_simt(st, sd, act, reinterpret_cast<const T*>(c->w_down[l]), M, d.d_model, d.d_ff, EpiResidual{h, d.d_model});
-        } else if (fused) {
-            const EpiSwiGLUNorm epi{reinterpret_cast<__half*>(act), d.d_ff, ssq, n_ssq, m_stride, d.d_model, d.rms_eps, c->err};
-            const int rc = plan_gemm(c, GEMM_GATE_UP, c->m_wgu[l], M, false).wide ? gemm_half_bn<256>(c, st, sd, c->map_a, c->m_wgu[l], M, epi, DEP_GATE_UP)
-                                                                                  : gemm_half_bn<64>(c, st, sd, c->map_a, c->m_wgu[l], M, epi, DEP_GATE_UP);
-            if (rc) return rc;
-            c->mark(st, l, PC_MARK_GATE_UP);
-            const GemmPlan gp = plan_gemm(c, GEMM_DOWN, c->m_wdown[l], M, true);
-            if (gp.splits == 1 && l + 1 < d.n_layers) {
-                // complete sums in every tile: the next layer's attention norm moves into this epilogue and the QKV epilogue
-                // (the sums of squares of the MLP norm were consumed by the gate/up projection above)
-                n_ssq_attn = (d.d_model + (gp.wide ? 256 : 64) - 1) / (gp.wide ? 256 : 64);
-                const EpiResNorm epi2{h, d.d_model, c->attn_norm[l + 1], reinterpret_cast<__half*>(a), ssq, m_stride, c->err};
-                const int rc2 = gp.wide ? gemm_half_bn<256>(c, st, sd, c->map_act, c->m_wdown[l], M, epi2, DEP_DOWN)
-                                        : gemm_half_bn<64>(c, st, sd, c->map_act, c->m_wdown[l], M, epi2, DEP_DOWN);
-                if (rc2) return rc2;
-            } else if (gp.splits == 1) {
-                if (int rc2 = gemm_bf16(c, st, sd, c->map_act, nullptr, c->m_wdown[l], M, gp, tc::EpiResidual{h, d.d_model}, half_gemm, DEP_DOWN)) return rc2;
-            } else {
-                pend = Partials{res_part, gp.splits, (size_t)M * d.d_model, d.d_model};
-                if (int rc2 = gemm_bf16(c, st, sd, c->map_act, nullptr, c->m_wdown[l], M, gp, tc::EpiPartial{res_part, d.d_model, pend.stride}, half_gemm, DEP_DOWN)) return rc2;
-            }
         } else {
             if (int rc = gemm_bf16(c, st, sd, c->map_a, nullptr, c->m_wgu[l], M, plan_gemm(c, GEMM_GATE_UP, c->m_wgu[l], M, false), tc::EpiSwiGLU{act, d.d_ff, half_gemm ? 1 : 0, c->err}, half_gemm, DEP_GATE_UP))
                 return rc;
@@ -862,7 +801,7 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
 
 // The factor of the final norm when the last down projection left the LM head's operand without it.
 pc::wt::RowScale folded_norm(const pc_ctx* c) {
-    return pc::wt::RowScale{reinterpret_cast<const float*>(c->ws + c->cv.ssq), c->d.d_model / pc::wt::FT,
+    return pc::wt::RowScale{reinterpret_cast<const float*>(c->ws + c->cv.ssq), (c->d.d_model + pc::wt::FT - 1) / pc::wt::FT,
                             std::max(std::max(c->max_rows, c->max_prefill), 1), c->d.d_model, c->d.rms_eps};
 }
 
