@@ -90,7 +90,7 @@ inline Geom make_geom(int M, int N, int K, int cg, int nt, int splits, int stage
 
 template <bool DUAL> __host__ __device__ constexpr int x_bytes(int nt, int cg) { return (nt / cg) * BK * 2 * (DUAL ? 2 : 1); }
 constexpr int SCALE_FLOATS = 2 * MAX_ROWS_TILE + 32;        // row scales of two tiles; rows behind the last are read, not used
-constexpr int SMEM_FIXED = 1024 /*align*/ + 512 /*barriers*/ + SCALE_FLOATS * 4;
+constexpr int SMEM_FIXED = 1024 /*align*/ + 512 /*barriers*/ + 2 * SCALE_FLOATS * 4 /*row scales, row slots*/;
 // Rows of a chunk of one epilogue group (unsplit tiles): NR for each of its four warps, or half of the tile when that is less.
 __host__ __device__ constexpr int chunk_rows(int nt, int nr) { return nt >= 32 ? 4 * nr : 8; }
 template <bool DUAL> __host__ __device__ constexpr int smem_bytes(int nt, int nr, int cg, int splits, int stages) {
@@ -233,6 +233,7 @@ struct Ctx {
     bool fv;                // they exist (the number of features is a multiple of 4, except for logits)
     int row0;               // first row of the tile
     const float* scale;     // RMSNorm factor per row of the tile
+    const int* slot;        // where each row of the tile goes (epilogues with kSlots)
 };
 // Rows r + j * step, j < NR, of the tile; those below `end` exist.
 struct Rows {
@@ -287,6 +288,7 @@ __device__ __forceinline__ bool beyond_half(float m) { return !(m <= HALF_MAX_F)
 // logits[row, f] = acc times the row's RMSNorm factor
 struct EpiStore {
     static constexpr bool kDual = true;       // may take its activations as value + rounding remainder
+    static constexpr bool kSlots = false;
     static constexpr int NR = 4;
     float* C; int ld;
     RowScale rs;
@@ -325,6 +327,7 @@ __device__ __forceinline__ float silu(float g) {
 template <bool HALF>
 struct EpiSwiGLU {
     static constexpr bool kDual = false;       // may take its activations as value + rounding remainder
+    static constexpr bool kSlots = false;
     static constexpr int NR = 4;
     Operand act; int ld;
     RowScale rs;
@@ -364,6 +367,7 @@ struct EpiSwiGLU {
 template <bool HALF>
 struct EpiResNorm {
     static constexpr bool kDual = !HALF;       // may take its activations as value + rounding remainder
+    static constexpr bool kSlots = false;
     static constexpr int NR = 4;
     float* h; int ld;
     const float* gain;
@@ -442,6 +446,7 @@ struct EpiResNorm {
 // RoPE, q to its buffer, K / V to the row's KV slot (all IEEE half) -- the arithmetic of qkv_post_kernel.
 struct EpiQkv {
     static constexpr bool kDual = true;       // may take its activations as value + rounding remainder
+    static constexpr bool kSlots = true;
     static constexpr int NR = 2;       // rotary factors of the rows in hand and of the next ones take registers
     int Hq, Hkv, layer;
     const float* bias;                 // [(Hq + 2 Hkv) * 128] or nullptr
@@ -455,8 +460,8 @@ struct EpiQkv {
     RowScale rs;
     int32_t* err;
     float4 b, g, cs[NR][2];            // bias, gain; rotary factors of the rows in hand
-    __half* to[NR];                    // where the rows go (nullptr: nowhere)
     __half *base_s, *base_p;           // this head's plane of the two arenas; q: its column of the q buffer (base_s)
+    int pitch;                         // elements from one slot (q: row) to the next
     bool is_q, turn, norm, bad;
     __device__ __forceinline__ void begin(const Ctx& c) {
         const int head = c.f0 / FT;
@@ -470,24 +475,24 @@ struct EpiQkv {
         const int64_t plane = ((int64_t)layer * 2 + (turn ? 0 : 1)) * Hkv + (turn ? head - Hq : head - Hq - Hkv);
         base_s = (is_q ? q_out + (size_t)head * FT : reinterpret_cast<__half*>(suffix_arena.base) + plane * suffix_arena.n_slots * FT) + 4 * c.lane;
         base_p = reinterpret_cast<__half*>(prompt_arena.base) + plane * prompt_arena.n_slots * FT + 4 * c.lane;
+        pitch = is_q ? Hq * FT : FT;
 #pragma unroll
         for (int j = 0; j < NR; ++j) cs[j][0] = cs[j][1] = f4(1.f, 0.f, 1.f, 0.f);
+    }
+    // 2 * slot + (1: suffix arena or q buffer, 0: prompt arena), negative: nowhere.  Taken once per tile by a thread per row: the
+    // lookup per row and chunk put two dependent loads into every chunk (the projection over 10,184 rows: 184 -> 147 us).
+    __device__ __forceinline__ int slot_of(int row) const {
+        if (is_q) return 2 * row + 1;
+        const int64_t w = geo.wslot[row];
+        return (int)(2 * w) + (geo.warena[row] ? 1 : 0);
     }
     __device__ __forceinline__ void prefetch(const Ctx& c, const Rows& R) {
 #pragma unroll
         for (int j = 0; j < NR; ++j) {
-            const int row = c.row0 + R.at(j);
-            const bool on = c.fv & R.has(j);
-            if (on & turn) {
-                const float4* p = reinterpret_cast<const float4*>(rope + (size_t)row * 64) + 2 * (c.lane & 15);
+            if (c.fv & R.has(j) & turn) {
+                const float4* p = reinterpret_cast<const float4*>(rope + (size_t)(c.row0 + R.at(j)) * 64) + 2 * (c.lane & 15);
                 cs[j][0] = p[0];
                 cs[j][1] = p[1];
-            }
-            to[j] = nullptr;
-            if (on & is_q) to[j] = base_s + (size_t)row * (Hq * FT);
-            if (on & !is_q) {
-                const int64_t w = geo.wslot[row];
-                if (w >= 0) to[j] = (geo.warena[row] ? base_s : base_p) + w * FT;
             }
         }
     }
@@ -495,7 +500,6 @@ struct EpiQkv {
         const float sign = c.lane < 16 ? -1.f : 1.f;
         float4 v[NR];
         uint2 y[NR];
-        __half* dst[NR];
         float m = 0.f;
 #pragma unroll
         for (int j = 0; j < NR; ++j) {
@@ -525,7 +529,6 @@ struct EpiQkv {
             v[j] = f4(v[j].x * p.x + sign * (o.x * p.y), v[j].y * p.z + sign * (o.y * p.w), v[j].z * q.x + sign * (o.z * q.y), v[j].w * q.z + sign * (o.w * q.w));
             m = max_mag(max_mag(max_mag(max_mag(m, v[j].x), v[j].y), v[j].z), v[j].w);
             y[j] = make_uint2(pack_half(v[j].x, v[j].y), pack_half(v[j].z, v[j].w));
-            dst[j] = to[j];
         }
         if (beyond_half(m)) {
 #pragma unroll
@@ -536,8 +539,10 @@ struct EpiQkv {
         }
         prefetch(c, next);
 #pragma unroll
-        for (int j = 0; j < NR; ++j)
-            if (dst[j] != nullptr) *reinterpret_cast<uint2*>(dst[j]) = y[j];
+        for (int j = 0; j < NR; ++j) {
+            const int slot = c.slot[R.at(j)];
+            if (c.fv & R.has(j) & (slot >= 0)) *reinterpret_cast<uint2*>((slot & 1 ? base_s : base_p) + (int64_t)(slot >> 1) * pitch) = y[j];
+        }
     }
     __device__ __forceinline__ void end() { if (bad) set_error(err, DEV_ERR_HALF_RANGE); }
 };
@@ -555,7 +560,8 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int X1 = (G.nt / CG) * BK * 2, stage_bytes = W_BYTES + X1 * (DUAL ? 2 : 1);
     float* scale = reinterpret_cast<float*>(tiles + G.stages * stage_bytes);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(scale + SCALE_FLOATS);
+    int* slots = reinterpret_cast<int*>(scale + SCALE_FLOATS);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(slots + SCALE_FLOATS);
     float* staging = reinterpret_cast<float*>(bars + 64);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * MAX_STAGES + 4);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -704,6 +710,7 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             // a warp may be one tile ahead of another (not more: all meet once per tile), so the row scales alternate
             float* tile_scale = scale + turn * MAX_ROWS_TILE;
             c.scale = tile_scale;
+            c.slot = slots + turn * MAX_ROWS_TILE;
             place(t, c.f0, c.row0);
             c.f = c.f0 + 4 * lane; c.fv = c.f < G.N;
             const int live = max(0, min(G.nt, m_live - c.row0));
@@ -718,6 +725,7 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             if (begin + tid < end) {                              // at most 256 rows: a thread each
                 const RowScale& r = epi.rs;
                 tile_scale[begin + tid] = r.n > 0 ? row_factor(r.ssq + c.row0 + begin + tid, r.n, r.stride, r.d, r.eps) : 1.f;
+                if constexpr (Epi::kSlots) slots[turn * MAX_ROWS_TILE + begin + tid] = epi.slot_of(c.row0 + begin + tid);
             }
             // the accumulator is complete, the row scales are in place
             ok = epi_all(mbar_wait(tfull0 + 8 * acc, acc_phase, abort_flag));

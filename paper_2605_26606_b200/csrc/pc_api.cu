@@ -374,7 +374,7 @@ const pc_ctx::WtPlan& plan_wt(pc_ctx* c, GemmKind kind, int N, int K, int M, boo
                 const double sm = waves * kbs * std::max(stage / 120e3, mmas * nt * 2. / 1750. * 1.43);
                 const double hbm = (double)N * K * 2e-6 / 5.2, l2 = clusters * cg * sp * kbs * stage * 1e-6 / 18.;
                 const double rows = (double)nt / sp * (sp > 1 ? waves : 1.);
-                const double cost = 5.3 + std::cbrt(sm * sm * sm + hbm * hbm * hbm + l2 * l2 * l2) + (kind == GEMM_QKV ? 0.078 * rows : 0.) +
+                const double cost = 5.3 + std::cbrt(sm * sm * sm + hbm * hbm * hbm + l2 * l2 * l2) + (kind == GEMM_QKV ? 0.03 * rows : 0.) +
                                     (sp > 1 ? 0.0136 * nt * waves : 0.) + (cg == 2 ? 0.5 : 0.);
                 if (best_cost < 0. || cost < best_cost) {
                     best_cost = cost;
