@@ -118,11 +118,11 @@ __device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t addr) {
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
@@ -133,7 +133,7 @@ __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volat
     uint64_t began = 0;
 #pragma unroll 1
     for (uint32_t it = 0; it < tc::WAIT_LIMIT; ++it) {
-        if (mbar_try_wait_cluster(bar, parity)) return true;
+        if (mbar_try_wait(bar, parity)) return true;
         if ((it & 63u) == 63u) {
             uint64_t now;
             asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
@@ -145,7 +145,23 @@ __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volat
     return false;
 }
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-    return mbar_try_wait_cluster(bar, parity) || mbar_wait_slow(bar, parity, abort_flag);
+    return mbar_try_wait(bar, parity) || mbar_wait_slow(bar, parity, abort_flag);
+}
+// The whole warp waits; the same answer in every lane.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)) != 0;
+}
+// True in one lane, the same one each time.  The producer and the MMA issuer run their loops with the whole warp and elect a lane
+// where they issue: control and addresses stay in uniform registers, and the compiler knows that one thread issues.  A loop of
+// lane 0 alone took 0.34 us per k-block whatever the tile, which bounded every pass (gate/up of 16 rows: 8.2 us for 24 k-blocks).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(r) :: "memory");
+    return r != 0;
 }
 template <int CG> __device__ __forceinline__ void tmem_alloc(uint32_t dst, uint32_t cols) {
     if constexpr (CG == 1) {
@@ -606,7 +622,7 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
         asm volatile("bar.arrive 4, %0;" ::"n"(THREADS) : "memory");      // the barriers exist; the others meet here, this warp goes on
         // ---------------- TMA producer ----------------
         // Before the wait for the previous kernel the weight tile of every stage is requested, and nothing else.
-        if (lane == 0) {
+        {
             bool ok = true;
             int tile = cluster, kb = kb0, f0, r0;
             place(tile, f0, r0);
@@ -614,8 +630,10 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             int s = 0;
 #pragma unroll 1
             for (; s < stages && tile < n_tiles; ++s) {
-                if (peer == 0) mbar_arrive_expect_tx(full0 + 8 * s, CG * stage_bytes);
-                load_tile<CG>(tiles_u32 + s * stage_bytes, &map_w, full_at + 8 * s, kb * BK, f0);
+                if (elect_one()) {
+                    if (peer == 0) mbar_arrive_expect_tx(full0 + 8 * s, CG * stage_bytes);
+                    load_tile<CG>(tiles_u32 + s * stage_bytes, &map_w, full_at + 8 * s, kb * BK, f0);
+                }
                 if (++kb == kb1) { kb = kb0; tile += n_clusters; place(tile, f0, r0); }
             }
             int ahead = s;                          // stages whose weights are requested
@@ -628,20 +646,22 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
 #pragma unroll 1
             while (tile < n_tiles) {
                 const uint32_t at = tiles_u32 + s * stage_bytes, bar = full_at + 8 * s;
-                if (ahead > 0) {
-                    --ahead;
-                } else {
-                    if (!mbar_wait(empty0 + 8 * s, phase, abort_flag)) { ok = false; break; }
-                    if (peer == 0) mbar_arrive_expect_tx(full0 + 8 * s, CG * stage_bytes);
-                    load_tile<CG>(at, &map_w, bar, kb * BK, f0);
+                const bool requested = ahead > 0;
+                --ahead;
+                if (!requested && !mbar_wait_warp(empty0 + 8 * s, phase, abort_flag)) { ok = false; break; }
+                if (elect_one()) {
+                    if (!requested) {
+                        if (peer == 0) mbar_arrive_expect_tx(full0 + 8 * s, CG * stage_bytes);
+                        load_tile<CG>(at, &map_w, bar, kb * BK, f0);
+                    }
+                    const int r = r0 + (int)peer * (G.nt / CG);
+                    load_tile<CG>(at + W_BYTES, &map_x, bar, kb * BK, r);
+                    if (DUAL) load_tile<CG>(at + W_BYTES + X1, &map_x_lo, bar, kb * BK, r);
                 }
-                const int r = r0 + (int)peer * (G.nt / CG);
-                load_tile<CG>(at + W_BYTES, &map_x, bar, kb * BK, r);
-                if (DUAL) load_tile<CG>(at + W_BYTES + X1, &map_x_lo, bar, kb * BK, r);
                 if (++s == stages) { s = 0; phase ^= 1u; }
                 if (++kb == kb1) { kb = kb0; tile += n_clusters; place(tile, f0, r0); }
             }
-            if (!ok) { *abort_flag = 1; set_error(err, DEV_ERR_WAIT_TIMEOUT); }
+            if (!ok && lane == 0) { *abort_flag = 1; set_error(err, DEV_ERR_WAIT_TIMEOUT); }
         }
         __syncwarp();
     }
@@ -655,38 +675,43 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
         grid_dep_wait();                            // residual stream, row geometry, buffers to be overwritten
     }
     if (warp == 1) {
-        if (lane == 0 && peer == 0) {
+        if (peer == 0) {
             // ---------------- MMA issuer ----------------
             const uint32_t idesc = tc::make_idesc(FT * CG, G.nt, G.half != 0);
             const uint32_t pair = 3u << leader;
+            const uint64_t dw0 = tc::make_smem_desc(tiles_u32);          // of stage 0; only the address field (16-byte units) changes
+            const uint32_t step = stage_bytes >> 4;
             uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
             bool ok = true;
 #pragma unroll 1
             for (int t = cluster; t < n_tiles && ok; t += n_clusters) {
-                if (!mbar_wait(tempty0 + 8 * acc, acc_phase ^ 1u, abort_flag)) { ok = false; break; }
+                if (!mbar_wait_warp(tempty0 + 8 * acc, acc_phase ^ 1u, abort_flag)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t d = tmem_base + acc * acc_cols;
+                uint32_t add = 0;
 #pragma unroll 1
                 for (int kb = kb0; kb < kb1; ++kb) {
-                    if (!mbar_wait(full0 + 8 * stage, phase, abort_flag)) { ok = false; break; }
+                    if (!mbar_wait_warp(full0 + 8 * stage, phase, abort_flag)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t sw = tiles_u32 + stage * stage_bytes, sx = sw + W_BYTES;
-                    const uint64_t dw = tc::make_smem_desc(sw), dx = tc::make_smem_desc(sx);
+                    if (elect_one()) {
+                        const uint64_t dw = dw0 + stage * step, dx = dw + (W_BYTES >> 4);
 #pragma unroll
-                    for (int kk = 0; kk < BK / 16; ++kk) mma<CG>(d, dw + 2 * kk, dx + 2 * kk, idesc, (kb > kb0 || kk > 0) ? 1u : 0u);
-                    if (DUAL) {
-                        const uint64_t dl = tc::make_smem_desc(sx + X1);
+                        for (int kk = 0; kk < BK / 16; ++kk) mma<CG>(d, dw + 2 * kk, dx + 2 * kk, idesc, kk > 0 ? 1u : add);
+                        if (DUAL) {
+                            const uint64_t dl = dx + (X1 >> 4);
 #pragma unroll
-                        for (int kk = 0; kk < BK / 16; ++kk) mma<CG>(d, dw + 2 * kk, dl + 2 * kk, idesc, 1u);
+                            for (int kk = 0; kk < BK / 16; ++kk) mma<CG>(d, dw + 2 * kk, dl + 2 * kk, idesc, 1u);
+                        }
+                        commit<CG>(empty0 + 8 * stage, pair);
                     }
-                    commit<CG>(empty0 + 8 * stage, pair);
+                    add = 1;
                     if (++stage == (uint32_t)G.stages) { stage = 0; phase ^= 1u; }
                 }
                 if (!ok) break;
-                commit<CG>(tfull0 + 8 * acc, pair);
+                if (elect_one()) commit<CG>(tfull0 + 8 * acc, pair);
                 if (++acc == (uint32_t)G.n_acc) { acc = 0; acc_phase ^= 1u; }
             }
-            if (!ok) { *abort_flag = 1; set_error(err, DEV_ERR_WAIT_TIMEOUT); }
+            if (!ok && lane == 0) { *abort_flag = 1; set_error(err, DEV_ERR_WAIT_TIMEOUT); }
         }
         __syncwarp();
     } else if (warp > 1) {
