@@ -147,8 +147,10 @@ attn_prefix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
     const int tile0 = my_part * per_part, n_tiles = max(0, min(tiles_all, tile0 + per_part) - tile0);
 
     bool ok = true;
+    // one answer per warp: tensor-memory accesses need all its lanes, and producer and issuer elect one where they issue
+    auto warp_wait = [&](uint32_t bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)) != 0; };
     if (warp == 5) {
-        if (lane == 0) {
+        {
             // ---------------- TMA producer ----------------
             const int64_t kv_start = g.p_start[row0];
             const int64_t krow = (((int64_t)layer * 2 + 0) * Hkv + kvh) * n_slots + kv_start, vrow = (((int64_t)layer * 2 + 1) * Hkv + kvh) * n_slots + kv_start;
@@ -156,52 +158,60 @@ attn_prefix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
             for (int t = 0; t < n_tiles; ++t) {
                 const int s = t % STAGES;
                 const uint32_t kb = kv_u32 + s * 2 * KV_BYTES, vb = kb + KV_BYTES, ph = (uint32_t)(t / STAGES - 1) & 1u;
-                if (t >= STAGES && !mbar_wait(kempty0 + 8 * s, ph, abort_flag)) { ok = false; break; }
-                mbar_arrive_expect_tx(kfull0 + 8 * s, KV_BYTES);
-                tma_load_2d(kb, &kv_map, kfull0 + 8 * s, 0, (int)(krow + (int64_t)(tile0 + t) * TK));
-                tma_load_2d(kb + TK * 128, &kv_map, kfull0 + 8 * s, 64, (int)(krow + (int64_t)(tile0 + t) * TK));
-                if (t >= STAGES && !mbar_wait(vempty0 + 8 * s, ph, abort_flag)) { ok = false; break; }
-                mbar_arrive_expect_tx(vfull0 + 8 * s, KV_BYTES);
-                tma_load_2d(vb, &kv_map, vfull0 + 8 * s, 0, (int)(vrow + (int64_t)(tile0 + t) * TK));
-                tma_load_2d(vb + TK * 128, &kv_map, vfull0 + 8 * s, 64, (int)(vrow + (int64_t)(tile0 + t) * TK));
+                if (t >= STAGES && !warp_wait(kempty0 + 8 * s, ph)) { ok = false; break; }
+                if (wt::elect_one()) {
+                    mbar_arrive_expect_tx(kfull0 + 8 * s, KV_BYTES);
+                    tma_load_2d(kb, &kv_map, kfull0 + 8 * s, 0, (int)(krow + (int64_t)(tile0 + t) * TK));
+                    tma_load_2d(kb + TK * 128, &kv_map, kfull0 + 8 * s, 64, (int)(krow + (int64_t)(tile0 + t) * TK));
+                }
+                if (t >= STAGES && !warp_wait(vempty0 + 8 * s, ph)) { ok = false; break; }
+                if (wt::elect_one()) {
+                    mbar_arrive_expect_tx(vfull0 + 8 * s, KV_BYTES);
+                    tma_load_2d(vb, &kv_map, vfull0 + 8 * s, 0, (int)(vrow + (int64_t)(tile0 + t) * TK));
+                    tma_load_2d(vb + TK * 128, &kv_map, vfull0 + 8 * s, 64, (int)(vrow + (int64_t)(tile0 + t) * TK));
+                }
             }
         }
         __syncwarp();
     } else if (warp == 4) {
-        if (lane == 0 && n_tiles > 0) {
+        if (n_tiles > 0) {
             // ---------------- MMA issuer: S of the next tile goes ahead of this tile's P V ----------------
             const uint32_t idesc_s = tc::make_idesc(QROWS, TK, true), idesc_o = tc::make_idesc(QROWS, HD, true) | (1u << 16) /* V: MN-major */;
             auto issue_s = [&](int t) {
                 const int s = t % STAGES;
-                if (!mbar_wait(kfull0 + 8 * s, (uint32_t)(t / STAGES) & 1u, abort_flag)) return false;
+                if (!warp_wait(kfull0 + 8 * s, (uint32_t)(t / STAGES) & 1u)) return false;
                 tc_fence_after();
-                const uint64_t dq = tc::make_smem_desc(q_u32), dk = tc::make_smem_desc(kv_u32 + s * 2 * KV_BYTES);
+                if (wt::elect_one()) {
+                    const uint64_t dq = tc::make_smem_desc(q_u32), dk = tc::make_smem_desc(kv_u32 + s * 2 * KV_BYTES);
 #pragma unroll
-                for (int kk = 0; kk < HD / 16; ++kk) {
-                    // 64-column blocks of Q (128 rows) and K (TK rows), 32 bytes per 16 columns inside a block
-                    const uint32_t aq = (kk >> 2) * (QROWS * 128 >> 4) + (kk & 3) * 2, ak = (kk >> 2) * (TK * 128 >> 4) + (kk & 3) * 2;
-                    tc::umma_bf16(tmem + HD + (t & 1) * TK, dq + aq, dk + ak, idesc_s, kk > 0 ? 1u : 0u);
+                    for (int kk = 0; kk < HD / 16; ++kk) {
+                        // 64-column blocks of Q (128 rows) and K (TK rows), 32 bytes per 16 columns inside a block
+                        const uint32_t aq = (kk >> 2) * (QROWS * 128 >> 4) + (kk & 3) * 2, ak = (kk >> 2) * (TK * 128 >> 4) + (kk & 3) * 2;
+                        tc::umma_bf16(tmem + HD + (t & 1) * TK, dq + aq, dk + ak, idesc_s, kk > 0 ? 1u : 0u);
+                    }
+                    tc::umma_commit(kempty0 + 8 * s);
+                    tc::umma_commit(sfull0 + 8 * (t & 1));
                 }
-                tc::umma_commit(kempty0 + 8 * s);
-                tc::umma_commit(sfull0 + 8 * (t & 1));
                 return true;
             };
-            ok = mbar_wait(qready, 0, abort_flag);
+            ok = warp_wait(qready, 0);
             tc_fence_after();
             if (ok) ok = issue_s(0);
 #pragma unroll 1
             for (int t = 0; t < n_tiles && ok; ++t) {
                 if (t + 1 < n_tiles && !issue_s(t + 1)) { ok = false; break; }
                 const int s = t % STAGES;
-                if (!mbar_wait(vfull0 + 8 * s, (uint32_t)(t / STAGES) & 1u, abort_flag) || !mbar_wait(pready, (uint32_t)t & 1u, abort_flag)) { ok = false; break; }
+                if (!warp_wait(vfull0 + 8 * s, (uint32_t)(t / STAGES) & 1u) || !warp_wait(pready, (uint32_t)t & 1u)) { ok = false; break; }
                 tc_fence_after();
-                const uint64_t dp = tc::make_smem_desc(p_u32), dv = make_mn_desc(kv_u32 + s * 2 * KV_BYTES + KV_BYTES, TK * 128);
-                const int steps = min(TK, max_len - (tile0 + t) * TK + 15) / 16;       // groups of 16 keys that hold a visible one
-#pragma unroll 1
-                for (int kk = 0; kk < steps; ++kk)
-                    tc::umma_bf16(tmem, dp + kk * 2, dv + kk * (16 * 128 >> 4), idesc_o, (t > 0 || kk > 0) ? 1u : 0u);
-                tc::umma_commit(vempty0 + 8 * s);
-                tc::umma_commit(odone);
+                if (wt::elect_one()) {
+                    const uint64_t dp = tc::make_smem_desc(p_u32), dv = make_mn_desc(kv_u32 + s * 2 * KV_BYTES + KV_BYTES, TK * 128);
+                    const int steps = (max_len - (tile0 + t) * TK + 15) / 16;       // groups of 16 keys that hold a visible one
+#pragma unroll
+                    for (int kk = 0; kk < TK / 16; ++kk)
+                        if (kk < steps) tc::umma_bf16(tmem, dp + kk * 2, dv + kk * (16 * 128 >> 4), idesc_o, (t > 0 || kk > 0) ? 1u : 0u);
+                    tc::umma_commit(vempty0 + 8 * s);
+                    tc::umma_commit(odone);
+                }
             }
         }
         __syncwarp();
@@ -221,8 +231,6 @@ attn_prefix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
         __syncwarp();
         if (lane == 0) mbar_arrive(qready);
         const uint32_t lanes = tmem + ((uint32_t)(warp * 32) << 16);
-        // (one answer per warp: the tensor-memory accesses below need all its lanes)
-        auto warp_wait = [&](uint32_t bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)); };
         float m = -INFINITY, l = 0.f;
 #pragma unroll 1
         for (int t = 0; t < n_tiles; ++t) {
