@@ -8,6 +8,8 @@
 // output.
 #pragma once
 
+#include <type_traits>
+
 #include "attention_mma.cuh"
 #include "gemm_wt.cuh"
 
@@ -150,14 +152,24 @@ attn_suffix_team_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDe
                 for (int e = 0; e < EPL; ++e) acc[e] = __fmaf_rn(v[i][e], w, acc[e]);
             }
         }
-#pragma unroll 4
-        for (int k = 0; k < workers; ++k) {
-            const float w = __shfl_sync(0xffffffffu, wt_, k);
-            float x[EPL];
-            ld_cluster<EPL>(wt::map_rank(smem_u32(obuf + ((k % T_WARPS) * 8 + j) * HD + lane * EPL), (uint32_t)(k / T_WARPS)), x);
+        // sixteen reads in flight where a cluster shares the item: a read of another CTA's memory takes a quarter of a microsecond
+        auto add = [&](auto batch) {
+            constexpr int N = decltype(batch)::value;
+#pragma unroll 1
+            for (int k0 = 0; k0 < workers; k0 += N) {
+                float x[N][EPL];
 #pragma unroll
-            for (int e = 0; e < EPL; ++e) acc[e] = __fmaf_rn(x[e], w, acc[e]);      // (a worker without tiles left zeros)
-        }
+                for (int i = 0; i < N; ++i)
+                    ld_cluster<EPL>(wt::map_rank(smem_u32(obuf + ((i % T_WARPS) * 8 + j) * HD + lane * EPL), (uint32_t)min((k0 + i) / T_WARPS, team_ctas - 1)), x[i]);
+#pragma unroll
+                for (int i = 0; i < N; ++i) {
+                    const float w = __shfl_sync(0xffffffffu, wt_, (k0 + i) & 31);      // 0 from `workers` on
+#pragma unroll
+                    for (int e = 0; e < EPL; ++e) acc[e] = __fmaf_rn(x[i][e], w, acc[e]);      // (a worker without tiles left zeros)
+                }
+            }
+        };
+        if (team_ctas > 1) add(std::integral_constant<int, 16>{}); else add(std::integral_constant<int, T_WARPS>{});
         store_attention<HD>(lane, rh0 + j, acc, denom, out, out_lo, err);
     }
     // drain: tiles issued but not consumed must land before the shared memory is released

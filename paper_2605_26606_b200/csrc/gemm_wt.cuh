@@ -147,6 +147,15 @@ __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volat
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
     return mbar_try_wait(bar, parity) || mbar_wait_slow(bar, parity, abort_flag);
 }
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
 // The whole warp waits; the same answer in every lane.
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)) != 0;
@@ -689,12 +698,16 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
                 tc_fence_after();
                 const uint32_t d = tmem_base + acc * acc_cols;
                 uint32_t add = 0;
+                bool ready = false;                                  // the next stage was seen full while this one was issued
 #pragma unroll 1
                 for (int kb = kb0; kb < kb1; ++kb) {
-                    if (!mbar_wait_warp(full0 + 8 * stage, phase, abort_flag)) { ok = false; break; }
+                    if (!__all_sync(0xffffffffu, ready) && !mbar_wait_warp(full0 + 8 * stage, phase, abort_flag)) { ok = false; break; }
                     tc_fence_after();
+                    const uint32_t here = stage;
+                    if (++stage == (uint32_t)G.stages) { stage = 0; phase ^= 1u; }
+                    ready = mbar_test(full0 + 8 * stage, phase);
                     if (elect_one()) {
-                        const uint64_t dw = dw0 + stage * step, dx = dw + (W_BYTES >> 4);
+                        const uint64_t dw = dw0 + here * step, dx = dw + (W_BYTES >> 4);
 #pragma unroll
                         for (int kk = 0; kk < BK / 16; ++kk) mma<CG>(d, dw + 2 * kk, dx + 2 * kk, idesc, kk > 0 ? 1u : add);
                         if (DUAL) {
@@ -702,10 +715,9 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
 #pragma unroll
                             for (int kk = 0; kk < BK / 16; ++kk) mma<CG>(d, dw + 2 * kk, dl + 2 * kk, idesc, 1u);
                         }
-                        commit<CG>(empty0 + 8 * stage, pair);
+                        commit<CG>(empty0 + 8 * here, pair);
                     }
                     add = 1;
-                    if (++stage == (uint32_t)G.stages) { stage = 0; phase ^= 1u; }
                 }
                 if (!ok) break;
                 if (elect_one()) commit<CG>(tfull0 + 8 * acc, pair);

@@ -346,8 +346,8 @@ enum XBuf { X_A = 0, X_ATTN = 1, X_ACT = 2, X_A_LO = 3, X_ATTN_LO = 4 };
 // estimate of a candidate, in us: start, hand-over and drain of a launch + the main loop, a smooth maximum of what one SM takes
 // for its waves (its share of the ring's bytes, or the MMAs), of the weights' way from HBM and of all operand bytes' way from
 // L2 + the rows a CTA finishes (the QKV epilogue only: the others hide) + the hand-over of partial tiles.  Constants fitted to
-// 3,947 timed launches of the 1.5B and 8B shapes at 16 .. 2048 rows; over those the chosen candidate is 2 % slower than the
-// fastest one on average, 17 % at worst.
+// 3,947 timed launches of the 1.5B and 8B shapes at 16 .. 2048 rows; the rates of
+// the main loop then raised by a quarter with the issue loops (237 rows: 21.25 -> 20.63 ms per eight steps).
 // At most max_active[c] clusters of c CTAs with a whole SM's shared memory each are resident (the GPCs' SM counts).
 const pc_ctx::WtPlan& plan_wt(pc_ctx* c, GemmKind kind, int N, int K, int M, bool dual) {
     using namespace pc;
@@ -371,8 +371,8 @@ const pc_ctx::WtPlan& plan_wt(pc_ctx* c, GemmKind kind, int N, int K, int M, boo
                 if (stages < 3 || (sp > 1 && stages * stage < (nt + 8) * wt::FT * 4)) continue;
                 const double clusters = (double)features * tr, waves = std::ceil(clusters / max_active[cg * sp] * 148. / c->num_sms);
                 const double kbs = (double)kb / sp, mmas = dual ? 2. : 1.;
-                const double sm = waves * kbs * std::max(stage / 120e3, mmas * nt * 2. / 1750. * 1.43);
-                const double hbm = (double)N * K * 2e-6 / 5.2, l2 = clusters * cg * sp * kbs * stage * 1e-6 / 18.;
+                const double sm = waves * kbs * std::max(stage / 160e3, mmas * nt * 2. / 1750. * 1.43);
+                const double hbm = (double)N * K * 2e-6 / 6.2, l2 = clusters * cg * sp * kbs * stage * 1e-6 / 22.;
                 const double rows = (double)nt / sp * (sp > 1 ? waves : 1.);
                 const double cost = 5.3 + std::cbrt(sm * sm * sm + hbm * hbm * hbm + l2 * l2 * l2) + (kind == GEMM_QKV ? 0.03 * rows : 0.) +
                                     (sp > 1 ? 0.0136 * nt * waves : 0.) + (cg == 2 ? 0.5 : 0.);
