@@ -192,26 +192,22 @@ PC_API int pc_selftest_wait_timeout(void* stream, uint32_t spin_limit, int32_t* 
  * stated, not checked (the default). */
 PC_API int pc_set_index_bounds(pc_ctx* ctx, int n_prompts, int64_t n_tokens);
 
-/* bf16 models with half_gemm = 1 and head_dim 128, passes of more than 256 rows.  1 (the default): two row-wise kernels
- * of every layer run inside GEMM epilogues instead -- bias / QK-norm / RoPE / KV append in the QKV projection's, and the residual add, the operand of the
- * gate/up projection and the RMSNorm's sum of squares in the output projection's, the norm's 1/rms being applied by the
- * gate/up epilogue (RMSNorm(h; g) W^T = rstd * ((h * g) W^T)).  The two projections then run without K split, which is why
- * smaller passes keep the separate kernels (their projections need the split to fill the GPU).  0: one kernel per
- * operation throughout, as for every other model type.  A value n > 1: the fused form from passes of n rows on (a
- * measurement aid: below 257 rows it is slower).  Same mathematics, different rounding order (both inside the
- * tolerances the tests state).  Drops captured decode steps.  The paper has no counterpart. */
+/* bf16 models with head_dim 128.  1 (the default): every row-wise step of a layer runs inside GEMM epilogues -- bias / QK-norm /
+ * RoPE / KV append in the QKV projection's, the residual add, the next operand and its RMSNorm's sum of squares in the output
+ * and down projections', the norm's 1/rms being applied by the projection that reads the operand (RMSNorm(h; g) W^T =
+ * rstd * ((h * g) W^T)).  0: one kernel per operation throughout, as for every other model type.  A value n > 1: the fused form
+ * from passes of n rows on (a measurement aid).  Same mathematics, different rounding order (both inside the tolerances the
+ * tests state).  Drops captured decode steps.  The paper has no counterpart. */
 PC_API int pc_set_fused_epilogues(pc_ctx* ctx, int on);
 
 /* bf16 models.  mask: one bit per kernel (1 QKV, 2 output, 4 gate/up, 8 down projection, 16 LM head, 32 shared-prefix
  * attention of decode steps), 0 .. 63; the default is 63.  A kernel whose bit is set is launched as a programmatic
- * dependent of the kernel before it (a row norm, the QKV post-processing, the attention merge or a projection, all of
- * which signal their dependents as soon as they start).  A projection's CTAs set up their barriers and tensor memory
- * and request their first weight tiles while that kernel is still running; the attention kernel requests its first
- * prompt K/V tiles (written by an earlier call).  Both wait for the kernel before them (griddepcontrol.wait) before they
- * touch activations or any output.  Results are bit-identical to mask 0 (plain stream order); only the start of each
- * kernel moves.  Projections of passes of 129 .. 256 rows (two row tiles: measured slower with it) and steps that record
- * phase events (pc_profile_step) run in plain stream order whatever the mask.  Drops captured decode steps.  The paper
- * has no counterpart. */
+ * dependent of the kernel before it.  A projection's CTAs set up their barriers and tensor memory and request their first
+ * weight tiles while that kernel is still running; the attention kernels request prompt K/V an earlier call wrote.  All
+ * wait for the kernel before them (griddepcontrol.wait) before they touch activations or any output, and release their own
+ * dependents only after that.  Results are bit-identical to mask 0 (plain stream order); only the start of each kernel moves.
+ * Steps that record phase events (pc_profile_step) run in plain stream order whatever the mask, and so do the projections of
+ * passes of 129 .. 256 rows with one kernel per operation.  Drops captured decode steps.  The paper has no counterpart. */
 PC_API int pc_set_dependent_launch(pc_ctx* ctx, int mask);
 
 /* bf16 models, decode steps that only sample (no logits_out, no log-probability buffer): 1 draws the token in
@@ -256,7 +252,8 @@ PC_API size_t pc_chain_trace_words(const pc_ctx* ctx);
  *   LM_BEGIN | final RMSNorm + LM head | LM_HEAD | sampler | SAMPLE
  * so the time of an operation is the elapsed time between the marks around it.  One-shot; the caller synchronises
  * and reads the times.  float32 models run one attention kernel: GROUP is recorded before it, SUFFIX and MERGE after
- * it.  The paper has no counterpart. */
+ * it.  The suffix attention merges by itself: MERGE follows SUFFIX at once.  A norm or post-processing inside an epilogue leaves
+ * its two marks together in the same way.  The paper has no counterpart. */
 enum {
     PC_MARK_LAYER_BEGIN = 0, PC_MARK_NORM_ATTN, PC_MARK_QKV, PC_MARK_POST, PC_MARK_GROUP, PC_MARK_SUFFIX, PC_MARK_MERGE, PC_MARK_O,
     PC_MARK_NORM_MLP, PC_MARK_GATE_UP, PC_MARK_DOWN, PC_MARK_LM_BEGIN, PC_MARK_LM_HEAD, PC_MARK_SAMPLE, PC_PROFILE_MARKS
