@@ -14,8 +14,9 @@
 //   attn_suffix_kernel  one warp per (rollout, KV head, range of the suffix) streams the rollout's own suffix K/V
 //                       through a 3-stage TMA ring.  Positions sit on the MMA M axis (S^T = K Q^T,
 //                       O^T = V^T P^T), so the 6-8 query heads fill the N = 8 axis and no MMA work is
-//                       padded; P is transposed between the two MMAs with movmatrix.  It leaves its
-//                       (m, l, unnormalised O) record next to the prefix records.
+//                       padded; P is transposed between the two MMAs with movmatrix.  The warp that has
+//                       an item's whole suffix, or the last of the few that share it, merges it with the
+//                       prefix records into the attention output.
 //
 // Scores are kept in the log2 domain (scaled by log2(e) / sqrt(head_dim)) so that exp2f is the only
 // transcendental.  Waits on mbarriers are bounded (see gemm_tc.cuh).
@@ -389,7 +390,7 @@ template <int HD> constexpr int suffix_smem_bytes() {
 // head) item (cpi) for a step whose longest suffix has max_slen slots: among 1..MERGE_CHUNKS chunks per item, the
 // choice that minimises (units the busiest warp gets) x (tiles per unit + 4), the + 4 standing for the fixed cost of a
 // unit (length lookup, first TMA round trip, record) in tile times.  The same value serves every row of the step, and
-// the merge kernel recomputes it from the same inputs.
+// the warp that merges recomputes it from the same inputs.
 struct SuffixPlan { int ct, cpi; };
 __device__ __forceinline__ SuffixPlan suffix_plan(int max_slen, int n_items, int n_warps) {
     const int ntiles = max(1, (max_slen + S_TP - 1) / S_TP);
