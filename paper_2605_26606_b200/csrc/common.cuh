@@ -89,6 +89,13 @@ __device__ __forceinline__ float half_guard(float x, int32_t* err) {
     return half_clamp(x);
 }
 
+// Power of two a projection's epilogue puts into the next norm's half operand in place of 1/rms, which it does not know yet: 2^-4
+// times this norm's, rounded down (gemm_wt.cuh, RowScale).
+__device__ __forceinline__ float operand_scale(float rstd) {
+    const float r = fminf(fmaxf(rstd, 0x1p-60f), 0x1p60f);          // (NaN: the lower bound)
+    return __uint_as_float((__float_as_uint(r) & 0x7f800000u) - (4u << 23));
+}
+
 template <typename T> __device__ __forceinline__ float to_f32(T v);
 template <> __device__ __forceinline__ float to_f32<float>(float v) { return v; }
 template <> __device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }

@@ -258,7 +258,7 @@ struct Ctx {
     int f;                  // first of this lane's four features
     bool fv;                // they exist (the number of features is a multiple of 4, except for logits)
     int row0;               // first row of the tile
-    const float* scale;     // RMSNorm factor per row of the tile
+    const float* scale;     // per row of the tile: RMSNorm factor (ResNorm: power of two of the operand)
     const int* slot;        // where each row of the tile goes (epilogues with kSlots)
 };
 // Rows r + j * step, j < NR, of the tile; those below `end` exist.
@@ -268,23 +268,81 @@ struct Rows {
     __device__ __forceinline__ bool has(int j) const { return r + j * step < end; }
 };
 
-// RMSNorm factor of a row, rsqrt(sum of squares / d + eps), from the sums a ResNorm epilogue left per feature tile.
+// The RMSNorm a ResNorm epilogue left unfinished.  It wrote half(h * gain * used) with a power of two per row and the row's sum of
+// squares per feature tile; what the accumulators still lack is rstd / used, rstd = rsqrt(sum / d + eps).
+//
+// The power of two keeps the operand inside half's range whatever the size of the residual stream: it is 2^-4 / rms, rounded down,
+// of the row one norm earlier (operand_scale), so the mantissas are those of half(h * gain) and the values are about 2^-4 times
+// the normalised ones.  That leaves room for an rms that grows 2^10-fold within a sublayer at a gain of 8 and a row whose
+// whole weight sits in one element, and for one that shrinks 2^6-fold (factor 2^10) before half's subnormals cost more than 2^-15 of
+// the row's rms, an eighth of its rounding.  A row outside that room is not multiplied from its operand: the ResNorm tile that met an
+// overflow leaves its sum with the sign set, row_factor answers with -rstd, and the consumer's epilogue takes the row's products
+// from the residual stream itself (rescue_rows), rounded as the plain norm rounds them.
+// Measured beside the same kernels without any of this: no case differs by more than two runs of one side (16 rows 10.51 -> 10.52 ms
+// per eight steps, 351-token prefill 2.10 -> 2.06 ms); the same rescue per row inside the chunk loop cost 2 % at 16-351 rows.
 struct RowScale {
     const float* ssq; int n, stride, d; float eps;      // ssq[n][stride]; n == 0: the operand is complete
+    const float* used;             // per row: the power of two in the operand (nullptr: none).  ResNorm: the one to put there
+    float* next;                   // per row: operand_scale of this norm, for the ResNorm that follows (or nullptr)
+    const void* w; const float* h; const float* gain;      // weights, residual stream and gain for rescue_rows
 };
 
-// The entries are added in order (every consumer gets the same bits), sixteen loads in flight at a time.
-__device__ __forceinline__ float row_factor(const float* __restrict__ p, int n, int stride, int d, float eps) {
-    float s = 0.f;
+constexpr float MAX_FACTOR = 1024.f;
+// What the accumulators of `row` are to be multiplied with, or -rstd (never zero) when the operand does not hold the row.  The
+// entries are added in order (every consumer gets the same bits), sixteen loads in flight at a time.
+__device__ __forceinline__ float row_factor(const RowScale& r, int row, bool keep_next) {
+    const float* __restrict__ p = r.ssq + row;
+    const float u = r.used != nullptr ? r.used[row] : 1.f;
+    float s = 0.f, low = 0.f;
 #pragma unroll 1
-    for (int e = 0; e < n; e += 16) {
+    for (int e = 0; e < r.n; e += 16) {
         float x[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) x[i] = e + i < n ? p[(size_t)(e + i) * stride] : 0.f;
+        for (int i = 0; i < 16; ++i) x[i] = e + i < r.n ? p[(size_t)(e + i) * r.stride] : 0.f;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) s += x[i];
+        for (int i = 0; i < 16; ++i) { s += fabsf(x[i]); low = fminf(low, x[i]); }
     }
-    return rsqrtf(s / (float)d + eps);
+    const float rstd = rsqrtf(s / (float)r.d + r.eps);
+    if (keep_next && r.next != nullptr) r.next[row] = operand_scale(rstd);
+    if (r.used == nullptr) return rstd;
+    const float f = rstd * __uint_as_float(0x7f000000u - __float_as_uint(u));       // 1 / u of a power of two
+    return (low < 0.f) | !(f <= MAX_FACTOR) ? -fmaxf(rstd, 1e-37f) : f;             // (a NaN row too)
+}
+
+// Rows of a complete accumulator tile whose operand does not hold them (scale < 0, that is -rstd): this CTA's share k0 .. k1 of their
+// products from the residual stream, the operand rounded as the plain norm rounds it (half, range-guarded), put in the place of
+// the accumulators, and the factor left is 1.  All epilogue threads; a thread has a feature, its group every other row.
+__device__ __forceinline__ void rescue_rows(const __half* __restrict__ w_row, const float* __restrict__ h, const float* __restrict__ gain, int K,
+                                            int k0, int k1, int live, float* scale, uint32_t taddr, int group, int32_t* err) {
+    int bad = 0;
+#pragma unroll 1
+    for (int p = group; p < live; p += 2) {
+        const float rstd = -scale[p];
+        if (!(rstd > 0.f)) continue;
+        const float* __restrict__ h_row = h + (size_t)p * K;
+        float y[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+        for (int k = k0; k < k1; k += 4) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float v = h_row[k + i] * rstd * gain[k + i];
+                bad |= half_bad(v);
+                const float a = __half2float(__float2half_rn(half_clamp(v)));
+                if (w_row != nullptr) y[i] = fmaf(a, __half2float(w_row[k + i]), y[i]);
+            }
+        }
+        const uint32_t sum = __float_as_uint((y[0] + y[1]) + (y[2] + y[3]));
+        __syncwarp();
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr + p), "r"(sum) : "memory");
+    }
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    if (bad) set_error(err, DEV_ERR_HALF_RANGE);
+    tc_fence_before();
+    asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory");
+    tc_fence_after();
+    for (int p = (int)threadIdx.x - 64; p < live; p += EPI_THREADS)
+        if (scale[p] < 0.f) scale[p] = 1.f;
+    asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory");
 }
 
 // A 16-bit GEMM operand: IEEE half (range-guarded), or bfloat16 with an optional rounding remainder.
@@ -302,6 +360,16 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 }
 __device__ __forceinline__ float bf16_rest(float v) { return v - __bfloat162float(__float2bfloat16_rn(v)); }
 __device__ __forceinline__ float4 f4(float a, float b, float c, float d) { return make_float4(a, b, c, d); }
+// Element products, two per instruction.
+__device__ __forceinline__ float4 mul4(float4 a, float4 b) {
+    float4 y;
+    asm("{\n\t.reg .b64 a, b;\n\t"
+        "mov.b64 a, {%4, %5}; mov.b64 b, {%8, %9}; mul.rn.f32x2 a, a, b; mov.b64 {%0, %1}, a;\n\t"
+        "mov.b64 a, {%6, %7}; mov.b64 b, {%10, %11}; mul.rn.f32x2 a, a, b; mov.b64 {%2, %3}, a;\n\t}"
+        : "=f"(y.x), "=f"(y.y), "=f"(y.z), "=f"(y.w)
+        : "f"(a.x), "f"(a.y), "f"(a.z), "f"(a.w), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w));
+    return y;
+}
 // Largest magnitude, NaN when there is one: one instruction per value finds whether a batch fits half; only a batch that does
 // not is clamped.
 __device__ __forceinline__ float max_mag(float m, float v) {
@@ -314,6 +382,7 @@ __device__ __forceinline__ bool beyond_half(float m) { return !(m <= HALF_MAX_F)
 // logits[row, f] = acc times the row's RMSNorm factor
 struct EpiStore {
     static constexpr bool kDual = true;       // may take its activations as value + rounding remainder
+    static constexpr bool kScaled = true;     // the operand may lack its norm's factor
     static constexpr bool kSlots = false;
     static constexpr int NR = 4;
     float* C; int ld;
@@ -353,6 +422,7 @@ __device__ __forceinline__ float silu(float g) {
 template <bool HALF>
 struct EpiSwiGLU {
     static constexpr bool kDual = false;       // may take its activations as value + rounding remainder
+    static constexpr bool kScaled = HALF;
     static constexpr bool kSlots = false;
     static constexpr int NR = 4;
     Operand act; int ld;
@@ -388,23 +458,22 @@ struct EpiSwiGLU {
     __device__ __forceinline__ void end() { if (HALF && bad) set_error(err, DEV_ERR_HALF_RANGE); }
 };
 
-// h[row, f] += acc;  the next norm's operand a[row, f] = h * gain WITHOUT its 1/rms factor;  ssq[f / 128][row] = the tile's
-// share of the row's sum of squares (the consumer applies rsqrt(sum / d + eps)).  gain == nullptr: only the residual add.
+// h[row, f] += acc;  the next norm's operand a[row, f] = h * gain (half: times the row's power of two) WITHOUT its 1/rms factor;
+// ssq[f / 128][row] = the tile's share of the row's sum of squares, with the sign set where the operand left half's range (see
+// RowScale).  gain == nullptr: only the residual add.
 template <bool HALF>
 struct EpiResNorm {
     static constexpr bool kDual = !HALF;       // may take its activations as value + rounding remainder
+    static constexpr bool kScaled = false;
     static constexpr bool kSlots = false;
     static constexpr int NR = 4;
     float* h; int ld;
     const float* gain;
     Operand a;
     float* ssq; int ssq_stride;
-    RowScale rs;                     // unused: the operand of these projections is complete
-    int32_t* err;
+    RowScale rs;                     // only `used`: the operand of these projections is complete
     float4 g, res[NR];
-    bool bad;
     __device__ __forceinline__ void begin(const Ctx& c) {
-        bad = false;
         g = gain != nullptr && c.fv ? *reinterpret_cast<const float4*>(gain + c.f) : f4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int j = 0; j < NR; ++j) res[j] = f4(0.f, 0.f, 0.f, 0.f);
@@ -433,16 +502,20 @@ struct EpiResNorm {
 #pragma unroll
         for (int j = 0; j < NR; ++j) {
             s[j] = v[j].x * v[j].x + v[j].y * v[j].y + v[j].z * v[j].z + v[j].w * v[j].w;
-            v[j] = f4(v[j].x * g.x, v[j].y * g.y, v[j].z * g.z, v[j].w * g.w);
+            v[j] = mul4(v[j], g);
+            if (HALF) { const float u = c.scale[R.at(j)]; v[j] = mul4(v[j], f4(u, u, u, u)); }
             if (HALF) m = max_mag(max_mag(max_mag(max_mag(m, v[j].x), v[j].y), v[j].z), v[j].w);
             y[j] = HALF ? make_uint2(pack_half(v[j].x, v[j].y), pack_half(v[j].z, v[j].w)) : make_uint2(pack_bf16(v[j].x, v[j].y), pack_bf16(v[j].z, v[j].w));
         }
-        if (HALF && beyond_half(m)) {
+        uint32_t sign = 0;               // of the sum this lane stores: set when its row does not fit half
+        if (HALF && __any_sync(0xffffffffu, beyond_half(m))) {
+            uint32_t over = 0;           // bit j: row j (rows behind the last hold anything and store nothing)
 #pragma unroll
             for (int j = 0; j < NR; ++j) {
-                bad |= R.has(j) & (beyond_half(v[j].x) | beyond_half(v[j].y) | beyond_half(v[j].z) | beyond_half(v[j].w));
+                if (c.fv & (beyond_half(v[j].x) | beyond_half(v[j].y) | beyond_half(v[j].z) | beyond_half(v[j].w))) over |= 1u << j;
                 y[j] = make_uint2(pack_half_clamped(v[j].x, v[j].y), pack_half_clamped(v[j].z, v[j].w));
             }
+            sign = __reduce_or_sync(0xffffffffu, over) >> (c.lane >> 3) << 31;
         }
 #pragma unroll
         for (int j = 0; j < NR; ++j, op += step)
@@ -463,15 +536,17 @@ struct EpiResNorm {
         t += __shfl_xor_sync(0xffffffffu, t, 2);
         t += __shfl_xor_sync(0xffffffffu, t, 1);
         const int j = c.lane >> 3;                       // lane bits 4 and 3 chose the row
+        if (HALF) t = __uint_as_float(__float_as_uint(t) ^ sign);
         if (((c.lane & 7) == 0) & R.has(j)) ssq[(size_t)(c.f0 / FT) * ssq_stride + c.row0 + R.at(j)] = t;
     }
-    __device__ __forceinline__ void end() { if (HALF && bad) set_error(err, DEV_ERR_HALF_RANGE); }
+    __device__ __forceinline__ void end() {}
 };
 
 // QKV projection, head_dim 128 = one feature tile per head: RMSNorm factor of the row, bias, per-head RMSNorm of q and k,
 // RoPE, q to its buffer, K / V to the row's KV slot (all IEEE half) -- the arithmetic of qkv_post_kernel.
 struct EpiQkv {
     static constexpr bool kDual = true;       // may take its activations as value + rounding remainder
+    static constexpr bool kScaled = true;
     static constexpr bool kSlots = true;
     static constexpr int NR = 2;       // rotary factors of the rows in hand and of the next ones take registers
     int Hq, Hkv, layer;
@@ -591,6 +666,7 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     float* staging = reinterpret_cast<float*>(bars + 64);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * MAX_STAGES + 4);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    volatile int* outside_tile = abort_flag + 1;       // [2] the last tile (plus one) of this parity that has rows its operand does not hold
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
@@ -617,6 +693,7 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
         mbar_init(tfull0, 1); mbar_init(tfull0 + 8, 1);
         mbar_init(tempty0, CG * EPI_WARPS); mbar_init(tempty0 + 8, CG * EPI_WARPS);
         *abort_flag = 0;
+        outside_tile[0] = outside_tile[1] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -738,6 +815,7 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
         const uint32_t tempty_at = CG == 2 ? map_rank(tempty0, leader) : tempty0;
         const int share = G.share;                               // rows of a tile this CTA finishes (all, or its share of a split)
         constexpr int NR = Epi::NR;
+        constexpr bool kRescue = Epi::kScaled && !DUAL;
         const int cw = chunk_rows(G.nt, NR);
         float* stage = staging + group * cw * FT;
         uint32_t acc = 0, acc_phase = 0;
@@ -760,16 +838,23 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             auto rows_of = [&](int p) { return G.splits > 1 ? Rows{p, 8, end} : Rows{p + quarter, 4, min(live, p + cw)}; };
             epi.begin(c);
             epi.prefetch(c, rows_of(at));
-            if (begin + tid < end) {                              // at most 256 rows: a thread each
+            if (tid < live) {                                     // at most 256 rows: a thread each
                 const RowScale& r = epi.rs;
-                tile_scale[begin + tid] = r.n > 0 ? row_factor(r.ssq + c.row0 + begin + tid, r.n, r.stride, r.d, r.eps) : 1.f;
-                if constexpr (Epi::kSlots) slots[turn * MAX_ROWS_TILE + begin + tid] = epi.slot_of(c.row0 + begin + tid);
+                const int row = c.row0 + tid;
+                const float s = r.n > 0 ? row_factor(r, row, c.f0 == 0 && split == 0) : (r.used != nullptr ? r.used[row] : 1.f);
+                tile_scale[tid] = s;
+                if (kRescue && s < 0.f) outside_tile[turn] = t + 1;
+                if constexpr (Epi::kSlots) slots[turn * MAX_ROWS_TILE + tid] = epi.slot_of(row);
             }
             // the accumulator is complete, the row scales are in place
             ok = epi_all(mbar_wait(tfull0 + 8 * acc, acc_phase, abort_flag));
             if (!ok) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * acc_cols;
+            if constexpr (kRescue)
+                if (outside_tile[turn] == t + 1)
+                    rescue_rows(c.f0 + lane128 < G.N ? reinterpret_cast<const __half*>(epi.rs.w) + (size_t)(c.f0 + lane128) * G.K : nullptr,
+                                epi.rs.h + (size_t)c.row0 * G.K, epi.rs.gain, G.K, kb0 * BK, kb1 * BK, live, tile_scale, taddr, group, err);
             if (G.splits > 1) {
                 // leave the partial tile in this CTA's shared memory (the operand ring is drained) for the cluster
                 float* part = reinterpret_cast<float*>(tiles) + lane128;

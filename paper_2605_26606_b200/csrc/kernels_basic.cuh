@@ -193,7 +193,7 @@ __device__ __forceinline__ float sq4(float4 v) {
 template <typename T>
 __device__ __forceinline__ void norm_row_warp(int lane, int d, float* __restrict__ h_row, Partials pend, size_t pend_row,
                                               const float* __restrict__ gain, float eps, T* __restrict__ a_row,
-                                              T* __restrict__ a_lo_row, int half_out, int32_t* err = nullptr) {
+                                              T* __restrict__ a_lo_row, int half_out, int32_t* err = nullptr, float* next_scale = nullptr) {
     const int n4 = d >> 2;
     float4* x = reinterpret_cast<float4*>(h_row);
     float seg[NORM_SEGS];
@@ -219,6 +219,7 @@ __device__ __forceinline__ void norm_row_warp(int lane, int d, float* __restrict
 #pragma unroll
         for (int g = 0; g < NORM_SEGS; ++g) ss = __fadd_rn(ss, warp_sum(seg[g]));
         const float rstd = rsqrtf(__fadd_rn(__fdiv_rn(ss, (float)d), eps));
+        if (next_scale != nullptr && lane == 0) *next_scale = operand_scale(rstd);
 #pragma unroll
         for (int k = 0; k < NORM_REG4; ++k) {
             const int i = lane + 32 * k;
@@ -245,6 +246,7 @@ __device__ __forceinline__ void norm_row_warp(int lane, int d, float* __restrict
 #pragma unroll
     for (int g = 0; g < NORM_SEGS; ++g) ss = __fadd_rn(ss, warp_sum(seg[g]));
     const float rstd = rsqrtf(__fadd_rn(__fdiv_rn(ss, (float)d), eps));
+    if (next_scale != nullptr && lane == 0) *next_scale = operand_scale(rstd);
     for (int i = lane; i < n4; i += 32) {
         const float4 v = x[i], gg = *reinterpret_cast<const float4*>(gain + 4 * i);     // this lane's own writes
         store_norm_out<T>(a_row, a_lo_row, i, make_float4(v.x * rstd * gg.x, v.y * rstd * gg.y, v.z * rstd * gg.z, v.w * rstd * gg.w), half_out, err);
@@ -258,7 +260,7 @@ __device__ __forceinline__ void norm_row_warp(int lane, int d, float* __restrict
 template <typename T, int KK>
 __device__ __forceinline__ bool norm_row_cta_kk(int w, int lane, int d, float* __restrict__ h_row, Partials pend, size_t pend_row,
                                                 const float* __restrict__ gain, float eps, T* __restrict__ a_row, T* __restrict__ a_lo_row,
-                                                int half_out, volatile float* red, int* counter, int32_t* err) {
+                                                int half_out, volatile float* red, int* counter, int32_t* err, float* next_scale) {
     const int n4 = d >> 2;
     float4* x = reinterpret_cast<float4*>(h_row);
     float4 v[KK], gg[KK];
@@ -296,6 +298,7 @@ __device__ __forceinline__ bool norm_row_cta_kk(int w, int lane, int d, float* _
 #pragma unroll
     for (int g = 0; g < NORM_SEGS; ++g) ss = __fadd_rn(ss, red[g]);
     const float rstd = rsqrtf(__fadd_rn(__fdiv_rn(ss, (float)d), eps));
+    if (next_scale != nullptr && w == 0 && lane == 0) *next_scale = operand_scale(rstd);
 #pragma unroll
     for (int kk = 0; kk < KK; ++kk) {
         const int i = lane + 32 * (w + NORM_SEGS * kk);
@@ -310,11 +313,11 @@ __device__ __forceinline__ bool norm_row_fits_cta(int d) { return ((d >> 2) + 31
 template <typename T>
 __device__ __forceinline__ bool norm_row_cta(int w, int lane, int d, float* __restrict__ h_row, Partials pend, size_t pend_row,
                                              const float* __restrict__ gain, float eps, T* __restrict__ a_row, T* __restrict__ a_lo_row,
-                                             int half_out, volatile float* red, int* counter, int32_t* err = nullptr) {
+                                             int half_out, volatile float* red, int* counter, int32_t* err = nullptr, float* next_scale = nullptr) {
     const int nk = ((d >> 2) + 31) / 32;
-    if (nk <= NORM_SEGS * 2) return norm_row_cta_kk<T, 2>(w, lane, d, h_row, pend, pend_row, gain, eps, a_row, a_lo_row, half_out, red, counter, err);
-    if (nk <= NORM_SEGS * 4) return norm_row_cta_kk<T, 4>(w, lane, d, h_row, pend, pend_row, gain, eps, a_row, a_lo_row, half_out, red, counter, err);
-    return norm_row_cta_kk<T, 8>(w, lane, d, h_row, pend, pend_row, gain, eps, a_row, a_lo_row, half_out, red, counter, err);
+    if (nk <= NORM_SEGS * 2) return norm_row_cta_kk<T, 2>(w, lane, d, h_row, pend, pend_row, gain, eps, a_row, a_lo_row, half_out, red, counter, err, next_scale);
+    if (nk <= NORM_SEGS * 4) return norm_row_cta_kk<T, 4>(w, lane, d, h_row, pend, pend_row, gain, eps, a_row, a_lo_row, half_out, red, counter, err, next_scale);
+    return norm_row_cta_kk<T, 8>(w, lane, d, h_row, pend, pend_row, gain, eps, a_row, a_lo_row, half_out, red, counter, err, next_scale);
 }
 
 // h_row[:] = E[token, :] as float (the residual stream), one warp per row; d is a multiple of 8.
@@ -330,12 +333,13 @@ __device__ __forceinline__ void embed_row_warp(int lane, int d, const T* __restr
 constexpr int ROW_WARPS = 8;         // items per block of the stand-alone per-(row, head) kernels
 constexpr int NORM_THREADS = NORM_SEGS * 32;
 
-// h[r, :] = E[token[r], :] (float residual stream); a[r, :] = RMSNorm(h[r, :]; gain) in storage type T.  One block per row.
+// h[r, :] = E[token[r], :] (float residual stream); a[r, :] = RMSNorm(h[r, :]; gain) in storage type T.  next_scale (or nullptr):
+// operand_scale per row, for the output projection's epilogue.  One block per row.
 template <typename T>
 __global__ void __launch_bounds__(NORM_THREADS) embed_rmsnorm_kernel(const StepDesc* __restrict__ sd, int d, const int32_t* token,
                                                                      const T* __restrict__ embed, const float* __restrict__ gain, float eps,
                                                                      float* __restrict__ h, T* __restrict__ a, T* __restrict__ a_lo, int half_out,
-                                                                     int32_t* err) {
+                                                                     int32_t* err, float* __restrict__ next_scale) {
     __shared__ float red[8];
     __shared__ int counter;
     const int r = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -343,6 +347,7 @@ __global__ void __launch_bounds__(NORM_THREADS) embed_rmsnorm_kernel(const StepD
     if (r >= sd->n_rows) return;
     if (threadIdx.x == 0) counter = 0;
     const T* e_row = embed + (size_t)token[r] * d;
+    float* next = next_scale ? next_scale + r : nullptr;
     float* h_row = h + (size_t)r * d;
     for (int i = threadIdx.x; i < (d >> 2); i += NORM_THREADS) {
         float v[4];
@@ -352,10 +357,10 @@ __global__ void __launch_bounds__(NORM_THREADS) embed_rmsnorm_kernel(const StepD
     __syncthreads();
     if (norm_row_fits_cta(d))
         norm_row_cta<T>(w, lane, d, h_row, Partials{nullptr, 0, 0, 0}, 0, gain, eps, a + (size_t)r * d, a_lo ? a_lo + (size_t)r * d : nullptr,
-                        half_out, red, &counter, err);
+                        half_out, red, &counter, err, next);
     else if (w == 0)
         norm_row_warp<T>(lane, d, h_row, Partials{nullptr, 0, 0, 0}, 0, gain, eps, a + (size_t)r * d, a_lo ? a_lo + (size_t)r * d : nullptr,
-                         half_out, err);
+                         half_out, err, next);
 }
 
 // Optional residual update followed by the norm:  h[row, :] += pending partial sums of row;  a[r, :] = RMSNorm(h[row, :]; gain)

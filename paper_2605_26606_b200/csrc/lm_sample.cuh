@@ -55,7 +55,7 @@ struct EpiSample {
     const int32_t* step_key;
     int32_t* row_bound;            // per row: running lower bound of the final second-best score (ordered-int form)
     const DecodeArgsDev* da;       // temperature and seed
-    wt::RowScale rs;               // RMSNorm factor the operand still lacks (n == 0: none)
+    const float* factor;           // per row: RMSNorm factor the operand still lacks (nullptr: none), from final_factor_kernel
     __device__ __forceinline__ void set_rows(int) {}
 
     // scored iff (2^23 - (w >> 9)) < the returned word: the candidate's noise could lift it above `second`
@@ -76,7 +76,7 @@ struct EpiSample {
             if (live) rec[(size_t)(2 * (n0_tile / BN) + part) * m_stride + row] = Top2Rec{-INFINITY, -INFINITY, 0x7fffffff, 0};
             return;
         }
-        const float scale = rs.n > 0 && live ? wt::row_factor(rs.ssq + row, rs.n, rs.stride, rs.d, rs.eps) : 1.f;
+        const float scale = factor != nullptr && live ? factor[row] : 1.f;
         float lmax = -INFINITY;
 #pragma unroll 1
         for (int c = 0; c < n_cols; c += 32) {
@@ -132,6 +132,26 @@ struct EpiSample {
         }
     }
 };
+
+// The factor of the final norm per row, for EpiSample.  A row whose operand does not hold it (wt::RowScale) gets the complete one
+// and the factor 1.  One block per row.
+constexpr int FINAL_FACTOR_THREADS = 128;
+__global__ void __launch_bounds__(FINAL_FACTOR_THREADS) final_factor_kernel(const StepDesc* __restrict__ sd, const wt::RowScale rs, uint16_t* __restrict__ a,
+                                                                            float* __restrict__ factor, int32_t* err) {
+    const int r = blockIdx.x;
+    grid_dep_launch_dependents();          // the LM head may set itself up and request its first weight tiles
+    if (r >= sd->n_rows) return;
+    const float f = wt::row_factor(rs, r, false);
+    if (threadIdx.x == 0) factor[r] = f >= 0.f ? f : 1.f;
+    if (f >= 0.f) return;
+    int bad = 0;
+    for (int i = threadIdx.x; i < rs.d; i += FINAL_FACTOR_THREADS) {
+        const float v = rs.h[(size_t)r * rs.d + i] * -f * rs.gain[i];
+        bad |= half_bad(v);
+        a[(size_t)r * rs.d + i] = __half_as_ushort(__float2half_rn(half_clamp(v)));
+    }
+    if (bad) set_error(err, DEV_ERR_HALF_RANGE);
+}
 
 // One block of 128 threads per row: folds the row's records of all half tiles (the merge is order-independent: equal scores
 // keep the lowest id) and stores the token.  A thread's loads are issued four at a time.

@@ -85,7 +85,7 @@ constexpr int kMaxSplits = pc::PARTIALS_MAX;
 struct Carve {
     size_t h, a, qkv, q, attn, act, logits, rope, pos, wslot, warena, p_start, p_len, s_start, s_len, token, last_row,
         part_m, part_l, part_o, arrived, res_part, step_desc, step_counter, max_slen, sample_scratch, a_lo, attn_lo, chain_layers, chain_glob,
-        chain_bar, dargs, key_prompt, key_rollout, key_step, out_index, group_start, sample_tiles, sample_bound, ssq, total;
+        chain_bar, dargs, key_prompt, key_rollout, key_step, out_index, group_start, sample_tiles, sample_bound, ssq, row_pow2, total;
 };
 
 // A captured decode step, replayable for every step that fits the same upper bounds on the same KV arenas.  The
@@ -226,6 +226,7 @@ Carve carve(const pc_ctx* c, int max_rows, int max_prefill) {
     v.out_index = take(M * 8);
     v.group_start = take((M + 1) * 4);
     v.ssq = take((size_t)((d.d_model + 63) / 64) * M * 4);       // per-tile sums of squares of the residual rows (EpiResNorm)
+    v.row_pow2 = take(3 * M * 4);       // powers of two of the attention and MLP norms' half operands, factors of the final norm (EpiSample)
     // fused LM head + sampler: one record per (vocabulary tile of the narrowest tile width, row)
     v.sample_tiles = take(2 * (size_t)((d.vocab + 63) / 64) * (size_t)std::max(max_rows, 1) * sizeof(pc::Top2Rec));   // one record per half tile
     v.sample_bound = take((size_t)std::max(max_rows, 1) * sizeof(int32_t));
@@ -652,6 +653,9 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
     const bool wt_path = !kF32 && use_wt(c, M);
     float* ssq = reinterpret_cast<float*>(w + c->cv.ssq);
     const int m_stride = std::max(std::max(c->max_rows, c->max_prefill), 1);
+    // half operands carry a power of two per row: of the attention norms' operands and of the MLP norms'
+    float* pow2_mlp = wt_path && half_gemm ? reinterpret_cast<float*>(w + c->cv.row_pow2) : nullptr;       // what the attention norms leave for the output projection
+    float* pow2_attn = pow2_mlp ? pow2_mlp + m_stride : nullptr;                                            // what the MLP norms leave for the down projection
     T* a_lo = kF32 || half_gemm ? nullptr : reinterpret_cast<T*>(w + c->cv.a_lo);          // rounding remainders (bf16 operands only)
     float2* rope = reinterpret_cast<float2*>(w + c->cv.rope);
     const RowGeom g = geom(c);
@@ -664,7 +668,7 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
     c->final_norm_pending = false;
     launch_k(rope_table_kernel, dim3((M * half + 255) / 256), dim3(256), 0, st, sd, half, (double)d.rope_theta, g.pos, rope);
     launch_k(embed_rmsnorm_kernel<T>, dim3(M), dim3(NORM_THREADS), 0, st, sd, d.d_model, g.token, reinterpret_cast<const T*>(c->embed), c->attn_norm[0],
-                                               d.rms_eps, h, a, a_lo, half_gemm ? 1 : 0, c->err);
+                                               d.rms_eps, h, a, a_lo, half_gemm ? 1 : 0, c->err, pow2_mlp);
     count_launches(2);
     PC_CUDA_CHECK_LAUNCH("embed_rmsnorm");
     for (int l = 0; l < d.n_layers; ++l) {
@@ -673,24 +677,29 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
             // Five projections' worth of work in four launches: every row-wise step around a projection is in its epilogue.
             const float* bias_l = d.qkv_bias ? c->bqkv[l] : nullptr;
             const int n_tiles = (d.d_model + wt::FT - 1) / wt::FT;
-            const wt::RowScale complete{nullptr, 0, 0, 1, 0.f}, scaled{ssq, n_tiles, m_stride, d.d_model, d.rms_eps};
+            const wt::RowScale complete{};
+            // the norm a projection finishes: the power of two in its operand, the one it leaves for the next, and where its products come
+            // from when the operand does not hold a row
+            auto scaled = [&](const float* used, float* next, const void* weights, const float* gain) {
+                return wt::RowScale{ssq, n_tiles, m_stride, d.d_model, d.rms_eps, used, next, weights, h, gain};
+            };
             c->mark(st, l, PC_MARK_NORM_ATTN);
             wt::EpiQkv eq{};
             eq.Hq = d.n_q_heads; eq.Hkv = d.n_kv_heads; eq.layer = l; eq.bias = bias_l;
             eq.q_gain = d.qk_norm ? c->q_norm[l] : nullptr; eq.k_gain = d.qk_norm ? c->k_norm[l] : nullptr; eq.eps = d.rms_eps;
             eq.rope = rope; eq.geo = g; eq.prompt_arena = prompt_arena; eq.suffix_arena = suffix_arena; eq.q_out = reinterpret_cast<__half*>(q);
-            eq.rs = l == 0 ? complete : scaled; eq.err = c->err;
+            eq.rs = l == 0 ? complete : scaled(pow2_attn, pow2_mlp, c->wqkv[l], c->attn_norm[l]); eq.err = c->err;
             if (int rc = gemm_wt(c, st, sd, GEMM_QKV, X_A, !half_gemm, c->m_wqkv[l], M, eq, DEP_QKV)) return rc;
             c->mark(st, l, PC_MARK_QKV);
             c->mark(st, l, PC_MARK_POST);
             if (int rc = attention_bf16<128>(c, st, sd, M, l, plan, prompt_arena, suffix_arena, q, attn)) return rc;
-            auto res_norm = [&](auto epi, const float* gain, void* lo) {
+            auto res_norm = [&](auto epi, const float* gain, void* lo, const float* pow2) {
                 epi.h = h; epi.ld = d.d_model; epi.gain = gain; epi.a = wt::Operand{a, lo}; epi.ssq = ssq; epi.ssq_stride = m_stride;
-                epi.rs = complete; epi.err = c->err;
+                epi.rs = complete; epi.rs.used = pow2;
                 return epi;
             };
-            int rc = half_gemm ? gemm_wt(c, st, sd, GEMM_O, X_ATTN, false, c->m_wo[l], M, res_norm(wt::EpiResNorm<true>{}, c->mlp_norm[l], nullptr), DEP_O)
-                               : gemm_wt(c, st, sd, GEMM_O, X_ATTN, true, c->m_wo[l], M, res_norm(wt::EpiResNorm<false>{}, nullptr, nullptr), DEP_O);
+            int rc = half_gemm ? gemm_wt(c, st, sd, GEMM_O, X_ATTN, false, c->m_wo[l], M, res_norm(wt::EpiResNorm<true>{}, c->mlp_norm[l], nullptr, pow2_mlp), DEP_O)
+                               : gemm_wt(c, st, sd, GEMM_O, X_ATTN, true, c->m_wo[l], M, res_norm(wt::EpiResNorm<false>{}, nullptr, nullptr, nullptr), DEP_O);
             if (rc) return rc;
             c->mark(st, l, PC_MARK_O);
             if (!half_gemm) {
@@ -701,7 +710,7 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
             }
             c->mark(st, l, PC_MARK_NORM_MLP);
             auto swiglu = [&](auto epi) {
-                epi.act = wt::Operand{act, nullptr}; epi.ld = d.d_ff; epi.rs = half_gemm ? scaled : complete; epi.err = c->err;
+                epi.act = wt::Operand{act, nullptr}; epi.ld = d.d_ff; epi.rs = half_gemm ? scaled(pow2_mlp, pow2_attn, c->w_gate_up[l], c->mlp_norm[l]) : complete; epi.err = c->err;
                 return epi;
             };
             rc = half_gemm ? gemm_wt(c, st, sd, GEMM_GATE_UP, X_A, false, c->m_wgu[l], M, swiglu(wt::EpiSwiGLU<true>{}), DEP_GATE_UP)
@@ -710,8 +719,8 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
             c->mark(st, l, PC_MARK_GATE_UP);
             const bool last = l + 1 == d.n_layers;
             const float* gain = !last ? c->attn_norm[l + 1] : (fold_final_norm ? c->final_norm : nullptr);
-            rc = half_gemm ? gemm_wt(c, st, sd, GEMM_DOWN, X_ACT, false, c->m_wdown[l], M, res_norm(wt::EpiResNorm<true>{}, gain, nullptr), DEP_DOWN)
-                           : gemm_wt(c, st, sd, GEMM_DOWN, X_ACT, false, c->m_wdown[l], M, res_norm(wt::EpiResNorm<false>{}, gain, a_lo), DEP_DOWN);
+            rc = half_gemm ? gemm_wt(c, st, sd, GEMM_DOWN, X_ACT, false, c->m_wdown[l], M, res_norm(wt::EpiResNorm<true>{}, gain, nullptr, pow2_attn), DEP_DOWN)
+                           : gemm_wt(c, st, sd, GEMM_DOWN, X_ACT, false, c->m_wdown[l], M, res_norm(wt::EpiResNorm<false>{}, gain, a_lo, nullptr), DEP_DOWN);
             if (rc) return rc;
             if (last) c->final_norm_pending = fold_final_norm;
             count_launches(4);
@@ -801,8 +810,10 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
 
 // The factor of the final norm when the last down projection left the LM head's operand without it.
 pc::wt::RowScale folded_norm(const pc_ctx* c) {
-    return pc::wt::RowScale{reinterpret_cast<const float*>(c->ws + c->cv.ssq), (c->d.d_model + pc::wt::FT - 1) / pc::wt::FT,
-                            std::max(std::max(c->max_rows, c->max_prefill), 1), c->d.d_model, c->d.rms_eps};
+    const int m_stride = std::max(std::max(c->max_rows, c->max_prefill), 1);
+    return pc::wt::RowScale{reinterpret_cast<const float*>(c->ws + c->cv.ssq), (c->d.d_model + pc::wt::FT - 1) / pc::wt::FT, m_stride, c->d.d_model,
+                            c->d.rms_eps, c->d.half_gemm ? reinterpret_cast<const float*>(c->ws + c->cv.row_pow2) + m_stride : nullptr, nullptr,
+                            c->lm_head, reinterpret_cast<const float*>(c->ws + c->cv.h), c->final_norm};
 }
 
 // logits[n, V] = RMSNorm(h[src[r]]; final_norm) * W_lm^T
@@ -824,7 +835,7 @@ int run_lm_head(pc_ctx* c, cudaStream_t st, int n, const pc::StepDesc* sd, const
         const T* wlm = reinterpret_cast<const T*>(d.tied_embed ? c->embed : c->lm_head);
         launch_gemm_simt(st, sd, a, wlm, n, d.vocab, d.d_model, EpiStoreF32{logits, d.vocab, nullptr});
     } else if (folded || use_wt(c, n)) {
-        wt::EpiStore epi{logits, d.vocab, {nullptr, 0, 0, 1, 0.f}};
+        wt::EpiStore epi{logits, d.vocab, {}};
         if (folded) epi.rs = folded_norm(c);
         if (int rc = gemm_wt(c, st, sd, GEMM_LM_HEAD, X_A, !half_gemm, c->m_lm, n, epi, DEP_LM_HEAD)) return rc;
     } else {
@@ -857,14 +868,19 @@ int run_lm_head_sample(pc_ctx* c, cudaStream_t st, int n, const pc::StepDesc* sd
     const GemmPlan gp = plan_gemm(c, GEMM_LM_HEAD, c->m_lm, n, false);
     Top2Rec* rec = reinterpret_cast<Top2Rec*>(c->ws + c->cv.sample_tiles);
     const int m_stride = std::max(c->max_rows, 1);
+    float* factor = nullptr;
+    if (folded) {
+        factor = reinterpret_cast<float*>(c->ws + c->cv.row_pow2) + 2 * std::max(std::max(c->max_rows, c->max_prefill), 1);
+        launch_k(final_factor_kernel, dim3(n), dim3(FINAL_FACTOR_THREADS), 0, st, sd, folded_norm(c), reinterpret_cast<uint16_t*>(a), factor, c->err);
+    }
     if (int rc = gemm_bf16(c, st, sd, c->map_a, half_gemm ? nullptr : &c->map_a_lo, c->m_lm, n, gp,
-                           EpiSample{rec, m_stride, keys.key_prompt, keys.rollout, keys.step_key, keys.sample_bound, da, folded ? folded_norm(c) : wt::RowScale{nullptr, 0, 0, 1, 0.f}},
+                           EpiSample{rec, m_stride, keys.key_prompt, keys.rollout, keys.step_key, keys.sample_bound, da, factor},
                            half_gemm, DEP_LM_HEAD))
         return rc;
     c->mark(st, -1, PC_MARK_LM_HEAD);
     const int bn = gp.wide ? 256 : 64;
     launch_k(sample_tiles_reduce_kernel, dim3(n), dim3(TILES_REDUCE_THREADS), 0, st, sd, 2 * ((d.vocab + bn - 1) / bn), rec, m_stride, keys.out_index, da);
-    count_launches(folded ? 2 : 3);
+    count_launches(3);
     c->mark(st, -1, PC_MARK_SAMPLE);
     PC_CUDA_CHECK_LAUNCH("lm head with sampler");
     return PC_OK;
