@@ -131,6 +131,10 @@ def _calls():
         except ImportError as e:
             raise RuntimeError("_pc_calls.so is missing or does not load: build it with `python -m paper_2605_26606_b200.build` "
                                "(there is no fallback path)") from e
+        from . import build
+        if _pc_calls.built_for != build.calls_key():
+            raise RuntimeError(f"_pc_calls.so is {_pc_calls.built_for}, not {build.calls_key()}: build it again with "
+                               "`python -m paper_2605_26606_b200.build`")
         _pc_calls.bind(*(C.cast(getattr(lib, n), C.c_void_p).value for n in
                          ("pc_reward_last_token", "pc_group_stats", "pc_allocate", "pc_allocate_variance", "pc_grpo_advantage")))
         _CALLS = _pc_calls

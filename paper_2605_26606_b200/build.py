@@ -1,6 +1,7 @@
 """Builds the CUDA library (libpc.so, sm_100a only) and the native call wrappers (_pc_calls.so) in-tree."""
 from __future__ import annotations
 
+import importlib.metadata
 import os
 import shutil
 import subprocess
@@ -30,16 +31,32 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def calls_key() -> str:
+    """What the call wrappers are compiled against beside their source: torch's C++ ABI and this interpreter's.  The text is
+    compiled in (the module's built_for)."""
+    return f"built for torch {importlib.metadata.version('torch')}, python {sys.version_info.major}.{sys.version_info.minor}"
+
+
+def _calls_stale() -> bool:
+    if not os.path.exists(CALLS):
+        return True
+    t = os.path.getmtime(CALLS)
+    if any(os.path.getmtime(d) > t for d in (CALLS_SOURCE, os.path.join(HERE, "..", "include", "pc.h"), __file__)):
+        return True
+    with open(CALLS, "rb") as f:
+        return calls_key().encode() + b"\0" not in f.read()
+
+
 def build_calls(force: bool = False) -> str:
     """The CPython extension of csrc/py_calls.cpp (host code only)."""
-    deps = [CALLS_SOURCE, os.path.join(HERE, "..", "include", "pc.h"), __file__]
-    if not force and os.path.exists(CALLS) and all(os.path.getmtime(d) <= os.path.getmtime(CALLS) for d in deps):
+    if not force and not _calls_stale():
         return CALLS
     import torch
     from torch.utils import cpp_extension
     lib = os.path.join(os.path.dirname(torch.__file__), "lib")
     cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_nvcc()))), "include")
-    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           f'-DPC_CALLS_KEY="{calls_key()}"']
     for inc in cpp_extension.include_paths() + [sysconfig.get_paths()["include"], cuda]:
         cmd += ["-isystem", inc]
     cmd += [CALLS_SOURCE, "-o", CALLS, "-L" + lib, "-ltorch_python", "-lc10", "-lc10_cuda", "-Wl,-rpath," + lib]

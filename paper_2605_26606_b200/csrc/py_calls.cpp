@@ -186,4 +186,11 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_pc_calls", nullptr, -1, methods, 
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__pc_calls() { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit__pc_calls() {
+    PyObject* m = PyModule_Create(&module);
+    if (m != nullptr && PyModule_AddStringConstant(m, "built_for", PC_CALLS_KEY) != 0) {
+        Py_DECREF(m);
+        return nullptr;
+    }
+    return m;
+}

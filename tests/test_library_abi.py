@@ -72,3 +72,21 @@ def test_binding_fails_loudly_without_the_library(monkeypatch, tmp_path):
     monkeypatch.setattr(B, "LIB_PATH", str(tmp_path / "missing.so"))
     with pytest.raises(RuntimeError, match="no fallback"):
         B.pc_status_string(0)
+
+
+def test_call_wrappers_of_another_torch_are_rebuilt(lib, monkeypatch, tmp_path):
+    """The wrappers are compiled against one torch's C++ ABI: with another torch installed the newer file counts as stale, and an
+    import of it is refused."""
+    copy = tmp_path / "_pc_calls.so"
+    copy.write_bytes(open(build.CALLS, "rb").read())
+    compiled = []
+    monkeypatch.setattr(build, "CALLS", str(copy))
+    monkeypatch.setattr(build.subprocess, "run", lambda cmd, **kw: compiled.append(cmd) or build.subprocess.CompletedProcess(cmd, 0, "", ""))
+    build.build_calls()
+    assert not compiled
+    monkeypatch.setattr(build.importlib.metadata, "version", lambda name: "2.10.0+cu126")
+    build.build_calls()
+    assert len(compiled) == 1
+    monkeypatch.setattr(B, "_CALLS", None)
+    with pytest.raises(RuntimeError, match="built for"):
+        B._calls()
