@@ -160,6 +160,7 @@ struct pc_ctx {
     struct WtPlan { int kind, M, dual; int cg, nt, splits, stages, clusters, n_acc; };
     std::vector<XMap> x_maps;
     std::vector<WtPlan> wt_plans;
+    int max_clusters[pc::wt::MAX_SPLITS + 1] = {};       // by size: clusters of CTAs with a whole SM's shared memory each that are resident at once
     bool final_norm_pending = false;         // the last down projection left half(h * final gain) without its 1/rms factor
 
     int fused_epilogues = 1;                 // half-operand models with head_dim 128: QKV post-processing and the MLP norm inside GEMM epilogues
@@ -349,12 +350,11 @@ enum XBuf { X_A = 0, X_ATTN = 1, X_ACT = 2, X_A_LO = 3, X_ATTN_LO = 4 };
 // L2 + the rows a CTA finishes (the QKV epilogue only: the others hide) + the hand-over of partial tiles.  Constants fitted to
 // 3,947 timed launches of the 1.5B and 8B shapes at 16 .. 2048 rows; the rates of
 // the main loop then raised by a quarter with the issue loops (237 rows: 21.25 -> 20.63 ms per eight steps).
-// At most max_active[c] clusters of c CTAs with a whole SM's shared memory each are resident (the GPCs' SM counts).
+// A wave is as many clusters as the device holds at once (max_clusters, asked for by pc_set_workspace: it depends on the GPCs' SM counts).
 const pc_ctx::WtPlan& plan_wt(pc_ctx* c, GemmKind kind, int N, int K, int M, bool dual) {
     using namespace pc;
     for (const auto& p : c->wt_plans)
         if (p.kind == kind && p.M == M && p.dual == (int)dual) return p;
-    static const int max_active[9] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
     const int kb = K / wt::BK;
     const bool may_split = kind == GEMM_QKV || kind == GEMM_O || kind == GEMM_DOWN;
     pc_ctx::WtPlan best{kind, M, dual ? 1 : 0, 1, 16, 1, 4, 1, 1};
@@ -370,7 +370,7 @@ const pc_ctx::WtPlan& plan_wt(pc_ctx* c, GemmKind kind, int N, int K, int M, boo
                 const int stage = wt::W_BYTES + (dual ? wt::x_bytes<true>(nt, cg) : wt::x_bytes<false>(nt, cg));
                 const int stages = std::min(wt::MAX_STAGES, (wt::SMEM_BUDGET - wt::smem_bytes<false>(nt, 4, cg, sp, 0)) / stage);
                 if (stages < 3 || (sp > 1 && stages * stage < (nt + 8) * wt::FT * 4)) continue;
-                const double clusters = (double)features * tr, waves = std::ceil(clusters / max_active[cg * sp] * 148. / c->num_sms);
+                const double clusters = (double)features * tr, waves = std::ceil(clusters / c->max_clusters[cg * sp]);
                 const double kbs = (double)kb / sp, mmas = dual ? 2. : 1.;
                 const double sm = waves * kbs * std::max(stage / 160e3, mmas * nt * 2. / 1750. * 1.43);
                 const double hbm = (double)N * K * 2e-6 / 6.2, l2 = clusters * cg * sp * kbs * stage * 1e-6 / 22.;
@@ -505,6 +505,23 @@ cudaError_t configure_wt_dual() {
     cudaError_t e = wt::configure<1, true, Epi>();
     if (e == cudaSuccess) e = wt::configure<2, true, Epi>();
     return e;
+}
+cudaError_t count_clusters(pc_ctx* c) {
+    using namespace pc;
+    for (int size = 1; size <= wt::MAX_SPLITS; ++size) {
+        cudaLaunchConfig_t cfg;
+        std::memset(&cfg, 0, sizeof(cfg));
+        cfg.gridDim = dim3((unsigned)(size * c->num_sms)); cfg.blockDim = dim3(wt::THREADS); cfg.dynamicSmemBytes = wt::SMEM_BUDGET;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = size; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        int n = 0;
+        const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, wt::gemm_wt_kernel<1, false, wt::EpiStore>, &cfg);
+        if (e != cudaSuccess) return e;
+        c->max_clusters[size] = std::max(n, 1);
+    }
+    return cudaSuccess;
 }
 cudaError_t configure_simt() {
     cudaError_t e = pc::configure_gemm_simt<pc::EpiStoreF32>();
@@ -1135,6 +1152,7 @@ int pc_set_workspace(pc_ctx* ctx, void* dev_ws, size_t bytes, int max_rows, int 
     }
     if (ctx->d.dtype == PC_DTYPE_BF16) {
         cudaError_t ce = configure_kernels();
+        if (ce == cudaSuccess) ce = count_clusters(ctx);
         if (ce != cudaSuccess) { ctx->ws = nullptr; return cuda_fail(ce, "kernel attributes"); }
         const uint64_t cap = (uint64_t)std::max(std::max(max_rows, max_prefill_tokens), 1);
         char* w = ctx->ws;
