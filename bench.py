@@ -225,7 +225,9 @@ def chain_trace(eng, B, torch, pp, rr, step):
 
 def phase_table(eng, B, n_layers):
     """Per-operation device time from the sampled decode steps: every sample holds the CUDA events pc_profile_step
-    recorded around the operations of one decoder layer and of the step's tail (LM head, sampler)."""
+    recorded around the operations of one decoder layer and of the step's tail (LM head, sampler).  The suffix attention merges by
+    itself, so the time between its two marks is that of an event alone; it is taken off every operation.  Operations that run
+    inside another kernel, with nothing between their marks either, have no line."""
     names = B.PROFILE_MARKS
     ix = {n: i for i, n in enumerate(names)}
     layer_ops = [("norm_attn", "layer_begin", "norm_attn"), ("qkv_gemm", "norm_attn", "qkv"), ("qkv_post", "qkv", "post"),
@@ -233,12 +235,18 @@ def phase_table(eng, B, n_layers):
                  ("o_gemm", "merge", "o"), ("norm_mlp", "o", "norm_mlp"), ("gate_up_gemm", "norm_mlp", "gate_up"),
                  ("down_gemm", "gate_up", "down")]
     tail_ops = [("lm_head", "lm_begin", "lm_head"), ("sampler", "lm_head", "sample")]
+    inside = {"attn_merge"}
+    if eng.model.dtype != wl.DTYPE_BF16:
+        inside |= {"attn_prefix"}
+    elif eng.model.head_dim == 128:
+        inside |= {"norm_attn", "qkv_post"} | ({"norm_mlp"} if eng.half_gemm else set())
+    layer_ops = [op for op in layer_ops if op[0] not in inside]
     tot = {k: 0.0 for k, _, _ in layer_ops + tail_ops}
     per_sample = []
     for evs, nr, npos in eng.profile_samples:
-        d = {}
+        d, event = {}, evs[ix["suffix"]].elapsed_time(evs[ix["merge"]])
         for k, a, b in layer_ops + tail_ops:
-            d[k] = evs[ix[a]].elapsed_time(evs[ix[b]])
+            d[k] = max(evs[ix[a]].elapsed_time(evs[ix[b]]) - event, 0.0)
             tot[k] += d[k]
         per_sample.append((d, nr, npos))
     n = max(len(per_sample), 1)
@@ -402,7 +410,7 @@ def main():
                                "traffic": SUFFIX_TRAFFIC_PER_ALGORITHMIC_BYTE * s_bytes / n_samp,
                                "traffic_note": "ncu capture of a smaller case scaled by algorithmic bytes (profiles/attn_suffix_kernel_ncu.md)",
                                "avg_launch_ms": s_ms / n_samp, "avg_algorithmic_bytes": s_bytes / n_samp},
-        "gemm_tc_kernel (QKV, O, gate/up, down of one layer)": {
+        "gemm_wt_kernel (QKV, O, gate/up, down of one layer)": {
             "bound": "hbm below about %d rows, tensor above" % int(tf_burst * 1e12 / (peak * 1e9) / 2 * m.elem_bytes),
             "avg_ms_per_layer": g_ms / n_samp, "weight_gbs": layer_w_bytes * n_samp / (g_ms * 1e-3) / 1e9 if g_ms > 0 else 0.0,
             "weight_frac_of_hbm_peak": (layer_w_bytes * n_samp / (g_ms * 1e-3) / 1e9 / peak) if g_ms > 0 else 0.0,
@@ -454,8 +462,8 @@ def main():
         "phase_ms": {"prefill_per_step": prefill_ms / max(args.steps, 1),
                      "sampled_decode_steps": len(per_sample), "per_launch_avg": per_op_ms,
                      "estimated_per_decode_step": est_ms,
-                     "note": "CUDA events around the operations of layer %d and the LM head / sampler in every 32nd decode step; "
-                             "a layer operation is counted n_layers times; the sampled steps run in plain stream order (an event between "
+                     "note": "CUDA events around the operations of layer %d and the LM head / sampler in every 32nd decode step, the time of an "
+                             "event with nothing behind it taken off; a layer operation is counted n_layers times; the sampled steps run in plain stream order (an event between "
                              "two kernels rules out the dependent launches the other steps use)" % eng.profile_layer},
         "live_rows_histogram": live_hist,
         "hbm_step": {"bytes_per_step": step_bytes, "achieved_gbs": step_bytes * args.steps / (dev_ms * 1e-3) / 1e9,
