@@ -161,10 +161,9 @@ def run_probe(args):
     eng = RolloutEngine(w.model, weights, max_rows=P * G, max_prefill_tokens=int(batch.prompt_offsets[-1]))
     eng.use_graphs = kv.get("graphs", "1") != "0"
     B.pc_set_decode_mode(eng.ctx, int(kv.get("mode", 0)))
-    B.pc_set_attention_overlap(eng.ctx, int(kv.get("overlap", 0)))
     B.pc_set_fused_sampler(eng.ctx, int(kv.get("fused", 0)))
     B.pc_set_fused_epilogues(eng.ctx, int(kv.get("epi", 1)))
-    B.pc_set_dependent_launch(eng.ctx, int(kv.get("dep", 1)))
+    B.pc_set_dependent_launch(eng.ctx, int(kv.get("dep", 63)))
     if "plan" in kv:            # forced GEMM plans, e.g. plan=qkv:128x1+o:64x1
         B.pc_set_gemm_plan(eng.ctx, kv["plan"].replace(":", "=").replace("+", ","))
     eng.load_batch(w, batch)
