@@ -61,6 +61,7 @@ def test_logits_after_a_prefill_of_many_row_tiles(cuda_device, prompt_len):
 
 
 UNTIED = dataclasses.replace(wl.SMALL_BF16, name="untied-bf16", tied_embed=False, qkv_bias=False)
+WIDE_MLP = dataclasses.replace(UNTIED, name="wide-mlp-bf16", d_model=1536, n_q_heads=12, d_ff=8960, vocab=1003)      # CTA pairs from 200 rows on
 
 
 def _scaled(model, factors):
@@ -112,17 +113,20 @@ def test_residual_stream_of_any_size(cuda_device, rows, matrices, values):
     assert worst <= 3 * ordinary, (worst, ordinary)
 
 
-@pytest.mark.parametrize("rows", [3, 130])
-@pytest.mark.parametrize("grown", [{"layers.0.w_up": 6, "layers.0.w_down": 14}, {"layers.1.w_up": 14, "layers.1.w_down": 18}], ids=["into-qkv", "into-lm-head"])
-def test_rows_that_outgrow_their_operand(cuda_device, rows, grown):
+@pytest.mark.parametrize("model,rows,grown", [(UNTIED, 3, {"layers.0.w_up": 6, "layers.0.w_down": 14}), (UNTIED, 130, {"layers.0.w_up": 6, "layers.0.w_down": 14}),
+                                              (UNTIED, 3, {"layers.1.w_up": 14, "layers.1.w_down": 18}), (UNTIED, 130, {"layers.1.w_up": 14, "layers.1.w_down": 18}),
+                                              (WIDE_MLP, 256, {})],
+                         ids=["into-qkv-3", "into-qkv-130", "into-lm-head-3", "into-lm-head-130", "into-cta-pairs-256"])
+def test_rows_that_outgrow_their_operand(cuda_device, model, rows, grown):
     """The residual stream grows 2^20-fold and more within a sublayer (layer 0's attention, then an MLP): the next operand does not
-    hold the rows and their products come from the stream itself.  Six roundings of 2^-11 on logits of rms 0.45, 4.5 standard
-    deviations: 2.5e-3; asserted with a factor 4."""
+    hold the rows and their products come from the stream itself.  Six roundings of 2^-11 on logits of rms 0.45 (0.78 with 1,536
+    features), 4.5 standard deviations: 2.5e-3 (4.3e-3); asserted with a factor 4."""
     ensure_built()
-    model = dataclasses.replace(UNTIED, rms_eps=1e-20)
+    bound = 1e-2 * (model.d_model / 512) ** 0.5
+    model = dataclasses.replace(model, rms_eps=1e-20)
     weights = _scaled(model, {"embed": -20, **grown})
     batch, tokens, logits = _pilot(model, weights, rows)
     worst = _worst(model, weights, batch, tokens, logits)
     print(f"max |dlogit| {worst:.5f}")
-    assert worst <= 1e-2, worst
+    assert worst <= bound, worst
     assert np.array_equal(np.stack(_pilot(model, weights, rows, fused_sampler=1)[1]), np.stack(tokens))

@@ -100,7 +100,8 @@ def test_small_bf16_models_teacher_forced(model, half_gemm):
 @pytest.mark.parametrize("spec", ["qkv=256x2,o=256x3,dn=256x4,gu=64x1,lm=64x1", "qkv=64x1,o=64x1,dn=64x8,gu=256x1,lm=256x1",
                                   "qkv=128x2,o=128x2,dn=128x4,gu=128x1"])
 def test_forced_gemm_plans_stay_within_tolerance(spec):
-    """pc_set_gemm_plan: tile width and K-split change the order of the float additions, nothing else; a bad spec is refused."""
+    """pc_set_gemm_plan: the rows-on-lanes kernels with a forced tile width and K-split stay within the tolerance of the oracle; a bad
+    spec is refused."""
     from paper_2605_26606_b200 import binding as B
     model = wl.SMALL_BF16
     w = dataclasses.replace(wl.WORKLOADS["config0"], model=model, n_prompts=3, prompt_len_lo=5, prompt_len_hi=70,
@@ -339,8 +340,8 @@ def test_bound_pass_bf16_logits_against_full_recompute():
 
 @pytest.mark.parametrize("model", [wl.SMALL_BF16, wl.SMALL_QKNORM_BF16, wl.TINY_BF16], ids=lambda m: m.name)
 def test_persistent_decode_kernel_equals_one_kernel_per_operation(model):
-    """pc_set_decode_mode: the persistent kernel (phases separated by grid barriers) runs the arithmetic of the separate
-    kernels in the same order, so a free-running Pilot-Commit step gives identical tokens and identical recorded logits; a
+    """pc_set_decode_mode: the persistent kernel (phases separated by grid barriers) runs the arithmetic of the form with one
+    kernel per operation (pc_set_fused_epilogues 0) in the same order, so a free-running Pilot-Commit step gives identical tokens and identical recorded logits; a
     missed barrier or a stale tile would show up as a difference."""
     from paper_2605_26606_b200 import binding as B
     w = dataclasses.replace(wl.WORKLOADS["config0"], model=model, n_prompts=5, prompt_len_lo=3, prompt_len_hi=90, group_size=40,
@@ -377,7 +378,7 @@ def test_dependent_launch_of_the_projections_changes_no_bit(model, group_size):
     while the kernel before it still runs, and waits for that kernel before it reads activations.  Tokens, recorded logits
     and advantages of a free-running Pilot-Commit step must be identical with the switch on (every projection and the shared-prefix attention), on for the
     gate/up projection only, on for the attention kernel only, and off; a projection that read its operand early would show up as a difference.  The
-    90-rollout groups take the commit stage above 256 rows, where the fused epilogues run."""
+    90-rollout groups take the commit stage above 256 rows, to other tilings and to the suffix kernel that merges inside a warp."""
     from paper_2605_26606_b200 import binding as B
     w = dataclasses.replace(wl.WORKLOADS["config0"], model=model, n_prompts=5, prompt_len_lo=3, prompt_len_hi=90, group_size=group_size,
                             n_pilot=8, max_new=40, cap_lo=1, cap_hi=40, data_seed=21,
