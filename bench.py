@@ -28,11 +28,10 @@ if ROOT not in sys.path:
 from paper_2605_26606_b200 import dist_util  # noqa: E402
 from paper_2605_26606_b200 import workloads as wl  # noqa: E402
 
-# DRAM traffic of the suffix attention kernel per algorithmic byte, from the ncu captures summarised in
-# profiles/attn_suffix_kernel_ncu.md (current build: 143.5 MB moved for 136.0 MB algorithmic at 256 rollouts x 513 slots, 1,157 MB
-# for 1,088 MB at 2048 x 513).  The kernel streams every (rollout, KV head) suffix once, so traffic grows in proportion to the
-# algorithmic bytes of a launch.
-SUFFIX_TRAFFIC_PER_ALGORITHMIC_BYTE = 1.06
+# DRAM traffic of the suffix attention kernel per algorithmic byte, from the ncu captures in profiles/decode_kernels_ncu.md: 145.9 MB
+# moved for 136.1 MB at 256 rollouts x 513 slots (1.045 at 64 x 513, 1.036 at 1,024 x 129).  The kernel streams every (rollout, KV
+# head) suffix once, so traffic grows in proportion to the algorithmic bytes of a launch.
+SUFFIX_TRAFFIC_PER_ALGORITHMIC_BYTE = 1.07
 METRIC = "generated tokens/s"
 UNIT = "tokens/s"
 
@@ -407,7 +406,7 @@ def main():
         "attn_suffix_kernel": {"bound": "hbm", "achieved": s_bytes / (s_ms * 1e-3) / 1e9 if s_ms > 0 else 0.0, "peak": peak, "unit": "GB/s",
                                "frac": (s_bytes / (s_ms * 1e-3) / 1e9 / peak) if s_ms > 0 else 0.0,
                                "traffic": SUFFIX_TRAFFIC_PER_ALGORITHMIC_BYTE * s_bytes / n_samp,
-                               "traffic_note": "ncu capture of a smaller case scaled by algorithmic bytes (profiles/attn_suffix_kernel_ncu.md)",
+                               "traffic_note": "ncu capture of a smaller case scaled by algorithmic bytes (profiles/decode_kernels_ncu.md)",
                                "avg_launch_ms": s_ms / n_samp, "avg_algorithmic_bytes": s_bytes / n_samp},
         "gemm_wt_kernel (QKV, O, gate/up, down of one layer)": {
             "bound": "hbm below about %d rows, tensor above" % int(tf_burst * 1e12 / (peak * 1e9) / 2 * m.elem_bytes),
@@ -449,8 +448,8 @@ def main():
         "roofline": {"bound": "hbm", "kernel": "decode steps of the Pilot-Commit step, all kernels (prefill excluded)",
                      "achieved": achieved_step, "peak": peak, "peak_kind": peak_kind, "unit": "GB/s", "frac": achieved_step / peak,
                      "frac_of_8tbs": achieved_step / 8000.0, "traffic": None,
-                     "traffic_note": "not captured for the 4,100-step job; ncu captures of single decode steps moved 1.22 x (256 rows x 512) "
-                                     "and 1.26 x (2048 rows x 512) their algorithmic bytes (profiles/decode_step_launch_list_config2.md)",
+                     "traffic_note": "not captured for the 4,100-step job; by the ncu captures of its kernels a single decode step of 256 rows x 512 "
+                                     "moves 1.14 x its algorithmic bytes (profiles/decode_kernels_ncu.md)",
                      "bytes_per_step": step_bytes, "decode_ms_per_step": decode_ms / max(args.steps, 1),
                      "parts": {"suffix_kv_read": suffix_reads, "prompt_kv_read": prompt_reads, "weights": weight_reads, "kv_write": kv_writes},
                      "target": 0.60},
