@@ -172,14 +172,14 @@ PC_API int pc_workspace_bytes(const pc_ctx* ctx, int max_rows, int max_prefill_t
 PC_API int pc_set_workspace(pc_ctx* ctx, void* dev_ws, size_t bytes, int max_rows, int max_prefill_tokens,
                      int32_t* dev_error_flag);
 
-/* Tuning aid: forces the tile width (64 or 256 output columns) and the number of K-slices of the bf16 tensor-core
- * GEMMs instead of the built-in choice.  spec (host string) is a comma-separated list of name=WIDTHxSLICES with name
- * in {qkv, o, gu, dn, lm} (QKV, output, gate/up, down projection, LM head), e.g. "dn=256x4,o=64x2"; names left out,
- * NULL or "" keep the built-in choice.  The slice count is clamped to what the workspace holds for the step's row
- * bound; gate/up and the LM head never split.  Where the QKV and output projections run with the fused epilogues
- * (pc_set_fused_epilogues) only the width applies to them: 128 or 256 for QKV (whole heads per tile; 128 is accepted for
- * this case only and otherwise read as 64), 64 or 256 for the output projection.  Results stay deterministic for a
- * fixed plan.  Drops captured decode steps.  The paper has no counterpart. */
+/* Tuning aid for the rows-on-lanes GEMMs (one kernel per operation): forces their tile width (64, 128 or 256 output columns)
+ * and number of K-slices.  spec (host string) is a comma-separated list of name=WIDTHxSLICES with name in {qkv, o, gu, dn, lm}
+ * (QKV, output, gate/up, down projection, LM head), e.g. "dn=256x4,o=64x2".  Any name takes ALL GEMMs of a bf16 model to those kernels,
+ * as pc_set_fused_epilogues(0) does, and those left out keep the choice built in there; to see what a plan changes, compare it
+ * with pc_set_fused_epilogues(0) and no plan.  NULL or "" returns to the default kernels.  The slice count is clamped to what
+ * the workspace holds for the step's row bound; gate/up and the LM head never split.  Width 128 exists for QKV, gate/up and split
+ * output and down projections with one operand matrix (half_gemm 1, or gate/up and down); elsewhere it is read as 64.  Results stay deterministic for a fixed
+ * plan.  Drops captured decode steps.  The paper has no counterpart. */
 PC_API int pc_set_gemm_plan(pc_ctx* ctx, const char* spec);
 
 /* Self-test of the bounded waits every kernel here uses on its mbarriers: launches one warp that waits, for at most
@@ -195,7 +195,7 @@ PC_API int pc_set_index_bounds(pc_ctx* ctx, int n_prompts, int64_t n_tokens);
 /* bf16 models with head_dim 128.  1 (the default): every row-wise step of a layer runs inside GEMM epilogues -- bias / QK-norm /
  * RoPE / KV append in the QKV projection's, the residual add, the next operand and its RMSNorm's sum of squares in the output
  * and down projections', the norm's 1/rms being applied by the projection that reads the operand (RMSNorm(h; g) W^T =
- * rstd * ((h * g) W^T)).  0: one kernel per operation throughout, as for every other model type.  A value n > 1: the fused form
+ * rstd * ((h * g) W^T); a half operand carries an exact power of two per row, so that it fits whatever the size of h).  0: one kernel per operation throughout, as for every other model type.  A value n > 1: the fused form
  * from passes of n rows on (a measurement aid).  Same mathematics, different rounding order (both inside the tolerances the
  * tests state).  Drops captured decode steps.  The paper has no counterpart. */
 PC_API int pc_set_fused_epilogues(pc_ctx* ctx, int on);
@@ -216,8 +216,8 @@ PC_API int pc_set_dependent_launch(pc_ctx* ctx, int mask);
  * back; 0 (the default) stores the logits and runs the stand-alone sampler on them.  Both draw exactly the same tokens
  * (Section 4.2: T = 1.0, top_p = 1.0; pc_sample states the rule): the tiles of a row share a running lower bound of the
  * row's second-best score, so which candidates a tile scores depends on timing, the folded result does not.  The
- * epilogue form is not the faster one on B200 (LM head + draw at 2048 rows: 2.37 ms against 0.90 + 0.60 ms; at 64 rows
- * 0.17 against 0.15 ms): the Philox arithmetic needs many warps per scheduler to reach the integer pipes' rate, and a
+ * epilogue form is not the faster one on B200 (whole decode steps of the 1.5B shape: 15.1 ms against 13.4 at 2048 rows, 3.58
+ * against 2.81 at 256; at 64 rows the two do not differ by more than their spread): the Philox arithmetic needs many warps per scheduler to reach the integer pipes' rate, and a
  * GEMM CTA has room for eight epilogue warps.  It is kept for callers that cannot afford the [rows, vocab] logits
  * buffer.  Drops captured steps. */
 PC_API int pc_set_fused_sampler(pc_ctx* ctx, int on);
@@ -230,8 +230,8 @@ PC_API int pc_set_attention_overlap(pc_ctx* ctx, int on);
  * attention calls of a step -- output projection, residual + RMSNorm, gate/up + SwiGLU, down projection, residual +
  * RMSNorm, QKV projection of the next layer and its bias / QK-norm / RoPE / KV append; embedding before the first
  * layer, LM head after the last -- runs as phases of ONE persistent cooperative kernel with grid-wide barriers, the
- * weight tiles of the next GEMM being requested across the barriers.  mode 0 (the default): one kernel per operation.  Both modes
- * run the same arithmetic in the same order and give identical results; models of other types always use mode 0.
+ * weight tiles of the next GEMM being requested across the barriers.  mode 0 (the default): separate kernels.  Mode 1 runs the
+ * arithmetic of pc_set_fused_epilogues(0) in the same order and gives identical results; models of other types always use mode 0.
  * Drops captured decode steps.  The paper has no counterpart. */
 PC_API int pc_set_decode_mode(pc_ctx* ctx, int mode);
 

@@ -9,9 +9,11 @@
 // The running reference of a row's softmax only moves when its maximum grows by more than 2^8 over it: O is then rescaled in
 // TMEM.  Below that P stays below 256, far inside half's range, and the reference cancels in the result.
 //
-// What bounds it: the exponentials (16 per clock and SM: 512 clocks per 128 x 64 tile) and, for short prompts, the chain
-// Q -> S -> softmax -> P V.  The mma.sync kernel (attn_group_kernel, kept for head_dim 64) needs 5,000 clocks for a tile of half
-// the rows.
+// What bounds it: chains, not a pipe.  Alone on the GPU (cold) a launch of 96-128 CTAs takes 12.5 us with three tiles a CTA (64 rows x
+// 640 keys) and 20.9 us with ten (1,024 rows): about 1.2 us or 2,400 clocks a tile, of which the exponentials (16 per clock and
+// SM) would be 512, and 9 us that no tile explains (launch, q, first K, record).  Prefill of 16 x 640 tokens, 960 CTAs of 5.5 tiles:
+// 67.6 us, 1.9 us of an SM's time per tile with a CTA's start and end in it.  Tensor pipe 9 / 16 / 19 %, DRAM 10 / 8 / 8 % busy.
+// The mma.sync kernel (attn_group_kernel, kept for head_dim 64) needs 5,000 clocks for a tile of half the rows.
 #pragma once
 
 #include "attention_mma.cuh"

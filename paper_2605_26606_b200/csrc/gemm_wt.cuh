@@ -21,12 +21,14 @@
 // barriers and TMEM and requests weight tiles; it releases its own dependents only after its wait, so whatever runs two
 // kernels back has finished when a kernel starts.
 //
-// What it measured against the rows-on-lanes kernel with separate norm and post-processing kernels (four projections and what
-// lies between them, per layer, B200): 16 rows 46 -> 34 us, 71 rows 50 -> 41, 237 rows 80 -> 57, 336 rows 78 -> 68; whole decode
-// steps of the 1.5B shape 2.03 -> 1.78 ms (16 rows), 3.76 -> 3.17 ms (237 rows), of the 8B shape 6.28 -> 5.22 ms (64 rows).
-// What bounds it: up to about 128 rows the weight stream (gate/up 6-7 TB/s of 6.5 copy rate, part of it requested before the
-// kernel's turn) and 4-5 us of fixed chain per launch (hand-over, first tile, drain, cluster hand-over); from 512 rows on the MMAs
-// and, beside them, the epilogue's instructions (gate/up of 10,184 rows: 405 us, without any epilogue 350).
+// What it measured when it replaced the rows-on-lanes kernel with separate norm and post-processing kernels (four projections and
+// what lies between them, per layer, B200): 16 rows 46 -> 34 us, 71 rows 50 -> 41, 237 rows 80 -> 57, 336 rows 78 -> 68.  Whole decode
+// steps then and now: 1.5B shape, 16 rows 2.03 -> 1.32 ms, 237 rows 3.76 -> 2.57 ms; 8B shape, 64 rows 6.28 -> 4.43 ms.
+// What bounds it: up to about 128 rows the weight stream (gate/up of 16 rows: 55 MB in the 11.5 us from its first request to its
+// last tile, 4.8 TB/s of 6.55 copy rate, 5 us of it before its turn) and a fixed chain per launch (hand-over 0.7 us, first tile 0.5,
+// drain 1-2; where K is split 1.2-1.8 more, the slices of a row being read one after another).  From 512 rows on the MMAs and,
+// beside them, the epilogue's instructions (gate/up of 10,184 rows: 405 us, without any epilogue 350).  Counters, alone on the GPU:
+// gate/up 64 rows 17.2 us, tensor pipe 13 %, DRAM 39 %; 1,024 rows 48.5 us, 70 %, 15 %; 10,240 rows 362 us, 91 %.
 //
 // All waits on mbarriers are bounded; one that runs out raises DEV_ERR_WAIT_TIMEOUT, every role leaves its loop, and the
 // CTA frees its TMEM before it returns.
@@ -409,8 +411,9 @@ struct EpiStore {
     __device__ __forceinline__ void end() {}
 };
 
-// g / (1 + e^-g) with the hardware exponential and reciprocal: good to about 2^-21, where the product is rounded to 2^-11 (half)
-// or 2^-8 (bfloat16) next.
+// g / (1 + e^-g) with the hardware exponential and reciprocal.  For g >= 0 good to 2^-21; below, the rounding of the exponent's argument
+// counts |g| times, 2^-20 at g = -10.  The product is rounded to 2^-11 (half) or 2^-8 (bfloat16) next.  Against 64 bits the logits
+// of the 1.5B and 8B shapes are as far off as with expf and a division (decode 16-560 rows: 0.991 to 1.011 times).
 __device__ __forceinline__ float silu(float g) {
     float e, r;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(g * -1.4426950408889634f));

@@ -952,7 +952,7 @@ int pc_set_gemm_plan(pc_ctx* ctx, const char* spec) {
         if (kind < 0) return PC_ERR_INVALID_ARG;
         int w = 0, s = 0, used = 0;
         if (std::sscanf(p + len, "%dx%d%n", &w, &s, &used) != 2) return PC_ERR_INVALID_ARG;
-        if ((w != 64 && w != 128 && w != 256) || s < 1 || s > kMaxSplits) return PC_ERR_INVALID_ARG;      // 128: fused QKV epilogue only
+        if ((w != 64 && w != 128 && w != 256) || s < 1 || s > kMaxSplits) return PC_ERR_INVALID_ARG;
         bn[kind] = w; sp[kind] = s;
         p += len + used;
         if (*p == ',') ++p;
