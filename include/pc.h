@@ -212,7 +212,7 @@ PC_API int pc_set_dependent_launch(pc_ctx* ctx, int mask);
 
 /* bf16 models, decode steps that only sample (no logits_out, no log-probability buffer): 1 draws the token in
  * the epilogue of the LM-head GEMM -- per half tile of the vocabulary the largest and second-largest perturbed score
- * and the arg-max, folded per row by a small second kernel -- so the step's [rows, vocab] logits are never written or read
+ * and the arg-max, folded per row by a small kernel behind it (one in front computes the rows' factors of the final norm) -- so the step's [rows, vocab] logits are never written or read
  * back; 0 (the default) stores the logits and runs the stand-alone sampler on them.  Both draw exactly the same tokens
  * (Section 4.2: T = 1.0, top_p = 1.0; pc_sample states the rule): the tiles of a row share a running lower bound of the
  * row's second-best score, so which candidates a tile scores depends on timing, the folded result does not.  The
