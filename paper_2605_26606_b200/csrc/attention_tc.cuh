@@ -6,8 +6,10 @@
 // first product, V the MN-major operand of the second.  Two S accumulators let the next S run under the softmax, and two CTAs
 // per SM (113 KB, 256 TMEM columns each) overlap one's softmax with the other's MMAs.
 //
-// The running reference of a row's softmax only moves when its maximum grows by more than 2^8 over it: O is then rescaled in
-// TMEM.  Below that P stays below 256, far inside half's range, and the reference cancels in the result.
+// The running reference of a row's softmax is its maximum so far; when that grows, O is rescaled in TMEM.  A reference that lags
+// behind it by up to 2^8 saves most of the rescaling (prefill of 351 tokens 2 %, 2,048 rows 1 %, fewer rows nothing) but costs precision:
+// the large P then lie anywhere between powers of two instead of just below 1, where half rounds finest, and the K and V of a prefill
+// were 0.22 % (+- 0.02) further from 64 bits.
 //
 // What bounds it: chains, not a pipe.  Alone on the GPU (cold) a launch of 96-128 CTAs takes 12.5 us with three tiles a CTA (64 rows x
 // 640 keys) and 20.9 us with ten (1,024 rows): about 1.2 us or 2,400 clocks a tile, of which the exponentials (16 per clock and
@@ -40,7 +42,6 @@ constexpr int Q_BYTES = QROWS * HD * 2, P_BYTES = QROWS * TK * 2, KV_BYTES = TK 
 constexpr int THREADS = 192;        // warps 0..3 softmax (TMEM lane quarter = warp), 4 MMA issuer, 5 TMA producer
 constexpr int TMEM_COLS = 256;      // O: columns 0..127, S: 128..191 and 192..255
 constexpr int SMEM_BYTES = Q_BYTES + P_BYTES + STAGES * 2 * KV_BYTES + 1024;      // 113 KB: half of an SM's 228 KB less the reserved KB
-constexpr float SLACK = 8.f;        // log2 growth of a row's maximum that is tolerated before its reference moves
 
 // Shared-memory descriptor of an MN-major 128-byte-swizzled operand: rows of 64 values along MN (128 bytes), 8-row groups along K
 // 1024 bytes apart, blocks of 64 along MN `mn_stride` bytes apart.
@@ -253,7 +254,7 @@ attn_prefix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
             // P's buffer and O are free once the previous P V is done
             if (t > 0 && !warp_wait(odone, (uint32_t)(t - 1) & 1u)) { ok = false; break; }
             tc_fence_after();
-            const bool move = mx > m + SLACK || (m == -INFINITY && mx > -INFINITY);
+            const bool move = mx > m;
             if (__any_sync(0xffffffffu, move)) {
                 const float corr = move ? (m == -INFINITY ? 0.f : ex2(m - mx)) : 1.f;
                 if (move) m = mx;

@@ -227,7 +227,7 @@ Carve carve(const pc_ctx* c, int max_rows, int max_prefill) {
     v.out_index = take(M * 8);
     v.group_start = take((M + 1) * 4);
     v.ssq = take((size_t)((d.d_model + 63) / 64) * M * 4);       // per-tile sums of squares of the residual rows (EpiResNorm)
-    v.row_pow2 = take(3 * M * 4);       // powers of two of the attention and MLP norms' half operands, factors of the final norm (EpiSample)
+    v.row_pow2 = take(3 * M * 4);       // powers of two in the MLP and the attention norms' half operands, factors of the final norm (EpiSample)
     // fused LM head + sampler: one record per (vocabulary tile of the narrowest tile width, row)
     v.sample_tiles = take(2 * (size_t)((d.vocab + 63) / 64) * (size_t)std::max(max_rows, 1) * sizeof(pc::Top2Rec));   // one record per half tile
     v.sample_bound = take((size_t)std::max(max_rows, 1) * sizeof(int32_t));

@@ -4,6 +4,7 @@ import dataclasses
 
 import numpy as np
 import pytest
+import torch
 
 from oracle.decoder import Decoder
 from paper_2605_26606_b200 import workloads as wl
@@ -38,3 +39,38 @@ def test_decode_logits_at_attention_tile_edges(cuda_device, model, prompt, rows,
             logits, rp, rr = eng.record_pilot_logits[s]
             row = int(np.flatnonzero((rp == p) & (rr == i))[0])
             assert np.max(np.abs(logits[row].cpu().numpy() - want[prompt + s])) <= 5e-2, (p, i, s)
+
+
+def test_probabilities_round_below_their_maximum(cuda_device):
+    """Half rounds a probability finest just below the row's largest, which is 1 and exact.  64 keys of one kind, then 200 whose score is
+    higher by log2(1.00044): as 1.00044 they would round to 1, a relative error of 4.4e-4 in every output; as 1, beside 0.99956 for
+    the others, they lose nothing.  Layer 1's V reads the outputs back: three half roundings each (rms 2^-11 / sqrt 3, zero mean), so the
+    mean error over 256 of them has a deviation of 3e-5 at most."""
+    ensure_built()
+    model = dataclasses.replace(wl.SMALL_QKNORM_BF16, name="two-kinds-of-keys", qk_norm=False, tied_embed=False, rms_eps=1e-12)
+    weights, rng = wl.gen_weights(model, seed=4, threads=4), np.random.default_rng(0)
+    d, hd = model.d_model, model.head_dim
+    zero = {n: np.zeros_like(weights[n]) for n in weights.names() if n.startswith("layers.") and "norm" not in n}
+    e = np.zeros((model.vocab, d), np.float32)
+    e[:, :128] = 2.0                                        # rms 1; the other coordinates receive the attention's outputs
+    e[0, 0] = -2.0                                          # token 0: the first kind of key, any other: the second
+    zero["layers.0.wq"][hd // 2 - 1::hd, 1] = 0.5           # the slowest rotary pair: q = 1 and k = -+ 0.00249 at every position
+    zero["layers.0.wk"][hd // 2 - 1::hd, 0] = 0.001244
+    c = (1 + rng.integers(0, 128, model.kv_dim) / 128).astype(np.float32)
+    zero["layers.0.wv"][:, 0] = zero["layers.0.wv"][:, 1] = c / 4            # V = 0 for the first kind, c for the second
+    zero["layers.0.wo"][128 + np.arange(384), np.arange(384)] = 0.25
+    zero["layers.1.wv"][np.arange(256), 128 + np.arange(256)] = 1.0
+    for name, a in {**zero, "embed": e}.items():
+        weights.put(name, a, True)
+    tokens = np.r_[np.zeros(64, np.int32), np.full(200, 7, np.int32)]
+    w = dataclasses.replace(wl.WORKLOADS["config0"], model=model, n_prompts=1, prompt_len_lo=264, prompt_len_hi=264, group_size=2, n_pilot=2,
+                            max_new=2, cap_lo=2, cap_hi=2, data_seed=5, forced_explicit=None)
+    batch = dataclasses.replace(wl.gen_batch(w), prompt_tokens=tokens)
+    eng = RolloutEngine(model, weights, max_rows=2, max_prefill_tokens=264)
+    eng.pilot_commit_step(w, batch)
+    _, kv = Decoder(model, weights).forward_full(tokens, return_kv=True, last_only=True)
+    got = eng.prompt_kv[1, 1, :, 263].contiguous().view(torch.float16).cpu().numpy().astype(np.float64).reshape(-1)
+    want = kv[1][1][263].reshape(-1)
+    off = float(np.mean(got / want - 1))
+    print(f"mean relative error {off:.2e}")
+    assert np.min(want) > 0.1 and abs(off) <= 1e-4, off
