@@ -11,10 +11,10 @@
 // the large P then lie anywhere between powers of two instead of just below 1, where half rounds finest, and the K and V of a prefill
 // were 0.22 % (+- 0.02) further from 64 bits.
 //
-// What bounds it: chains, not a pipe.  Alone on the GPU (cold) a launch of 96-128 CTAs takes 12.5 us with three tiles a CTA (64 rows x
-// 640 keys) and 20.9 us with ten (1,024 rows): about 1.2 us or 2,400 clocks a tile, of which the exponentials (16 per clock and
+// What bounds it: chains, not a pipe.  Alone on the GPU (cold) a launch of 96-128 CTAs takes 12.8 us with three tiles a CTA (64 rows x
+// 640 keys) and 22.5 us with ten (1,024 rows): about 1.4 us or 2,700 clocks a tile, of which the exponentials (16 per clock and
 // SM) would be 512, and 9 us that no tile explains (launch, q, first K, record).  Prefill of 16 x 640 tokens, 960 CTAs of 5.5 tiles:
-// 67.6 us, 1.9 us of an SM's time per tile with a CTA's start and end in it.  Tensor pipe 9 / 16 / 19 %, DRAM 10 / 8 / 8 % busy.
+// 71.3 us, 2.0 us of an SM's time per tile with a CTA's start and end in it.  Tensor pipe 8 / 15 / 17 %, DRAM 10 / 8 / 7 % busy.
 // The mma.sync kernel (attn_group_kernel, kept for head_dim 64) needs 5,000 clocks for a tile of half the rows.
 #pragma once
 

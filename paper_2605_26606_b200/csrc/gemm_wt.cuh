@@ -28,7 +28,7 @@
 // last tile, 4.8 TB/s of 6.55 copy rate, 5 us of it before its turn) and a fixed chain per launch (hand-over 0.7 us, first tile 0.5,
 // drain 1-2; where K is split 1.2-1.8 more, the slices of a row being read one after another).  From 512 rows on the MMAs and,
 // beside them, the epilogue's instructions (gate/up of 10,184 rows: 405 us, without any epilogue 350).  Counters, alone on the GPU:
-// gate/up 64 rows 17.2 us, tensor pipe 13 %, DRAM 39 %; 1,024 rows 48.5 us, 70 %, 15 %; 10,240 rows 362 us, 91 %.
+// gate/up 64 rows 17.6 us, tensor pipe 13 %, DRAM 38 %; 1,024 rows 49.1 us, 70 %, 15 %; 10,240 rows 368 us, 91 %.
 //
 // All waits on mbarriers are bounded; one that runs out raises DEV_ERR_WAIT_TIMEOUT, every role leaves its loop, and the
 // CTA frees its TMEM before it returns.
