@@ -60,7 +60,7 @@ struct EpiSample {
 
     // scored iff (2^23 - (w >> 9)) < the returned word: the candidate's noise could lift it above `second`
     static __device__ __forceinline__ uint32_t pass_word(float second, float lmax) {
-        const float T = second - lmax - 1e-3f * (1.f + fabsf(second) + fabsf(lmax));      // conservative, as in scan_blocks
+        const float T = second - lmax - 1e-3f * (1.f + fabsf(second) + fabsf(lmax));      // conservative: far above the float error of its evaluation
         const float d = -expm1f(-expf(-T)) * 8388608.f;
         return d >= 8388608.f ? 0xffffffffu : (uint32_t)(d * 1.001f + 2.f);
     }

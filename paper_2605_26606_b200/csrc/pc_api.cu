@@ -1450,7 +1450,7 @@ int decode_launches(pc_ctx* ctx, cudaStream_t st, int m_bound, int groups_bound,
             pc::Top2Rec* scratch = reinterpret_cast<pc::Top2Rec*>(ctx->ws + ctx->cv.sample_scratch);
             launch_k(pc::sample_partial_kernel, dim3(dim3(m_bound, chunks)), dim3(256), 0, st, sd, ctx->d.vocab, chunks, logits, nullptr, 1.f, 0u, 0u,
                                                                              keys.key_prompt, keys.rollout, keys.step_key, 0, scratch, nullptr, da);
-            launch_k(pc::sample_reduce_kernel, dim3((m_bound + 127) / 128), dim3(128), 0, st, sd, m_bound, chunks, scratch, nullptr, keys.out_index, 0,
+            launch_k(pc::sample_reduce_kernel, dim3((m_bound + pc::REDUCE_ROWS - 1) / pc::REDUCE_ROWS), dim3(32 * pc::REDUCE_ROWS), 0, st, sd, m_bound, chunks, scratch, nullptr, keys.out_index, 0,
                                                                             nullptr, da);
             count_launches(2);
         }
@@ -1612,7 +1612,7 @@ int pc_sample(void* stream, int n_rows, int vocab, const float* logits, const in
         pc::Top2Rec* rec = static_cast<pc::Top2Rec*>(scratch);
         launch_k(pc::sample_partial_kernel, dim3(dim3(n_rows, chunks)), dim3(256), 0, st, nullptr, vocab, chunks, logits, logits_row, temperature, k0, k1,
                                                                         row_prompt, row_rollout, row_step, 0, rec, nullptr, nullptr);
-        launch_k(pc::sample_reduce_kernel, dim3((n_rows + 127) / 128), dim3(128), 0, st, nullptr, n_rows, chunks, rec, out_tokens, out_index, 0,
+        launch_k(pc::sample_reduce_kernel, dim3((n_rows + pc::REDUCE_ROWS - 1) / pc::REDUCE_ROWS), dim3(32 * pc::REDUCE_ROWS), 0, st, nullptr, n_rows, chunks, rec, out_tokens, out_index, 0,
                                                                        out_top2_gap, nullptr);
         count_launches(2);
     }
@@ -1744,7 +1744,7 @@ int pc_sample_static(void* stream, int n_rows, int vocab, const float* logits, c
     // every record the second kernel reads is written by the first one in this same call: nothing has to start at zero
     launch_k(pc::sample_partial_kernel, dim3(dim3(n_rows, chunks)), dim3(256), 0, st, nullptr, vocab, chunks, logits, logits_row, temperature, k0, k1,
                                                                     row_prompt, row_rollout, row_step, 0, rec, nullptr, nullptr);
-    launch_k(pc::sample_reduce_kernel, dim3((n_rows + 127) / 128), dim3(128), 0, st, nullptr, n_rows, chunks, rec, out_tokens, out_index, 0, out_top2_gap, nullptr);
+    launch_k(pc::sample_reduce_kernel, dim3((n_rows + pc::REDUCE_ROWS - 1) / pc::REDUCE_ROWS), dim3(32 * pc::REDUCE_ROWS), 0, st, nullptr, n_rows, chunks, rec, out_tokens, out_index, 0, out_top2_gap, nullptr);
     count_launches(2);
     PC_CUDA_CHECK_LAUNCH("sample (static scratch)");
     return PC_OK;

@@ -24,6 +24,29 @@ __device__ __forceinline__ Philox4 philox4x32_10(uint32_t c0, uint32_t c1, uint3
     return Philox4{c0, c1, c2, c3};
 }
 
+// The same with the round keys in registers (as the compiler would have it, they are added up again in every block: 18 of 100
+// instructions).
+struct PhiloxKeys {
+    uint32_t a[10], b[10];
+    __device__ __forceinline__ PhiloxKeys(uint32_t k0, uint32_t k1) {
+#pragma unroll
+        for (int r = 0; r < 10; ++r) {
+            a[r] = k0 + (uint32_t)r * 0x9E3779B9u;
+            b[r] = k1 + (uint32_t)r * 0xBB67AE85u;
+            asm volatile("" : "+r"(a[r]), "+r"(b[r]));
+        }
+    }
+};
+__device__ __forceinline__ Philox4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, const PhiloxKeys& k) {
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+        const uint64_t p0 = (uint64_t)0xD2511F53u * c0, p1 = (uint64_t)0xCD9E8D57u * c2;
+        const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ k.a[r], n2 = (uint32_t)(p0 >> 32) ^ c3 ^ k.b[r];
+        c0 = n0; c1 = (uint32_t)p1; c2 = n2; c3 = (uint32_t)p0;
+    }
+    return Philox4{c0, c1, c2, c3};
+}
+
 // u = ((w >> 9) + 1/2) / 2^23 is exact in float and lies strictly inside (0, 1).
 __device__ __forceinline__ float gumbel_from_word(uint32_t w) {
     const float u = ((float)(w >> 9) + 0.5f) * 1.1920928955078125e-07f;   // 2^-23
@@ -68,29 +91,60 @@ __device__ __forceinline__ Top2 top2_warp_reduce(Top2 t) {
     return t;
 }
 
-// Scores the 4-id blocks b0, b0 + stride, ... < b1 of one row and folds them into t.
+// Scores the 4-id blocks b_begin .. b_end - 1 of one row (a thread block of SAMPLE_THREADS) and folds them into t.
 //
-// Almost every candidate is rejected without evaluating its Gumbel noise: v can enter the thread's top two only if
-// logit_v / T + g_v > t.second, hence only if g_v > t.second - lmax (lmax >= every logit_v / T of the range), i.e. only if
-// 1 - u_v < 1 - exp(-exp(-(t.second - lmax))).  u_v is an affine function of the random word, so this is one integer
-// comparison per candidate against a bound that is refreshed whenever the thread's second-best score rises.  The bound
-// carries a slack far above the float error of its evaluation, and candidates that pass are scored exactly as before, so
-// the result is identical to scoring everything.
+// Almost every candidate is rejected without evaluating its Gumbel noise.  v can enter the row's top two only if
+// logit_v / T + g_v > s for every lower bound s of the row's second-best score, that is only if
+// 1 - u_v < 1 - exp(-x), x = exp(logit_v / T - s), and 1 - exp(-x) <= x.  u_v is an affine function of the random word, so a block of four
+// ids costs one exponential (of its largest logit) and one comparison (of its largest word).  s is the best second-best score any warp
+// of the thread block has found, through one word of shared memory.  The bound carries a slack far above the float error of its
+// evaluation, a comparison with a NaN passes, and candidates that pass are scored in full, so the result is identical to scoring
+// everything.
+//
+// What bounds it: the issue slots (123 instructions per 128 ids; Philox is 20 multiplications and 20 three-way XORs of them, the 32 x 32 -> 64
+// multiplications alone half of the time), then the logits, which are read once.  With one bound per warp from the largest logit of the whole
+// range -- a pass of its own over the row -- most blocks of 128 ids still held a candidate, and voting on, queueing and scoring those was
+// half of the 245 instructions.  Vocabulary 151,936, both kernels of a draw, then and now: 16 rows 26 -> 16 us, 71 rows 57 -> 30,
+// 256 rows 127 -> 69, 2,048 rows 577 -> 375.
+constexpr int SAMPLE_THREADS = 256;
+constexpr int SAMPLE_BLOCKS = 4;        // resident per SM
 constexpr int SAMPLE_QUEUE = 160;       // per-warp queue of candidates that passed the bound: 32 waiting + up to 128 new
 
+// Bound of the words (as 2^23 + (w >> 9)) below which no candidate with a logit up to l can beat the score s; unit = log2(e) / T and
+// shift = -s log2(e) plus the slack of 1e-3 (1 + |s|), the slack of 1e-3 |l / T| is added here.
+__device__ __forceinline__ float word_limit(float l, float unit, float shift) {
+    const float y = l * unit;
+    float x;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(fmaf(fabsf(y), 1e-3f, y) + shift));
+    return fmaf(x, -8388608.f * 1.001f, 16777214.f);       // 2^24 - (2^23 x 1.001 + 2)
+}
+__device__ __forceinline__ float word_value(uint32_t w) { return __uint_as_float(0x4b000000u | (w >> 9)); }       // 2^23 + (w >> 9)
+
 __device__ __forceinline__ void scan_blocks(Top2& t, const float* __restrict__ lg, int vocab, int b_begin, int b_end,
-                                            float temperature, float lmax, uint32_t c1, uint32_t c2, uint32_t c3,
-                                            uint32_t k0, uint32_t k1, uint2* __restrict__ queue /*this warp's SAMPLE_QUEUE slots*/) {
-    // The bound uses the largest second-best score of the warp: the final second-best is at least that, so a candidate
-    // below it can change neither the winner nor the gap.  Candidates that pass are not scored where they are found (a
-    // lane or two would drag the whole warp through the logarithms on most draws) but parked in a warp-private queue
-    // and scored 32 at a time, one per lane.  Trip counts are warp-uniform (shuffles and ballots need every lane).
-    int pass_above = -1;                        // a candidate is scored iff (int)(w >> 9) > pass_above  (-1: every candidate)
-    float bound_for = -INFINITY;                // warp-wide score the bound was computed for
-    bool stale = true;                          // a score was folded since the bound was computed (warp-uniform)
+                                            float temperature, uint32_t c1, uint32_t c2, uint32_t c3, uint32_t k0, uint32_t k1,
+                                            uint2* __restrict__ queue /*this warp's SAMPLE_QUEUE slots*/, volatile int32_t* bound /*of the thread block, ordered form; -inf*/) {
+    constexpr int U = 2;                        // blocks of a thread in hand; as many more are on their way from memory
+    constexpr float LOG2E = 1.4426950408889634f;
     const int lane = threadIdx.x & 31;
     const uint32_t lt_mask = (1u << lane) - 1u;
+    const PhiloxKeys keys(k0, k1);
+    const float unit = LOG2E / temperature;
+    int32_t bound_for = score_to_ordered(-INFINITY);
+    float shift = INFINITY;                     // of the bound in use: -inf, everything passes
     int queued = 0;                             // warp-uniform
+    auto set_bound = [&](int32_t b) {
+        bound_for = b;
+        const float s = ordered_to_score(b);
+        shift = fmaf(-s, LOG2E, 1e-3f * LOG2E * (1.f + fabsf(s)));
+    };
+    auto share_bound = [&](float best, float second) {          // second-best of the warp's scores: a lower bound of the row's
+        const Top2 w = top2_warp_reduce(Top2{best, second, 0});
+        if (w.second > ordered_to_score(bound_for)) {
+            const int32_t b = score_to_ordered(w.second);
+            if (lane == 0) atomicMax(const_cast<int32_t*>(bound), b);
+            set_bound(b);
+        }
+    };
     auto drain = [&](int keep) {                // scores queued candidates, 32 at a time, until at most `keep` remain
         while (queued > keep) {
             const int take = min(32, queued);
@@ -100,45 +154,80 @@ __device__ __forceinline__ void scan_blocks(Top2& t, const float* __restrict__ l
                 top2_push_unordered(t, lg[c.x] / temperature + gumbel_from_word(c.y), (int)c.x);
             }
             queued -= take;
-            stale = true;
+            share_bound(t.best, t.second);
             __syncwarp();
         }
     };
-    for (int base = b_begin + (threadIdx.x - lane); base < b_end; base += blockDim.x) {
-        if (stale) {                             // the second-best scores only move when candidates were scored
-            stale = false;
-            const float ws = warp_max(t.second);
-            if (ws > bound_for) {
-                bound_for = ws;
-                const float T = ws - lmax - 1e-3f * (1.f + fabsf(ws) + fabsf(lmax));     // conservative
-                // (1 - U0) * 2^23 with U0 = exp(-exp(-T)); expm1f keeps the relative accuracy when U0 is close to 1
-                const float d = -expm1f(-expf(-T)) * 8388608.f;
-                // scored iff 2^23 - (w >> 9) < d * 1.001 + 2, i.e. iff (w >> 9) > 2^23 - (that bound)
-                pass_above = d >= 8388608.f ? -1 : 8388608 - (int)(uint32_t)(d * 1.001f + 2.f);
-            }
-        }
-        const int b = base + lane;
-        Philox4 w{0, 0, 0, 0};
-        if (b < b_end) w = philox4x32_10((uint32_t)b, c1, c2, c3, k0, k1);
-        // Almost every block holds no candidate above the bound: one comparison on the block's largest word and one vote
-        // decide that for the whole warp; only blocks that may hold one go through the per-word test and the queue.
+    // one candidate per lane, the one with the largest word, for a first bound (not folded: it is scored again later)
+    auto seed = [&](bool in, const Philox4& w, const float4& l) {
         const uint32_t top = max(max(w.x, w.y), max(w.z, w.w));
-        if (!__any_sync(0xffffffffu, b < b_end && (int)(top >> 9) > pass_above)) continue;
+        const float at = top == w.x ? l.x : (top == w.y ? l.y : (top == w.z ? l.z : l.w));
+        const float s = in ? at / temperature + gumbel_from_word(top) : -INFINITY;
+        share_bound(s > -INFINITY ? s : -INFINITY /*NaN too*/, -INFINITY);
+    };
+    auto consider = [&](bool in, int b, const Philox4& w, const float4& l) {
+        const uint32_t top = max(max(w.x, w.y), max(w.z, w.w));
+        const float most = fmaxf(fmaxf(l.x, l.y), fmaxf(l.z, l.w));
+        if (!__any_sync(0xffffffffu, in && !(word_value(top) <= word_limit(most, unit, shift)))) return;
         const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+        const float ll[4] = {l.x, l.y, l.z, l.w};
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int v = b * 4 + i;
-            const bool pass = b < b_end && v < vocab && (int)(ww[i] >> 9) > pass_above;
+            const bool pass = in && v < vocab && !(word_value(ww[i]) <= word_limit(ll[i], unit, shift));
             const uint32_t m = __ballot_sync(0xffffffffu, pass);
             if (pass) queue[queued + __popc(m & lt_mask)] = make_uint2((uint32_t)v, ww[i]);
             queued += __popc(m);
         }
         drain(31);
+    };
+    auto refresh = [&]() {
+        const int32_t b = *bound;
+        if (__any_sync(0xffffffffu, b > bound_for)) set_bound(__reduce_max_sync(0xffffffffu, b));
+    };
+    bool first = true;
+    int base = b_begin + (int)(threadIdx.x - lane);          // trip counts are warp-uniform (shuffles and ballots need every lane)
+    // rounds in which all of the warp's blocks are whole and their logits can be read as vectors
+    const int whole = (reinterpret_cast<uintptr_t>(lg) & 15u) == 0 ? min(b_end, vocab >> 2) - ((U - 1) * SAMPLE_THREADS + 31) : 0;
+    if (base < whole) {
+        const float4* p = reinterpret_cast<const float4*>(lg) + base + lane;
+        float4 next[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) next[u] = p[u * SAMPLE_THREADS];
+#pragma unroll 1
+        for (; base < whole; base += U * SAMPLE_THREADS) {
+            float4 l[U];
+            Philox4 w[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) l[u] = next[u];
+            p += U * SAMPLE_THREADS;
+            if (base + U * SAMPLE_THREADS < whole)
+#pragma unroll
+                for (int u = 0; u < U; ++u) next[u] = p[u * SAMPLE_THREADS];
+#pragma unroll
+            for (int u = 0; u < U; ++u) w[u] = philox4x32_10((uint32_t)(base + u * SAMPLE_THREADS + lane), c1, c2, c3, keys);
+            refresh();
+            if (first) { first = false; seed(true, w[0], l[0]); }
+#pragma unroll
+            for (int u = 0; u < U; ++u) consider(true, base + u * SAMPLE_THREADS + lane, w[u], l[u]);
+        }
+    }
+#pragma unroll 1
+    for (; base < b_end; base += SAMPLE_THREADS) {
+        const int b = base + lane;
+        float l[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) l[i] = b < b_end && 4 * b + i < vocab ? lg[4 * b + i] : -INFINITY;
+        const float4 l4 = make_float4(l[0], l[1], l[2], l[3]);
+        const Philox4 w = philox4x32_10((uint32_t)b, c1, c2, c3, keys);
+        refresh();
+        if (first) { first = false; seed(b < b_end, w, l4); }
+        consider(b < b_end, b, w, l4);
     }
     drain(0);
 }
 
-// Largest logit / T over the blocks a thread block will scan (block-wide); `red` is 33 floats of shared memory.
+// Largest logit / T of v0 <= v < v1 (block-wide); `red` is 33 floats of shared memory.
 __device__ __forceinline__ float range_max(const float* __restrict__ lg, int v0, int v1, float temperature, float* red) {
     float m = -INFINITY;
     // 16-byte loads, four in flight per thread: a row is hundreds of KB and one scalar load per thread at a time would
@@ -169,7 +258,7 @@ __device__ __forceinline__ float range_max(const float* __restrict__ lg, int v0,
 }
 
 // One block per row.
-__global__ void __launch_bounds__(256) sample_kernel(const StepDesc* __restrict__ sd, int vocab, const float* __restrict__ logits,
+__global__ void __launch_bounds__(SAMPLE_THREADS, SAMPLE_BLOCKS) sample_kernel(const StepDesc* __restrict__ sd, int vocab, const float* __restrict__ logits,
                                                      const int32_t* __restrict__ logits_row, float temperature,
                                                      uint32_t k0, uint32_t k1, const int32_t* __restrict__ row_prompt,
                                                      const int32_t* __restrict__ row_rollout, const int32_t* __restrict__ row_step,
@@ -188,10 +277,11 @@ __global__ void __launch_bounds__(256) sample_kernel(const StepDesc* __restrict_
                    c3 = (uint32_t)(prompt_key ? prompt_key[row_prompt[ro]] : row_prompt[ro]);    // key id of the prompt
     Top2 t{-INFINITY, -INFINITY, 0x7fffffff};
     const int n_blocks = (vocab + 3) >> 2;
-    __shared__ float red[33];
-    __shared__ uint2 queue[8][SAMPLE_QUEUE];
-    const float lmax = range_max(lg, 0, vocab, temperature, red);
-    scan_blocks(t, lg, vocab, 0, n_blocks, temperature, lmax, c1, c2, c3, k0, k1, queue[threadIdx.x >> 5]);
+    __shared__ int32_t bound;
+    __shared__ uint2 queue[SAMPLE_THREADS / 32][SAMPLE_QUEUE];
+    if (threadIdx.x == 0) bound = score_to_ordered(-INFINITY);
+    __syncthreads();
+    scan_blocks(t, lg, vocab, 0, n_blocks, temperature, c1, c2, c3, k0, k1, queue[threadIdx.x >> 5], &bound);
     t = top2_warp_reduce(t);
     __shared__ Top2 sh[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -215,7 +305,7 @@ __global__ void __launch_bounds__(256) sample_kernel(const StepDesc* __restrict_
 // ---------------------------------------------------------------------------------------------
 struct Top2Rec { float best, second; int idx; int pad; };
 
-__global__ void __launch_bounds__(256) sample_partial_kernel(const StepDesc* __restrict__ sd, int vocab, int n_chunks,
+__global__ void __launch_bounds__(SAMPLE_THREADS, SAMPLE_BLOCKS) sample_partial_kernel(const StepDesc* __restrict__ sd, int vocab, int n_chunks,
                                                              const float* __restrict__ logits, const int32_t* __restrict__ logits_row,
                                                              float temperature, uint32_t k0, uint32_t k1,
                                                              const int32_t* __restrict__ row_prompt, const int32_t* __restrict__ row_rollout,
@@ -232,10 +322,11 @@ __global__ void __launch_bounds__(256) sample_partial_kernel(const StepDesc* __r
     const int n_blocks = (vocab + 3) >> 2;
     const int per_chunk = (n_blocks + n_chunks - 1) / n_chunks;
     const int b_end = min(n_blocks, (chunk + 1) * per_chunk);
-    __shared__ float red[33];
-    __shared__ uint2 queue[8][SAMPLE_QUEUE];
-    const float lmax = range_max(lg, min(vocab, chunk * per_chunk * 4), min(vocab, b_end * 4), temperature, red);
-    scan_blocks(t, lg, vocab, chunk * per_chunk, b_end, temperature, lmax, c1, c2, c3, k0, k1, queue[threadIdx.x >> 5]);
+    __shared__ int32_t bound;
+    __shared__ uint2 queue[SAMPLE_THREADS / 32][SAMPLE_QUEUE];
+    if (threadIdx.x == 0) bound = score_to_ordered(-INFINITY);
+    __syncthreads();
+    scan_blocks(t, lg, vocab, chunk * per_chunk, b_end, temperature, c1, c2, c3, k0, k1, queue[threadIdx.x >> 5], &bound);
     t = top2_warp_reduce(t);
     __shared__ Top2 sh[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -248,18 +339,22 @@ __global__ void __launch_bounds__(256) sample_partial_kernel(const StepDesc* __r
     }
 }
 
-__global__ void sample_reduce_kernel(const StepDesc* __restrict__ sd, int n_rows, int n_chunks, const Top2Rec* __restrict__ scratch,
-                                     int32_t* __restrict__ out_tokens, const int64_t* __restrict__ out_index,
+// A warp per row, a record per lane (at most SAMPLE_MAX_CHUNKS = 32; the merge is order-independent: equal scores keep the lowest id).
+constexpr int REDUCE_ROWS = 4;          // rows (warps) of a block
+__global__ void __launch_bounds__(32 * REDUCE_ROWS) sample_reduce_kernel(const StepDesc* __restrict__ sd, int n_rows, int n_chunks,
+                                     const Top2Rec* __restrict__ scratch, int32_t* __restrict__ out_tokens, const int64_t* __restrict__ out_index,
                                      int64_t out_index_offset, float* __restrict__ out_gap, const DecodeArgsDev* __restrict__ da) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    const int r = blockIdx.x * REDUCE_ROWS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int64_t ro = r;
     if (r >= (sd != nullptr ? sd->n_rows : n_rows)) return;
     if (da != nullptr) out_tokens = da->tokens;
     Top2 t{-INFINITY, -INFINITY, 0x7fffffff};
-    for (int c = 0; c < n_chunks; ++c) {
-        const Top2Rec x = scratch[(size_t)r * n_chunks + c];
-        t = top2_merge(t, Top2{x.best, x.second, x.idx});
+    if (lane < n_chunks) {
+        const Top2Rec x = scratch[(size_t)r * n_chunks + lane];
+        t = Top2{x.best, x.second, x.idx};
     }
+    t = top2_warp_reduce(t);
+    if (lane != 0) return;
     const int64_t at = out_index ? out_index[ro] + out_index_offset : (int64_t)r;
     if (at >= 0) out_tokens[at] = t.idx;
     if (out_gap) out_gap[r] = t.best - t.second;
@@ -311,10 +406,17 @@ __global__ void __launch_bounds__(256) token_logprob_kernel(const StepDesc* __re
 }
 
 constexpr int SAMPLE_MAX_CHUNKS = 32;
-// Ranges per row so that about four blocks per SM are in flight; 1 means the one-pass kernel is the better choice.
+// Ranges per row: the number that minimises (waves of the grid) x (a range's share of the row + its fixed cost, 2 % of a row of 152,000
+// ids); 1 means the one-pass kernel.  (As many as give four blocks per SM or the next more: 768 blocks in two waves at 256 rows.)
 inline int sample_chunks(int n_rows, int num_sms) {
-    const int want = (4 * num_sms + n_rows - 1) / (n_rows > 0 ? n_rows : 1);
-    return want < 2 ? 1 : (want > SAMPLE_MAX_CHUNKS ? SAMPLE_MAX_CHUNKS : want);
+    const long long slots = (long long)SAMPLE_BLOCKS * num_sms;
+    int best = 1;
+    double best_cost = -1.;
+    for (int c = 1; c <= SAMPLE_MAX_CHUNKS; ++c) {
+        const double cost = (double)(((long long)n_rows * c + slots - 1) / slots) * (1. / c + 0.02);
+        if (best_cost < 0. || cost < best_cost * 0.98) { best_cost = cost; best = c; }
+    }
+    return best;
 }
 
 }  // namespace pc

@@ -54,6 +54,42 @@ def test_sample_matches_oracle(vocab, temperature):
             assert np.isinf(gap[r])
 
 
+@pytest.mark.parametrize("vocab", [5, 1003, 4100, 151936])
+@pytest.mark.parametrize("temperature", [1.0, 1e-3, 50.0])
+def test_sample_of_masked_and_extreme_logits(vocab, temperature):
+    """Rows whose scores leave the ordinary range: the bound that spares candidates their noise must not lose the winner."""
+    rng = np.random.default_rng(vocab)
+    low = np.finfo(np.float32).min
+    rows = (rng.normal(size=(8, vocab)) * 2).astype(np.float32)
+    rows[0, :] = -np.inf
+    rows[0, vocab // 2] = -7.0                              # one id allowed
+    rows[1, :] = low                                        # the noise is absorbed: all scores equal, or -inf where low / T overflows
+    rows[2, rng.random(vocab) < 0.9] = low
+    rows[3, rng.random(vocab) < 0.9] = -np.inf
+    rows[4, [vocab - 1, vocab // 3]] = np.inf               # two certain ids: the lower one
+    rows[5, rng.random(vocab) < 0.5] = np.nan               # never drawn
+    rows[6, :] = -np.inf                                    # nothing allowed: id 0, as for any tie
+    rows[7, :] *= 1e4
+    rows[2:6, vocab // 3 + 1] = 0.25
+    n = len(rows)
+    prompt, roll, step, seed = rng.integers(0, 50, n), rng.integers(0, 128, n), rng.integers(0, 2048, n), 99
+    got = []
+    for scratch in (None, torch.empty(n * 32 * 16, dtype=torch.uint8, device="cuda"), torch.empty(n * 3 * 16, dtype=torch.uint8, device="cuda")):
+        out, gap = torch.zeros(n, dtype=torch.int32, device="cuda"), torch.zeros(n, device="cuda")
+        B.pc_sample(n, vocab, torch.from_numpy(rows).cuda(), None, temperature, seed, _i32(prompt), _i32(roll), _i32(step), out, None, gap, scratch)
+        got.append((out.cpu().numpy(), gap.cpu().numpy()))
+    for out, gap in got[1:]:
+        assert np.array_equal(out, got[0][0]) and np.array_equal(gap, got[0][1], equal_nan=True)
+    out, gap = got[0]
+    assert list(out[[0, 1, 4, 6]]) == [vocab // 2, 0, vocab // 3, 0]
+    for r in (2, 3, 5, 7):
+        tok, g = osampler.sample(np.nan_to_num(rows[r].astype(np.float64), nan=-1e300, neginf=-1e300), temperature, seed, int(prompt[r]), int(roll[r]), int(step[r]))
+        # a float score of size |l / T| is rounded by 2^-24 of it, the noise by less than 1e-5
+        ordinary = rows[r][np.isfinite(rows[r]) & (rows[r] > low)].astype(np.float64)
+        if g > 1e-4 + 4 * 2.0 ** -24 * np.abs(ordinary).max() / temperature:
+            assert out[r] == tok
+
+
 def test_sample_row_mapping_and_scatter():
     rng = np.random.default_rng(0)
     V, P, G = 512, 3, 5
