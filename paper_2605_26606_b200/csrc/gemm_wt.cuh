@@ -26,7 +26,7 @@
 // steps then and now: 1.5B shape, 16 rows 2.03 -> 1.32 ms, 237 rows 3.76 -> 2.57 ms; 8B shape, 64 rows 6.28 -> 4.43 ms.
 // What bounds it: up to about 128 rows the weight stream (gate/up of 16 rows: 55 MB in the 11.5 us from its first request to its
 // last tile, 4.8 TB/s of 6.55 copy rate, 5 us of it before its turn) and a fixed chain per launch (hand-over 0.7 us, first tile 0.5,
-// drain 1-2; where K is split 1.2-1.8 more, the slices of a row being read one after another).  From 512 rows on the MMAs and,
+// drain 1-2; where K is split about 1 more for the hand-over of the partial tiles).  From 512 rows on the MMAs and,
 // beside them, the epilogue's instructions (gate/up of 10,184 rows: 405 us, without any epilogue 350).  Counters, alone on the GPU:
 // gate/up 64 rows 17.6 us, tensor pipe 13 %, DRAM 38 %; 1,024 rows 49.1 us, 70 %, 15 %; 10,240 rows 368 us, 91 %.
 //
@@ -385,6 +385,7 @@ __device__ __forceinline__ bool beyond_half(float m) { return !(m <= HALF_MAX_F)
 struct EpiStore {
     static constexpr bool kDual = true;       // may take its activations as value + rounding remainder
     static constexpr bool kScaled = true;     // the operand may lack its norm's factor
+    static constexpr bool kSplit = false;      // K may be split over a cluster
     static constexpr bool kSlots = false;
     static constexpr int NR = 4;
     float* C; int ld;
@@ -427,6 +428,7 @@ template <bool HALF>
 struct EpiSwiGLU {
     static constexpr bool kDual = false;       // may take its activations as value + rounding remainder
     static constexpr bool kScaled = HALF;
+    static constexpr bool kSplit = false;      // K may be split over a cluster
     static constexpr bool kSlots = false;
     static constexpr int NR = 4;
     Operand act; int ld;
@@ -469,6 +471,7 @@ template <bool HALF>
 struct EpiResNorm {
     static constexpr bool kDual = !HALF;       // may take its activations as value + rounding remainder
     static constexpr bool kScaled = false;
+    static constexpr bool kSplit = true;      // K may be split over a cluster (CTA pairs: never)
     static constexpr bool kSlots = false;
     static constexpr int NR = 4;
     float* h; int ld;
@@ -551,6 +554,7 @@ struct EpiResNorm {
 struct EpiQkv {
     static constexpr bool kDual = true;       // may take its activations as value + rounding remainder
     static constexpr bool kScaled = true;
+    static constexpr bool kSplit = true;      // K may be split over a cluster (CTA pairs: never)
     static constexpr bool kSlots = true;
     static constexpr int NR = 2;       // rotary factors of the rows in hand and of the next ones take registers
     int Hq, Hkv, layer;
@@ -658,7 +662,7 @@ struct EpiQkv {
 __device__ __forceinline__ int quotient(int x, uint64_t inverse) { return (int)(((uint64_t)(uint32_t)x * inverse) >> 32); }
 
 template <int CG, bool DUAL, class Epi>
-__global__ void __launch_bounds__(THREADS, 2)
+__global__ void __launch_bounds__(THREADS, 1)
 gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
                const __grid_constant__ CUtensorMap map_x_lo, const StepDesc* __restrict__ sd, const Geom G, Epi epi, int32_t* err) {
     extern __shared__ uint8_t smem_raw[];
@@ -673,6 +677,7 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     volatile int* outside_tile = abort_flag + 1;       // [2] the last tile (plus one) of this parity that has rows its operand does not hold
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool splitting = Epi::kSplit && CG == 1 && G.splits > 1;
     const uint32_t rank = cluster_rank();
     const uint32_t peer = CG == 2 ? rank & 1u : 0u, leader = rank - peer;
     const int split = (int)rank / CG;
@@ -837,9 +842,9 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             const int begin = min(live, split * share), end = min(live, begin + share);
             // The rows of this warp.  Whole tile: the groups take chunks of cw rows in turn, a warp every fourth row of a chunk.
             // Split tile: a warp takes every eighth row of the share.
-            int at = G.splits > 1 ? begin + warp - 2 : group * cw;
-            const int advance = G.splits > 1 ? 8 * NR : 2 * cw;
-            auto rows_of = [&](int p) { return G.splits > 1 ? Rows{p, 8, end} : Rows{p + quarter, 4, min(live, p + cw)}; };
+            int at = splitting ? begin + warp - 2 : group * cw;
+            const int advance = splitting ? 8 * NR : 2 * cw;
+            auto rows_of = [&](int p) { return splitting ? Rows{p, 8, end} : Rows{p + quarter, 4, min(live, p + cw)}; };
             epi.begin(c);
             epi.prefetch(c, rows_of(at));
             if (tid < live) {                                     // at most 256 rows: a thread each
@@ -859,7 +864,7 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
                 if (outside_tile[turn] == t + 1)
                     rescue_rows(c.f0 + lane128 < G.N ? reinterpret_cast<const __half*>(epi.rs.w) + (size_t)(c.f0 + lane128) * G.K : nullptr,
                                 epi.rs.h + (size_t)c.row0 * G.K, epi.rs.gain, G.K, kb0 * BK, kb1 * BK, live, tile_scale, taddr, group, err);
-            if (G.splits > 1) {
+            if (splitting) {
                 // leave the partial tile in this CTA's shared memory (the operand ring is drained) for the cluster
                 float* part = reinterpret_cast<float*>(tiles) + lane128;
 #pragma unroll 1
@@ -871,23 +876,37 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
                 }
                 cluster_sync();
             }
-            const int stop = G.splits > 1 ? end : live;
+            const int stop = splitting ? end : live;
 #pragma unroll 1
             for (; at < stop; at += advance) {
                 const Rows R = rows_of(at);
                 float4 x[NR];
-                if (G.splits > 1) {
-                    // the K ranges' partial sums of these rows, added in range order
+                if (splitting) {
+                    // the K ranges' partial sums of these rows, added in range order; all ranges of two rows are in flight together (a
+                    // read of another CTA's memory takes a quarter of a microsecond: one range after another took 1.2 us with six and
+                    // 1.8 us with eight, eight decode steps of 16 rows 10.51 -> 9.93 ms, of 237 rows 20.06 -> 19.73)
 #pragma unroll
                     for (int j = 0; j < NR; ++j) x[j] = f4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 1
-                    for (int s = 0; s < G.splits; ++s) {
-                        const uint32_t from = map_rank(tiles_u32 + (uint32_t)(R.r * FT + 4 * lane) * 4, (uint32_t)(s * CG) + peer);
 #pragma unroll
-                        for (int j = 0; j < NR; ++j)
-                            if (R.has(j)) {
-                                const float4 y = ld_cluster_f32x4(from + j * (8 * FT * 4));
-                                x[j] = f4(x[j].x + y.x, x[j].y + y.y, x[j].z + y.z, x[j].w + y.w);
+                    for (int j = 0; j < NR; j += 2) {
+                        if (!R.has(j)) break;
+                        const bool both = R.has(j + 1);
+                        const uint32_t at_row = tiles_u32 + (uint32_t)(R.at(j) * FT + 4 * lane) * 4;
+                        float4 y[MAX_SPLITS][2];
+#pragma unroll
+                        for (int s = 0; s < MAX_SPLITS; ++s) {
+                            y[s][0] = y[s][1] = f4(0.f, 0.f, 0.f, 0.f);
+                            if (s < G.splits) {
+                                const uint32_t from = map_rank(at_row, (uint32_t)s);
+                                y[s][0] = ld_cluster_f32x4(from);
+                                if (both) y[s][1] = ld_cluster_f32x4(from + 8 * FT * 4);
+                            }
+                        }
+#pragma unroll
+                        for (int s = 0; s < MAX_SPLITS; ++s)
+#pragma unroll
+                            for (int i = 0; i < 2; ++i) {
+                                x[j + i] = f4(x[j + i].x + y[s][i].x, x[j + i].y + y[s][i].y, x[j + i].z + y[s][i].z, x[j + i].w + y[s][i].w);
                             }
                     }
                 } else {
@@ -905,7 +924,7 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
                 }
                 epi.rows(c, x, R, rows_of(at + advance));
             }
-            if (G.splits == 1) {
+            if (!splitting) {
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) { if (CG == 2) mbar_arrive_cluster(tempty_at + 8 * acc); else mbar_arrive(tempty0 + 8 * acc); }
@@ -915,10 +934,10 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
         }
         if (!ok) {
             if (lane == 0) { *abort_flag = 1; set_error(err, DEV_ERR_WAIT_TIMEOUT); }
-            if (G.splits > 1) cluster_sync();                    // the meeting point this role would have reached
+            if (splitting) cluster_sync();                    // the meeting point this role would have reached
         }
     }
-    if (G.splits > 1 && warp < 2) cluster_sync();                // partial tiles are in place
+    if (splitting && warp < 2) cluster_sync();                // partial tiles are in place
     tc_fence_before();
     __syncthreads();
     if (*abort_flag) {
@@ -926,7 +945,7 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
         for (int i = 0; i < 2000; ++i) __nanosleep(1000);        // copies in flight land before the shared memory is released
         __syncthreads();
     }
-    if (G.splits > 1 || CG == 2) cluster_sync();                 // nobody leaves while a peer reads its memory or signals it
+    if (splitting || CG == 2) cluster_sync();                 // nobody leaves while a peer reads its memory or signals it
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
