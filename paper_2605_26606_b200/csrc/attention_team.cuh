@@ -1,11 +1,16 @@
-// Suffix attention of small decode batches: a cluster of C CTAs (C = 1, 2, 4 or 8) takes one (rollout, KV head), its 4 C warps
-// stream the item's tiles in turn, and the cluster merges their partial softmaxes and the item's shared-prefix records over
-// distributed shared memory into the attention output -- no records of its own, no merge kernel (a launch and three L2 round
-// trips: 5 us of a 60 us layer at 16 rows).  At 113 KB a CTA fits beside one of the shared-prefix kernel, whose programmatic
-// dependent it is: the two run side by side and this one waits for the records only when it merges.
+// Attention of small decode batches: a cluster of C CTAs (C = 1, 2, 4 or 8) takes one (rollout, KV head), its 4 C warps
+// stream the item's tiles in turn, and the cluster merges their partial softmaxes over distributed shared memory into the attention
+// output -- no records of its own, no merge kernel (a launch and three L2 round trips: 5 us of a 60 us layer at 16 rows).
 //
-// What bounds it: latency.  16 rows x 1,100: four tiles per warp (0.5 us each), the hand-over, and the chain record -> weights ->
-// output.
+//   JOINT   the tiles are the prompt's and then the suffix's, from two arenas: the kernel is the whole attention of a layer.  It follows the
+//           QKV projection; every tile but the one that projection writes into is requested before the wait.
+//   else    the tiles are the suffix's, and the item's shared-prefix records join the merge.  At 113 KB a CTA fits beside one of the
+//           shared-prefix kernel, whose programmatic dependent it is: the two run side by side and this one waits for the records
+//           only when it merges.
+// When which is taken: joint_attention in pc_api.cu.
+//
+// What bounds it: latency.  16 rows, 640 + 1,100 positions, four CTAs: seven tiles per warp (0.5 us each), the hand-over, and the chain
+// partial softmax -> weights -> output.
 #pragma once
 
 #include <type_traits>
@@ -31,9 +36,9 @@ template <int EPL> __device__ __forceinline__ void ld_cluster(uint32_t addr, flo
     }
 }
 
-template <int HD>
+template <int HD, bool JOINT>
 __global__ void __launch_bounds__(T_WARPS * 32, 2)
-attn_suffix_team_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* __restrict__ sd, int64_t n_slots, int Hq, int Hkv,
+attn_suffix_team_kernel(const __grid_constant__ CUtensorMap kv_map, const __grid_constant__ CUtensorMap prompt_map, int64_t prompt_slots, const StepDesc* __restrict__ sd, int64_t n_slots, int Hq, int Hkv,
                         int layer, const __nv_bfloat16* __restrict__ q, RowGeom g, float scale_log2, PrefixPartial part, int team_ctas,
                         __nv_bfloat16* __restrict__ out, __nv_bfloat16* __restrict__ out_lo, int32_t* err) {
     constexpr int KS = HD / 16, DT = HD / 16, EPL = HD / 32;
@@ -63,21 +68,30 @@ attn_suffix_team_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDe
     }
     __syncthreads();
 
-    const int n = g.s_len[row], tiles = (n + S_TP - 1) / S_TP;
+    const int n = g.s_len[row], n_prompt = JOINT ? g.p_len[row] : 0;
+    const int p_tiles = (n_prompt + S_TP - 1) / S_TP, tiles = p_tiles + (n + S_TP - 1) / S_TP;      // the prompt's tiles first
     const int workers = team_ctas * T_WARPS, me = rank * T_WARPS + warp;
     const int64_t krow = ((int64_t)layer * 2 * Hkv + kvh) * n_slots + g.s_start[row];
+    const int64_t prow = JOINT ? ((int64_t)layer * 2 * Hkv + kvh) * prompt_slots + g.p_start[row] : 0;
     int next = me, issued = 0, consumed = 0;
     auto issue = [&]() {
         const int stage = issued % T_STAGES;
         if (lane == 0) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             mbar_arrive_expect_tx(full0 + 8 * stage, 2 * TILE_BYTES);
-            tma_load_kv(tiles_u32 + stage * 2 * TILE_BYTES, &kv_map, full0 + 8 * stage, (int)(krow + (int64_t)next * S_TP));
+            if (JOINT && next < p_tiles) tma_load_kv(tiles_u32 + stage * 2 * TILE_BYTES, &prompt_map, full0 + 8 * stage, (int)(prow + (int64_t)next * S_TP));
+            else tma_load_kv(tiles_u32 + stage * 2 * TILE_BYTES, &kv_map, full0 + 8 * stage, (int)(krow + (int64_t)(next - p_tiles) * S_TP));
         }
         ++issued;
         next += workers;
     };
-    for (int i = 0; i < T_STAGES && next < tiles; ++i) issue();
+    if (JOINT) {
+        // all but the last tile, which holds the position the QKV projection is writing, were there before this step
+        while (issued < T_STAGES && next < tiles - 1) issue();
+        grid_dep_wait();
+        grid_dep_launch_dependents();          // the output projection may request its weights
+    }
+    while (issued < T_STAGES && next < tiles) issue();
     uint32_t qb[KS][2];
     {
         const int hq = lane >> 2;
@@ -97,7 +111,7 @@ attn_suffix_team_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDe
         const int stage = consumed % T_STAGES;
         if (!mbar_wait(full0 + 8 * stage, (uint32_t)(consumed / T_STAGES) & 1u, abort_flag)) { ok = false; break; }
         const uint32_t kb = tiles_u32 + stage * 2 * TILE_BYTES;
-        suffix_tile<HD>(kb, kb + TILE_BYTES, lane, min(S_TP, n - tile * S_TP), scale_log2, qb, o, mh, lh, [&]() {
+        suffix_tile<HD>(kb, kb + TILE_BYTES, lane, min(S_TP, tile < p_tiles ? n_prompt - tile * S_TP : n - (tile - p_tiles) * S_TP), scale_log2, qb, o, mh, lh, [&]() {
             ++consumed;
             __syncwarp();
             if (next < tiles) issue();
@@ -106,10 +120,12 @@ attn_suffix_team_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDe
     suffix_finish<HD>(lane, o, mh, lh, ml + warp * 16, ml + warp * 16 + 8, obuf + warp * 8 * HD);
     if (!ok) { *abort_flag = 1; if (lane == 0) set_error(err, DEV_ERR_WAIT_TIMEOUT); }
 
-    grid_dep_wait();                           // the shared-prefix kernel's records
-    grid_dep_launch_dependents();              // the output projection may request its weights
+    if (!JOINT) {
+        grid_dep_wait();                       // the shared-prefix kernel's records
+        grid_dep_launch_dependents();          // the output projection may request its weights
+    }
     const size_t rh0 = (size_t)row * Hq + (size_t)kvh * n_rep;
-    const int np = part.n_parts;
+    const int np = JOINT ? 0 : part.n_parts;
     // this warp's heads: me, me + workers, ...; the records of the first are requested before the cluster meets
     auto records = [&](int j, float& pm, float& pl, float (&v)[MAX_PREFIX_PARTS][EPL]) {
         pm = lane < np ? __ldcg(part.m + (size_t)lane * part.stride + rh0 + j) : -INFINITY;
@@ -127,10 +143,10 @@ attn_suffix_team_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDe
         }
     };
     float pm = -INFINITY, pl = 0.f, v[MAX_PREFIX_PARTS][EPL];
-    if (me < n_rep) records(me, pm, pl, v);
+    if (!JOINT && me < n_rep) records(me, pm, pl, v);
     if (team_ctas > 1) wt::cluster_sync(); else __syncthreads();
     for (int j = me; j < n_rep; j += workers) {
-        if (j != me) records(j, pm, pl, v);
+        if (!JOINT && j != me) records(j, pm, pl, v);
         // lane w holds m and l of worker w (at most 32)
         float tm = -INFINITY, tl = 0.f;
         if (lane < workers) {
@@ -145,7 +161,7 @@ attn_suffix_team_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDe
 #pragma unroll
         for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
 #pragma unroll
-        for (int i = 0; i < MAX_PREFIX_PARTS; ++i) {
+        for (int i = 0; i < (JOINT ? 0 : MAX_PREFIX_PARTS); ++i) {
             const float w = __shfl_sync(0xffffffffu, wp, i);
             if (w > 0.f) {                     // a record with m = -inf was left by an empty range: its output is not defined
 #pragma unroll

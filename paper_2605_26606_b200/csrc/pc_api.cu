@@ -92,7 +92,7 @@ struct Carve {
 // caller's row arrays, token buffer and sampling parameters are not part of the key: the captured kernels read them
 // from the device-resident argument block (DecodeArgsDev) that every call rewrites.
 struct GraphKey {
-    int m_bound, groups_bound, group_rows_bound, sample, logprobs, decode_mode;
+    int m_bound, groups_bound, group_rows_bound, sample, logprobs, decode_mode, joint;
     const void* prompt_kv; int64_t prompt_slots;
     const void* suffix_kv; int64_t suffix_slots;
 };
@@ -131,7 +131,7 @@ struct pc_ctx {
     CUtensorMap map_a, map_attn, map_act, map_a_lo, map_attn_lo;
     int num_sms = 148;
     // TMA descriptors of the KV arenas, rebuilt when a call brings another arena
-    const void* prompt_arena_ptr = nullptr; int64_t prompt_arena_slots = -1; CUtensorMap map_prompt_kv;
+    const void* prompt_arena_ptr = nullptr; int64_t prompt_arena_slots = -1; CUtensorMap map_prompt_kv, map_prompt_tiles;
     const void* suffix_arena_ptr = nullptr; int64_t suffix_arena_slots = -1; CUtensorMap map_suffix_kv;
     // one-shot profiling request (pc_profile_step): events recorded at the phase boundaries of one layer and of the step's tail
     int prof_layer = -1;                     // armed when >= 0
@@ -449,14 +449,30 @@ struct AttnPlan {
     int n_groups;                      // upper bound used for the grid; the live count is in the step descriptor
     const int32_t* group_row_start;    // device; the step's entries start at the descriptor's group_off
     int max_group_rows;                // upper bound
+    bool joint;                        // decode: every row attends its prompt itself (joint_attention)
 };
+
+// Whether a decode step's attention takes a team of CTAs per (row, KV head).
+bool suffix_teams(const pc_ctx* c, int M) { return M * c->d.n_kv_heads <= 2 * c->num_sms; }
+
+// Whether the teams read the prompt too, once per row instead of once per group, and there is no shared-prefix kernel.  With so few rows
+// that kernel and the hand-over of its records (7 + 4 us of a 40 us layer at 16 rows) cost more than the reads, which L2 serves, up to prompts of
+// about 1,024 tokens.  Eight decode steps of the 1.5B shape, with it and without: 16 rows x 640 tokens 8.92 / 9.75 ms, 36 x 640 10.23 / 10.72, 36 x
+// 1,024 10.66 / 10.64, 72 x 1,024 12.50 / 12.67, 128 x 640 13.93 / 14.09, 128 x 1,024 13.78 / 14.02, 72 x 4,096 19.23 / 14.39; 8B shape, 32 x 512 28.6 / 29.3.
+// The lengths are on the device; the host knows the arena, which holds the prompts (at least the step's groups) and may hold more.
+constexpr int64_t JOINT_MAX_PROMPT = 1024;
+bool joint_attention(const pc_ctx* c, int M, int n_groups, int64_t prompt_slots) {
+    const int64_t prompts = c->n_prompts_hint > 0 ? c->n_prompts_hint : n_groups;
+    return suffix_teams(c, M) && prompt_slots <= JOINT_MAX_PROMPT * prompts;
+}
 
 int arena_maps(pc_ctx* c, const void* prompt_kv, int64_t prompt_slots, const void* suffix_kv, int64_t suffix_slots) {
     const pc_model_desc& d = c->d;
     const uint64_t planes = (uint64_t)d.n_layers * 2 * d.n_kv_heads;
     if (prompt_kv != c->prompt_arena_ptr || prompt_slots != c->prompt_arena_slots) {
         if (planes * (uint64_t)prompt_slots >= (1ull << 31)) return PC_ERR_CAPACITY;
-        if (!pc::make_bf16_map(&c->map_prompt_kv, prompt_kv, planes * prompt_slots, d.head_dim, pc::am::G_TK)) {
+        if (!pc::make_bf16_map(&c->map_prompt_kv, prompt_kv, planes * prompt_slots, d.head_dim, pc::am::G_TK) ||
+            !pc::make_kv_tile_map(&c->map_prompt_tiles, prompt_kv, planes, prompt_slots, d.n_kv_heads, d.head_dim, pc::am::S_TP)) {
             g_cuda_error = "cuTensorMapEncodeTiled failed for the prompt KV arena";
             return PC_ERR_CUDA;
         }
@@ -489,7 +505,9 @@ cudaError_t configure_attention() {
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(am::attn_suffix_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::suffix_smem_bytes<HD>());
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(am::attn_suffix_team_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::TEAM_SMEM_BYTES);
+        e = cudaFuncSetAttribute(am::attn_suffix_team_kernel<HD, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::TEAM_SMEM_BYTES);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(am::attn_suffix_team_kernel<HD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::TEAM_SMEM_BYTES);
     return e;
 }
 template <class Epi>
@@ -584,7 +602,7 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
     const int base_ctas = std::max(1, q_tiles * d.n_kv_heads * plan.n_groups);
     // batches whose items occupy the suffix kernel's warps with few ranges each; smaller ones take a team of CTAs per item
     const int items = M * d.n_kv_heads;
-    const bool teams = items <= 2 * c->num_sms;
+    const bool teams = suffix_teams(c, M);
     const int n_parts = plan.prefill ? 1 : std::max(1, std::min(teams ? am::MAX_PREFIX_PARTS : am::MAX_MERGED_PARTS, c->num_sms / base_ctas));
     am::PrefixPartial part{reinterpret_cast<float*>(c->ws + c->cv.part_m), reinterpret_cast<float*>(c->ws + c->cv.part_l),
                            reinterpret_cast<float*>(c->ws + c->cv.part_o), n_parts, (size_t)std::max(c->max_rows, 1) * d.n_q_heads,
@@ -605,19 +623,23 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
     // The shared-prefix kernel depends on the QKV projection (or its post-processing), the suffix kernel on the shared-prefix
     // kernel; each may start when the one before it has begun, and reads what it needs of it after its wait.
     const bool group_dep = !after_chain && dependent_launch(c, DEP_GROUP, M);
-    if constexpr (HD == 128)
-        launch_k_dep(group_dep, at::attn_prefix_kernel<false>, ggrid, dim3(at::THREADS), at::SMEM_BYTES, st,
-            c->map_prompt_kv, sd, prompt_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, plan.group_row_start, g, scale_log2, part, q_tiles,
-            attn, attn_lo, c->err);
-    else
-        launch_k_dep(group_dep, am::attn_group_kernel<HD, false>, ggrid, dim3(am::G_THREADS), am::group_smem_bytes<HD>(), st,
-            c->map_prompt_kv, sd, prompt_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, plan.group_row_start, g, scale_log2, part,
-            attn, attn_lo, c->err);
+    if (!plan.joint) {
+        if constexpr (HD == 128)
+            launch_k_dep(group_dep, at::attn_prefix_kernel<false>, ggrid, dim3(at::THREADS), at::SMEM_BYTES, st,
+                c->map_prompt_kv, sd, prompt_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, plan.group_row_start, g, scale_log2, part, q_tiles,
+                attn, attn_lo, c->err);
+        else
+            launch_k_dep(group_dep, am::attn_group_kernel<HD, false>, ggrid, dim3(am::G_THREADS), am::group_smem_bytes<HD>(), st,
+                c->map_prompt_kv, sd, prompt_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, plan.group_row_start, g, scale_log2, part,
+                attn, attn_lo, c->err);
+        count_launches(1);
+    }
     c->mark(st, layer, PC_MARK_GROUP);
     if (teams) {
-        // a cluster of CTAs per (row, KV head): as many as fit beside the shared-prefix kernel, one CTA of each per SM
-        int team = 8;
-        while (team > 1 && items * team > c->num_sms) team >>= 1;
+        // a cluster of CTAs per (row, KV head): as many as fit beside the shared-prefix kernel, one CTA of each per SM; on its own, two
+        // CTAs per SM and at most four of an item (eight decode steps of 16 rows with eight 9.87 ms, four 8.92, two 9.40)
+        int team = plan.joint ? 4 : 8;
+        while (team > 1 && items * team > (plan.joint ? 2 * c->num_sms : c->num_sms)) team >>= 1;
         cudaLaunchConfig_t cfg;
         std::memset(&cfg, 0, sizeof(cfg));
         cfg.gridDim = dim3((unsigned)(items * team)); cfg.blockDim = dim3(am::T_WARPS * 32);
@@ -635,7 +657,8 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
             ++n_attr;
         }
         cfg.attrs = attr; cfg.numAttrs = n_attr;
-        const cudaError_t e = cudaLaunchKernelEx(&cfg, am::attn_suffix_team_kernel<HD>, c->map_suffix_kv, sd, suffix_arena.n_slots, d.n_q_heads,
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, plan.joint ? am::attn_suffix_team_kernel<HD, true> : am::attn_suffix_team_kernel<HD, false>,
+                                                 c->map_suffix_kv, c->map_prompt_tiles, prompt_arena.n_slots, sd, suffix_arena.n_slots, d.n_q_heads,
                                                  d.n_kv_heads, layer, q, g, scale_log2, part, team, attn, attn_lo, c->err);
         if (e != cudaSuccess) return cuda_fail(e, "suffix attention");
     } else {
@@ -647,7 +670,7 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
     }
     c->mark(st, layer, PC_MARK_SUFFIX);
     c->mark(st, layer, PC_MARK_MERGE);
-    count_launches(2);
+    count_launches(1);
     return PC_OK;
 }
 
@@ -1217,7 +1240,7 @@ int pc_prefill_shared(pc_ctx* ctx, void* stream, int n_prompts, const int32_t* p
     count_launches(2);
     PC_CUDA_CHECK_LAUNCH("prep_prefill_rows");
     const pc::KvArena pa{prompt_kv, prompt_slots}, sa{prompt_kv, prompt_slots};
-    const AttnPlan plan{true, n_prompts, prompt_offsets, max_prompt_len};
+    const AttnPlan plan{true, n_prompts, prompt_offsets, max_prompt_len, false};
     int rc = PC_OK;
     if (ctx->d.dtype == PC_DTYPE_F32) {
         rc = run_layers<float>(ctx, st, total_tokens, sd, pa, sa, plan);
@@ -1422,7 +1445,7 @@ int decode_launches(pc_ctx* ctx, cudaStream_t st, int m_bound, int groups_bound,
     PC_CUDA_CHECK_LAUNCH("prep_decode_rows");
     const pc::KvArena pa{const_cast<void*>(a.prompt_kv), a.prompt_slots}, sa{a.suffix_kv, a.suffix_slots};
     const bool f32 = ctx->d.dtype == PC_DTYPE_F32;
-    const AttnPlan plan{false, groups_bound, keys.group_start, group_rows_bound};
+    const AttnPlan plan{false, groups_bound, keys.group_start, group_rows_bound, joint_attention(ctx, m_bound, groups_bound, a.prompt_slots)};
     float* logits = logits_out ? logits_out : reinterpret_cast<float*>(ctx->ws + ctx->cv.logits);
     int rc;
     if (!f32 && ctx->decode_mode == 1 && ctx->chain_ready) {
@@ -1545,6 +1568,7 @@ int pc_decode_run(pc_ctx* ctx, void* stream, int n_steps, const pc_step_desc* st
         std::memset(&key, 0, sizeof(key));
         key.m_bound = m_bound; key.groups_bound = groups_bound; key.group_rows_bound = group_rows_bound;
         key.sample = a.sample; key.logprobs = a.logprobs != nullptr; key.decode_mode = ctx->decode_mode;
+        key.joint = joint_attention(ctx, m_bound, groups_bound, a.prompt_slots);
         key.prompt_kv = a.prompt_kv; key.prompt_slots = a.prompt_slots; key.suffix_kv = a.suffix_kv; key.suffix_slots = a.suffix_slots;
         cudaGraphExec_t exec = nullptr;
         for (auto& ent : ctx->graphs)

@@ -18,7 +18,9 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("model,prompt,rows,depth,half", [(wl.SMALL_BF16, 1, 1, 2, True), (wl.SMALL_BF16, 16, 63, 18, True),
                                                           (wl.SMALL_QKNORM_BF16, 63, 64, 5, True), (wl.SMALL_BF16, 64, 65, 3, False),
                                                           (wl.SMALL_QKNORM_BF16, 65, 2, 34, True), (wl.SMALL_BF16, 191, 129, 3, True),
-                                                          (wl.SMALL_BF16, 600, 3, 66, True), (wl.TINY_BF16, 130, 40, 18, True)],
+                                                          (wl.SMALL_BF16, 600, 3, 66, True), (wl.TINY_BF16, 130, 40, 18, True),
+                                                          # prompts past the length up to which few rows read them themselves
+                                                          (wl.SMALL_BF16, 1024, 3, 17, True), (wl.SMALL_BF16, 1025, 3, 17, True), (wl.TINY_BF16, 1100, 20, 17, True)],
                          ids=lambda v: getattr(v, "name", str(v)))
 def test_decode_logits_at_attention_tile_edges(cuda_device, model, prompt, rows, depth, half):
     ensure_built()
