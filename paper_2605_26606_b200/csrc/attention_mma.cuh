@@ -377,12 +377,13 @@ attn_group_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* __
 // A warp's tile -- ldmatrix, two rounds of MMAs, the softmax between them -- is one chain of about 900 clocks for 8 KB, so a warp
 // of its own per scheduler cannot keep up with HBM (4 warps, 32 positions at a time: 4.35 TB/s at 237 rows x 512); two per
 // scheduler can.  192 KB of tiles are in flight per SM.
-constexpr int S_WARPS = 8;
+constexpr int S_WARPS = 4;
+constexpr int S_CTAS = 2;           // per SM
 constexpr int S_TP = 16;            // positions per stage: one MMA tile
 constexpr int S_STAGES = 3;
-template <int HD> constexpr int suffix_smem_bytes() {
-    return S_WARPS * (S_STAGES * 2 * S_TP * HD * 2 + 8 * HD * 4) + 1024 + 256;
-}
+template <int HD> __host__ __device__ constexpr int suffix_smem_need() { return S_WARPS * (S_STAGES * 2 * S_TP * HD * 2 + 8 * HD * 4) + 512; }
+constexpr int SUFFIX_SMEM_BYTES = 113 * 1024;      // half of an SM's 228 KB less the reserved KB
+static_assert(suffix_smem_need<128>() <= SUFFIX_SMEM_BYTES, "suffix buffers");
 
 // With few rollouts there are about as many (rollout, KV head) streams as warps on the GPU, and one stream more than
 // warps doubles the kernel's time.  The suffix of a rollout is therefore cut into ranges of tiles ("chunks") that
@@ -618,7 +619,7 @@ struct SuffixMerge {
 };
 
 template <int HD>
-__global__ void __launch_bounds__(S_WARPS * 32, 1)
+__global__ void __launch_bounds__(S_WARPS * 32, S_CTAS)
 attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* __restrict__ sd, int64_t n_slots, int Hq, int Hkv,
                    int layer, const __nv_bfloat16* __restrict__ q, RowGeom g, float scale_log2, PrefixPartial part, SuffixMerge mg, int32_t* err) {
     constexpr int KS = HD / 16;                   // k-steps of K Q^T
@@ -630,13 +631,18 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t* my_tiles = base + warp * WARP_BYTES;
     float* obuf = reinterpret_cast<float*>(base + S_WARPS * WARP_BYTES) + warp * 8 * HD;      // [8 heads][HD]
-    uint64_t* bars = reinterpret_cast<uint64_t*>(base + S_WARPS * (WARP_BYTES + 8 * HD * 4)) + warp * S_STAGES;
-    __shared__ float s_ml[S_WARPS][16];
-    __shared__ int s_abort;
+    float* ml = reinterpret_cast<float*>(base + S_WARPS * (WARP_BYTES + 8 * HD * 4)) + warp * 16;      // m of 8 heads, l of 8 heads
+    uint64_t* bars = reinterpret_cast<uint64_t*>(base + S_WARPS * (WARP_BYTES + 8 * HD * 4 + 64)) + warp * S_STAGES;
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(base + S_WARPS * (WARP_BYTES + 8 * HD * 4 + 64 + 8 * S_STAGES));
+    if ((int)(base - smem_raw) + suffix_smem_need<HD>() > SUFFIX_SMEM_BYTES) {        // (the shared memory window is not where it should be)
+        if (threadIdx.x == 0) set_error(err, DEV_ERR_GROUP_RANGE);
+        grid_dep_wait();
+        return;
+    }
     const uint32_t tiles_u32 = smem_u32(my_tiles), full0 = smem_u32(bars);
     const int n_rep = Hq / Hkv;
 
-    if (threadIdx.x == 0) s_abort = 0;
+    if (threadIdx.x == 0) *abort_flag = 0;
     if (lane == 0) {
         for (int s = 0; s < S_STAGES; ++s) mbar_init(full0 + 8 * s, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -731,7 +737,7 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
         for (int tile = t0; tile < t1; ++tile) {
             const int stage = consumed % S_STAGES;
             const uint32_t phase = (uint32_t)(consumed / S_STAGES) & 1u;
-            if (!mbar_wait(full0 + 8 * stage, phase, &s_abort)) { ok = false; break; }
+            if (!mbar_wait(full0 + 8 * stage, phase, abort_flag)) { ok = false; break; }
             const uint32_t kb = tiles_u32 + stage * 2 * TILE_BYTES, vb = kb + TILE_BYTES;
             suffix_tile<HD>(kb, vb, lane, min(S_TP, n - tile * S_TP), scale_log2, qb, o, mh, lh, [&]() {
                 ++consumed;
@@ -741,7 +747,7 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
         }
         if (!ok) break;
 
-        suffix_finish<HD>(lane, o, mh, lh, s_ml[warp], s_ml[warp] + 8, obuf);
+        suffix_finish<HD>(lane, o, mh, lh, ml, ml + 8, obuf);
         __syncwarp();
         constexpr int EPL = HD / 32;
         const size_t rh0 = (size_t)row * Hq + (size_t)kvh * n_rep;
@@ -752,11 +758,11 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
             waited = true;
         }
         if (n_own == 1) {
-            merge_heads_warp<HD>(lane, rh0, n_rep, part, part.n_parts, s_ml[warp], s_ml[warp] + 8, obuf, mg.out, mg.out_lo, err);
+            merge_heads_warp<HD>(lane, rh0, n_rep, part, part.n_parts, ml, ml + 8, obuf, mg.out, mg.out_lo, err);
         } else {
             // leave this chunk as record number part.n_parts + chunk, next to the prefix records
             const size_t base = (size_t)(part.n_parts + chunk) * part.stride + rh0;
-            if (lane < n_rep) { part.m[base + lane] = s_ml[warp][lane]; part.l[base + lane] = s_ml[warp][8 + lane]; }
+            if (lane < n_rep) { part.m[base + lane] = ml[lane]; part.l[base + lane] = ml[8 + lane]; }
             for (int j = 0; j < n_rep; ++j) {
                 float* dst = part.o + (base + j) * HD + lane * EPL;
                 const float* src = obuf + j * HD + lane * EPL;
@@ -776,14 +782,14 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
         }
         __syncwarp();
     }
-    if (!ok) { s_abort = 1; if (lane == 0) set_error(err, DEV_ERR_WAIT_TIMEOUT); }
+    if (!ok) { *abort_flag = 1; if (lane == 0) set_error(err, DEV_ERR_WAIT_TIMEOUT); }
     // drain: tiles issued but not consumed must land before the shared memory is released
     while (ok && consumed < issued) {
         const int stage = consumed % S_STAGES;
-        if (!mbar_wait(full0 + 8 * stage, (uint32_t)(consumed / S_STAGES) & 1u, &s_abort)) break;
+        if (!mbar_wait(full0 + 8 * stage, (uint32_t)(consumed / S_STAGES) & 1u, abort_flag)) break;
         ++consumed;
     }
-    if (s_abort) {
+    if (*abort_flag) {
         for (int i = 0; i < 2000; ++i) __nanosleep(1000);
     }
     __syncthreads();

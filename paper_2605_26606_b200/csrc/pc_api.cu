@@ -503,7 +503,7 @@ cudaError_t configure_attention() {
             e = cudaFuncSetAttribute(am::attn_group_kernel<HD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::group_smem_bytes<HD>());
     }
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(am::attn_suffix_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::suffix_smem_bytes<HD>());
+        e = cudaFuncSetAttribute(am::attn_suffix_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::SUFFIX_SMEM_BYTES);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(am::attn_suffix_team_kernel<HD, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::TEAM_SMEM_BYTES);
     if (e == cudaSuccess)
@@ -606,7 +606,7 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
     const int n_parts = plan.prefill ? 1 : std::max(1, std::min(teams ? am::MAX_PREFIX_PARTS : am::MAX_MERGED_PARTS, c->num_sms / base_ctas));
     am::PrefixPartial part{reinterpret_cast<float*>(c->ws + c->cv.part_m), reinterpret_cast<float*>(c->ws + c->cv.part_l),
                            reinterpret_cast<float*>(c->ws + c->cv.part_o), n_parts, (size_t)std::max(c->max_rows, 1) * d.n_q_heads,
-                           d.n_kv_heads, c->num_sms * am::S_WARPS};
+                           d.n_kv_heads, c->num_sms * am::S_CTAS * am::S_WARPS};
     const dim3 ggrid = HD == 128 ? dim3(q_tiles * n_parts * d.n_kv_heads * plan.n_groups) : dim3(q_tiles * n_parts, d.n_kv_heads, plan.n_groups);
     if (plan.prefill) {
         if constexpr (HD == 128)
@@ -665,7 +665,7 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
         // one warp per (rollout, KV head, range of the suffix); how the suffixes are cut into ranges is decided on the device for
         // the warps of this grid (the longest suffix of the step is only known there)
         const am::SuffixMerge mg{reinterpret_cast<int32_t*>(c->ws + c->cv.arrived), attn, attn_lo};
-        launch_k_dep(group_dep, am::attn_suffix_kernel<HD>, dim3(c->num_sms), dim3(am::S_WARPS * 32), am::suffix_smem_bytes<HD>(), st,
+        launch_k_dep(group_dep, am::attn_suffix_kernel<HD>, dim3(am::S_CTAS * c->num_sms), dim3(am::S_WARPS * 32), am::SUFFIX_SMEM_BYTES, st,
             c->map_suffix_kv, sd, suffix_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, g, scale_log2, part, mg, c->err);
     }
     c->mark(st, layer, PC_MARK_SUFFIX);
