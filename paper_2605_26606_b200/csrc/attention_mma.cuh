@@ -103,13 +103,10 @@ struct PrefixPartial {
     float* o;               // [n_parts][stride * head_dim]
     int n_parts;
     size_t stride;          // rows capacity * Hq
-    int n_kv_heads;
-    int n_suffix_warps;     // warps of the suffix kernel's grid: how suffixes are cut into ranges is planned for this many
+    int32_t* done;          // CTAs of the shared-prefix kernel that have left their records (a hint), or nullptr
 };
-constexpr int MAX_PREFIX_PARTS = 8, MAX_MERGED_PARTS = 4;      // (the second where the suffix kernel merges)
-constexpr int MERGE_CHUNKS = 3;
-constexpr int MAX_MERGED_RECORDS = MAX_MERGED_PARTS + MERGE_CHUNKS;
-constexpr int MAX_RECORDS = MAX_PREFIX_PARTS > MAX_MERGED_RECORDS ? MAX_PREFIX_PARTS : MAX_MERGED_RECORDS;
+constexpr int MAX_PREFIX_PARTS = 8, MAX_MERGED_PARTS = 4;      // (the second where attn_suffix_kernel merges)
+constexpr int MAX_RECORDS = MAX_PREFIX_PARTS > MAX_MERGED_PARTS + 1 ? MAX_PREFIX_PARTS : MAX_MERGED_PARTS + 1;
 
 // ---------------------------------------------------------------------------------------------
 // Group (shared-prefix / causal-prefill) kernel
@@ -376,39 +373,15 @@ attn_group_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* __
 // ---------------------------------------------------------------------------------------------
 // A warp's tile -- ldmatrix, two rounds of MMAs, the softmax between them -- is one chain of about 900 clocks for 8 KB, so a warp
 // of its own per scheduler cannot keep up with HBM (4 warps, 32 positions at a time: 4.35 TB/s at 237 rows x 512); two per
-// scheduler can.  192 KB of tiles are in flight per SM.
+// scheduler can.  192 KB of tiles are in flight per SM, in two CTAs, so that one fits beside a CTA of the shared-prefix kernel.
 constexpr int S_WARPS = 4;
 constexpr int S_CTAS = 2;           // per SM
 constexpr int S_TP = 16;            // positions per stage: one MMA tile
 constexpr int S_STAGES = 3;
-template <int HD> __host__ __device__ constexpr int suffix_smem_need() { return S_WARPS * (S_STAGES * 2 * S_TP * HD * 2 + 8 * HD * 4) + 512; }
+constexpr int S_SLOTS = 8;          // items a CTA knows of: the one in hand and those its rings reach into
+template <int HD> __host__ __device__ constexpr int suffix_smem_need() { return S_WARPS * (S_STAGES * 2 * S_TP * HD * 2 + 8 * HD * 4) + 768; }
 constexpr int SUFFIX_SMEM_BYTES = 113 * 1024;      // half of an SM's 228 KB less the reserved KB
 static_assert(suffix_smem_need<128>() <= SUFFIX_SMEM_BYTES, "suffix buffers");
-
-// With few rollouts there are about as many (rollout, KV head) streams as warps on the GPU, and one stream more than
-// warps doubles the kernel's time.  The suffix of a rollout is therefore cut into ranges of tiles ("chunks") that
-// are spread over the warps; every chunk leaves its own record.  Tiles per chunk (ct) and chunk slots per (row, KV
-// head) item (cpi) for a step whose longest suffix has max_slen slots: among 1..MERGE_CHUNKS chunks per item, the
-// choice that minimises (units the busiest warp gets) x (tiles per unit + 4), the + 4 standing for the fixed cost of a
-// unit (length lookup, first TMA round trip, record) in tile times.  The same value serves every row of the step, and
-// the warp that merges recomputes it from the same inputs.
-struct SuffixPlan { int ct, cpi; };
-__device__ __forceinline__ SuffixPlan suffix_plan(int max_slen, int n_items, int n_warps) {
-    const int ntiles = max(1, (max_slen + S_TP - 1) / S_TP);
-    SuffixPlan best{ntiles, 1};
-    long long best_cost = -1;
-    for (int c = 1; c <= MERGE_CHUNKS; ++c) {
-        const int ct = (ntiles + c - 1) / c;
-        const int cc = (ntiles + ct - 1) / ct;
-        const long long cost = (long long)((n_items * cc + n_warps - 1) / max(n_warps, 1)) * (ct + 4);
-        if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = SuffixPlan{ct, cc}; }
-    }
-    return best;
-}
-__device__ __forceinline__ int suffix_chunks(int n, int ct) {             // records a row with n suffix slots leaves
-    const int ntiles = (n + S_TP - 1) / S_TP;
-    return (ntiles + ct - 1) / ct;
-}
 
 // One tile of 16 positions: K fragments against the heads' queries, online softmax, V.  loaded() is called once the tile is in
 // registers (its ring slot is free).
@@ -528,272 +501,298 @@ __device__ __forceinline__ void store_attention(int lane, size_t rh, float* acc,
     }
 }
 
-// Merge of records 0 .. n-1 of all n_rep (<= 8) query heads of one row and KV head by a warp, in index order, by their
-// log-sum-exp:  M = max m_i,  out = sum_i O_i 2^(m_i - M) / sum_i l_i 2^(m_i - M).  m and l of all (record, head) pairs come in one
-// round trip, the outputs of two records in another each.  own_*: one more record, the last, that is still in shared memory ([8]
-// values, [8][HD] outputs), or nullptr.
-template <int HD>
-__device__ __forceinline__ void merge_heads_warp(int lane, size_t rh0, int n_rep, const PrefixPartial& part, int n, const float* own_m,
-                                                 const float* own_l, const float* own_o, __nv_bfloat16* __restrict__ out,
-                                                 __nv_bfloat16* __restrict__ out_lo, int32_t* err) {
-    constexpr int EPL = HD / 32, NH = 8, B = 2, MR = (MAX_MERGED_RECORDS + 3) / 4;
-    const int hj = lane & 7, pi = lane >> 3;        // lane 8 p + j holds records p, p + 4, ... of head j
-    float m[MR], l[MR], M = own_m != nullptr && hj < n_rep ? own_m[hj] : -INFINITY;
-#pragma unroll
-    for (int k = 0; k < MR; ++k) {
-        const int i = pi + 4 * k;
-        const bool on = i < n && hj < n_rep;
-        m[k] = on ? __ldcg(part.m + (size_t)i * part.stride + rh0 + hj) : -INFINITY;
-        l[k] = on ? __ldcg(part.l + (size_t)i * part.stride + rh0 + hj) : 0.f;
-    }
-#pragma unroll
-    for (int k = 0; k < MR; ++k) M = fmaxf(M, m[k]);
-    M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 8));
-    M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 16));
-#pragma unroll
-    for (int k = 0; k < MR; ++k) m[k] = exp2_safe(m[k], M);        // weights
-    float acc[NH][EPL], denom = 0.f;
-#pragma unroll
-    for (int j = 0; j < NH; ++j)
-#pragma unroll
-        for (int e = 0; e < EPL; ++e) acc[j][e] = 0.f;
-#pragma unroll
-    for (int k = 0; k < MR; ++k) {
-#pragma unroll
-        for (int p0 = 0; p0 < 4; p0 += B) {
-            if (4 * k + p0 >= n) break;
-            float v[B][NH][EPL];
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
-                const float* src = part.o + ((size_t)(4 * k + p0 + b) * part.stride + rh0) * HD + lane * EPL;
-#pragma unroll
-                for (int j = 0; j < NH; ++j) {
-                    // a record with m = -inf was left by an empty range: its output is not defined
-                    const bool have = j < n_rep && __shfl_sync(0xffffffffu, m[k], 8 * (p0 + b) + j) > 0.f;
-                    if (EPL == 4) {
-                        const float4 x = have ? __ldcg(reinterpret_cast<const float4*>(src + j * HD)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                        v[b][j][0] = x.x; v[b][j][1] = x.y; v[b][j][EPL - 2] = x.z; v[b][j][EPL - 1] = x.w;
-                    } else {
-                        const float2 x = have ? __ldcg(reinterpret_cast<const float2*>(src + j * HD)) : make_float2(0.f, 0.f);
-                        v[b][j][0] = x.x; v[b][j][1] = x.y;
-                    }
-                }
-            }
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
-                denom = __fmaf_rn(__shfl_sync(0xffffffffu, l[k], 8 * (p0 + b) + hj), __shfl_sync(0xffffffffu, m[k], 8 * (p0 + b) + hj), denom);
-#pragma unroll
-                for (int j = 0; j < NH; ++j) {
-                    const float wj = __shfl_sync(0xffffffffu, m[k], 8 * (p0 + b) + j);
-#pragma unroll
-                    for (int e = 0; e < EPL; ++e) acc[j][e] = __fmaf_rn(v[b][j][e], wj, acc[j][e]);
-                }
-            }
-        }
-    }
-    float wo = 0.f;
-    if (own_m != nullptr && hj < n_rep) {
-        wo = exp2_safe(own_m[hj], M);
-        denom = __fmaf_rn(own_l[hj], wo, denom);
-    }
-#pragma unroll
-    for (int j = 0; j < NH; ++j) {
-        const float wj = __shfl_sync(0xffffffffu, wo, j), dj = __shfl_sync(0xffffffffu, denom, j);
-        if (j < n_rep) {
-            if (own_o != nullptr) {
-#pragma unroll
-                for (int e = 0; e < EPL; ++e) acc[j][e] = __fmaf_rn(own_o[j * HD + lane * EPL + e], wj, acc[j][e]);
-            }
-            store_attention<HD>(lane, rh0 + j, acc[j], dj, out, out_lo, err);
-        }
-    }
-}
-
-// A warp that holds an item's whole suffix merges it with the prefix records from shared memory; of the few warps that share an
-// item (at most MERGE_CHUNKS) each leaves its record and the last one merges.  For batches with enough items to occupy the warps
-// that way; smaller ones take attn_suffix_team_kernel.
-struct SuffixMerge {
-    int32_t* arrived;           // [rows capacity * Hkv]: warps that have left their record of an item; 0 between launches
+// Suffix attention of batches with more than two (row, KV head) items per SM (smaller ones take attn_suffix_team_kernel).  A team of
+// T warps takes an item at a time, each warp every T-th tile, and merges the warps' shares and the item's shared-prefix records
+// by their log-sum-exp:  M = max m_i,  out = sum_i O_i 2^(m_i - M) / sum_i l_i 2^(m_i - M).  T: suffix_team_warps in pc_api.cu.
+//
+// The items are claimed as the teams get to them.  A CTA that starts beside the shared-prefix kernel (113 KB each) streams while
+// that one computes and takes more of them than one that has to wait for its place; an item that is finished before the shared-prefix
+// records are there is left as a record too and merged at the end.  A warp's ring runs on into the next item while its team merges.
+//
+// What bounds it: HBM, but for the first and the last few microseconds.  237 rows x 512 (118 MB, 18 us at the copy rate): from the end of the
+// projection before 33 us with the shared-prefix kernel inside (12 of them); first tile at 4, last item begun at 24.  With one
+// 192 KB CTA per SM, which had to wait for the shared-prefix CTAs, and a suffix per warp cut into ranges, merged between two ranges by the last
+// warp (5-13 us, every warp at the same time), eight steps took: 237 rows x 512 19.8 -> 19.1 ms, 336 x 900 30.6 -> 29.0, 2,048 x 512 101.2 -> 95.5.
+// Halving the last items so that the CTAs end closer together cost more (records, fences, a second merge) than it gave.
+struct SuffixWork {
+    int32_t* next;              // the layer's next item; 0 at the start of a step
+    int32_t* link;              // [rows capacity * Hkv]: items put off, a list per CTA
+    int prefix_ctas;            // value of part.done once the shared-prefix records are there
     __nv_bfloat16* out;
     __nv_bfloat16* out_lo;
 };
+struct SuffixItem {
+    int64_t krow;               // first K row of the suffix in the arena's (plane, slot) rows
+    int item, n;                // (row, KV head), or -1: there are no more; suffix length
+};
 
-template <int HD>
+template <int HD, int T>
 __global__ void __launch_bounds__(S_WARPS * 32, S_CTAS)
 attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* __restrict__ sd, int64_t n_slots, int Hq, int Hkv,
-                   int layer, const __nv_bfloat16* __restrict__ q, RowGeom g, float scale_log2, PrefixPartial part, SuffixMerge mg, int32_t* err) {
+                   int layer, const __nv_bfloat16* __restrict__ q, RowGeom g, float scale_log2, PrefixPartial part, SuffixWork wk, int32_t* err) {
     constexpr int KS = HD / 16;                   // k-steps of K Q^T
     constexpr int DT = HD / 16;                   // 16-dim m-tiles of O^T
+    constexpr int EPL = HD / 32;
+    constexpr int H = 8 / T;                      // heads of an item a warp merges
     constexpr int TILE_BYTES = S_TP * HD * 2;
-    constexpr int WARP_BYTES = S_STAGES * 2 * TILE_BYTES;
+    constexpr int RING_BYTES = S_STAGES * 2 * TILE_BYTES;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint8_t* my_tiles = base + warp * WARP_BYTES;
-    float* obuf = reinterpret_cast<float*>(base + S_WARPS * WARP_BYTES) + warp * 8 * HD;      // [8 heads][HD]
-    float* ml = reinterpret_cast<float*>(base + S_WARPS * (WARP_BYTES + 8 * HD * 4)) + warp * 16;      // m of 8 heads, l of 8 heads
-    uint64_t* bars = reinterpret_cast<uint64_t*>(base + S_WARPS * (WARP_BYTES + 8 * HD * 4 + 64)) + warp * S_STAGES;
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(base + S_WARPS * (WARP_BYTES + 8 * HD * 4 + 64 + 8 * S_STAGES));
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, team = warp / T, me = warp % T;
+    float* obufs = reinterpret_cast<float*>(base + S_WARPS * RING_BYTES);              // [warp][8 heads][HD]
+    float* mls = obufs + S_WARPS * 8 * HD;                                              // [warp][m of 8 heads, l of 8 heads]
+    float *obuf = obufs + team * T * 8 * HD, *ml = mls + team * T * 16;                // of the team
+    SuffixItem* all_slots = reinterpret_cast<SuffixItem*>(mls + S_WARPS * 16);
+    SuffixItem* slots = all_slots + team * S_SLOTS;
+    uint64_t* all_bars = reinterpret_cast<uint64_t*>(all_slots + S_WARPS / T * S_SLOTS);
+    uint64_t* bars = all_bars + warp * S_STAGES;
+    // of the team: a wait ran out, items its first warp has entered in the slots so far, the shared-prefix records are there
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(all_bars + S_WARPS * S_STAGES) + team * 4;
+    volatile int *known = abort_flag + 1, *records_there = abort_flag + 2;
+    auto team_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(T * 32) : "memory"); };
     if ((int)(base - smem_raw) + suffix_smem_need<HD>() > SUFFIX_SMEM_BYTES) {        // (the shared memory window is not where it should be)
         if (threadIdx.x == 0) set_error(err, DEV_ERR_GROUP_RANGE);
         grid_dep_wait();
         return;
     }
-    const uint32_t tiles_u32 = smem_u32(my_tiles), full0 = smem_u32(bars);
-    const int n_rep = Hq / Hkv;
+    // A team's first warp claims: lane 0 asks for an item while the last tiles of the one before are requested, and enters it when the ring gets there.
+    int claim = 0;
+    auto request = [&]() { if (lane == 0) claim = atomicAdd(wk.next, 1); };
+    if (me == 0) request();
+    const uint32_t tiles_u32 = smem_u32(base + warp * RING_BYTES), full0 = smem_u32(bars);
+    const int n_rep = Hq / Hkv, n_items = sd->n_rows * Hkv;
 
-    if (threadIdx.x == 0) *abort_flag = 0;
+    if (threadIdx.x == 32) asm volatile("prefetch.tensormap [%0];" ::"l"(&kv_map) : "memory");
+    if (me == 0 && lane == 0) { *abort_flag = 0; *known = 0; *records_there = part.done == nullptr; }
     if (lane == 0) {
         for (int s = 0; s < S_STAGES; ++s) mbar_init(full0 + 8 * s, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
+    auto enter = [&](int seq) {                   // slot of the seq-th item of this team
+        int item = __shfl_sync(0xffffffffu, claim, 0), n = 0;
+        int64_t start = 0;
+        while (item < n_items) {
+            const int row = item / Hkv;
+            n = g.s_len[row]; start = g.s_start[row];
+            if (n > 0) break;                     // (a row that was refused has no suffix and its outputs are not defined)
+            request();
+            item = __shfl_sync(0xffffffffu, claim, 0);
+        }
+        if (lane == 0) {
+            const int kvh = item % Hkv;
+            slots[seq % S_SLOTS] = SuffixItem{((int64_t)layer * 2 * Hkv + kvh) * n_slots + start, item < n_items ? item : -1, n};
+            __threadfence_block();
+            *known = seq + 1;
+        }
+        __syncwarp();
+    };
+    if (me == 0) enter(0);
     __syncthreads();
 
-    bool waited = false;                   // the prefix records are there
-    // work unit u = (item, chunk), item = (row, kv head); units of one item are consecutive, so they land on different warps
-    const int max_slen = *g.max_slen;
-    const SuffixPlan sp = suffix_plan(max_slen, sd->n_rows * Hkv, part.n_suffix_warps);
-    const int ct = sp.ct, cpi = sp.cpi;                                                            // tiles per chunk, unit slots per item
-    const int n_items = sd->n_rows * Hkv * cpi;
-    const int item_stride = gridDim.x * S_WARPS;
-    const int first_item = warp * gridDim.x + blockIdx.x;          // few units: one per SM before a second one
-    // tile range [t0, t1) of unit u for a row with n suffix slots; empty when the row has fewer chunks
-    auto unit_range = [&](int u, int n, int& t0, int& t1) {
-        const int ntiles = (n + S_TP - 1) / S_TP;
-        t0 = min(ntiles, (u % cpi) * ct);
-        t1 = min(ntiles, t0 + ct);
-    };
-
-    // producer cursor (tracked identically by every lane; lane 0 issues)
-    int p_item = first_item, p_tile = 0, p_ntiles = 0;
+    // producer cursor: item p_seq, tile p_tile (tracked identically by every lane; lane 0 issues)
+    int p_seq = 0, p_tile = me, p_tiles = 0, issued = 0, consumed = 0;
     int64_t p_krow = 0;
-    auto p_load_item = [&]() {
-        while (p_item < n_items) {
-            const int it = p_item / cpi;
-            const int row = it / Hkv, kvh = it - row * Hkv;
-            int t0, t1;
-            unit_range(p_item, g.s_len[row], t0, t1);
-            if (t1 > t0) {
-                p_ntiles = t1;
-                p_krow = ((int64_t)layer * 2 * Hkv + kvh) * n_slots + g.s_start[row];
-                p_tile = t0;
-                return;
+    bool p_asked = false, p_open = false;
+    auto refill = [&]() {
+        while (issued - consumed < S_STAGES) {
+            if (!p_open) {
+                if (p_seq >= __shfl_sync(0xffffffffu, *known, 0)) {
+                    if (me != 0) return;          // the first warp has not got there: again at the next tile or item
+                    enter(p_seq);
+                }
+                __syncwarp();
+                const SuffixItem s = slots[p_seq % S_SLOTS];
+                if (s.item < 0) return;
+                p_krow = s.krow; p_tiles = (s.n + S_TP - 1) / S_TP; p_tile = me;
+                p_open = true; p_asked = false;
             }
-            p_item += item_stride;
+            if (me == 0 && !p_asked && p_tile + 2 * T >= p_tiles) { request(); p_asked = true; }
+            if (p_tile >= p_tiles) { ++p_seq; p_open = false; continue; }
+            const int stage = issued % S_STAGES;
+            if (lane == 0) {
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                mbar_arrive_expect_tx(full0 + 8 * stage, 2 * TILE_BYTES);
+                tma_load_kv(tiles_u32 + stage * 2 * TILE_BYTES, &kv_map, full0 + 8 * stage, (int)(p_krow + (int64_t)p_tile * S_TP));
+            }
+            ++issued;
+            p_tile += T;
         }
-        p_ntiles = 0;
     };
-    int issued = 0;
-    auto p_issue = [&]() {          // loads the producer cursor's tile into the next ring slot and advances the cursor
-        const int stage = issued % S_STAGES;
-        if (lane == 0) {
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            mbar_arrive_expect_tx(full0 + 8 * stage, 2 * TILE_BYTES);
-            tma_load_kv(tiles_u32 + stage * 2 * TILE_BYTES, &kv_map, full0 + 8 * stage, (int)(p_krow + (int64_t)p_tile * S_TP));
-        }
-        ++issued;
-        if (++p_tile == p_ntiles) { p_item += item_stride; p_load_item(); }
-    };
-    p_load_item();
-    for (int i = 0; i < S_STAGES && p_item < n_items; ++i) p_issue();
 
-    int consumed = 0;
-    bool ok = true;
-    // Q^T fragments (B operand): head = lane / 4, dims ks*16 + (lane%4)*2 (+8).  The next item's fragments and
-    // length are fetched while the current item streams, so that an item does not start with a global-memory stall.
-    uint32_t qn[KS][2];
-    int n_next = 0;
-    auto fetch_item = [&](int item) {
-        if (item >= n_items) return;
-        const int it = item / cpi;
-        const int row = it / Hkv, kvh = it - row * Hkv;
-        n_next = g.s_len[row];
-        const int hq = lane >> 2;
+    bool waited = false, ok = true;
+    int later = -1;                               // first lane of the team: head of the list of items put off
+    auto wait_prefix = [&]() {
+        grid_dep_wait();
+        grid_dep_launch_dependents();          // the output projection may request its weights once there is room for it
+        waited = true;
+    };
+    // Merges: heads me, me + T, ... of an item, side by side.  Lane 8 h + i holds m and l of source i of the h-th of them: the shares of the
+    // team's warps and up to four records, or records alone (at most five).
+    constexpr int R = MAX_MERGED_PARTS + 1;
+    float rec[H][R][EPL], rm = -INFINITY, rl = 0.f;
+    auto fetch_records = [&](size_t rh0, int np, int first) {       // first: source number of record 0
+#pragma unroll
+        for (int h = 0; h < H; ++h)
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                const bool on = i < np && me + T * h < n_rep;
+                const float* src = part.o + ((size_t)i * part.stride + rh0 + me + T * h) * HD + lane * EPL;
+                if (EPL == 4) {
+                    const float4 x = on ? __ldcg(reinterpret_cast<const float4*>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    rec[h][i][0] = x.x; rec[h][i][1] = x.y; rec[h][i][EPL - 2] = x.z; rec[h][i][EPL - 1] = x.w;
+                } else {
+                    const float2 x = on ? __ldcg(reinterpret_cast<const float2*>(src)) : make_float2(0.f, 0.f);
+                    rec[h][i][0] = x.x; rec[h][i][1] = x.y;
+                }
+            }
+        const int i = (lane & 7) - first, j = me + T * (lane >> 3);
+        const bool on = i >= 0 && i < np && lane < 8 * H && j < n_rep;
+        rm = on ? __ldcg(part.m + (size_t)i * part.stride + rh0 + j) : -INFINITY;
+        rl = on ? __ldcg(part.l + (size_t)i * part.stride + rh0 + j) : 0.f;
+    };
+    // record >= 0: the merged heads become that record, else the item's output
+    auto merge = [&](size_t rh0, bool shares, int record) {
+        float m = rm, l = rl;
+        if (shares && (lane & 7) < T && lane < 8 * H) {
+            const float* at = ml + (lane & 7) * 16 + ((me + T * (lane >> 3)) & 7);
+            m = at[0]; l = at[8];
+        }
+        float M = m;
+#pragma unroll
+        for (int d = 1; d < 8; d <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, d));
+        const float w = exp2_safe(m, M);
+        float denom = l * w;
+#pragma unroll
+        for (int d = 1; d < 8; d <<= 1) denom += __shfl_xor_sync(0xffffffffu, denom, d);
+        float acc[H][EPL];
+#pragma unroll
+        for (int h = 0; h < H; ++h)
+#pragma unroll
+            for (int e = 0; e < EPL; ++e) acc[h][e] = 0.f;
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                const float x = __shfl_sync(0xffffffffu, w, 8 * h + (shares ? min(T + i, 7) : i));
+                // a record with m = -inf was left by an empty range: its output is not defined
+                const float f = shares && i >= MAX_MERGED_PARTS ? 0.f : x;
+#pragma unroll
+                for (int e = 0; e < EPL; ++e) acc[h][e] = __fmaf_rn(f > 0.f ? rec[h][i][e] : 0.f, f, acc[h][e]);
+            }
+            if (shares) {
+#pragma unroll
+                for (int i = 0; i < T; ++i) {
+                    const float x = __shfl_sync(0xffffffffu, w, 8 * h + i);
+                    const float* src = obuf + (i * 8 + ((me + T * h) & 7)) * HD + lane * EPL;
+#pragma unroll
+                    for (int e = 0; e < EPL; ++e) acc[h][e] = __fmaf_rn(src[e], x, acc[h][e]);      // (a warp without tiles left zeros)
+                }
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            const int j = me + T * h;
+            const float Mh = __shfl_sync(0xffffffffu, M, 8 * h), dh = __shfl_sync(0xffffffffu, denom, 8 * h);
+            if (j >= n_rep) break;
+            if (record < 0) {
+                store_attention<HD>(lane, rh0 + j, acc[h], dh, wk.out, wk.out_lo, err);
+            } else {
+                const size_t at = (size_t)record * part.stride + rh0 + j;
+                if (lane == 0) { part.m[at] = Mh; part.l[at] = dh; }
+                float* dst = part.o + at * HD + lane * EPL;
+                if (EPL == 4) *reinterpret_cast<float4*>(dst) = make_float4(acc[h][0], acc[h][1], acc[h][EPL - 2], acc[h][EPL - 1]);
+                else *reinterpret_cast<float2*>(dst) = make_float2(acc[h][0], acc[h][1]);
+            }
+        }
+    };
+
+    uint32_t qn[KS][2];                           // Q^T fragments (B operand) of item q_seq: head = lane / 4, dims ks*16 + (lane%4)*2 (+8)
+    int q_seq = -1;
+    auto fetch_q = [&](int seq) {
+        const int item = slots[seq % S_SLOTS].item;
+        if (item < 0) return;
+        const int row = item / Hkv, kvh = item - row * Hkv, hq = lane >> 2;
         const __nv_bfloat16* qp = q + ((size_t)row * Hq + (size_t)kvh * n_rep + hq) * HD + (lane & 3) * 2;
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks) {
             qn[ks][0] = hq < n_rep ? *reinterpret_cast<const uint32_t*>(qp + ks * 16) : 0u;
             qn[ks][1] = hq < n_rep ? *reinterpret_cast<const uint32_t*>(qp + ks * 16 + 8) : 0u;
         }
+        q_seq = seq;
     };
-    fetch_item(first_item);
-    for (int item = first_item; item < n_items && ok; item += item_stride) {
-        const int it = item / cpi, chunk = item - it * cpi;
-        const int row = it / Hkv, kvh = it - row * Hkv;
-        const int n = n_next;
-        int t0, t1;
-        unit_range(item, n, t0, t1);
+    refill();
+    for (int seq = 0;; ++seq) {
+        const SuffixItem it = slots[seq % S_SLOTS];
+        if (it.item < 0) break;
+        const int row = it.item / Hkv, kvh = it.item - row * Hkv, tiles = (it.n + S_TP - 1) / S_TP;
+        if (q_seq != seq) fetch_q(seq);
         uint32_t qb[KS][2];
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks) { qb[ks][0] = qn[ks][0]; qb[ks][1] = qn[ks][1]; }
-        fetch_item(item + item_stride);
-        if (t1 <= t0) continue;      // this row has fewer chunks: nothing to leave
+        refill();
         float o[DT][4];
 #pragma unroll
         for (int t = 0; t < DT; ++t) { o[t][0] = o[t][1] = o[t][2] = o[t][3] = 0.f; }
         float mh[2] = {-INFINITY, -INFINITY}, lh[2] = {0.f, 0.f};      // heads (lane%4)*2 + {0, 1}
-
-        for (int tile = t0; tile < t1; ++tile) {
+#pragma unroll 1
+        for (int tile = me; tile < tiles; tile += T) {
             const int stage = consumed % S_STAGES;
-            const uint32_t phase = (uint32_t)(consumed / S_STAGES) & 1u;
-            if (!mbar_wait(full0 + 8 * stage, phase, abort_flag)) { ok = false; break; }
-            const uint32_t kb = tiles_u32 + stage * 2 * TILE_BYTES, vb = kb + TILE_BYTES;
-            suffix_tile<HD>(kb, vb, lane, min(S_TP, n - tile * S_TP), scale_log2, qb, o, mh, lh, [&]() {
+            if (!__all_sync(0xffffffffu, mbar_wait(full0 + 8 * stage, (uint32_t)(consumed / S_STAGES) & 1u, abort_flag))) { ok = false; break; }
+            const uint32_t kb = tiles_u32 + stage * 2 * TILE_BYTES;
+            suffix_tile<HD>(kb, kb + TILE_BYTES, lane, min(S_TP, it.n - tile * S_TP), scale_log2, qb, o, mh, lh, [&]() {
                 ++consumed;
                 __syncwarp();
-                if (p_item < n_items) p_issue();      // refill the slot just drained
+                refill();
             });
         }
-        if (!ok) break;
-
-        suffix_finish<HD>(lane, o, mh, lh, ml, ml + 8, obuf);
-        __syncwarp();
-        constexpr int EPL = HD / 32;
-        const size_t rh0 = (size_t)row * Hq + (size_t)kvh * n_rep;
-        const int n_own = suffix_chunks(n, ct);
-        if (!waited) {
-            grid_dep_wait();
-            grid_dep_launch_dependents();          // the output projection may request its weights once there is room for it
-            waited = true;
-        }
-        if (n_own == 1) {
-            merge_heads_warp<HD>(lane, rh0, n_rep, part, part.n_parts, ml, ml + 8, obuf, mg.out, mg.out_lo, err);
-        } else {
-            // leave this chunk as record number part.n_parts + chunk, next to the prefix records
-            const size_t base = (size_t)(part.n_parts + chunk) * part.stride + rh0;
-            if (lane < n_rep) { part.m[base + lane] = ml[lane]; part.l[base + lane] = ml[8 + lane]; }
-            for (int j = 0; j < n_rep; ++j) {
-                float* dst = part.o + (base + j) * HD + lane * EPL;
-                const float* src = obuf + j * HD + lane * EPL;
-                if (EPL == 4) *reinterpret_cast<float4*>(dst) = *reinterpret_cast<const float4*>(src);
-                else *reinterpret_cast<float2*>(dst) = *reinterpret_cast<const float2*>(src);
-            }
-            __threadfence();                   // the record is visible before this warp counts as arrived
-            __syncwarp();
-            int last = 0;
+        if (me == 0) {
+            if (ok && p_seq == seq) refill();     // (its last tile was requested, the next item may not have been looked up)
             if (lane == 0) {
-                last = atomicAdd(mg.arrived + it, 1) == n_own - 1;
-                if (last) mg.arrived[it] = 0;  // for the next layer
-                __threadfence();
+                if (!ok) *abort_flag = 1;
+                if (*records_there == 0 && *reinterpret_cast<volatile int32_t*>(part.done) >= wk.prefix_ctas) *records_there = 1;
             }
-            if (__shfl_sync(0xffffffffu, last, 0))
-                merge_heads_warp<HD>(lane, rh0, n_rep, part, part.n_parts + n_own, nullptr, nullptr, nullptr, mg.out, mg.out_lo, err);
         }
-        __syncwarp();
+        if (!ok) *abort_flag = 1;
+        const size_t rh0 = (size_t)row * Hq + (size_t)kvh * n_rep;
+        if (waited) fetch_records(rh0, part.n_parts, T);      // (they travel while the warps meet)
+        team_sync();                              // the item before has been merged; the next is known
+        if (*abort_flag) { ok = false; break; }
+        suffix_finish<HD>(lane, o, mh, lh, ml + me * 16, ml + me * 16 + 8, obuf + me * 8 * HD);
+        if (*known > seq + 1) fetch_q(seq + 1);
+        const bool now = *records_there != 0;
+        if (now && !waited) {
+            wait_prefix();
+            fetch_records(rh0, part.n_parts, T);
+        }
+        team_sync();
+        merge(rh0, true, now ? -1 : part.n_parts);
+        if (!now && me == 0 && lane == 0) { wk.link[it.item] = later; later = it.item; }
     }
-    if (!ok) { *abort_flag = 1; if (lane == 0) set_error(err, DEV_ERR_WAIT_TIMEOUT); }
+    if (!ok && lane == 0) { *abort_flag = 1; set_error(err, DEV_ERR_WAIT_TIMEOUT); }
+    if (!waited) wait_prefix();                   // (every CTA waits on every path)
+    if (me == 0 && lane == 0) *known = later;
+    team_sync();
+    // items put off: a head was left by the warp that merges it now
+    for (int item = *known; item >= 0 && ok;) {
+        const int row = item / Hkv, kvh = item - row * Hkv;
+        const size_t rh0 = (size_t)row * Hq + (size_t)kvh * n_rep;
+        const int next = __ldcg(wk.link + item);
+        fetch_records(rh0, part.n_parts + 1, 0);
+        merge(rh0, false, -1);
+        item = next;
+    }
     // drain: tiles issued but not consumed must land before the shared memory is released
     while (ok && consumed < issued) {
         const int stage = consumed % S_STAGES;
         if (!mbar_wait(full0 + 8 * stage, (uint32_t)(consumed / S_STAGES) & 1u, abort_flag)) break;
         ++consumed;
     }
+    __syncthreads();
     if (*abort_flag) {
         for (int i = 0; i < 2000; ++i) __nanosleep(1000);
     }
     __syncthreads();
-    if (!waited) grid_dep_wait();          // decode steps start this kernel when the shared-prefix kernel's CTAs leave: that one ends first
 }
 
 }  // namespace am

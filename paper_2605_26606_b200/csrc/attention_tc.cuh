@@ -41,6 +41,8 @@ constexpr int STAGES = 2;           // K / V tiles in flight
 constexpr int Q_BYTES = QROWS * HD * 2, P_BYTES = QROWS * TK * 2, KV_BYTES = TK * HD * 2;
 constexpr int THREADS = 192;        // warps 0..3 softmax (TMEM lane quarter = warp), 4 MMA issuer, 5 TMA producer
 constexpr int TMEM_COLS = 256;      // O: columns 0..127, S: 128..191 and 192..255
+constexpr int REC_PITCH = HD * 4 + 16;      // rows of an output on its way out: eight threads' 16 bytes in different banks
+static_assert(QROWS * REC_PITCH <= Q_BYTES + P_BYTES + STAGES * 2 * KV_BYTES, "rows of a record");
 constexpr int SMEM_BYTES = Q_BYTES + P_BYTES + STAGES * 2 * KV_BYTES + 1024;      // 113 KB: half of an SM's 228 KB less the reserved KB
 
 // Shared-memory descriptor of an MN-major 128-byte-swizzled operand: rows of 64 values along MN (128 bytes), 8-row groups along K
@@ -108,6 +110,7 @@ attn_prefix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
         if (q0 < n_q && threadIdx.x == 0) set_error(err, DEV_ERR_GROUP_RANGE);        // (the shared memory window is not where it should be)
         grid_dep_wait();
         grid_dep_launch_dependents();
+        if (!FINAL && part.done != nullptr && threadIdx.x == 0) atomicAdd(part.done, 1);
         return;
     }
 
@@ -305,6 +308,9 @@ attn_prefix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
             const size_t ph = (size_t)my_part * part.stride + rh;
             const float inv = FINAL ? (l > 0.f ? 1.f / l : 0.f) : 1.f;
             if (!FINAL && valid) { part.m[ph] = m; part.l[ph] = l; }
+            // a record's output (512 bytes, a row per thread) leaves through shared memory, where nothing is in use any more: stored by
+            // the threads, 16 bytes each of 32 rows at a time, it took 2 us
+            float* rec_row = reinterpret_cast<float*>(base + threadIdx.x * REC_PITCH);
             if (n_tiles > 0) {               // an empty range leaves (m, l) = (-inf, 0); its output is never read
 #pragma unroll 1
                 for (int c = 0; c < HD; c += 32) {
@@ -312,7 +318,7 @@ attn_prefix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
                     tc::tmem_ld32(lanes + c, o);
                     if (!valid) continue;
                     if (!FINAL) {
-                        float4* dst = reinterpret_cast<float4*>(part.o + ph * HD + c);
+                        float4* dst = reinterpret_cast<float4*>(rec_row + c);
 #pragma unroll
                         for (int i = 0; i < 8; ++i) dst[i] = make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
                         continue;
@@ -338,6 +344,13 @@ attn_prefix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
                         }
                     }
                 }
+                if (!FINAL && valid) {
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
+                                 ::"l"(__cvta_generic_to_global(part.o + ph * HD)), "r"(smem_u32(rec_row)), "r"(HD * 4) : "memory");
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+                }
             } else if (FINAL && valid) {
                 for (int c = 0; c < HD; c += 8) {
                     *reinterpret_cast<uint4*>(out + rh * HD + c) = make_uint4(0u, 0u, 0u, 0u);
@@ -349,6 +362,8 @@ attn_prefix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
     if (!ok && lane == 0) { *abort_flag = 1; set_error(err, DEV_ERR_WAIT_TIMEOUT); }
     tc_fence_before();
     __syncthreads();
+    // Tells suffix warps that started beside this kernel when to stop putting off their merges.  (They still wait for the kernel's end.)
+    if (!FINAL && part.done != nullptr && threadIdx.x == 0) atomicAdd(part.done, 1);
     if (*abort_flag) {
 #pragma unroll 1
         for (int i = 0; i < 2000; ++i) __nanosleep(1000);    // copies in flight land before the shared memory is released

@@ -45,12 +45,13 @@ __global__ void load_step_desc(const DecodeArgsDev* __restrict__ da, int32_t* co
 // Also compacts the row's sampling key, the position of its next token and the step's group boundaries into the
 // workspace.  A row whose indices do not fit their arrays is switched off (no KV access, token 0) and flagged.
 __global__ void prep_decode_rows(const StepDesc* __restrict__ sd, const DecodeArgsDev* __restrict__ da, int64_t prompt_slots,
-                                 int64_t suffix_slots, int vocab, RowGeom g, RowKeys keys, int32_t* __restrict__ arrived, int Hkv, int32_t* err) {
+                                 int64_t suffix_slots, int vocab, RowGeom g, RowKeys keys,
+                                 int32_t* __restrict__ sched, int n_sched, int32_t* err) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     const int n_rows = sd->n_rows;
+    for (int i = r; i < n_sched; i += gridDim.x * blockDim.x) sched[i] = 0;        // work counters of the layers' attention
     if (r <= sd->n_groups) keys.group_start[r] = da->group_row_start[sd->group_off + r];
     if (r >= n_rows) return;
-    for (int k = 0; k < Hkv; ++k) arrived[r * Hkv + k] = 0;        // (attn_suffix_kernel leaves them 0 after every complete layer)
     const int64_t ro = sd->row_off + r;
     int p = da->row_prompt[ro];
     const int step = da->row_step[ro];

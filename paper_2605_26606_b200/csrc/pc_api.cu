@@ -84,7 +84,7 @@ constexpr int kMaxSplits = pc::PARTIALS_MAX;
 
 struct Carve {
     size_t h, a, qkv, q, attn, act, logits, rope, pos, wslot, warena, p_start, p_len, s_start, s_len, token, last_row,
-        part_m, part_l, part_o, arrived, res_part, step_desc, step_counter, max_slen, sample_scratch, a_lo, attn_lo, chain_layers, chain_glob,
+        part_m, part_l, part_o, put_off, sched, res_part, step_desc, step_counter, max_slen, sample_scratch, a_lo, attn_lo, chain_layers, chain_glob,
         chain_bar, dargs, key_prompt, key_rollout, key_step, out_index, group_start, sample_tiles, sample_bound, ssq, row_pow2, total;
 };
 
@@ -236,7 +236,8 @@ Carve carve(const pc_ctx* c, int max_rows, int max_prefill) {
     v.part_m = take(pc::am::MAX_RECORDS * R * d.n_q_heads * 4);
     v.part_l = take(pc::am::MAX_RECORDS * R * d.n_q_heads * 4);
     v.part_o = take(pc::am::MAX_RECORDS * R * d.n_q_heads * d.head_dim * 4);
-    v.arrived = take(R * d.n_kv_heads * 4);
+    v.put_off = take(R * d.n_kv_heads * 4);             // lists of attn_suffix_kernel
+    v.sched = take(2 * (size_t)d.n_layers * 4);         // per layer: next item of the suffix attention, finished CTAs of the shared-prefix attention
     v.total = off;
     return v;
 }
@@ -455,6 +456,15 @@ struct AttnPlan {
 // Whether a decode step's attention takes a team of CTAs per (row, KV head).
 bool suffix_teams(const pc_ctx* c, int M) { return M * c->d.n_kv_heads <= 2 * c->num_sms; }
 
+// Warps that share an item of attn_suffix_kernel: two, so that a CTA has two items in hand and one is streamed while the other is merged;
+// four where the items would be one to two rounds of the pairs, the second of them partly empty.  Eight decode steps with pairs / with
+// four, 1.5B shape, 296 CTAs = 592 pairs: 237 rows x 512 (474 items) 19.03 / 19.25 ms, 336 x 900 (672) 29.9 / 29.4, 2,048 x 512 (4,096) 95.1 /
+// 96.7; 8B shape, 64 x 300 (512) 34.7 / 35.3.
+int suffix_team_warps(const pc_ctx* c, int items) {
+    const int pairs = c->num_sms * pc::am::S_CTAS * pc::am::S_WARPS / 2;
+    return items > pairs && items <= 2 * pairs ? 4 : 2;
+}
+
 // Whether the teams read the prompt too, once per row instead of once per group, and there is no shared-prefix kernel.  With so few rows
 // that kernel and the hand-over of its records (7 + 4 us of a 40 us layer at 16 rows) cost more than the reads, which L2 serves, up to prompts of
 // about 1,024 tokens.  Eight decode steps of the 1.5B shape, with it and without: 16 rows x 640 tokens 8.92 / 9.75 ms, 36 x 640 10.23 / 10.72, 36 x
@@ -503,7 +513,9 @@ cudaError_t configure_attention() {
             e = cudaFuncSetAttribute(am::attn_group_kernel<HD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::group_smem_bytes<HD>());
     }
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(am::attn_suffix_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::SUFFIX_SMEM_BYTES);
+        e = cudaFuncSetAttribute(am::attn_suffix_kernel<HD, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::SUFFIX_SMEM_BYTES);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(am::attn_suffix_kernel<HD, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::SUFFIX_SMEM_BYTES);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(am::attn_suffix_team_kernel<HD, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, am::TEAM_SMEM_BYTES);
     if (e == cudaSuccess)
@@ -606,7 +618,7 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
     const int n_parts = plan.prefill ? 1 : std::max(1, std::min(teams ? am::MAX_PREFIX_PARTS : am::MAX_MERGED_PARTS, c->num_sms / base_ctas));
     am::PrefixPartial part{reinterpret_cast<float*>(c->ws + c->cv.part_m), reinterpret_cast<float*>(c->ws + c->cv.part_l),
                            reinterpret_cast<float*>(c->ws + c->cv.part_o), n_parts, (size_t)std::max(c->max_rows, 1) * d.n_q_heads,
-                           d.n_kv_heads, c->num_sms * am::S_CTAS * am::S_WARPS};
+                           HD == 128 && !teams && !plan.prefill ? reinterpret_cast<int32_t*>(c->ws + c->cv.sched) + 2 * layer + 1 : nullptr};
     const dim3 ggrid = HD == 128 ? dim3(q_tiles * n_parts * d.n_kv_heads * plan.n_groups) : dim3(q_tiles * n_parts, d.n_kv_heads, plan.n_groups);
     if (plan.prefill) {
         if constexpr (HD == 128)
@@ -662,11 +674,11 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
                                                  d.n_kv_heads, layer, q, g, scale_log2, part, team, attn, attn_lo, c->err);
         if (e != cudaSuccess) return cuda_fail(e, "suffix attention");
     } else {
-        // one warp per (rollout, KV head, range of the suffix); how the suffixes are cut into ranges is decided on the device for
-        // the warps of this grid (the longest suffix of the step is only known there)
-        const am::SuffixMerge mg{reinterpret_cast<int32_t*>(c->ws + c->cv.arrived), attn, attn_lo};
-        launch_k_dep(group_dep, am::attn_suffix_kernel<HD>, dim3(am::S_CTAS * c->num_sms), dim3(am::S_WARPS * 32), am::SUFFIX_SMEM_BYTES, st,
-            c->map_suffix_kv, sd, suffix_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, g, scale_log2, part, mg, c->err);
+        const am::SuffixWork work{reinterpret_cast<int32_t*>(c->ws + c->cv.sched) + 2 * layer, reinterpret_cast<int32_t*>(c->ws + c->cv.put_off),
+                                  (int)ggrid.x, attn, attn_lo};
+        launch_k_dep(group_dep, suffix_team_warps(c, items) == 4 ? am::attn_suffix_kernel<HD, 4> : am::attn_suffix_kernel<HD, 2>, dim3(am::S_CTAS * c->num_sms),
+            dim3(am::S_WARPS * 32), am::SUFFIX_SMEM_BYTES, st, c->map_suffix_kv, sd, suffix_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, g, scale_log2,
+            part, work, c->err);
     }
     c->mark(st, layer, PC_MARK_SUFFIX);
     c->mark(st, layer, PC_MARK_MERGE);
@@ -1440,7 +1452,7 @@ int decode_launches(pc_ctx* ctx, cudaStream_t st, int m_bound, int groups_bound,
     if (cap == cudaStreamCaptureStatusNone && ctx->prof_layer >= 0) { ctx->prof_active_layer = ctx->prof_layer; ctx->prof_layer = -1; }
     struct Disarm { pc_ctx* c; ~Disarm() { c->prof_active_layer = -1; } } disarm{ctx};
     launch_k(pc::prep_decode_rows, dim3((m_bound + 128) / 128), dim3(128), 0, st, sd, da, a.prompt_slots, a.suffix_slots, ctx->d.vocab, g, keys,
-             reinterpret_cast<int32_t*>(ctx->ws + ctx->cv.arrived), ctx->d.n_kv_heads, ctx->err);
+             reinterpret_cast<int32_t*>(ctx->ws + ctx->cv.sched), 2 * ctx->d.n_layers, ctx->err);
     count_launches(1);
     PC_CUDA_CHECK_LAUNCH("prep_decode_rows");
     const pc::KvArena pa{const_cast<void*>(a.prompt_kv), a.prompt_slots}, sa{a.suffix_kv, a.suffix_slots};

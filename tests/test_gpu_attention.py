@@ -43,6 +43,15 @@ def test_decode_logits_at_attention_tile_edges(cuda_device, model, prompt, rows,
             assert np.max(np.abs(logits[row].cpu().numpy() - want[prompt + s])) <= 5e-2, (p, i, s)
 
 
+@pytest.mark.parametrize("model,prompt,rows,depth,half", [(wl.SMALL_BF16, 600, 150, 3, True), (wl.SMALL_QKNORM_BF16, 40, 150, 66, True),
+                                                          (wl.SMALL_BF16, 300, 160, 35, False), (wl.SMALL_BF16, 64, 300, 18, True),
+                                                          (wl.TINY_BF16, 130, 160, 34, True)], ids=lambda v: getattr(v, "name", str(v)))
+def test_decode_logits_where_suffix_items_are_claimed(cuda_device, model, prompt, rows, depth, half):
+    """600 to 1,200 (row, KV head) items: up to one, between one and two, and more than two rounds of warp pairs.  Long prompts beside short
+    suffixes: items are finished before the shared-prefix records are there, and some warps have no tile."""
+    test_decode_logits_at_attention_tile_edges(cuda_device, model, prompt, rows, depth, half)
+
+
 def test_probabilities_round_below_their_maximum(cuda_device):
     """Half rounds a probability finest just below the row's largest, which is 1 and exact.  64 keys of one kind, then 200 whose score is
     higher by log2(1.00044): as 1.00044 they would round to 1, a relative error of 4.4e-4 in every output; as 1, beside 0.99956 for
