@@ -17,18 +17,29 @@ constexpr int ATTN_MAX_REP = 8;   // query heads per KV head supported
 constexpr int ATTN_WARPS = 8;
 constexpr int ATTN_CHUNK = 8;     // positions a warp works on together
 
+// POST (decode): the q|k|v projection comes as it left its GEMM, and the block finishes its own heads first -- bias, QK-norm, RoPE, q to
+// its buffer, K and V to the row's slot, which no other row attends (a kernel of its own was 4 us per layer).
 // HD = head_dim (64 or 128); each lane owns EPL = HD / 32 consecutive dims of every K/V row.  REP: query heads per KV head, rounded
 // up to 2, 4 or 8.
-template <int HD, int REP>
-__global__ void __launch_bounds__(32 * ATTN_WARPS) attn_row_simt_kernel(const StepDesc* __restrict__ sd, int Hq, int Hkv, int layer, const float* __restrict__ q,
+template <int HD, int REP, bool POST>
+__global__ void __launch_bounds__(32 * ATTN_WARPS) attn_row_simt_kernel(const StepDesc* __restrict__ sd, int Hq, int Hkv, int layer, const float* q,
                                                                         RowGeom g, KvArena prompt_arena, KvArena suffix_arena,
-                                                                        float scale, float* __restrict__ out) {
+                                                                        float scale, float* __restrict__ out, QkvPostArgs<float> post) {
     constexpr int EPL = HD / 32, CH = ATTN_CHUNK;
     const int r = blockIdx.x, kvh = blockIdx.y;
+    grid_dep_wait();
+    grid_dep_launch_dependents();
     if (r >= sd->n_rows) return;
     const int n_rep = Hq / Hkv;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
+    if (POST) {
+        for (int j = warp; j < n_rep + 2; j += ATTN_WARPS) {
+            const int head = j < n_rep ? kvh * n_rep + j : Hq + kvh + (j - n_rep) * Hkv;
+            qkv_post_items_warp<float, 1>(lane, post, &r, &head, 1);
+        }
+        __syncthreads();
+    }
     float qf[REP][EPL], acc[REP][EPL], mx[REP], ls[REP];
 #pragma unroll
     for (int j = 0; j < REP; ++j) {
@@ -137,14 +148,19 @@ __global__ void __launch_bounds__(32 * ATTN_WARPS) attn_row_simt_kernel(const St
     }
 }
 
-template <int HD>
-inline void launch_attn_row_simt(cudaStream_t st, const StepDesc* sd, int M, int Hq, int Hkv, int layer, const float* q, RowGeom g, KvArena prompt_arena,
-                                 KvArena suffix_arena, float scale, float* out) {
+template <int HD, bool POST>
+inline cudaError_t launch_attn_row_simt(cudaStream_t st, bool dep, const StepDesc* sd, int M, int Hq, int Hkv, int layer, const float* q, RowGeom g,
+                                        KvArena prompt_arena, KvArena suffix_arena, float scale, float* out, const QkvPostArgs<float>& post) {
     const int rep = Hq / Hkv;
-    const dim3 grid(M, Hkv);
-    if (rep <= 2) attn_row_simt_kernel<HD, 2><<<grid, 32 * ATTN_WARPS, 0, st>>>(sd, Hq, Hkv, layer, q, g, prompt_arena, suffix_arena, scale, out);
-    else if (rep <= 4) attn_row_simt_kernel<HD, 4><<<grid, 32 * ATTN_WARPS, 0, st>>>(sd, Hq, Hkv, layer, q, g, prompt_arena, suffix_arena, scale, out);
-    else attn_row_simt_kernel<HD, 8><<<grid, 32 * ATTN_WARPS, 0, st>>>(sd, Hq, Hkv, layer, q, g, prompt_arena, suffix_arena, scale, out);
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(M, Hkv); cfg.blockDim = dim3(32 * ATTN_WARPS); cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = dep ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, rep <= 2 ? attn_row_simt_kernel<HD, 2, POST> : rep <= 4 ? attn_row_simt_kernel<HD, 4, POST> : attn_row_simt_kernel<HD, 8, POST>,
+                              sd, Hq, Hkv, layer, q, g, prompt_arena, suffix_arena, scale, out, post);
 }
 
 }  // namespace pc

@@ -95,7 +95,6 @@ attn_prefix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
     int* s_maxlen = reinterpret_cast<int*>(tmem_slot + 2);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    if (FINAL) grid_dep_wait();             // K and V of this very pass; decode: the prompt's were written by an earlier call
     const int n_rep = Hq / Hkv;
     const int n_parts = FINAL ? 1 : part.n_parts;
     const int unit = blockIdx.x;
@@ -158,6 +157,7 @@ attn_prefix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
     if (warp == 5) {
         {
             // ---------------- TMA producer ----------------
+            if (FINAL) grid_dep_wait();             // K and V of this very pass; decode: the prompt's were written by an earlier call
             const int64_t kv_start = g.p_start[row0];
             const int64_t krow = (((int64_t)layer * 2 + 0) * Hkv + kvh) * n_slots + kv_start, vrow = (((int64_t)layer * 2 + 1) * Hkv + kvh) * n_slots + kv_start;
 #pragma unroll 1

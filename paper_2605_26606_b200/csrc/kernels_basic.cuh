@@ -24,6 +24,7 @@ struct RowGeom {
 // launched with STEP_DESC_THREADS threads).
 constexpr int STEP_DESC_THREADS = 128;
 __global__ void set_step_desc(StepDesc* sd, int n_rows, int n_groups, int max_group_rows, int32_t* max_slen, int32_t* bar, int n_bar) {
+    grid_dep_launch_dependents();
     for (int i = threadIdx.x; i < n_bar; i += blockDim.x) bar[i] = 0;
     if (threadIdx.x != 0) return;
     *max_slen = 0;
@@ -32,6 +33,7 @@ __global__ void set_step_desc(StepDesc* sd, int n_rows, int n_groups, int max_gr
 }
 // First node of a captured decode step: takes the next descriptor of the caller's schedule.
 __global__ void load_step_desc(const DecodeArgsDev* __restrict__ da, int32_t* counter, StepDesc* sd, int32_t* max_slen, int32_t* bar, int n_bar) {
+    grid_dep_launch_dependents();
     for (int i = threadIdx.x; i < n_bar; i += blockDim.x) bar[i] = 0;
     if (threadIdx.x != 0) return;
     *max_slen = 0;
@@ -47,6 +49,8 @@ __global__ void load_step_desc(const DecodeArgsDev* __restrict__ da, int32_t* co
 __global__ void prep_decode_rows(const StepDesc* __restrict__ sd, const DecodeArgsDev* __restrict__ da, int64_t prompt_slots,
                                  int64_t suffix_slots, int vocab, RowGeom g, RowKeys keys,
                                  int32_t* __restrict__ sched, int n_sched, int32_t* err) {
+    grid_dep_wait();
+    grid_dep_launch_dependents();
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     const int n_rows = sd->n_rows;
     for (int i = r; i < n_sched; i += gridDim.x * blockDim.x) sched[i] = 0;        // work counters of the layers' attention
@@ -91,6 +95,8 @@ __global__ void prep_decode_rows(const StepDesc* __restrict__ sd, const DecodeAr
 __global__ void prep_prefill_rows(int n_prompts, const int32_t* prompt_tokens, const int32_t* prompt_offsets,
                                   const int64_t* prompt_kv_start, int64_t prompt_slots, int vocab, RowGeom g,
                                   int32_t* last_row, int32_t* err) {
+    grid_dep_wait();
+    grid_dep_launch_dependents();
     const int p = blockIdx.x;
     const int b = prompt_offsets[p], e = prompt_offsets[p + 1];
     const int64_t ps = prompt_kv_start[p];
@@ -113,14 +119,17 @@ __global__ void prep_prefill_rows(int n_prompts, const int32_t* prompt_tokens, c
 }
 
 // cos/sin of pos * theta^(-2i/hd), evaluated in double so that long positions keep float accuracy.
+__device__ __forceinline__ float2 rope_entry(int pos, int i, int half, double theta) {
+    const double inv_freq = pow(theta, -(double)i / (double)half);
+    double s, c;
+    sincos((double)pos * inv_freq, &s, &c);
+    return make_float2((float)c, (float)s);
+}
 __global__ void rope_table_kernel(const StepDesc* __restrict__ sd, int half, double theta, const int32_t* pos, float2* table) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= sd->n_rows * half) return;
     const int r = idx / half, i = idx - r * half;
-    const double inv_freq = pow(theta, -(double)i / (double)half);
-    double s, c;
-    sincos((double)pos[r] * inv_freq, &s, &c);
-    table[idx] = make_float2((float)c, (float)s);
+    table[idx] = rope_entry(pos[r], i, half, theta);
 }
 
 // K-slice sums left by a split GEMM: value(row, col) = sum over s < n of p[s * stride + row * ld + col], added in
@@ -334,16 +343,19 @@ __device__ __forceinline__ void embed_row_warp(int lane, int d, const T* __restr
 constexpr int ROW_WARPS = 8;         // items per block of the stand-alone per-(row, head) kernels
 constexpr int NORM_THREADS = NORM_SEGS * 32;
 
-// h[r, :] = E[token[r], :] (float residual stream); a[r, :] = RMSNorm(h[r, :]; gain) in storage type T.  next_scale (or nullptr):
+// h[r, :] = E[token[r], :] (float residual stream); a[r, :] = RMSNorm(h[r, :]; gain) in storage type T (a == nullptr: the projection
+// applies it); the row's rotary factors.  next_scale (or nullptr):
 // operand_scale per row, for the output projection's epilogue.  One block per row.
 template <typename T>
 __global__ void __launch_bounds__(NORM_THREADS) embed_rmsnorm_kernel(const StepDesc* __restrict__ sd, int d, const int32_t* token,
                                                                      const T* __restrict__ embed, const float* __restrict__ gain, float eps,
                                                                      float* __restrict__ h, T* __restrict__ a, T* __restrict__ a_lo, int half_out,
-                                                                     int32_t* err, float* __restrict__ next_scale) {
+                                                                     int32_t* err, float* __restrict__ next_scale, int half, double theta,
+                                                                     const int32_t* __restrict__ pos, float2* __restrict__ rope) {
     __shared__ float red[8];
     __shared__ int counter;
     const int r = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    grid_dep_wait();
     grid_dep_launch_dependents();          // the projection that follows may set itself up and request its first weight tiles
     if (r >= sd->n_rows) return;
     if (threadIdx.x == 0) counter = 0;
@@ -355,6 +367,9 @@ __global__ void __launch_bounds__(NORM_THREADS) embed_rmsnorm_kernel(const StepD
         VecLoad<T, 4>::load(e_row + 4 * i, v);
         reinterpret_cast<float4*>(h_row)[i] = make_float4(v[0], v[1], v[2], v[3]);
     }
+    // (the warps at the end: they have the fewest elements of the row)
+    for (int i = NORM_THREADS - 1 - threadIdx.x; i < half; i += NORM_THREADS) rope[(size_t)r * half + i] = rope_entry(pos[r], i, half, theta);
+    if (a == nullptr) return;
     __syncthreads();
     if (norm_row_fits_cta(d))
         norm_row_cta<T>(w, lane, d, h_row, Partials{nullptr, 0, 0, 0}, 0, gain, eps, a + (size_t)r * d, a_lo ? a_lo + (size_t)r * d : nullptr,
@@ -520,6 +535,7 @@ template <typename T>
 __global__ void __launch_bounds__(ROW_WARPS * 32) qkv_post_kernel(const StepDesc* __restrict__ sd, QkvPostArgs<T> A) {
     const int n_heads = A.Hq + 2 * A.Hkv;
     const int item = blockIdx.x * ROW_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    grid_dep_wait();
     grid_dep_launch_dependents();          // the shared-prefix attention kernel may request its first prompt K/V tiles
     if (item >= sd->n_rows * n_heads) return;
     const int row = item / n_heads, head = item - row * n_heads;

@@ -622,7 +622,7 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
     const dim3 ggrid = HD == 128 ? dim3(q_tiles * n_parts * d.n_kv_heads * plan.n_groups) : dim3(q_tiles * n_parts, d.n_kv_heads, plan.n_groups);
     if (plan.prefill) {
         if constexpr (HD == 128)
-            launch_k(at::attn_prefix_kernel<true>, ggrid, dim3(at::THREADS), at::SMEM_BYTES, st,
+            launch_k_dep(dependent_launch(c, DEP_GROUP, M), at::attn_prefix_kernel<true>, ggrid, dim3(at::THREADS), at::SMEM_BYTES, st,
                 c->map_prompt_kv, sd, prompt_arena.n_slots, d.n_q_heads, d.n_kv_heads, layer, q, plan.group_row_start, g, scale_log2,
                 part, q_tiles, attn, attn_lo, c->err);
         else
@@ -718,10 +718,12 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
     Partials pend = none;
 
     c->final_norm_pending = false;
-    launch_k(rope_table_kernel, dim3((M * half + 255) / 256), dim3(256), 0, st, sd, half, (double)d.rope_theta, g.pos, rope);
-    launch_k(embed_rmsnorm_kernel<T>, dim3(M), dim3(NORM_THREADS), 0, st, sd, d.d_model, g.token, reinterpret_cast<const T*>(c->embed), c->attn_norm[0],
-                                               d.rms_eps, h, a, a_lo, half_gemm ? 1 : 0, c->err, pow2_mlp);
-    count_launches(2);
+    // Row-wise kernels that wait for the one before them first and release the next one then: launched as programmatic dependents, but not in
+    // steps that record phase events (an event between two kernels is no kernel-to-kernel edge).
+    const bool dep = c->dep_launch != 0 && c->prof_active_layer < 0;
+    launch_k_dep(dep, embed_rmsnorm_kernel<T>, dim3(M), dim3(NORM_THREADS), 0, st, sd, d.d_model, g.token, reinterpret_cast<const T*>(c->embed), c->attn_norm[0],
+                 d.rms_eps, h, kF32 ? nullptr : a, a_lo, half_gemm ? 1 : 0, c->err, pow2_mlp, half, (double)d.rope_theta, g.pos, rope);
+    count_launches(1);
     PC_CUDA_CHECK_LAUNCH("embed_rmsnorm");
     for (int l = 0; l < d.n_layers; ++l) {
         c->mark(st, l, PC_MARK_LAYER_BEGIN);
@@ -780,7 +782,7 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
             PC_CUDA_CHECK_LAUNCH("decoder layer");
             continue;
         }
-        if (l > 0) {
+        if (!kF32 && l > 0) {
             launch_k(rmsnorm_kernel<T>, dim3(M), dim3(NORM_THREADS), 0, st, sd, M, d.d_model, h, nullptr, pend, c->attn_norm[l], d.rms_eps, a, a_lo, half_gemm ? 1 : 0, c->err);
             pend = none;
             count_launches(1);
@@ -789,8 +791,8 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
         const float* bias = d.qkv_bias ? c->bqkv[l] : nullptr;
         Partials qkv_parts{qkv, 1, (size_t)M * c->n_qkv(), c->n_qkv()};
         if constexpr (kF32) {
-            launch_gemm_simt(st, sd, a, reinterpret_cast<const T*>(c->wqkv[l]), M, c->n_qkv(), d.d_model,
-                                EpiStoreF32{qkv, c->n_qkv(), nullptr});
+            launch_gemm_simt(st, dep, sd, h, reinterpret_cast<const T*>(c->wqkv[l]), M, c->n_qkv(), d.d_model,
+                                SimtNorm{c->attn_norm[l], d.rms_eps, nullptr}, EpiStoreF32{qkv, c->n_qkv(), nullptr});
         } else {
             const GemmPlan gp = plan_gemm(c, GEMM_QKV, c->m_wqkv[l], M, true);
             qkv_parts.n = gp.splits;
@@ -799,20 +801,30 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
                 return rc;
         }
         c->mark(st, l, PC_MARK_QKV);
-        const int post_items = M * (d.n_q_heads + 2 * d.n_kv_heads);
-        launch_k(qkv_post_kernel<T>, dim3((post_items + ROW_WARPS - 1) / ROW_WARPS), dim3(ROW_WARPS * 32), 0, st,
-            sd, QkvPostArgs<T>{d.n_q_heads, d.n_kv_heads, d.head_dim, l, qkv_parts, bias, d.qk_norm ? c->q_norm[l] : nullptr,
-                               d.qk_norm ? c->k_norm[l] : nullptr, d.rms_eps, rope, g, prompt_arena, suffix_arena, q, c->err});
-        count_launches(2);
+        const QkvPostArgs<T> post{d.n_q_heads, d.n_kv_heads, d.head_dim, l, qkv_parts, bias, d.qk_norm ? c->q_norm[l] : nullptr,
+                                  d.qk_norm ? c->k_norm[l] : nullptr, d.rms_eps, rope, g, prompt_arena, suffix_arena, q, c->err};
+        const bool post_in_attention = kF32 && !plan.prefill;          // (a prefill's rows attend one another)
+        if (!post_in_attention) {
+            const int post_items = M * (d.n_q_heads + 2 * d.n_kv_heads);
+            launch_k_dep(kF32 && dep, qkv_post_kernel<T>, dim3((post_items + ROW_WARPS - 1) / ROW_WARPS), dim3(ROW_WARPS * 32), 0, st, sd, post);
+            count_launches(1);
+        }
+        count_launches(1);
         c->mark(st, l, PC_MARK_POST);
         if constexpr (kF32) {
             c->mark(st, l, PC_MARK_GROUP);
-            if (d.head_dim == 128) launch_attn_row_simt<128>(st, sd, M, d.n_q_heads, d.n_kv_heads, l, q, g, prompt_arena, suffix_arena, scale, attn);
-            else launch_attn_row_simt<64>(st, sd, M, d.n_q_heads, d.n_kv_heads, l, q, g, prompt_arena, suffix_arena, scale, attn);
+            auto attend = [&](auto hd, auto fused) {
+                return launch_attn_row_simt<decltype(hd)::value, decltype(fused)::value>(st, dep, sd, M, d.n_q_heads, d.n_kv_heads, l, q, g, prompt_arena, suffix_arena,
+                                                                                         scale, attn, post);
+            };
+            using H64 = std::integral_constant<int, 64>;
+            using H128 = std::integral_constant<int, 128>;
+            if (d.head_dim == 128) post_in_attention ? attend(H128{}, std::true_type{}) : attend(H128{}, std::false_type{});
+            else post_in_attention ? attend(H64{}, std::true_type{}) : attend(H64{}, std::false_type{});
             c->mark(st, l, PC_MARK_SUFFIX);
             c->mark(st, l, PC_MARK_MERGE);
             count_launches(1);
-            launch_gemm_simt(st, sd, attn, reinterpret_cast<const T*>(c->wo[l]), M, d.d_model, c->q_dim(), EpiResidual{h, d.d_model});
+            launch_gemm_simt(st, dep, sd, attn, reinterpret_cast<const T*>(c->wo[l]), M, d.d_model, c->q_dim(), SimtNorm{}, EpiResidual{h, d.d_model});
         } else {
             int rc = d.head_dim == 128
                          ? attention_bf16<128>(c, st, sd, M, l, plan, prompt_arena, suffix_arena, q, attn)
@@ -831,15 +843,18 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
             }
         }
         c->mark(st, l, PC_MARK_O);
-        launch_k(rmsnorm_kernel<T>, dim3(M), dim3(NORM_THREADS), 0, st, sd, M, d.d_model, h, nullptr, pend, c->mlp_norm[l], d.rms_eps, a, nullptr, half_gemm ? 1 : 0, c->err);
-        pend = none;
-        count_launches(2);
+        if constexpr (!kF32) {
+            launch_k(rmsnorm_kernel<T>, dim3(M), dim3(NORM_THREADS), 0, st, sd, M, d.d_model, h, nullptr, pend, c->mlp_norm[l], d.rms_eps, a, nullptr, half_gemm ? 1 : 0, c->err);
+            pend = none;
+            count_launches(1);
+        }
+        count_launches(1);
         c->mark(st, l, PC_MARK_NORM_MLP);
         if constexpr (kF32) {
-            launch_gemm_simt(st, sd, a, reinterpret_cast<const T*>(c->w_gate_up[l]), M, 2 * d.d_ff, d.d_model,
-                                EpiSwiGLU{act, d.d_ff});
+            launch_gemm_simt(st, dep, sd, h, reinterpret_cast<const T*>(c->w_gate_up[l]), M, 2 * d.d_ff, d.d_model,
+                                SimtNorm{c->mlp_norm[l], d.rms_eps, nullptr}, EpiSwiGLU{act, d.d_ff});
             c->mark(st, l, PC_MARK_GATE_UP);
-            launch_gemm_simt(st, sd, act, reinterpret_cast<const T*>(c->w_down[l]), M, d.d_model, d.d_ff, EpiResidual{h, d.d_model});
+            launch_gemm_simt(st, dep, sd, act, reinterpret_cast<const T*>(c->w_down[l]), M, d.d_model, d.d_ff, SimtNorm{}, EpiResidual{h, d.d_model});
         } else {
             if (int rc = gemm_bf16(c, st, sd, c->map_a, nullptr, c->m_wgu[l], M, plan_gemm(c, GEMM_GATE_UP, c->m_wgu[l], M, false), tc::EpiSwiGLU{act, d.d_ff, half_gemm ? 1 : 0, c->err}, half_gemm, DEP_GATE_UP))
                 return rc;
@@ -880,12 +895,14 @@ int run_lm_head(pc_ctx* c, cudaStream_t st, int n, const pc::StepDesc* sd, const
     c->mark(st, -1, PC_MARK_LM_BEGIN);
     const bool folded = c->final_norm_pending;         // only the 1/rms factor is still to be applied: the LM head's epilogue does
     c->final_norm_pending = false;
-    if (!folded)
+    const bool in_head = std::is_same<T, float>::value;      // the norm is applied by the LM head's GEMM
+    if (!folded && !in_head)
         launch_k(rmsnorm_kernel<T>, dim3(n), dim3(NORM_THREADS), 0, st, sd, n, d.d_model, h, src, c->pend, c->final_norm, d.rms_eps, a, a_lo, half_gemm ? 1 : 0, c->err);
     c->pend = pc::Partials{nullptr, 0, 0, 0};
     if constexpr (std::is_same<T, float>::value) {
         const T* wlm = reinterpret_cast<const T*>(d.tied_embed ? c->embed : c->lm_head);
-        launch_gemm_simt(st, sd, a, wlm, n, d.vocab, d.d_model, EpiStoreF32{logits, d.vocab, nullptr});
+        launch_gemm_simt(st, c->dep_launch != 0 && c->prof_active_layer < 0, sd, h, wlm, n, d.vocab, d.d_model, SimtNorm{c->final_norm, d.rms_eps, src},
+                            EpiStoreF32{logits, d.vocab, nullptr});
     } else if (folded || use_wt(c, n)) {
         wt::EpiStore epi{logits, d.vocab, {}};
         if (folded) epi.rs = folded_norm(c);
@@ -895,7 +912,7 @@ int run_lm_head(pc_ctx* c, cudaStream_t st, int n, const pc::StepDesc* sd, const
                                tc::EpiStoreF32{logits, d.vocab, nullptr}, half_gemm, DEP_LM_HEAD))
             return rc;
     }
-    count_launches(folded ? 1 : 2);
+    count_launches(folded || in_head ? 1 : 2);
     c->mark(st, -1, PC_MARK_LM_HEAD);
     PC_CUDA_CHECK_LAUNCH("lm head");
     return PC_OK;
@@ -1247,7 +1264,7 @@ int pc_prefill_shared(pc_ctx* ctx, void* stream, int n_prompts, const int32_t* p
     int32_t* last_row = reinterpret_cast<int32_t*>(ctx->ws + ctx->cv.last_row);
     pc::StepDesc* sd = reinterpret_cast<pc::StepDesc*>(ctx->ws + ctx->cv.step_desc);
     pc::set_step_desc<<<1, pc::STEP_DESC_THREADS, 0, st>>>(sd, total_tokens, n_prompts, max_prompt_len, g.max_slen, nullptr, 0);
-    launch_k(pc::prep_prefill_rows, dim3(n_prompts), dim3(256), 0, st, n_prompts, prompt_tokens, prompt_offsets, prompt_kv_start, prompt_slots,
+    launch_k_dep(ctx->dep_launch != 0, pc::prep_prefill_rows, dim3(n_prompts), dim3(256), 0, st, n_prompts, prompt_tokens, prompt_offsets, prompt_kv_start, prompt_slots,
                                                      ctx->d.vocab, g, last_row, ctx->err);
     count_launches(2);
     PC_CUDA_CHECK_LAUNCH("prep_prefill_rows");
@@ -1451,7 +1468,8 @@ int decode_launches(pc_ctx* ctx, cudaStream_t st, int m_bound, int groups_bound,
     ctx->prof_active_layer = -1;
     if (cap == cudaStreamCaptureStatusNone && ctx->prof_layer >= 0) { ctx->prof_active_layer = ctx->prof_layer; ctx->prof_layer = -1; }
     struct Disarm { pc_ctx* c; ~Disarm() { c->prof_active_layer = -1; } } disarm{ctx};
-    launch_k(pc::prep_decode_rows, dim3((m_bound + 128) / 128), dim3(128), 0, st, sd, da, a.prompt_slots, a.suffix_slots, ctx->d.vocab, g, keys,
+    const bool dep = ctx->dep_launch != 0 && ctx->prof_active_layer < 0;
+    launch_k_dep(dep, pc::prep_decode_rows, dim3((m_bound + 128) / 128), dim3(128), 0, st, sd, da, a.prompt_slots, a.suffix_slots, ctx->d.vocab, g, keys,
              reinterpret_cast<int32_t*>(ctx->ws + ctx->cv.sched), 2 * ctx->d.n_layers, ctx->err);
     count_launches(1);
     PC_CUDA_CHECK_LAUNCH("prep_decode_rows");
@@ -1478,19 +1496,19 @@ int decode_launches(pc_ctx* ctx, cudaStream_t st, int m_bound, int groups_bound,
         // keys, output positions, token buffer, temperature and seed come from the workspace copies / the argument block
         const int chunks = pc::sample_chunks(m_bound, ctx->num_sms);
         if (chunks == 1) {
-            launch_k(pc::sample_kernel, dim3(m_bound), dim3(256), 0, st, sd, ctx->d.vocab, logits, nullptr, 1.f, 0u, 0u, keys.key_prompt, keys.rollout,
+            launch_k_dep(dep, pc::sample_kernel, dim3(m_bound), dim3(256), 0, st, sd, ctx->d.vocab, logits, nullptr, 1.f, 0u, 0u, keys.key_prompt, keys.rollout,
                                                        keys.step_key, 0, nullptr, keys.out_index, 0, nullptr, nullptr, da);
             count_launches(1);
         } else {
             pc::Top2Rec* scratch = reinterpret_cast<pc::Top2Rec*>(ctx->ws + ctx->cv.sample_scratch);
-            launch_k(pc::sample_partial_kernel, dim3(dim3(m_bound, chunks)), dim3(256), 0, st, sd, ctx->d.vocab, chunks, logits, nullptr, 1.f, 0u, 0u,
+            launch_k_dep(dep, pc::sample_partial_kernel, dim3(dim3(m_bound, chunks)), dim3(256), 0, st, sd, ctx->d.vocab, chunks, logits, nullptr, 1.f, 0u, 0u,
                                                                              keys.key_prompt, keys.rollout, keys.step_key, 0, scratch, nullptr, da);
-            launch_k(pc::sample_reduce_kernel, dim3((m_bound + pc::REDUCE_ROWS - 1) / pc::REDUCE_ROWS), dim3(32 * pc::REDUCE_ROWS), 0, st, sd, m_bound, chunks, scratch, nullptr, keys.out_index, 0,
+            launch_k_dep(dep, pc::sample_reduce_kernel, dim3((m_bound + pc::REDUCE_ROWS - 1) / pc::REDUCE_ROWS), dim3(32 * pc::REDUCE_ROWS), 0, st, sd, m_bound, chunks, scratch, nullptr, keys.out_index, 0,
                                                                             nullptr, da);
             count_launches(2);
         }
         if (a.logprobs != nullptr) {
-            launch_k(pc::token_logprob_kernel, dim3(m_bound), dim3(256), 0, st, sd, ctx->d.vocab, logits, nullptr, 1.f, nullptr, keys.out_index, 0, nullptr,
+            launch_k_dep(dep, pc::token_logprob_kernel, dim3(m_bound), dim3(256), 0, st, sd, ctx->d.vocab, logits, nullptr, 1.f, nullptr, keys.out_index, 0, nullptr,
                                                               keys.out_index, 0, da);
             count_launches(1);
         }

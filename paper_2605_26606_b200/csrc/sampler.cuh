@@ -266,6 +266,8 @@ __global__ void __launch_bounds__(SAMPLE_THREADS, SAMPLE_BLOCKS) sample_kernel(c
                                                      const int64_t* __restrict__ out_index, int64_t out_index_offset,
                                                      float* __restrict__ out_gap, const int32_t* __restrict__ prompt_key,
                                                      const DecodeArgsDev* __restrict__ da) {
+    grid_dep_wait();
+    grid_dep_launch_dependents();
     const int r = blockIdx.x;
     const int64_t ro = r;                   // index into the row arrays
     if (sd != nullptr && r >= sd->n_rows) return;
@@ -311,6 +313,8 @@ __global__ void __launch_bounds__(SAMPLE_THREADS, SAMPLE_BLOCKS) sample_partial_
                                                              const int32_t* __restrict__ row_prompt, const int32_t* __restrict__ row_rollout,
                                                              const int32_t* __restrict__ row_step, int step_offset, Top2Rec* __restrict__ scratch,
                                                              const int32_t* __restrict__ prompt_key, const DecodeArgsDev* __restrict__ da) {
+    grid_dep_wait();
+    grid_dep_launch_dependents();
     const int r = blockIdx.x, chunk = blockIdx.y;
     const int64_t ro = r;
     if (sd != nullptr && r >= sd->n_rows) return;
@@ -344,6 +348,8 @@ constexpr int REDUCE_ROWS = 4;          // rows (warps) of a block
 __global__ void __launch_bounds__(32 * REDUCE_ROWS) sample_reduce_kernel(const StepDesc* __restrict__ sd, int n_rows, int n_chunks,
                                      const Top2Rec* __restrict__ scratch, int32_t* __restrict__ out_tokens, const int64_t* __restrict__ out_index,
                                      int64_t out_index_offset, float* __restrict__ out_gap, const DecodeArgsDev* __restrict__ da) {
+    grid_dep_wait();
+    grid_dep_launch_dependents();
     const int r = blockIdx.x * REDUCE_ROWS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int64_t ro = r;
     if (r >= (sd != nullptr ? sd->n_rows : n_rows)) return;
@@ -368,6 +374,8 @@ __global__ void __launch_bounds__(256) token_logprob_kernel(const StepDesc* __re
                                                             int64_t tok_index_offset, float* __restrict__ out,
                                                             const int64_t* __restrict__ out_index, int64_t out_index_offset,
                                                             const DecodeArgsDev* __restrict__ da) {
+    grid_dep_wait();
+    grid_dep_launch_dependents();
     const int r = blockIdx.x;
     const int64_t ro = r;
     if (sd != nullptr && r >= sd->n_rows) return;
