@@ -55,6 +55,16 @@ constexpr int SIMT_LD = SIMT_BK + 4;        // padded row of a tile: eight lanes
 template <int RT> __host__ __device__ constexpr int simt_stages() { return RT >= 64 ? 4 : 8; }
 template <int RT> __host__ __device__ constexpr int simt_stage_floats() { return (RT + SIMT_BN + 1) * SIMT_LD; }      // activations, weights, gain
 template <int RT> __host__ __device__ constexpr int simt_smem_bytes() { return simt_stages<RT>() * simt_stage_floats<RT>() * 4; }
+// A launch of more CTAs than two per SM gets only the stages it fills (K = 256: four), so that more of them fit an SM: vocabulary 2,048 x
+// 128 rows are 512 CTAs, two rounds with eight stages (11.6 us), one with four (6.6).  Smaller launches keep them all: a dependent
+// CTA that settles beside those still at work slows them (down projection of 128 rows 4.0 -> 5.2 us).
+constexpr int SIMT_SPREAD_CTAS = 2 * 148;
+template <int RT> inline int simt_smem_bytes(int K, long long ctas) {
+    if (ctas <= SIMT_SPREAD_CTAS) return simt_smem_bytes<RT>();
+    const int blocks = (K + SIMT_BK - 1) / SIMT_BK, used = blocks < simt_stages<RT>() ? blocks : simt_stages<RT>();
+    const int tiles = used * simt_stage_floats<RT>() * 4, sums = SIMT_WARPS * RT * (SIMT_BN + 1) * 4;
+    return tiles > sums ? tiles : sums;
+}
 // RMSNorm in front of a GEMM (Epi::kNorm):  RMSNorm(x; gain) W^T = rstd * (x (gain * W)^T).  Every CTA has its rows' squares in hand anyway; a
 // norm kernel of its own was 4 us of a float32 decode step, five times.
 struct SimtNorm {
@@ -193,7 +203,7 @@ inline cudaError_t launch_gemm_simt_rt(cudaStream_t st, bool dep, const StepDesc
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((N + SIMT_BN - 1) / SIMT_BN, (M + RT - 1) / RT); cfg.blockDim = dim3(32 * SIMT_WARPS);
-    cfg.dynamicSmemBytes = simt_smem_bytes<RT>(); cfg.stream = st;
+    cfg.dynamicSmemBytes = simt_smem_bytes<RT>(K, (long long)cfg.gridDim.x * cfg.gridDim.y); cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;

@@ -17,26 +17,23 @@ struct RowGeom {
     int64_t* s_start;    // [M] first suffix-arena slot attended
     int32_t* s_len;      // [M] number of suffix-arena slots attended
     int32_t* token;      // [M] input token id
-    int32_t* max_slen;   // [1] largest s_len of the step (decode only)
 };
 
 // Both step-descriptor kernels also zero the grid-barrier words of the persistent decode kernel (bar, n_bar words;
 // launched with STEP_DESC_THREADS threads).
 constexpr int STEP_DESC_THREADS = 128;
-__global__ void set_step_desc(StepDesc* sd, int n_rows, int n_groups, int max_group_rows, int32_t* max_slen, int32_t* bar, int n_bar) {
+__global__ void set_step_desc(StepDesc* sd, int n_rows, int n_groups, int max_group_rows, int32_t* bar, int n_bar) {
     grid_dep_launch_dependents();
     for (int i = threadIdx.x; i < n_bar; i += blockDim.x) bar[i] = 0;
     if (threadIdx.x != 0) return;
-    *max_slen = 0;
     sd->n_rows = n_rows; sd->n_groups = n_groups; sd->max_group_rows = max_group_rows; sd->reserved = 0;
     sd->row_off = 0; sd->group_off = 0;
 }
-// First node of a captured decode step: takes the next descriptor of the caller's schedule.
-__global__ void load_step_desc(const DecodeArgsDev* __restrict__ da, int32_t* counter, StepDesc* sd, int32_t* max_slen, int32_t* bar, int n_bar) {
+// Takes the next descriptor of the caller's schedule (steps without rows, and the persistent decode kernel's steps; else decode_begin_kernel).
+__global__ void load_step_desc(const DecodeArgsDev* __restrict__ da, int32_t* counter, StepDesc* sd, int32_t* bar, int n_bar) {
     grid_dep_launch_dependents();
     for (int i = threadIdx.x; i < n_bar; i += blockDim.x) bar[i] = 0;
     if (threadIdx.x != 0) return;
-    *max_slen = 0;
     const int i = *counter;
     *sd = da->steps[i];
     *counter = i + 1;
@@ -44,19 +41,10 @@ __global__ void load_step_desc(const DecodeArgsDev* __restrict__ da, int32_t* co
 
 // Decode: row r of prompt p with `step` suffix tokens cached attends prompt slots [start_p, start_p + Lp)
 // and suffix slots [kv_start_r, kv_start_r + step + 1); its own K/V goes to suffix slot kv_start_r + step.
-// Also compacts the row's sampling key, the position of its next token and the step's group boundaries into the
-// workspace.  A row whose indices do not fit their arrays is switched off (no KV access, token 0) and flagged.
-__global__ void prep_decode_rows(const StepDesc* __restrict__ sd, const DecodeArgsDev* __restrict__ da, int64_t prompt_slots,
-                                 int64_t suffix_slots, int vocab, RowGeom g, RowKeys keys,
-                                 int32_t* __restrict__ sched, int n_sched, int32_t* err) {
-    grid_dep_wait();
-    grid_dep_launch_dependents();
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    const int n_rows = sd->n_rows;
-    for (int i = r; i < n_sched; i += gridDim.x * blockDim.x) sched[i] = 0;        // work counters of the layers' attention
-    if (r <= sd->n_groups) keys.group_start[r] = da->group_row_start[sd->group_off + r];
-    if (r >= n_rows) return;
-    const int64_t ro = sd->row_off + r;
+// Also compacts the row's sampling key and the position of its next token into the workspace.  Returns the row's token and position.
+__device__ __forceinline__ int2 prep_decode_row(const StepDesc& sd, int r, const DecodeArgsDev* __restrict__ da, int64_t prompt_slots, int64_t suffix_slots,
+                                                int vocab, const RowGeom& g, const RowKeys& keys, int32_t* err) {
+    const int64_t ro = sd.row_off + r;
     int p = da->row_prompt[ro];
     const int step = da->row_step[ro];
     const int64_t ti = da->row_tok_index[ro];
@@ -88,7 +76,23 @@ __global__ void prep_decode_rows(const StepDesc* __restrict__ sd, const DecodeAr
     keys.step_key[r] = step + 1;
     keys.out_index[r] = ok ? ti + 1 : -1;            // -1: nothing is stored for this row
     keys.sample_bound[r] = score_to_ordered(-INFINITY);      // no tile of the row has reported a second-best score yet
-    if (ok) atomicMax(g.max_slen, step + 1);
+    return make_int2(tok, Lp + step);
+}
+// The step's group boundaries and the attention's work counters, by threads tid = 0 .. n - 1.
+__device__ __forceinline__ void prep_decode_step(const StepDesc& sd, int tid, int n, const DecodeArgsDev* __restrict__ da, const RowKeys& keys,
+                                                 int32_t* __restrict__ sched, int n_sched) {
+    for (int i = tid; i < n_sched; i += n) sched[i] = 0;
+    for (int i = tid; i <= sd.n_groups; i += n) keys.group_start[i] = da->group_row_start[sd.group_off + i];
+}
+// The steps of the persistent decode kernel (which embeds by itself).
+__global__ void prep_decode_rows(const StepDesc* __restrict__ sd, const DecodeArgsDev* __restrict__ da, int64_t prompt_slots,
+                                 int64_t suffix_slots, int vocab, RowGeom g, RowKeys keys,
+                                 int32_t* __restrict__ sched, int n_sched, int32_t* err) {
+    grid_dep_wait();
+    grid_dep_launch_dependents();
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    prep_decode_step(*sd, r, gridDim.x * blockDim.x, da, keys, sched, n_sched);
+    if (r < sd->n_rows) prep_decode_row(*sd, r, da, prompt_slots, suffix_slots, vocab, g, keys, err);
 }
 
 // Prefill: packed token t of prompt p at position i attends prompt slots [start_p, start_p + i + 1).
@@ -343,40 +347,89 @@ __device__ __forceinline__ void embed_row_warp(int lane, int d, const T* __restr
 constexpr int ROW_WARPS = 8;         // items per block of the stand-alone per-(row, head) kernels
 constexpr int NORM_THREADS = NORM_SEGS * 32;
 
-// h[r, :] = E[token[r], :] (float residual stream); a[r, :] = RMSNorm(h[r, :]; gain) in storage type T (a == nullptr: the projection
-// applies it); the row's rotary factors.  next_scale (or nullptr):
-// operand_scale per row, for the output projection's epilogue.  One block per row.
+// h[r, :] = E[token, :] (float residual stream); a[r, :] = RMSNorm(h[r, :]; gain) in storage type T (a == nullptr: the projection
+// applies it); the row's rotary factors.  next_scale (or nullptr): operand_scale per row, for the output projection's epilogue.  A block.
 template <typename T>
-__global__ void __launch_bounds__(NORM_THREADS) embed_rmsnorm_kernel(const StepDesc* __restrict__ sd, int d, const int32_t* token,
-                                                                     const T* __restrict__ embed, const float* __restrict__ gain, float eps,
-                                                                     float* __restrict__ h, T* __restrict__ a, T* __restrict__ a_lo, int half_out,
-                                                                     int32_t* err, float* __restrict__ next_scale, int half, double theta,
-                                                                     const int32_t* __restrict__ pos, float2* __restrict__ rope) {
-    __shared__ float red[8];
-    __shared__ int counter;
-    const int r = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    grid_dep_wait();
-    grid_dep_launch_dependents();          // the projection that follows may set itself up and request its first weight tiles
-    if (r >= sd->n_rows) return;
-    if (threadIdx.x == 0) counter = 0;
-    const T* e_row = embed + (size_t)token[r] * d;
-    float* next = next_scale ? next_scale + r : nullptr;
-    float* h_row = h + (size_t)r * d;
+struct EmbedArgs {
+    int d;
+    const T* embed; const float* gain; float eps;
+    float* h; T* a; T* a_lo; int half_out;
+    float* next_scale;
+    int half; double theta; float2* rope;
+};
+template <typename T>
+__device__ __forceinline__ void embed_row_block(const EmbedArgs<T>& E, int r, int token, int pos, float* red, int* counter, int32_t* err) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, d = E.d;
+    const T* e_row = E.embed + (size_t)token * d;
+    float* h_row = E.h + (size_t)r * d;
     for (int i = threadIdx.x; i < (d >> 2); i += NORM_THREADS) {
         float v[4];
         VecLoad<T, 4>::load(e_row + 4 * i, v);
         reinterpret_cast<float4*>(h_row)[i] = make_float4(v[0], v[1], v[2], v[3]);
     }
     // (the warps at the end: they have the fewest elements of the row)
-    for (int i = NORM_THREADS - 1 - threadIdx.x; i < half; i += NORM_THREADS) rope[(size_t)r * half + i] = rope_entry(pos[r], i, half, theta);
-    if (a == nullptr) return;
+    for (int i = NORM_THREADS - 1 - threadIdx.x; i < E.half; i += NORM_THREADS) E.rope[(size_t)r * E.half + i] = rope_entry(pos, i, E.half, E.theta);
+    if (E.a == nullptr) return;
     __syncthreads();
+    T* a_lo = E.a_lo ? E.a_lo + (size_t)r * d : nullptr;
+    float* next = E.next_scale ? E.next_scale + r : nullptr;
     if (norm_row_fits_cta(d))
-        norm_row_cta<T>(w, lane, d, h_row, Partials{nullptr, 0, 0, 0}, 0, gain, eps, a + (size_t)r * d, a_lo ? a_lo + (size_t)r * d : nullptr,
-                        half_out, red, &counter, err, next);
+        norm_row_cta<T>(w, lane, d, h_row, Partials{nullptr, 0, 0, 0}, 0, E.gain, E.eps, E.a + (size_t)r * d, a_lo, E.half_out, red, counter, err, next);
     else if (w == 0)
-        norm_row_warp<T>(lane, d, h_row, Partials{nullptr, 0, 0, 0}, 0, gain, eps, a + (size_t)r * d, a_lo ? a_lo + (size_t)r * d : nullptr,
-                         half_out, err, next);
+        norm_row_warp<T>(lane, d, h_row, Partials{nullptr, 0, 0, 0}, 0, E.gain, E.eps, E.a + (size_t)r * d, a_lo, E.half_out, err, next);
+}
+
+// Prefill: one block per row.
+template <typename T>
+__global__ void __launch_bounds__(NORM_THREADS) embed_rmsnorm_kernel(const StepDesc* __restrict__ sd, const int32_t* __restrict__ token, const int32_t* __restrict__ pos,
+                                                                     EmbedArgs<T> E, int32_t* err) {
+    __shared__ float red[8];
+    __shared__ int counter;
+    const int r = blockIdx.x;
+    grid_dep_wait();
+    grid_dep_launch_dependents();          // the projection that follows may set itself up and request its first weight tiles
+    if (r >= sd->n_rows) return;
+    if (threadIdx.x == 0) counter = 0;
+    embed_row_block<T>(E, r, token[r], pos[r], red, &counter, err);
+}
+
+// First kernel of a decode step, one block per row (and one at least): the step's descriptor, its rows' geometry and sampling keys, their
+// embeddings, norm and rotary factors -- a chain of four kernels of 3-6 us each when every one of them is a launch.
+// schedule != nullptr: [0] the index of the step in the caller's schedule, advanced by the last block that has read it, [1] blocks that
+// have (0 between steps); nullptr: the descriptor is in *sd.
+template <typename T>
+__global__ void __launch_bounds__(NORM_THREADS) decode_begin_kernel(StepDesc* sd, int32_t* schedule, const DecodeArgsDev* __restrict__ da, int64_t prompt_slots,
+                                                                    int64_t suffix_slots, int vocab, RowGeom g, RowKeys keys,
+                                                                    int32_t* __restrict__ sched, int n_sched, EmbedArgs<T> E, int32_t* err) {
+    __shared__ float red[8];
+    __shared__ int counter;
+    __shared__ StepDesc s_sd;
+    __shared__ int2 s_row;
+    grid_dep_wait();
+    grid_dep_launch_dependents();
+    const int r = blockIdx.x;
+    if (threadIdx.x == 0) {
+        counter = 0;
+        StepDesc step;
+        if (schedule != nullptr) {
+            const int i = *reinterpret_cast<volatile int32_t*>(schedule);
+            step = da->steps[i];
+            __threadfence();
+            if (atomicAdd(schedule + 1, 1) == (int)gridDim.x - 1) {
+                schedule[1] = 0;
+                schedule[0] = i + 1;
+            }
+            if (r == 0) *sd = step;
+        } else {
+            step = *sd;
+        }
+        s_sd = step;
+        if (r < step.n_rows) s_row = prep_decode_row(step, r, da, prompt_slots, suffix_slots, vocab, g, keys, err);
+    }
+    __syncthreads();
+    if (r == 0) prep_decode_step(s_sd, threadIdx.x, NORM_THREADS, da, keys, sched, n_sched);
+    if (r >= s_sd.n_rows) return;
+    embed_row_block<T>(E, r, s_row.x, s_row.y, red, &counter, err);
 }
 
 // Optional residual update followed by the norm:  h[row, :] += pending partial sums of row;  a[r, :] = RMSNorm(h[row, :]; gain)

@@ -84,7 +84,7 @@ constexpr int kMaxSplits = pc::PARTIALS_MAX;
 
 struct Carve {
     size_t h, a, qkv, q, attn, act, logits, rope, pos, wslot, warena, p_start, p_len, s_start, s_len, token, last_row,
-        part_m, part_l, part_o, put_off, sched, res_part, step_desc, step_counter, max_slen, sample_scratch, a_lo, attn_lo, chain_layers, chain_glob,
+        part_m, part_l, part_o, put_off, sched, res_part, step_desc, step_counter, sample_scratch, a_lo, attn_lo, chain_layers, chain_glob,
         chain_bar, dargs, key_prompt, key_rollout, key_step, out_index, group_start, sample_tiles, sample_bound, ssq, row_pow2, total;
 };
 
@@ -203,8 +203,7 @@ Carve carve(const pc_ctx* c, int max_rows, int max_prefill) {
     v.chain_glob = take(sizeof(pc::chain::GlobalTab));
     v.chain_bar = take(chain_bar_words(d.n_layers) * 4);
     v.step_desc = take(sizeof(pc::StepDesc));
-    v.step_counter = take(4);
-    v.max_slen = take(4);
+    v.step_counter = take(8);             // decode_begin_kernel: index of the step, blocks that have read it
     v.sample_scratch = take((size_t)std::max(max_rows, 1) * pc::SAMPLE_MAX_CHUNKS * sizeof(pc::Top2Rec));
     v.q = take(M * c->q_dim() * eb);
     v.attn = take(M * c->q_dim() * eb);
@@ -253,7 +252,6 @@ pc::RowGeom geom(const pc_ctx* c) {
     g.s_start = reinterpret_cast<int64_t*>(w + c->cv.s_start);
     g.s_len = reinterpret_cast<int32_t*>(w + c->cv.s_len);
     g.token = reinterpret_cast<int32_t*>(w + c->cv.token);
-    g.max_slen = reinterpret_cast<int32_t*>(w + c->cv.max_slen);
     return g;
 }
 
@@ -688,9 +686,10 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
 
 // The decoder layers over the rows whose geometry is already in the workspace; leaves the residual stream in ws.h.
 // M is the row count grids and GEMM plans are sized for; the live count (<= M) is read from *sd on the device.
-template <typename T>
+// begin(embed arguments, dependent launch): launches the kernel that leaves the rows' geometry (decode), embeddings and rotary factors.
+template <typename T, class Begin>
 int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::KvArena prompt_arena, pc::KvArena suffix_arena,
-               const AttnPlan& plan, bool fold_final_norm = false) {
+               const AttnPlan& plan, bool fold_final_norm, Begin begin) {
     using namespace pc;
     constexpr bool kF32 = std::is_same<T, float>::value;
     const pc_model_desc& d = c->d;
@@ -721,8 +720,8 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
     // Row-wise kernels that wait for the one before them first and release the next one then: launched as programmatic dependents, but not in
     // steps that record phase events (an event between two kernels is no kernel-to-kernel edge).
     const bool dep = c->dep_launch != 0 && c->prof_active_layer < 0;
-    launch_k_dep(dep, embed_rmsnorm_kernel<T>, dim3(M), dim3(NORM_THREADS), 0, st, sd, d.d_model, g.token, reinterpret_cast<const T*>(c->embed), c->attn_norm[0],
-                 d.rms_eps, h, kF32 ? nullptr : a, a_lo, half_gemm ? 1 : 0, c->err, pow2_mlp, half, (double)d.rope_theta, g.pos, rope);
+    begin(EmbedArgs<T>{d.d_model, reinterpret_cast<const T*>(c->embed), c->attn_norm[0], d.rms_eps, h, kF32 ? nullptr : a, a_lo, half_gemm ? 1 : 0, pow2_mlp,
+                       half, (double)d.rope_theta, rope}, dep);
     count_launches(1);
     PC_CUDA_CHECK_LAUNCH("embed_rmsnorm");
     for (int l = 0; l < d.n_layers; ++l) {
@@ -874,6 +873,9 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
     c->pend = pend;        // folded into h by the final norm
     return PC_OK;
 }
+
+template <typename T> auto embed_kernel(const pc::EmbedArgs<T>&) { return pc::embed_rmsnorm_kernel<T>; }
+template <typename T> auto decode_begin(const pc::EmbedArgs<T>&) { return pc::decode_begin_kernel<T>; }
 
 // The factor of the final norm when the last down projection left the LM head's operand without it.
 pc::wt::RowScale folded_norm(const pc_ctx* c) {
@@ -1263,7 +1265,7 @@ int pc_prefill_shared(pc_ctx* ctx, void* stream, int n_prompts, const int32_t* p
     const pc::RowGeom g = geom(ctx);
     int32_t* last_row = reinterpret_cast<int32_t*>(ctx->ws + ctx->cv.last_row);
     pc::StepDesc* sd = reinterpret_cast<pc::StepDesc*>(ctx->ws + ctx->cv.step_desc);
-    pc::set_step_desc<<<1, pc::STEP_DESC_THREADS, 0, st>>>(sd, total_tokens, n_prompts, max_prompt_len, g.max_slen, nullptr, 0);
+    pc::set_step_desc<<<1, pc::STEP_DESC_THREADS, 0, st>>>(sd, total_tokens, n_prompts, max_prompt_len, nullptr, 0);
     launch_k_dep(ctx->dep_launch != 0, pc::prep_prefill_rows, dim3(n_prompts), dim3(256), 0, st, n_prompts, prompt_tokens, prompt_offsets, prompt_kv_start, prompt_slots,
                                                      ctx->d.vocab, g, last_row, ctx->err);
     count_launches(2);
@@ -1271,11 +1273,14 @@ int pc_prefill_shared(pc_ctx* ctx, void* stream, int n_prompts, const int32_t* p
     const pc::KvArena pa{prompt_kv, prompt_slots}, sa{prompt_kv, prompt_slots};
     const AttnPlan plan{true, n_prompts, prompt_offsets, max_prompt_len, false};
     int rc = PC_OK;
+    auto embed = [&](const auto& E, bool dep) {
+        launch_k_dep(dep, embed_kernel(E), dim3(total_tokens), dim3(pc::NORM_THREADS), 0, st, sd, g.token, g.pos, E, ctx->err);
+    };
     if (ctx->d.dtype == PC_DTYPE_F32) {
-        rc = run_layers<float>(ctx, st, total_tokens, sd, pa, sa, plan);
+        rc = run_layers<float>(ctx, st, total_tokens, sd, pa, sa, plan, false, embed);
     } else {
         rc = arena_maps(ctx, prompt_kv, prompt_slots, nullptr, 0);
-        if (rc == PC_OK) rc = run_layers<__nv_bfloat16>(ctx, st, total_tokens, sd, pa, sa, plan);
+        if (rc == PC_OK) rc = run_layers<__nv_bfloat16>(ctx, st, total_tokens, sd, pa, sa, plan, false, embed);
     }
     if (rc) return rc;
     // only the last position of every prompt goes through the LM head: its row count is known on the host
@@ -1454,13 +1459,23 @@ int run_decode_chained(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd
     return PC_OK;
 }
 
-// The kernels of one decode step.  Grids and GEMM plans are sized for (m_bound rows, groups_bound groups of at most
+// Next descriptor of the schedule to the workspace.
+void load_step(pc_ctx* ctx, cudaStream_t st, int32_t* schedule, bool chained) {
+    pc::load_step_desc<<<1, pc::STEP_DESC_THREADS, 0, st>>>(reinterpret_cast<const pc::DecodeArgsDev*>(ctx->ws + ctx->cv.dargs), schedule,
+                                                            reinterpret_cast<pc::StepDesc*>(ctx->ws + ctx->cv.step_desc),
+                                                            chained ? reinterpret_cast<int32_t*>(ctx->ws + ctx->cv.chain_bar) : nullptr,
+                                                            chained ? (int)chain_bar_words(ctx->d.n_layers) : 0);
+    count_launches(1);
+}
+
+// The kernels of one decode step.  schedule: the step's descriptor is taken from the caller's schedule (pc_decode_run), else it is in
+// the workspace.  Grids and GEMM plans are sized for (m_bound rows, groups_bound groups of at most
 // group_rows_bound rows); the live counts and the offsets into the caller's row arrays are in the step descriptor.
 int decode_launches(pc_ctx* ctx, cudaStream_t st, int m_bound, int groups_bound, int group_rows_bound, const DecodeArgs& a,
-                    float* logits_out) {
+                    float* logits_out, int32_t* schedule) {
     const pc::RowGeom g = geom(ctx);
     const pc::RowKeys keys = row_keys(ctx);
-    const pc::StepDesc* sd = reinterpret_cast<const pc::StepDesc*>(ctx->ws + ctx->cv.step_desc);
+    pc::StepDesc* sd = reinterpret_cast<pc::StepDesc*>(ctx->ws + ctx->cv.step_desc);
     const pc::DecodeArgsDev* da = reinterpret_cast<const pc::DecodeArgsDev*>(ctx->ws + ctx->cv.dargs);
     // a profiling request is served by the first step issued outside a capture (a captured step never carries the events)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -1469,21 +1484,28 @@ int decode_launches(pc_ctx* ctx, cudaStream_t st, int m_bound, int groups_bound,
     if (cap == cudaStreamCaptureStatusNone && ctx->prof_layer >= 0) { ctx->prof_active_layer = ctx->prof_layer; ctx->prof_layer = -1; }
     struct Disarm { pc_ctx* c; ~Disarm() { c->prof_active_layer = -1; } } disarm{ctx};
     const bool dep = ctx->dep_launch != 0 && ctx->prof_active_layer < 0;
-    launch_k_dep(dep, pc::prep_decode_rows, dim3((m_bound + 128) / 128), dim3(128), 0, st, sd, da, a.prompt_slots, a.suffix_slots, ctx->d.vocab, g, keys,
-             reinterpret_cast<int32_t*>(ctx->ws + ctx->cv.sched), 2 * ctx->d.n_layers, ctx->err);
-    count_launches(1);
-    PC_CUDA_CHECK_LAUNCH("prep_decode_rows");
+    int32_t* sched = reinterpret_cast<int32_t*>(ctx->ws + ctx->cv.sched);
+    const int n_sched = 2 * ctx->d.n_layers;
     const pc::KvArena pa{const_cast<void*>(a.prompt_kv), a.prompt_slots}, sa{a.suffix_kv, a.suffix_slots};
     const bool f32 = ctx->d.dtype == PC_DTYPE_F32;
     const AttnPlan plan{false, groups_bound, keys.group_start, group_rows_bound, joint_attention(ctx, m_bound, groups_bound, a.prompt_slots)};
     float* logits = logits_out ? logits_out : reinterpret_cast<float*>(ctx->ws + ctx->cv.logits);
     int rc;
     if (!f32 && ctx->decode_mode == 1 && ctx->chain_ready) {
+        if (schedule != nullptr) load_step(ctx, st, schedule, true);
+        launch_k_dep(dep, pc::prep_decode_rows, dim3((m_bound + 128) / 128), dim3(128), 0, st, sd, da, a.prompt_slots, a.suffix_slots, ctx->d.vocab, g, keys,
+                     sched, n_sched, ctx->err);
+        count_launches(1);
+        PC_CUDA_CHECK_LAUNCH("prep_decode_rows");
         rc = run_decode_chained(ctx, st, m_bound, sd, pa, sa, plan, logits);
         if (rc) return rc;
     } else {
         const bool draw_in_head = !f32 && a.sample && logits_out == nullptr && a.logprobs == nullptr && ctx->fused_sampler;
-        rc = f32 ? run_layers<float>(ctx, st, m_bound, sd, pa, sa, plan) : run_layers<__nv_bfloat16>(ctx, st, m_bound, sd, pa, sa, plan, true);
+        auto begin = [&](const auto& E, bool dependent) {
+            launch_k_dep(dependent, decode_begin(E), dim3(m_bound), dim3(pc::NORM_THREADS), 0, st, sd, schedule, da, a.prompt_slots, a.suffix_slots, ctx->d.vocab, g,
+                         keys, sched, n_sched, E, ctx->err);
+        };
+        rc = f32 ? run_layers<float>(ctx, st, m_bound, sd, pa, sa, plan, false, begin) : run_layers<__nv_bfloat16>(ctx, st, m_bound, sd, pa, sa, plan, true, begin);
         if (rc) return rc;
         if (draw_in_head) {
             // nobody asked for the logits: the draw happens in the LM head's epilogue and they are never stored
@@ -1544,14 +1566,13 @@ int pc_decode_step(pc_ctx* ctx, void* stream, int n_rows, const int32_t* row_pro
         if (int rc = arena_maps(ctx, prompt_kv, prompt_slots, suffix_kv, suffix_slots)) return rc;
     if (int rc = upload_decode_args(ctx, st, a, nullptr)) return rc;
     pc::set_step_desc<<<1, pc::STEP_DESC_THREADS, 0, st>>>(reinterpret_cast<pc::StepDesc*>(ctx->ws + ctx->cv.step_desc), n_rows, n_groups,
-                                                           max_group_rows, reinterpret_cast<int32_t*>(ctx->ws + ctx->cv.max_slen),
-                                                           reinterpret_cast<int32_t*>(ctx->ws + ctx->cv.chain_bar),
+                                                           max_group_rows, reinterpret_cast<int32_t*>(ctx->ws + ctx->cv.chain_bar),
                                                            (int)chain_bar_words(ctx->d.n_layers));
     count_launches(1);
     int groups_bound, group_rows_bound;
     const int m_bound = row_class(ctx, n_rows);
     canonical_group_bounds(ctx, n_groups, max_group_rows, m_bound, &groups_bound, &group_rows_bound);
-    return decode_launches(ctx, st, m_bound, groups_bound, group_rows_bound, a, logits_out);
+    return decode_launches(ctx, st, m_bound, groups_bound, group_rows_bound, a, logits_out, nullptr);
 }
 
 int pc_decode_run(pc_ctx* ctx, void* stream, int n_steps, const pc_step_desc* steps_host, const pc_step_desc* steps_dev,
@@ -1582,13 +1603,11 @@ int pc_decode_run(pc_ctx* ctx, void* stream, int n_steps, const pc_step_desc* st
     pc::StepDesc* sd = reinterpret_cast<pc::StepDesc*>(ctx->ws + ctx->cv.step_desc);
     if (int rc = upload_decode_args(ctx, st, a, steps_dev)) return rc;
     const pc::DecodeArgsDev* da = reinterpret_cast<const pc::DecodeArgsDev*>(ctx->ws + ctx->cv.dargs);
-    cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int32_t), st);
+    cudaError_t e = cudaMemsetAsync(counter, 0, 2 * sizeof(int32_t), st);
     if (e != cudaSuccess) return cuda_fail(e, "reset step counter");
     for (int s = 0; s < n_steps; ++s) {
         if (steps_host[s].n_rows == 0) {          // keep the device counter in step with the host loop
-            pc::load_step_desc<<<1, pc::STEP_DESC_THREADS, 0, st>>>(da, counter, sd, reinterpret_cast<int32_t*>(ctx->ws + ctx->cv.max_slen),
-                                                                    nullptr, 0);
-            count_launches(1);
+            load_step(ctx, st, counter, false);
             continue;
         }
         const int m_bound = row_class(ctx, steps_host[s].n_rows);
@@ -1614,12 +1633,7 @@ int pc_decode_run(pc_ctx* ctx, void* stream, int n_steps, const pc_step_desc* st
             e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
             if (e != cudaSuccess) return cuda_fail(e, "begin graph capture");
             g_capture_launches = 0;                // launches are recorded into the graph, not run
-            pc::load_step_desc<<<1, pc::STEP_DESC_THREADS, 0, cs>>>(da, counter, sd,
-                                                                    reinterpret_cast<int32_t*>(ctx->ws + ctx->cv.max_slen),
-                                                                    reinterpret_cast<int32_t*>(ctx->ws + ctx->cv.chain_bar),
-                                                                    (int)chain_bar_words(ctx->d.n_layers));
-            count_launches(1);
-            const int rc = decode_launches(ctx, cs, m_bound, groups_bound, group_rows_bound, a, nullptr);
+            const int rc = decode_launches(ctx, cs, m_bound, groups_bound, group_rows_bound, a, nullptr, counter);
             e = cudaStreamEndCapture(cs, &graph);
             const int captured = (int)g_capture_launches;
             g_capture_launches = -1;
