@@ -87,6 +87,13 @@ __device__ __forceinline__ void tma_load_kv(uint32_t dst, const CUtensorMap* map
         ::"r"(dst), "l"(map), "r"(bar), "r"(0), "r"(row)
         : "memory");
 }
+// The same for tiles that are read once.
+__device__ __forceinline__ void tma_load_kv_once(uint32_t dst, const CUtensorMap* map, uint32_t bar, int row, uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %3, %3}], [%2], %5;"
+        ::"r"(dst), "l"(map), "r"(bar), "r"(0), "r"(row), "l"(policy)
+        : "memory");
+}
 // Byte offset of (row r, dim d) (d a multiple of 8) in a swizzled tile of ROWS rows: boxes of 64 dims,
 // rows of 128 bytes, 16-byte chunk index XORed with (r mod 8).
 template <int ROWS>
@@ -591,6 +598,7 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
     __syncthreads();
 
     // producer cursor: item p_seq, tile p_tile (tracked identically by every lane; lane 0 issues)
+    const uint64_t policy = policy_evict_first();
     int p_seq = 0, p_tile = me, p_tiles = 0, issued = 0, consumed = 0;
     int64_t p_krow = 0;
     bool p_asked = false, p_open = false;
@@ -613,7 +621,7 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
             if (lane == 0) {
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 mbar_arrive_expect_tx(full0 + 8 * stage, 2 * TILE_BYTES);
-                tma_load_kv(tiles_u32 + stage * 2 * TILE_BYTES, &kv_map, full0 + 8 * stage, (int)(p_krow + (int64_t)p_tile * S_TP));
+                tma_load_kv_once(tiles_u32 + stage * 2 * TILE_BYTES, &kv_map, full0 + 8 * stage, (int)(p_krow + (int64_t)p_tile * S_TP), policy);
             }
             ++issued;
             p_tile += T;

@@ -73,6 +73,7 @@ attn_suffix_team_kernel(const __grid_constant__ CUtensorMap kv_map, const __grid
     const int workers = team_ctas * T_WARPS, me = rank * T_WARPS + warp;
     const int64_t krow = ((int64_t)layer * 2 * Hkv + kvh) * n_slots + g.s_start[row];
     const int64_t prow = JOINT ? ((int64_t)layer * 2 * Hkv + kvh) * prompt_slots + g.p_start[row] : 0;
+    const uint64_t policy = policy_evict_first();
     int next = me, issued = 0, consumed = 0;
     auto issue = [&]() {
         const int stage = issued % T_STAGES;
@@ -80,7 +81,7 @@ attn_suffix_team_kernel(const __grid_constant__ CUtensorMap kv_map, const __grid
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             mbar_arrive_expect_tx(full0 + 8 * stage, 2 * TILE_BYTES);
             if (JOINT && next < p_tiles) tma_load_kv(tiles_u32 + stage * 2 * TILE_BYTES, &prompt_map, full0 + 8 * stage, (int)(prow + (int64_t)next * S_TP));
-            else tma_load_kv(tiles_u32 + stage * 2 * TILE_BYTES, &kv_map, full0 + 8 * stage, (int)(krow + (int64_t)(next - p_tiles) * S_TP));
+            else tma_load_kv_once(tiles_u32 + stage * 2 * TILE_BYTES, &kv_map, full0 + 8 * stage, (int)(krow + (int64_t)(next - p_tiles) * S_TP), policy);
         }
         ++issued;
         next += workers;

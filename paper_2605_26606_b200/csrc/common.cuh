@@ -75,6 +75,11 @@ __device__ __forceinline__ float ordered_to_score(int32_t i) { return __int_as_f
 __device__ __forceinline__ void grid_dep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Cache policies for TMA loads: data read once per pass (the suffix K/V, weights that one CTA reads) is the first to leave L2, so that it
+// does not drive out activations, records and the kernels' own instructions.  Eight decode steps: 16 rows 9.46 -> 9.31 ms, 71 rows 11.01 -> 10.74,
+// 336 rows x 900 29.1 -> 28.5, 2,048 x 512 95.3 -> 94.4, 8B shape 64 rows 34.9 -> 34.3.
+__device__ __forceinline__ uint64_t policy_evict_first() { uint64_t p; asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p)); return p; }
+
 __device__ __forceinline__ void set_error(int32_t* flag, int32_t code) {
     if (flag != nullptr) atomicCAS(flag, 0, code);
 }

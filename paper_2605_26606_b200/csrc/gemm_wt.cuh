@@ -219,6 +219,16 @@ template <int CG> __device__ __forceinline__ void load_tile(uint32_t dst, const 
             ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1) : "memory");
     }
 }
+// A weight tile that is read once.
+template <int CG> __device__ __forceinline__ void load_weights_once(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, uint64_t policy) {
+    if constexpr (CG == 1) {
+        asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;"
+                     ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "l"(policy) : "memory");
+    } else {
+        asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;"
+                     ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "l"(policy) : "memory");
+    }
+}
 // 8 consecutive accumulator columns of this thread's TMEM lane
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
     uint32_t r[8];
@@ -661,7 +671,8 @@ struct EpiQkv {
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ int quotient(int x, uint64_t inverse) { return (int)(((uint64_t)(uint32_t)x * inverse) >> 32); }
 
-template <int CG, bool DUAL, class Epi>
+// ONCE: one row tile, every weight is read once per pass (with a choice at run time in the loop the 8B shape lost 2 %, large prefills 1 %).
+template <int CG, bool DUAL, bool ONCE, class Epi>
 __global__ void __launch_bounds__(THREADS, 1)
 gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
                const __grid_constant__ CUtensorMap map_x_lo, const StepDesc* __restrict__ sd, const Geom G, Epi epi, int32_t* err) {
@@ -720,6 +731,11 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
         // Before the wait for the previous kernel the weight tile of every stage is requested, and nothing else.
         {
             bool ok = true;
+            const uint64_t policy = ONCE ? policy_evict_first() : 0;
+            auto weights = [&](uint32_t dst, uint32_t bar, int c0, int c1) {
+                if constexpr (ONCE) load_weights_once<CG>(dst, &map_w, bar, c0, c1, policy);
+                else load_tile<CG>(dst, &map_w, bar, c0, c1);
+            };
             int tile = cluster, kb = kb0, f0, r0;
             place(tile, f0, r0);
             const int stages = G.stages;
@@ -728,7 +744,7 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             for (; s < stages && tile < n_tiles; ++s) {
                 if (elect_one()) {
                     if (peer == 0) mbar_arrive_expect_tx(full0 + 8 * s, CG * stage_bytes);
-                    load_tile<CG>(tiles_u32 + s * stage_bytes, &map_w, full_at + 8 * s, kb * BK, f0);
+                    weights(tiles_u32 + s * stage_bytes, full_at + 8 * s, kb * BK, f0);
                 }
                 if (++kb == kb1) { kb = kb0; tile += n_clusters; place(tile, f0, r0); }
             }
@@ -748,7 +764,7 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
                 if (elect_one()) {
                     if (!requested) {
                         if (peer == 0) mbar_arrive_expect_tx(full0 + 8 * s, CG * stage_bytes);
-                        load_tile<CG>(at, &map_w, bar, kb * BK, f0);
+                        weights(at, bar, kb * BK, f0);
                     }
                     const int r = r0 + (int)peer * (G.nt / CG);
                     load_tile<CG>(at + W_BYTES, &map_x, bar, kb * BK, r);
@@ -955,7 +971,8 @@ gemm_wt_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
 
 template <int CG, bool DUAL, class Epi>
 inline cudaError_t configure() {
-    return cudaFuncSetAttribute(gemm_wt_kernel<CG, DUAL, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    const cudaError_t e = cudaFuncSetAttribute(gemm_wt_kernel<CG, DUAL, false, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(gemm_wt_kernel<CG, DUAL, true, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
 }
 
 // map_w: boxes of 128 weight rows; map_x (and map_x_lo when DUAL): boxes of nt / CG activation rows.
@@ -979,7 +996,7 @@ inline cudaError_t launch(cudaStream_t st, const CUtensorMap& map_w, const CUten
         ++n;
     }
     cfg.attrs = attr; cfg.numAttrs = n;
-    return cudaLaunchKernelEx(&cfg, gemm_wt_kernel<CG, DUAL, Epi>, map_w, map_x, map_x_lo, sd, g, epi, err);
+    return cudaLaunchKernelEx(&cfg, g.tiles_r == 1 ? gemm_wt_kernel<CG, DUAL, true, Epi> : gemm_wt_kernel<CG, DUAL, false, Epi>, map_w, map_x, map_x_lo, sd, g, epi, err);
 }
 
 }  // namespace wt

@@ -545,7 +545,7 @@ cudaError_t count_clusters(pc_ctx* c) {
         attr[0].val.clusterDim.x = size; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr; cfg.numAttrs = 1;
         int n = 0;
-        const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, wt::gemm_wt_kernel<1, false, wt::EpiStore>, &cfg);
+        const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, wt::gemm_wt_kernel<1, false, false, wt::EpiStore>, &cfg);
         if (e != cudaSuccess) return e;
         c->max_clusters[size] = std::max(n, 1);
     }
