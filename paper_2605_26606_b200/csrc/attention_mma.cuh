@@ -11,12 +11,11 @@
 //                       query row carries its own number of visible prompt slots, which also makes this
 //                       the causal prefill kernel.  Decode: leaves (m, l, unnormalised O) per query row
 //                       in scratch.  Prefill: writes the normalised output.
-//   attn_suffix_kernel  one warp per (rollout, KV head, range of the suffix) streams the rollout's own suffix K/V
-//                       through a 3-stage TMA ring.  Positions sit on the MMA M axis (S^T = K Q^T,
+//   attn_suffix_kernel  teams of two or four warps claim (rollout, KV head) items and stream their suffix K/V through
+//                       3-stage TMA rings, beside the shared-prefix kernel.  Positions sit on the MMA M axis (S^T = K Q^T,
 //                       O^T = V^T P^T), so the 6-8 query heads fill the N = 8 axis and no MMA work is
-//                       padded; P is transposed between the two MMAs with movmatrix.  The warp that has
-//                       an item's whole suffix, or the last of the few that share it, merges it with the
-//                       prefix records into the attention output.
+//                       padded; P is transposed between the two MMAs with movmatrix.  A team merges its warps' shares
+//                       and the shared-prefix records into the attention output.
 //
 // Scores are kept in the log2 domain (scaled by log2(e) / sqrt(head_dim)) so that exp2f is the only
 // transcendental.  Waits on mbarriers are bounded (see gemm_tc.cuh).
@@ -141,7 +140,7 @@ attn_group_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* __
     // it depends on would let the next kernel start too early).  The prefill form reads K/V of this very pass: it waits first.
     if (FINAL) grid_dep_wait();
     if (grp >= sd->n_groups) { grid_dep_wait(); return; }
-    // group_row_start holds this pass's groups from entry 0 on (decode: the copy prep_decode_rows leaves in the workspace)
+    // group_row_start holds this pass's groups from entry 0 on (decode: the copy in the workspace)
     const int row0 = group_row_start[grp], n_rows = group_row_start[grp + 1] - row0;
     const int n_rep = Hq / Hkv;
     const int n_parts = FINAL ? 1 : part.n_parts;

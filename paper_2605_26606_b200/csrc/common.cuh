@@ -50,7 +50,7 @@ struct DecodeArgsDev {
     int64_t n_tokens;                 // length of the token buffer (0: unknown, not checked)
 };
 
-// Per-row sampling keys and output positions of a decode step, compacted into the workspace by prep_decode_rows.
+// Per-row sampling keys and output positions of a decode step, compacted into the workspace by prep_decode_row.
 struct RowKeys {
     int32_t* key_prompt;     // [M] prompt id of the sampling key
     int32_t* rollout;        // [M]
@@ -76,8 +76,8 @@ __device__ __forceinline__ void grid_dep_launch_dependents() { asm volatile("gri
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Cache policies for TMA loads: data read once per pass (the suffix K/V, weights that one CTA reads) is the first to leave L2, so that it
-// does not drive out activations, records and the kernels' own instructions.  Eight decode steps: 16 rows 9.46 -> 9.31 ms, 71 rows 11.01 -> 10.74,
-// 336 rows x 900 29.1 -> 28.5, 2,048 x 512 95.3 -> 94.4, 8B shape 64 rows 34.9 -> 34.3.
+// does not drive out activations, records and the kernels' own instructions.  Eight decode steps: 16 rows 9.48 -> 9.31 ms, 71 rows
+// 11.02 -> 10.66, 237 rows x 512 19.00 -> 18.55, 336 x 900 28.46 -> 27.78, 2,048 x 512 92.3 -> 91.4, 8B shape 64 rows 34.26 -> 33.56.
 __device__ __forceinline__ uint64_t policy_evict_first() { uint64_t p; asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p)); return p; }
 
 __device__ __forceinline__ void set_error(int32_t* flag, int32_t code) {
