@@ -634,17 +634,19 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
         grid_dep_launch_dependents();          // the output projection may request its weights once there is room for it
         waited = true;
     };
-    // Merges: heads me, me + T, ... of an item, side by side.  Lane 8 h + i holds m and l of source i of the h-th of them: the shares of the
-    // team's warps and up to four records, or records alone (at most five).
-    constexpr int R = MAX_MERGED_PARTS + 1;
-    float rec[H][R][EPL], rm = -INFINITY, rl = 0.f;
-    auto fetch_records = [&](size_t rh0, int np, int first) {       // first: source number of record 0
+    // Merges: heads me, me + T, ... of an item, side by side.  Lane 8 h + i holds m and l of source i of the h-th of them: up to four
+    // shared-prefix records and, as source OWN, the suffix.  The team's shares are folded into that one source first, whether it then stays in
+    // registers or is put off as a record: which of the two an item meets is a matter of timing, its sums are not.
+    constexpr int OWN = MAX_MERGED_PARTS;
+    float rec[H][OWN + 1][EPL], rm = -INFINITY, rl = 0.f;
+    auto fetch_records = [&](size_t rh0, bool own) {        // own: the suffix too, which was put off
+        const int np = part.n_parts;
 #pragma unroll
         for (int h = 0; h < H; ++h)
 #pragma unroll
-            for (int i = 0; i < R; ++i) {
-                const bool on = i < np && me + T * h < n_rep;
-                const float* src = part.o + ((size_t)i * part.stride + rh0 + me + T * h) * HD + lane * EPL;
+            for (int i = 0; i <= OWN; ++i) {
+                const bool on = (i < OWN ? i < np : own) && me + T * h < n_rep;
+                const float* src = part.o + ((size_t)(i < OWN ? i : np) * part.stride + rh0 + me + T * h) * HD + lane * EPL;
                 if (EPL == 4) {
                     const float4 x = on ? __ldcg(reinterpret_cast<const float4*>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
                     rec[h][i][0] = x.x; rec[h][i][1] = x.y; rec[h][i][EPL - 2] = x.z; rec[h][i][EPL - 1] = x.w;
@@ -653,64 +655,72 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
                     rec[h][i][0] = x.x; rec[h][i][1] = x.y;
                 }
             }
-        const int i = (lane & 7) - first, j = me + T * (lane >> 3);
-        const bool on = i >= 0 && i < np && lane < 8 * H && j < n_rep;
-        rm = on ? __ldcg(part.m + (size_t)i * part.stride + rh0 + j) : -INFINITY;
-        rl = on ? __ldcg(part.l + (size_t)i * part.stride + rh0 + j) : 0.f;
+        const int i = lane & 7, j = me + T * (lane >> 3);
+        const bool on = (i < OWN ? i < np : i == OWN && own) && lane < 8 * H && j < n_rep;
+        const size_t at = (size_t)(i < OWN ? i : np) * part.stride + rh0 + j;
+        rm = on ? __ldcg(part.m + at) : -INFINITY;
+        rl = on ? __ldcg(part.l + at) : 0.f;
     };
-    // record >= 0: the merged heads become that record, else the item's output
-    auto merge = [&](size_t rh0, bool shares, int record) {
-        float m = rm, l = rl;
-        if (shares && (lane & 7) < T && lane < 8 * H) {
-            const float* at = ml + (lane & 7) * 16 + ((me + T * (lane >> 3)) & 7);
-            m = at[0]; l = at[8];
-        }
-        float M = m;
+    // over the eight lanes of a head, the same bits in each
+    auto head_max = [&](float m) {
 #pragma unroll
-        for (int d = 1; d < 8; d <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, d));
-        const float w = exp2_safe(m, M);
-        float denom = l * w;
+        for (int d = 1; d < 8; d <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
+        return m;
+    };
+    auto head_sum = [&](float l) {
 #pragma unroll
-        for (int d = 1; d < 8; d <<= 1) denom += __shfl_xor_sync(0xffffffffu, denom, d);
-        float acc[H][EPL];
-#pragma unroll
-        for (int h = 0; h < H; ++h)
-#pragma unroll
-            for (int e = 0; e < EPL; ++e) acc[h][e] = 0.f;
+        for (int d = 1; d < 8; d <<= 1) l = __fadd_rn(l, __shfl_xor_sync(0xffffffffu, l, d));
+        return l;
+    };
+    auto fold_shares = [&]() {                    // the shares of the team's warps -> source OWN
+        const bool on = (lane & 7) < T && lane < 8 * H;
+        const float* at = ml + (lane & (T - 1)) * 16 + ((me + T * (lane >> 3)) & 7);
+        const float m = on ? at[0] : -INFINITY, l = on ? at[8] : 0.f;
+        const float M = head_max(m), w = exp2_safe(m, M), sum = head_sum(__fmul_rn(l, w));
+        if ((lane & 7) == OWN) { rm = M; rl = sum; }
 #pragma unroll
         for (int h = 0; h < H; ++h) {
 #pragma unroll
-            for (int i = 0; i < R; ++i) {
-                const float x = __shfl_sync(0xffffffffu, w, 8 * h + (shares ? min(T + i, 7) : i));
-                // a record with m = -inf was left by an empty range: its output is not defined
-                const float f = shares && i >= MAX_MERGED_PARTS ? 0.f : x;
+            for (int e = 0; e < EPL; ++e) rec[h][OWN][e] = 0.f;
 #pragma unroll
-                for (int e = 0; e < EPL; ++e) acc[h][e] = __fmaf_rn(f > 0.f ? rec[h][i][e] : 0.f, f, acc[h][e]);
-            }
-            if (shares) {
+            for (int i = 0; i < T; ++i) {
+                const float x = __shfl_sync(0xffffffffu, w, 8 * h + i);
+                const float* src = obuf + (i * 8 + ((me + T * h) & 7)) * HD + lane * EPL;
 #pragma unroll
-                for (int i = 0; i < T; ++i) {
-                    const float x = __shfl_sync(0xffffffffu, w, 8 * h + i);
-                    const float* src = obuf + (i * 8 + ((me + T * h) & 7)) * HD + lane * EPL;
-#pragma unroll
-                    for (int e = 0; e < EPL; ++e) acc[h][e] = __fmaf_rn(src[e], x, acc[h][e]);      // (a warp without tiles left zeros)
-                }
+                for (int e = 0; e < EPL; ++e) rec[h][OWN][e] = __fmaf_rn(src[e], x, rec[h][OWN][e]);      // (a warp without tiles left zeros)
             }
         }
+    };
+    auto put_off = [&](size_t rh0) {              // source OWN -> record n_parts
 #pragma unroll
         for (int h = 0; h < H; ++h) {
             const int j = me + T * h;
-            const float Mh = __shfl_sync(0xffffffffu, M, 8 * h), dh = __shfl_sync(0xffffffffu, denom, 8 * h);
+            const float m = __shfl_sync(0xffffffffu, rm, 8 * h + OWN), l = __shfl_sync(0xffffffffu, rl, 8 * h + OWN);
             if (j >= n_rep) break;
-            if (record < 0) {
-                store_attention<HD>(lane, rh0 + j, acc[h], dh, wk.out, wk.out_lo, err);
-            } else {
-                const size_t at = (size_t)record * part.stride + rh0 + j;
-                if (lane == 0) { part.m[at] = Mh; part.l[at] = dh; }
-                float* dst = part.o + at * HD + lane * EPL;
-                if (EPL == 4) *reinterpret_cast<float4*>(dst) = make_float4(acc[h][0], acc[h][1], acc[h][EPL - 2], acc[h][EPL - 1]);
-                else *reinterpret_cast<float2*>(dst) = make_float2(acc[h][0], acc[h][1]);
+            const size_t at = (size_t)part.n_parts * part.stride + rh0 + j;
+            if (lane == 0) { part.m[at] = m; part.l[at] = l; }
+            float* dst = part.o + at * HD + lane * EPL;
+            if (EPL == 4) *reinterpret_cast<float4*>(dst) = make_float4(rec[h][OWN][0], rec[h][OWN][1], rec[h][OWN][EPL - 2], rec[h][OWN][EPL - 1]);
+            else *reinterpret_cast<float2*>(dst) = make_float2(rec[h][OWN][0], rec[h][OWN][1]);
+        }
+    };
+    auto merge = [&](size_t rh0) {                // all sources -> the item's output
+        const float M = head_max(rm), w = exp2_safe(rm, M), denom = head_sum(__fmul_rn(rl, w));
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            float acc[EPL];
+#pragma unroll
+            for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
+#pragma unroll
+            for (int i = 0; i <= OWN; ++i) {
+                const float f = __shfl_sync(0xffffffffu, w, 8 * h + i);
+                // a record with m = -inf was left by an empty range: its output is not defined
+#pragma unroll
+                for (int e = 0; e < EPL; ++e) acc[e] = __fmaf_rn(f > 0.f ? rec[h][i][e] : 0.f, f, acc[e]);
             }
+            const float dh = __shfl_sync(0xffffffffu, denom, 8 * h);
+            if (me + T * h >= n_rep) break;
+            store_attention<HD>(lane, rh0 + me + T * h, acc, dh, wk.out, wk.out_lo, err);
         }
     };
 
@@ -762,7 +772,7 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
         }
         if (!ok) *abort_flag = 1;
         const size_t rh0 = (size_t)row * Hq + (size_t)kvh * n_rep;
-        if (waited) fetch_records(rh0, part.n_parts, T);      // (they travel while the warps meet)
+        if (waited) fetch_records(rh0, false);    // (they travel while the warps meet)
         team_sync();                              // the item before has been merged; the next is known
         if (*abort_flag) { ok = false; break; }
         suffix_finish<HD>(lane, o, mh, lh, ml + me * 16, ml + me * 16 + 8, obuf + me * 8 * HD);
@@ -770,11 +780,16 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
         const bool now = *records_there != 0;
         if (now && !waited) {
             wait_prefix();
-            fetch_records(rh0, part.n_parts, T);
+            fetch_records(rh0, false);
         }
         team_sync();
-        merge(rh0, true, now ? -1 : part.n_parts);
-        if (!now && me == 0 && lane == 0) { wk.link[it.item] = later; later = it.item; }
+        fold_shares();
+        if (now) {
+            merge(rh0);
+        } else {
+            put_off(rh0);
+            if (me == 0 && lane == 0) { wk.link[it.item] = later; later = it.item; }
+        }
     }
     if (!ok && lane == 0) { *abort_flag = 1; set_error(err, DEV_ERR_WAIT_TIMEOUT); }
     if (!waited) wait_prefix();                   // (every CTA waits on every path)
@@ -785,8 +800,8 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
         const int row = item / Hkv, kvh = item - row * Hkv;
         const size_t rh0 = (size_t)row * Hq + (size_t)kvh * n_rep;
         const int next = __ldcg(wk.link + item);
-        fetch_records(rh0, part.n_parts + 1, 0);
-        merge(rh0, false, -1);
+        fetch_records(rh0, true);
+        merge(rh0);
         item = next;
     }
     // drain: tiles issued but not consumed must land before the shared memory is released

@@ -7,6 +7,7 @@ import pytest
 import torch
 
 from oracle.decoder import Decoder
+from paper_2605_26606_b200 import binding as B
 from paper_2605_26606_b200 import workloads as wl
 from paper_2605_26606_b200.engine import RolloutEngine
 
@@ -50,6 +51,48 @@ def test_decode_logits_where_suffix_items_are_claimed(cuda_device, model, prompt
     """600 to 1,200 (row, KV head) items: up to one, between one and two, and more than two rounds of warp pairs.  Long prompts beside short
     suffixes: items are finished before the shared-prefix records are there, and some warps have no tile."""
     test_decode_logits_at_attention_tile_edges(cuda_device, model, prompt, rows, depth, half)
+
+
+_heads = lambda base, hq, hkv: dataclasses.replace(base, name=f"{base.name}-{hq}-{hkv}", n_q_heads=hq, n_kv_heads=hkv)
+
+
+@pytest.mark.parametrize("model,rows,prompts,caps", [(wl.SMALL_BF16, 150, (600, 1000), (2, 20)),                    # 640 items
+                                                     (wl.SMALL_QKNORM_BF16, 110, (700, 1500), (3, 70)),              # 448
+                                                     (_heads(wl.SMALL_BF16, 12, 2), 300, (500, 900), (2, 24)),       # 1,280; six query heads per KV head
+                                                     (_heads(wl.SMALL_QKNORM_BF16, 32, 8), 30, (500, 900), (20, 40)),   # 512; four
+                                                     (_heads(wl.SMALL_BF16, 16, 2), 160, (400, 800), (2, 40)),       # 640; eight
+                                                     (_heads(wl.TINY_BF16, 16, 2), 110, (300, 700), (2, 50)),        # 448, head_dim 64
+                                                     (_heads(wl.TINY_BF16, 8, 2), 160, (300, 700), (2, 50))],        # 640, head_dim 64
+                         ids=lambda v: getattr(v, "name", str(v)))
+def test_claimed_suffix_items_give_the_same_bits_whenever_they_finish(cuda_device, model, rows, prompts, caps):
+    """Ragged groups of long prompts beside short suffixes: some items are finished before the shared-prefix records are there and are
+    merged later, others at once, and which is a matter of timing.  Tokens, log-probabilities and every K and V (layer 1's are made of layer
+    0's attention outputs) are the same in every run, and with the kernels in plain stream order (mask 0: all merged at once); a few
+    rollouts are compared with the oracle."""
+    ensure_built()
+    w = dataclasses.replace(wl.WORKLOADS["config0"], model=model, n_prompts=2, prompt_len_lo=prompts[0], prompt_len_hi=prompts[1], group_size=rows,
+                            n_pilot=rows, max_new=caps[1], cap_lo=caps[0], cap_hi=caps[1], data_seed=5, forced_explicit=None)
+    weights = wl.gen_weights(model, seed=4, threads=4, gain_jitter=0.1)
+    batch = wl.gen_batch(w)
+    eng = RolloutEngine(model, weights, max_rows=2 * rows, max_prefill_tokens=int(batch.prompt_offsets[-1]))
+    eng.collect_logprobs = True
+    eng.pilot_commit_step(w, batch)                       # (the arena exists now)
+    want = None
+    for mask in (0, 63, 63, 63, 63, 63):
+        B.pc_set_dependent_launch(eng.ctx, mask)
+        eng.suffix_kv.zero_()
+        out = eng.pilot_commit_step(w, batch)
+        got = (eng.tokens.clone(), eng.logprobs.clone(), eng.suffix_kv.view(torch.int16).clone())
+        want = want or got
+        for name, a, b in zip(("tokens", "log-probabilities", "K and V"), got, want):
+            assert torch.equal(a, b), (mask, name)
+    logp, dec = want[1].cpu().numpy().reshape(2, rows, w.max_new), Decoder(model, weights)
+    for p, i in {(0, 0), (1, rows - 1), (1, rows // 2)}:
+        toks = out["tokens"][p][i]
+        pt = batch.prompt_tokens[batch.prompt_offsets[p]:batch.prompt_offsets[p + 1]]
+        logits = dec.forward_full(np.concatenate([pt, toks[:-1]]))[len(pt) - 1:].astype(np.float64)
+        ref = logits[np.arange(len(toks)), toks] - np.logaddexp.reduce(logits, axis=1)
+        assert np.max(np.abs(logp[p, i, :len(toks)] - ref)) <= 1e-1        # two logits' worth of 5e-2
 
 
 def test_probabilities_round_below_their_maximum(cuda_device):
