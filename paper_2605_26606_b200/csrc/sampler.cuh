@@ -111,11 +111,12 @@ constexpr int SAMPLE_BLOCKS = 4;        // resident per SM
 constexpr int SAMPLE_QUEUE = 160;       // per-warp queue of candidates that passed the bound: 32 waiting + up to 128 new
 
 // Bound of the words (as 2^23 + (w >> 9)) below which no candidate with a logit up to l can beat the score s; unit = log2(e) / T and
-// shift = -s log2(e) plus the slack of 1e-3 (1 + |s|), the slack of 1e-3 |l / T| is added here.
+// shift = -s log2(e) plus a slack of 5e-4 (18 + |s|).  (The noise lies between -2.9 and 16.7, so only where |l / T| < |s| + 18 does the slack have to
+// cover the float error of l / T - s, which is 1e-6 of the two.)  With a finite shift a logit of -inf is refused, and one that overflows to it:
+// masked ids cost what others do (when they passed, as a NaN: 256 rows, 90 % of 151,936 ids at -inf, 441 us against 73).
 __device__ __forceinline__ float word_limit(float l, float unit, float shift) {
-    const float y = l * unit;
     float x;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(fmaf(fabsf(y), 1e-3f, y) + shift));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(fmaf(l, unit, shift)));
     return fmaf(x, -8388608.f * 1.001f, 16777214.f);       // 2^24 - (2^23 x 1.001 + 2)
 }
 __device__ __forceinline__ float word_value(uint32_t w) { return __uint_as_float(0x4b000000u | (w >> 9)); }       // 2^23 + (w >> 9)
@@ -128,18 +129,23 @@ __device__ __forceinline__ void scan_blocks(Top2& t, const float* __restrict__ l
     const int lane = threadIdx.x & 31;
     const uint32_t lt_mask = (1u << lane) - 1u;
     const PhiloxKeys keys(k0, k1);
-    const float unit = LOG2E / temperature;
+    // While no bound is known every id passes: shift = +inf, or ALL_BUT_INF once seed() has noted the lowest id that could be the answer
+    // where every score is -inf (unit is then small enough for every other logit to pass).
+    constexpr float ALL_BUT_INF = 3e38f;
     int32_t bound_for = score_to_ordered(-INFINITY);
-    float shift = INFINITY;                     // of the bound in use: -inf, everything passes
+    float unit = 1e-3f, shift = INFINITY;
     int queued = 0;                             // warp-uniform
     auto set_bound = [&](int32_t b) {
         bound_for = b;
         const float s = ordered_to_score(b);
-        shift = fmaf(-s, LOG2E, 1e-3f * LOG2E * (1.f + fabsf(s)));
+        unit = LOG2E / temperature;
+        shift = unit < INFINITY ? fmaf(-s, LOG2E, 5e-4f * LOG2E * (18.f + fabsf(s))) : NAN /*a temperature without a reciprocal: everything passes*/;
     };
     auto share_bound = [&](float best, float second) {          // second-best of the warp's scores: a lower bound of the row's
+        const float now = ordered_to_score(bound_for);
+        if (__popc(__ballot_sync(0xffffffffu, best > now)) + __popc(__ballot_sync(0xffffffffu, second > now)) < 2) return;
         const Top2 w = top2_warp_reduce(Top2{best, second, 0});
-        if (w.second > ordered_to_score(bound_for)) {
+        if (w.second > now) {
             const int32_t b = score_to_ordered(w.second);
             if (lane == 0) atomicMax(const_cast<int32_t*>(bound), b);
             set_bound(b);
@@ -158,11 +164,17 @@ __device__ __forceinline__ void scan_blocks(Top2& t, const float* __restrict__ l
             __syncwarp();
         }
     };
-    // one candidate per lane, the one with the largest word, for a first bound (not folded: it is scored again later)
-    auto seed = [&](bool in, const Philox4& w, const float4& l) {
+    // One candidate per lane, the one with the largest word, for a first bound (not folded: it is scored again later), and the lowest id of
+    // each lane that is a number, as a candidate of score -inf.
+    auto seed = [&](bool in, int b, const Philox4& w, const float4& l) {
         const uint32_t top = max(max(w.x, w.y), max(w.z, w.w));
         const float at = top == w.x ? l.x : (top == w.y ? l.y : (top == w.z ? l.z : l.w));
         const float s = in ? at / temperature + gumbel_from_word(top) : -INFINITY;
+        const float ll[4] = {l.x, l.y, l.z, l.w};
+#pragma unroll
+        for (int i = 3; i >= 0; --i)
+            if (in && b * 4 + i < vocab && ll[i] == ll[i]) t.idx = b * 4 + i;
+        if (bound_for == score_to_ordered(-INFINITY) && __any_sync(0xffffffffu, t.idx != 0x7fffffff)) shift = ALL_BUT_INF;
         share_bound(s > -INFINITY ? s : -INFINITY /*NaN too*/, -INFINITY);
     };
     auto consider = [&](bool in, int b, const Philox4& w, const float4& l) {
@@ -207,7 +219,7 @@ __device__ __forceinline__ void scan_blocks(Top2& t, const float* __restrict__ l
 #pragma unroll
             for (int u = 0; u < U; ++u) w[u] = philox4x32_10((uint32_t)(base + u * SAMPLE_THREADS + lane), c1, c2, c3, keys);
             refresh();
-            if (first) { first = false; seed(true, w[0], l[0]); }
+            if (first) { first = false; seed(true, base + lane, w[0], l[0]); }
 #pragma unroll
             for (int u = 0; u < U; ++u) consider(true, base + u * SAMPLE_THREADS + lane, w[u], l[u]);
         }
@@ -221,7 +233,7 @@ __device__ __forceinline__ void scan_blocks(Top2& t, const float* __restrict__ l
         const float4 l4 = make_float4(l[0], l[1], l[2], l[3]);
         const Philox4 w = philox4x32_10((uint32_t)b, c1, c2, c3, keys);
         refresh();
-        if (first) { first = false; seed(b < b_end, w, l4); }
+        if (first) { first = false; seed(b < b_end, b, w, l4); }
         consider(b < b_end, b, w, l4);
     }
     drain(0);

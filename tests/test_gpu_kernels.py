@@ -90,6 +90,56 @@ def test_sample_of_masked_and_extreme_logits(vocab, temperature):
             assert out[r] == tok
 
 
+def _draw(rows, temperature, seed, scratch=None):
+    """Tokens and gaps of one pc_sample call with the keys (row, 1, 2)."""
+    n, vocab = rows.shape
+    out, gap = torch.zeros(n, dtype=torch.int32, device="cuda"), torch.zeros(n, device="cuda")
+    key = lambda v: torch.full((n,), v, dtype=torch.int32, device="cuda")
+    B.pc_sample(n, vocab, rows, None, temperature, seed, torch.arange(n, dtype=torch.int32, device="cuda"), key(1), key(2), out, None, gap, scratch)
+    return out, gap
+
+
+@pytest.mark.parametrize("vocab", [133, 4096, 20001])
+def test_sample_where_whole_ranges_are_masked(vocab):
+    """Ids of logit -inf are passed over unless nothing else is there, whatever stands before them."""
+    low, inf, nan = float(np.finfo(np.float32).min), float("inf"), float("nan")
+    rows = torch.full((6, vocab), -inf, device="cuda")
+    rows[0, :vocab // 2] = nan                              # the lowest id that is a number
+    rows[1, vocab - 1] = low                                # the only finite one
+    rows[2, vocab // 3] = 3.0
+    rows[3] = nan
+    rows[3, vocab - 2] = -inf
+    rows[4, [2, vocab - 1]] = torch.tensor([0.0, 60.0], device="cuda")     # noise spans less than 20
+    rows[5, vocab // 2:] = torch.randn(vocab - vocab // 2, device="cuda", generator=torch.Generator("cuda").manual_seed(0))
+    want = [vocab // 2, vocab - 1, vocab // 3, vocab - 2, vocab - 1, None]
+    want[5] = int(osampler.sample(np.nan_to_num(rows[5].double().cpu().numpy(), neginf=-1e300), 1.0, 7, 5, 1, 2)[0])
+    for scratch in (None, torch.empty(6 * 32 * 16, dtype=torch.uint8, device="cuda")):
+        assert _draw(rows, 1.0, 7, scratch)[0].tolist() == want
+    cold = torch.full((1, vocab), -1e-3, device="cuda")     # a temperature without a finite reciprocal: the scores are -1e36
+    cold[0, vocab - 3] = -5e-4
+    assert _draw(cold, 1e-39, 7)[0].item() == vocab - 3
+
+
+@pytest.mark.parametrize("masked,share,ordered", [(-np.inf, 0.5, False), (-np.inf, 0.9, False), (np.finfo(np.float32).min, 0.9, False), (-np.inf, 0.9, True)])
+def test_masked_logits_cost_no_more_than_others(masked, share, ordered):
+    """Scoring every masked id took four to six times as long as a vocabulary without a mask."""
+    g = torch.Generator("cuda").manual_seed(0)
+    plain = torch.randn((256, 151936), device="cuda", generator=g)
+    rows = plain.clone()
+    rows[(torch.arange(rows.shape[1], device="cuda") >= (1 - share) * rows.shape[1]).expand_as(rows) if ordered
+         else torch.rand(rows.shape, device="cuda", generator=g) < share] = float(masked)
+    scratch = torch.empty(256 * 32 * 16, dtype=torch.uint8, device="cuda")
+    best = {}
+    for name, x in (("plain", plain), ("masked", rows)) * 10:
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        ev[0].record()
+        _draw(x, 1.0, 7, scratch)
+        ev[1].record()
+        torch.cuda.synchronize()
+        best[name] = min(best.get(name, 1e9), ev[0].elapsed_time(ev[1]))
+    assert best["masked"] <= 1.8 * best["plain"], best
+
+
 def test_sample_row_mapping_and_scatter():
     rng = np.random.default_rng(0)
     V, P, G = 512, 3, 5
