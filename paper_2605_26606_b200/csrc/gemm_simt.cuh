@@ -56,11 +56,10 @@ template <int RT> __host__ __device__ constexpr int simt_stages() { return RT >=
 template <int RT> __host__ __device__ constexpr int simt_stage_floats() { return (RT + SIMT_BN + 1) * SIMT_LD; }      // activations, weights, gain
 template <int RT> __host__ __device__ constexpr int simt_smem_bytes() { return simt_stages<RT>() * simt_stage_floats<RT>() * 4; }
 // A launch of more CTAs than two per SM gets only the stages it fills (K = 256: four), so that more of them fit an SM: vocabulary 2,048 x
-// 128 rows are 512 CTAs, two rounds with eight stages (11.6 us), one with four (6.6).  Smaller launches keep them all: a dependent
+// 128 rows are 512 CTAs, on 148 SMs two rounds with eight stages (11.6 us), one with four (6.6).  Smaller launches keep them all: a dependent
 // CTA that settles beside those still at work slows them (down projection of 128 rows 4.0 -> 5.2 us).
-constexpr int SIMT_SPREAD_CTAS = 2 * 148;
-template <int RT> inline int simt_smem_bytes(int K, long long ctas) {
-    if (ctas <= SIMT_SPREAD_CTAS) return simt_smem_bytes<RT>();
+template <int RT> inline int simt_smem_bytes(int K, long long ctas, int num_sms) {
+    if (ctas <= 2 * num_sms) return simt_smem_bytes<RT>();
     const int blocks = (K + SIMT_BK - 1) / SIMT_BK, used = blocks < simt_stages<RT>() ? blocks : simt_stages<RT>();
     const int tiles = used * simt_stage_floats<RT>() * 4, sums = SIMT_WARPS * RT * (SIMT_BN + 1) * 4;
     return tiles > sums ? tiles : sums;
@@ -199,11 +198,11 @@ inline cudaError_t configure_gemm_simt() {
 }
 
 template <int RT, class Epi>
-inline cudaError_t launch_gemm_simt_rt(cudaStream_t st, bool dep, const StepDesc* sd, const float* A, const float* W, int M, int N, int K, SimtNorm nm, Epi epi) {
+inline cudaError_t launch_gemm_simt_rt(cudaStream_t st, bool dep, int num_sms, const StepDesc* sd, const float* A, const float* W, int M, int N, int K, SimtNorm nm, Epi epi) {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((N + SIMT_BN - 1) / SIMT_BN, (M + RT - 1) / RT); cfg.blockDim = dim3(32 * SIMT_WARPS);
-    cfg.dynamicSmemBytes = simt_smem_bytes<RT>(K, (long long)cfg.gridDim.x * cfg.gridDim.y); cfg.stream = st;
+    cfg.dynamicSmemBytes = simt_smem_bytes<RT>(K, (long long)cfg.gridDim.x * cfg.gridDim.y, num_sms); cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -214,12 +213,12 @@ inline cudaError_t launch_gemm_simt_rt(cudaStream_t st, bool dep, const StepDesc
 // Rows per CTA: 64 read the weights fewest times and are for passes with several waves of such tiles (at one wave, 2048 columns x
 // 128 rows, the tile's own latency shows: 11.5 us); 16 from about a CTA per SM on.
 template <class Epi>
-inline cudaError_t launch_gemm_simt(cudaStream_t st, bool dep, const StepDesc* sd, const float* A, const float* W, int M, int N, int K, SimtNorm nm, Epi epi) {
+inline cudaError_t launch_gemm_simt(cudaStream_t st, bool dep, int num_sms, const StepDesc* sd, const float* A, const float* W, int M, int N, int K, SimtNorm nm, Epi epi) {
     if (M <= 0 || N <= 0) return cudaSuccess;
     const long long cols = (N + SIMT_BN - 1) / SIMT_BN;
-    if (cols * ((M + 63) / 64) >= 512) return launch_gemm_simt_rt<64>(st, dep, sd, A, W, M, N, K, nm, epi);
-    if (cols * ((M + 15) / 16) >= 128) return launch_gemm_simt_rt<16>(st, dep, sd, A, W, M, N, K, nm, epi);
-    return launch_gemm_simt_rt<8>(st, dep, sd, A, W, M, N, K, nm, epi);
+    if (cols * ((M + 63) / 64) >= 512) return launch_gemm_simt_rt<64>(st, dep, num_sms, sd, A, W, M, N, K, nm, epi);
+    if (cols * ((M + 15) / 16) >= 128) return launch_gemm_simt_rt<16>(st, dep, num_sms, sd, A, W, M, N, K, nm, epi);
+    return launch_gemm_simt_rt<8>(st, dep, num_sms, sd, A, W, M, N, K, nm, epi);
 }
 
 }  // namespace pc

@@ -790,7 +790,7 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
         const float* bias = d.qkv_bias ? c->bqkv[l] : nullptr;
         Partials qkv_parts{qkv, 1, (size_t)M * c->n_qkv(), c->n_qkv()};
         if constexpr (kF32) {
-            launch_gemm_simt(st, dep, sd, h, reinterpret_cast<const T*>(c->wqkv[l]), M, c->n_qkv(), d.d_model,
+            launch_gemm_simt(st, dep, c->num_sms, sd, h, reinterpret_cast<const T*>(c->wqkv[l]), M, c->n_qkv(), d.d_model,
                                 SimtNorm{c->attn_norm[l], d.rms_eps, nullptr}, EpiStoreF32{qkv, c->n_qkv(), nullptr});
         } else {
             const GemmPlan gp = plan_gemm(c, GEMM_QKV, c->m_wqkv[l], M, true);
@@ -823,7 +823,7 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
             c->mark(st, l, PC_MARK_SUFFIX);
             c->mark(st, l, PC_MARK_MERGE);
             count_launches(1);
-            launch_gemm_simt(st, dep, sd, attn, reinterpret_cast<const T*>(c->wo[l]), M, d.d_model, c->q_dim(), SimtNorm{}, EpiResidual{h, d.d_model});
+            launch_gemm_simt(st, dep, c->num_sms, sd, attn, reinterpret_cast<const T*>(c->wo[l]), M, d.d_model, c->q_dim(), SimtNorm{}, EpiResidual{h, d.d_model});
         } else {
             int rc = d.head_dim == 128
                          ? attention_bf16<128>(c, st, sd, M, l, plan, prompt_arena, suffix_arena, q, attn)
@@ -850,10 +850,10 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
         count_launches(1);
         c->mark(st, l, PC_MARK_NORM_MLP);
         if constexpr (kF32) {
-            launch_gemm_simt(st, dep, sd, h, reinterpret_cast<const T*>(c->w_gate_up[l]), M, 2 * d.d_ff, d.d_model,
+            launch_gemm_simt(st, dep, c->num_sms, sd, h, reinterpret_cast<const T*>(c->w_gate_up[l]), M, 2 * d.d_ff, d.d_model,
                                 SimtNorm{c->mlp_norm[l], d.rms_eps, nullptr}, EpiSwiGLU{act, d.d_ff});
             c->mark(st, l, PC_MARK_GATE_UP);
-            launch_gemm_simt(st, dep, sd, act, reinterpret_cast<const T*>(c->w_down[l]), M, d.d_model, d.d_ff, SimtNorm{}, EpiResidual{h, d.d_model});
+            launch_gemm_simt(st, dep, c->num_sms, sd, act, reinterpret_cast<const T*>(c->w_down[l]), M, d.d_model, d.d_ff, SimtNorm{}, EpiResidual{h, d.d_model});
         } else {
             if (int rc = gemm_bf16(c, st, sd, c->map_a, nullptr, c->m_wgu[l], M, plan_gemm(c, GEMM_GATE_UP, c->m_wgu[l], M, false), tc::EpiSwiGLU{act, d.d_ff, half_gemm ? 1 : 0, c->err}, half_gemm, DEP_GATE_UP))
                 return rc;
@@ -903,7 +903,7 @@ int run_lm_head(pc_ctx* c, cudaStream_t st, int n, const pc::StepDesc* sd, const
     c->pend = pc::Partials{nullptr, 0, 0, 0};
     if constexpr (std::is_same<T, float>::value) {
         const T* wlm = reinterpret_cast<const T*>(d.tied_embed ? c->embed : c->lm_head);
-        launch_gemm_simt(st, c->dep_launch != 0 && c->prof_active_layer < 0, sd, h, wlm, n, d.vocab, d.d_model, SimtNorm{c->final_norm, d.rms_eps, src},
+        launch_gemm_simt(st, c->dep_launch != 0 && c->prof_active_layer < 0, c->num_sms, sd, h, wlm, n, d.vocab, d.d_model, SimtNorm{c->final_norm, d.rms_eps, src},
                             EpiStoreF32{logits, d.vocab, nullptr});
     } else if (folded || use_wt(c, n)) {
         wt::EpiStore epi{logits, d.vocab, {}};
@@ -1150,15 +1150,18 @@ int pc_create(const pc_model_desc* desc, const pc_weights* wts, pc_ctx** out) {
         c->w_gate_up.push_back(wts->w_gate_up[l]);
         c->w_down.push_back(wts->w_down[l]);
     }
-    if (d.dtype == PC_DTYPE_BF16) {
-        if (c->q_dim() % 64 != 0) { delete c; return PC_ERR_SHAPE; }
-        int dev = 0, sms = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) {
-            delete c;
-            return cuda_fail(cudaGetLastError(), "no CUDA device for a bf16 model");
-        }
+    if (d.dtype == PC_DTYPE_BF16 && c->q_dim() % 64 != 0) { delete c; return PC_ERR_SHAPE; }
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0) {
         c->num_sms = sms;
+    } else {
+        const cudaError_t e = cudaGetLastError();
+        if (d.dtype == PC_DTYPE_BF16) {
+            delete c;
+            return cuda_fail(e, "no CUDA device for a bf16 model");
+        }
+    }
+    if (d.dtype == PC_DTYPE_BF16) {
         bool ok = true;
         c->m_wqkv.resize(d.n_layers); c->m_wo.resize(d.n_layers); c->m_wgu.resize(d.n_layers); c->m_wdown.resize(d.n_layers);
         for (int l = 0; l < d.n_layers && ok; ++l) {
