@@ -153,6 +153,7 @@ struct pc_ctx {
     unsigned long long captures = 0;         // decode steps captured and instantiated so far (pc_capture_count)
     int32_t n_prompts_hint = 0;              // pc_set_index_bounds: sizes of the caller's per-prompt arrays and token buffer (0: unknown)
     int64_t n_tokens_hint = 0;
+    int32_t prompt_bound = 0;                // pc_set_prompt_bound: no prompt of the decode steps is longer (0: unknown)
 
     // weight-on-lanes projections (gemm_wt.cuh): descriptors of the activation buffers by box height, built when first used, and
     // the tilings chosen so far
@@ -467,11 +468,15 @@ int suffix_team_warps(const pc_ctx* c, int items) {
 // that kernel and the hand-over of its records (7 + 4 us of a 40 us layer at 16 rows) cost more than the reads, which L2 serves, up to prompts of
 // about 1,024 tokens.  Eight decode steps of the 1.5B shape, with it and without: 16 rows x 640 tokens 8.92 / 9.75 ms, 36 x 640 10.23 / 10.72, 36 x
 // 1,024 10.66 / 10.64, 72 x 1,024 12.50 / 12.67, 128 x 640 13.93 / 14.09, 128 x 1,024 13.78 / 14.02, 72 x 4,096 19.23 / 14.39; 8B shape, 32 x 512 28.6 / 29.3.
-// The lengths are on the device; the host knows the arena, which holds the prompts (at least the step's groups) and may hold more.
+// The lengths are on the device.  A caller that states the longest (pc_set_prompt_bound; the engine does, per stage) gets the choice by it: rows
+// of one long prompt among short ones would read it once each.  Else the host knows only the arena, which holds the prompts (at least the step's groups)
+// and may hold more: the average decides.
 constexpr int64_t JOINT_MAX_PROMPT = 1024;
 bool joint_attention(const pc_ctx* c, int M, int n_groups, int64_t prompt_slots) {
+    if (!suffix_teams(c, M)) return false;
+    if (c->prompt_bound > 0) return c->prompt_bound <= JOINT_MAX_PROMPT;
     const int64_t prompts = c->n_prompts_hint > 0 ? c->n_prompts_hint : n_groups;
-    return suffix_teams(c, M) && prompt_slots <= JOINT_MAX_PROMPT * prompts;
+    return prompt_slots <= JOINT_MAX_PROMPT * prompts;
 }
 
 int arena_maps(pc_ctx* c, const void* prompt_kv, int64_t prompt_slots, const void* suffix_kv, int64_t suffix_slots) {
@@ -1077,6 +1082,12 @@ int pc_set_index_bounds(pc_ctx* ctx, int n_prompts, int64_t n_tokens) {
     if (ctx == nullptr || n_prompts < 0 || n_tokens < 0) return PC_ERR_INVALID_ARG;
     ctx->n_prompts_hint = n_prompts;
     ctx->n_tokens_hint = n_tokens;
+    return PC_OK;
+}
+
+int pc_set_prompt_bound(pc_ctx* ctx, int max_prompt_len) {
+    if (ctx == nullptr || max_prompt_len < 0) return PC_ERR_INVALID_ARG;
+    ctx->prompt_bound = max_prompt_len;
     return PC_OK;
 }
 

@@ -270,6 +270,7 @@ class RolloutEngine:
         if n == 0:
             return 0
         sp = B.SampleParams(wl.temperature, wl.sample_seed)
+        B.pc_set_prompt_bound(self.ctx, int(self.batch.prompt_lens[prompts].max()))
         rid = prompts.astype(np.int64) * wl.group_size + rollouts
         key = prompts if self.prompt_key_host is None else self.prompt_key_host[prompts]
         sch, (d_first, d_p, d_r, d_key, d_zero) = self._build_schedule(

@@ -95,6 +95,39 @@ def test_claimed_suffix_items_give_the_same_bits_whenever_they_finish(cuda_devic
         assert np.max(np.abs(logp[p, i, :len(toks)] - ref)) <= 1e-1        # two logits' worth of 5e-2
 
 
+def test_few_rows_read_a_long_prompt_once_per_group(cuda_device):
+    """Prompts of 40 tokens and one of 1,500: on average they are short enough for every row to read its own, but the long one is not.  The
+    step then has the shared-prefix kernel, one launch per layer more than a step of short prompts; logits against the oracle."""
+    ensure_built()
+    model, rows, steps = wl.SMALL_BF16, 8, 4
+    weights = wl.gen_weights(model, seed=4, threads=4, gain_jitter=0.1)
+    eng = RolloutEngine(model, weights, max_rows=4 * rows, max_prefill_tokens=1700)
+    eng.use_graphs = False
+    dec, launches = Decoder(model, weights), {}
+    for longest in (40, 1500):
+        w = dataclasses.replace(wl.WORKLOADS["config0"], model=model, n_prompts=4, prompt_len_lo=longest, prompt_len_hi=longest, group_size=rows,
+                                n_pilot=rows, max_new=steps + 1, cap_lo=steps + 1, cap_hi=steps + 1, data_seed=5, forced_explicit=None)
+        batch = wl.gen_batch(w)
+        lens = np.array([40, 40, longest, 40], np.int32)
+        keep = np.concatenate([np.arange(o, o + n) for o, n in zip(batch.prompt_offsets, lens)])
+        batch = dataclasses.replace(batch, prompt_lens=lens, prompt_offsets=np.r_[0, np.cumsum(lens)].astype(np.int32), prompt_tokens=batch.prompt_tokens[keep])
+        eng.load_batch(w, batch)
+        eng.prefill()
+        eng.record_pilot_logits = {steps - 1: None}
+        before = B.pc_launch_count()
+        prompts, rollouts = np.repeat(np.arange(4), rows), np.tile(np.arange(rows), 4)
+        eng.run_stage(prompts, rollouts, record_logits=eng.record_pilot_logits)
+        launches[longest] = B.pc_launch_count() - before
+        eng.check_error_flag()
+        logits = eng.record_pilot_logits[steps - 1][0].cpu().numpy()
+        toks = eng.tokens.cpu().numpy().reshape(4, rows, w.max_new)
+        for p in (1, 2):
+            pt = batch.prompt_tokens[batch.prompt_offsets[p]:batch.prompt_offsets[p + 1]]
+            want = dec.forward_full(np.concatenate([pt, toks[p, 3, :-1]]), last_only=True)[0]
+            assert np.max(np.abs(logits[p * rows + 3] - want)) <= 5e-2, p
+    assert launches[1500] - launches[40] == steps * model.n_layers, launches
+
+
 def test_probabilities_round_below_their_maximum(cuda_device):
     """Half rounds a probability finest just below the row's largest, which is 1 and exact.  64 keys of one kind, then 200 whose score is
     higher by log2(1.00044): as 1.00044 they would round to 1, a relative error of 4.4e-4 in every output; as 1, beside 0.99956 for
