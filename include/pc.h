@@ -194,7 +194,7 @@ PC_API int pc_set_index_bounds(pc_ctx* ctx, int n_prompts, int64_t n_tokens);
 
 /* Length of the longest prompt the following decode steps attend, 0 (the default) = not stated.  No limit and not checked: small batches of a bf16
  * model (up to two (row, KV head) pairs per SM) choose by it between two forms of the attention, in which every row reads its prompt itself
- * (prompts of up to 1,024 tokens) or a kernel of its own reads a group's prompt once.  Not stated, they choose by the average over the arena
+ * (prompts of up to 1,024 tokens, the smallest batches 4,096) or a kernel of its own reads a group's prompt once.  Not stated, they choose by the average over the arena
  * (prompt_slots over the n_prompts of pc_set_index_bounds or, without that, the step's groups), which is the wrong form for rows of one long
  * prompt among many short ones.  The two differ in the last bits.  The paper has no counterpart. */
 PC_API int pc_set_prompt_bound(pc_ctx* ctx, int max_prompt_len);

@@ -466,15 +466,27 @@ int suffix_team_warps(const pc_ctx* c, int items) {
 
 // Whether the teams read the prompt too, once per row instead of once per group, and there is no shared-prefix kernel.  With so few rows
 // that kernel and the hand-over of its records (7 + 4 us of a 40 us layer at 16 rows) cost more than the reads, which L2 serves, up to prompts of
-// about 1,024 tokens.  Eight decode steps of the 1.5B shape, with it and without: 16 rows x 640 tokens 8.92 / 9.75 ms, 36 x 640 10.23 / 10.72, 36 x
+// about 1,024 tokens (more with fewer rows).  Eight decode steps of the 1.5B shape, with it and without: 16 rows x 640 tokens 8.92 / 9.75 ms, 36 x 640 10.23 / 10.72, 36 x
 // 1,024 10.66 / 10.64, 72 x 1,024 12.50 / 12.67, 128 x 640 13.93 / 14.09, 128 x 1,024 13.78 / 14.02, 72 x 4,096 19.23 / 14.39; 8B shape, 32 x 512 28.6 / 29.3.
 // The lengths are on the device.  A caller that states the longest (pc_set_prompt_bound; the engine does, per stage) gets the choice by it: rows
 // of one long prompt among short ones would read it once each.  Else the host knows only the arena, which holds the prompts (at least the step's groups)
 // and may hold more: the average decides.
 constexpr int64_t JOINT_MAX_PROMPT = 1024;
+// CTAs of a team: on its own two per SM and at most four of an item (eight decode steps of 16 rows with eight 9.87 ms, four 8.92, two 9.40).
+int joint_team(const pc_ctx* c, int items) {
+    int team = 4;
+    while (team > 1 && items * team > 2 * c->num_sms) team >>= 1;
+    return team;
+}
 bool joint_attention(const pc_ctx* c, int M, int n_groups, int64_t prompt_slots) {
     if (!suffix_teams(c, M)) return false;
-    if (c->prompt_bound > 0) return c->prompt_bound <= JOINT_MAX_PROMPT;
+    if (c->prompt_bound > 0) {
+        // the more warps share an item, the longer the prompts.  All rows of one prompt, four CTAs: 16 rows x 4,096 10.73 / 11.05 ms, x 8,192 12.98 /
+        // 12.89, 32 x 4,096 11.20 / 12.39; two: 40 x 1,100 10.52 / 11.03, x 2,048 11.60 /
+        // 11.30, 8B shape 16 x 1,100 27.75 / 27.63, x 1,536 28.4 / 27.7; one: above, 8B shape 24 x 1,100 29.5 / 28.6
+        const int team = joint_team(c, M * c->d.n_kv_heads);
+        return c->prompt_bound <= (team >= 4 ? 4096 : team >= 2 ? 1280 : JOINT_MAX_PROMPT);
+    }
     const int64_t prompts = c->n_prompts_hint > 0 ? c->n_prompts_hint : n_groups;
     return prompt_slots <= JOINT_MAX_PROMPT * prompts;
 }
@@ -651,10 +663,9 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
     }
     c->mark(st, layer, PC_MARK_GROUP);
     if (teams) {
-        // a cluster of CTAs per (row, KV head): as many as fit beside the shared-prefix kernel, one CTA of each per SM; on its own, two
-        // CTAs per SM and at most four of an item (eight decode steps of 16 rows with eight 9.87 ms, four 8.92, two 9.40)
-        int team = plan.joint ? 4 : 8;
-        while (team > 1 && items * team > (plan.joint ? 2 * c->num_sms : c->num_sms)) team >>= 1;
+        // a cluster of CTAs per (row, KV head): as many as fit beside the shared-prefix kernel, one CTA of each per SM, or joint_team
+        int team = plan.joint ? joint_team(c, items) : 8;
+        while (!plan.joint && team > 1 && items * team > c->num_sms) team >>= 1;
         cudaLaunchConfig_t cfg;
         std::memset(&cfg, 0, sizeof(cfg));
         cfg.gridDim = dim3((unsigned)(items * team)); cfg.blockDim = dim3(am::T_WARPS * 32);

@@ -95,11 +95,18 @@ def test_claimed_suffix_items_give_the_same_bits_whenever_they_finish(cuda_devic
         assert np.max(np.abs(logp[p, i, :len(toks)] - ref)) <= 1e-1        # two logits' worth of 5e-2
 
 
+@pytest.mark.parametrize("model,prompt,rows", [(wl.SMALL_BF16, 4096, 3), (wl.SMALL_BF16, 4097, 3), (wl.TINY_BF16, 1280, 20), (wl.TINY_BF16, 1281, 20),
+                                               (wl.SMALL_QKNORM_BF16, 1281, 20), (wl.SMALL_BF16, 1025, 50)], ids=lambda v: getattr(v, "name", str(v)))
+def test_decode_logits_on_both_sides_of_the_longest_prompt_rows_read_themselves(cuda_device, model, prompt, rows):
+    """4,096 tokens with four CTAs to a (row, KV head), 1,280 with two, 1,024 with one."""
+    test_decode_logits_at_attention_tile_edges(cuda_device, model, prompt, rows, 17, True)
+
+
 def test_few_rows_read_a_long_prompt_once_per_group(cuda_device):
     """Prompts of 40 tokens and one of 1,500: on average they are short enough for every row to read its own, but the long one is not.  The
     step then has the shared-prefix kernel, one launch per layer more than a step of short prompts; logits against the oracle."""
     ensure_built()
-    model, rows, steps = wl.SMALL_BF16, 8, 4
+    model, rows, steps = wl.SMALL_BF16, 30, 4
     weights = wl.gen_weights(model, seed=4, threads=4, gain_jitter=0.1)
     eng = RolloutEngine(model, weights, max_rows=4 * rows, max_prefill_tokens=1700)
     eng.use_graphs = False
