@@ -1541,7 +1541,7 @@ int decode_launches(pc_ctx* ctx, cudaStream_t st, int m_bound, int groups_bound,
     }
     if (a.sample) {
         // keys, output positions, token buffer, temperature and seed come from the workspace copies / the argument block
-        const int chunks = pc::sample_chunks(m_bound, ctx->num_sms);
+        const int chunks = pc::sample_chunks(m_bound, ctx->d.vocab, ctx->num_sms);
         if (chunks == 1) {
             launch_k_dep(dep, pc::sample_kernel, dim3(m_bound), dim3(256), 0, st, sd, ctx->d.vocab, logits, nullptr, 1.f, 0u, 0u, keys.key_prompt, keys.rollout,
                                                        keys.step_key, 0, nullptr, keys.out_index, 0, nullptr, nullptr, da);
@@ -1694,7 +1694,7 @@ int pc_sample(void* stream, int n_rows, int vocab, const float* logits, const in
     if (scratch != nullptr) {
         int dev = 0, sms = 0;
         if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
-            chunks = pc::sample_chunks(n_rows, sms);
+            chunks = pc::sample_chunks(n_rows, vocab, sms);
         while (chunks > 1 && (size_t)n_rows * chunks * sizeof(pc::Top2Rec) > scratch_bytes) --chunks;    // use what fits
     }
     if (chunks == 1) {
@@ -1831,7 +1831,7 @@ int pc_sample_static(void* stream, int n_rows, int vocab, const float* logits, c
         g_static_scratch_addr[dev] = p;
     }
     pc::Top2Rec* rec = static_cast<pc::Top2Rec*>(g_static_scratch_addr[dev]);
-    const int chunks = pc::sample_chunks(n_rows, g_static_scratch_sms[dev]);
+    const int chunks = pc::sample_chunks(n_rows, vocab, g_static_scratch_sms[dev]);
     const uint32_t k0 = (uint32_t)(seed & 0xffffffffu), k1 = (uint32_t)(seed >> 32);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // every record the second kernel reads is written by the first one in this same call: nothing has to start at zero

@@ -140,6 +140,29 @@ def test_masked_logits_cost_no_more_than_others(masked, share, ordered):
     assert best["masked"] <= 1.8 * best["plain"], best
 
 
+def _best_times(calls, runs=10):
+    best = {}
+    for name, call in list(calls.items()) * runs:
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        ev[0].record()
+        call()
+        ev[1].record()
+        torch.cuda.synchronize()
+        best[name] = min(best.get(name, 1e9), ev[0].elapsed_time(ev[1]))
+    return best
+
+
+@pytest.mark.parametrize("n,vocab", [(600, 2048), (1024, 2048), (2048, 512)])
+def test_many_short_rows_are_not_cut_into_ranges(n, vocab):
+    """With scratch a row may be drawn in several ranges.  Where there are more rows than resident blocks and the rows are short, that took
+    twice as long as the one pass without scratch."""
+    rows = torch.randn((n, vocab), device="cuda", generator=torch.Generator("cuda").manual_seed(0))
+    scratch = torch.empty(n * 32 * 16, dtype=torch.uint8, device="cuda")
+    assert torch.equal(_draw(rows, 1.0, 7, scratch)[0], _draw(rows, 1.0, 7)[0])
+    best = _best_times({"one pass": lambda: _draw(rows, 1.0, 7), "scratch": lambda: _draw(rows, 1.0, 7, scratch)}, 30)
+    assert best["scratch"] <= 1.4 * best["one pass"], best
+
+
 def test_sample_row_mapping_and_scatter():
     rng = np.random.default_rng(0)
     V, P, G = 512, 3, 5
