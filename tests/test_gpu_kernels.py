@@ -152,6 +152,17 @@ def _best_times(calls, runs=10):
     return best
 
 
+def test_rows_with_certain_ids_cost_no_more_than_others():
+    """Logits of +inf: from the second one on nothing else can be drawn.  Scoring every id after it took three times as long."""
+    plain = torch.randn((256, 151936), device="cuda", generator=torch.Generator("cuda").manual_seed(0))
+    rows = plain.clone()
+    rows[:, 5:2000:7] = float("inf")
+    scratch = torch.empty(256 * 32 * 16, dtype=torch.uint8, device="cuda")
+    assert _draw(rows, 1.0, 7, scratch)[0].tolist() == [5] * 256
+    best = _best_times({"plain": lambda: _draw(plain, 1.0, 7, scratch), "certain": lambda: _draw(rows, 1.0, 7, scratch)})
+    assert best["certain"] <= 1.8 * best["plain"], best
+
+
 @pytest.mark.parametrize("n,vocab", [(600, 2048), (1024, 2048), (2048, 512)])
 def test_many_short_rows_are_not_cut_into_ranges(n, vocab):
     """With scratch a row may be drawn in several ranges.  Where there are more rows than resident blocks and the rows are short, that took
