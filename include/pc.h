@@ -207,12 +207,16 @@ PC_API int pc_set_prompt_bound(pc_ctx* ctx, int max_prompt_len);
  * tests state).  Drops captured decode steps.  The paper has no counterpart. */
 PC_API int pc_set_fused_epilogues(pc_ctx* ctx, int on);
 
-/* bf16 models.  mask: one bit per kernel (1 QKV, 2 output, 4 gate/up, 8 down projection, 16 LM head, 32 shared-prefix
- * attention of decode steps), 0 .. 63; the default is 63.  A kernel whose bit is set is launched as a programmatic
- * dependent of the kernel before it.  A projection's CTAs set up their barriers and tensor memory and request their first
- * weight tiles while that kernel is still running; the attention kernels request prompt K/V an earlier call wrote.  All
- * wait for the kernel before them (griddepcontrol.wait) before they touch activations or any output, and release their own
- * dependents only after that.  Results are bit-identical to mask 0 (plain stream order); only the start of each kernel moves.
+/* mask 0 .. 63; the default is 63.  bf16 models have one bit per kernel (1 QKV, 2 output, 4 gate/up, 8 down projection, 16 LM
+ * head, 32 attention); a kernel whose bit is set is launched as a programmatic dependent of the kernel before it.  The small
+ * kernels have no bit and are dependents whenever the mask is not 0: the first kernel of a step and of a prefill, samplers
+ * and log-probabilities, and every kernel of a float32 model.  0 is plain stream order.  A projection's CTAs set up
+ * their barriers and tensor memory and request their first weight tiles while the kernel before is still running; the
+ * attention kernels request K/V an earlier kernel wrote.  All wait for the kernel before them (griddepcontrol.wait) before they touch
+ * anything that it writes, and release their own dependents only after that.  So what ran two kernels back has finished when
+ * a kernel starts, and the suffix attention of large batches, which starts beside the shared-prefix kernel, reads what the QKV
+ * projection wrote, claims its items, and leaves records and lists that only it reads, before its wait.  Results are
+ * bit-identical to mask 0; only the start of each kernel moves.
  * Steps that record phase events (pc_profile_step) run in plain stream order whatever the mask, and so do the projections of
  * passes of 129 .. 256 rows with one kernel per operation.  Drops captured decode steps.  The paper has no counterpart. */
 PC_API int pc_set_dependent_launch(pc_ctx* ctx, int mask);

@@ -627,7 +627,7 @@ int attention_bf16(pc_ctx* c, cudaStream_t st, const pc::StepDesc* sd, int M, in
     // a group with few query rows keeps few CTAs busy: cut its prompt into ranges so that about one CTA per SM runs
     const int q_tiles = (plan.max_group_rows * n_rep + prefix_q_rows(HD) - 1) / prefix_q_rows(HD);
     const int base_ctas = std::max(1, q_tiles * d.n_kv_heads * plan.n_groups);
-    // batches whose items occupy the suffix kernel's warps with few ranges each; smaller ones take a team of CTAs per item
+    // large batches: teams of warps claim the items; smaller ones: a team of CTAs per item
     const int items = M * d.n_kv_heads;
     const bool teams = suffix_teams(c, M);
     const int n_parts = plan.prefill ? 1 : std::max(1, std::min(teams ? am::MAX_PREFIX_PARTS : am::MAX_MERGED_PARTS, c->num_sms / base_ctas));
@@ -739,7 +739,7 @@ int run_layers(pc_ctx* c, cudaStream_t st, int M, const pc::StepDesc* sd, pc::Kv
     begin(EmbedArgs<T>{d.d_model, reinterpret_cast<const T*>(c->embed), c->attn_norm[0], d.rms_eps, h, kF32 ? nullptr : a, a_lo, half_gemm ? 1 : 0, pow2_mlp,
                        half, (double)d.rope_theta, rope}, dep);
     count_launches(1);
-    PC_CUDA_CHECK_LAUNCH("embed_rmsnorm");
+    PC_CUDA_CHECK_LAUNCH("first kernel of the pass");
     for (int l = 0; l < d.n_layers; ++l) {
         c->mark(st, l, PC_MARK_LAYER_BEGIN);
         if constexpr (!kF32) if (wt_path) {
@@ -907,17 +907,19 @@ int run_lm_head(pc_ctx* c, cudaStream_t st, int n, const pc::StepDesc* sd, const
     using namespace pc;
     const pc_model_desc& d = c->d;
     float* h = reinterpret_cast<float*>(c->ws + c->cv.h);
-    T* a = reinterpret_cast<T*>(c->ws + c->cv.a);
-    const bool half_gemm = !std::is_same<T, float>::value && d.half_gemm != 0;
-    T* a_lo = std::is_same<T, float>::value || half_gemm ? nullptr : reinterpret_cast<T*>(c->ws + c->cv.a_lo);
+    constexpr bool in_head = std::is_same<T, float>::value;      // the norm is applied by the LM head's GEMM
+    const bool half_gemm = !in_head && d.half_gemm != 0;
     c->mark(st, -1, PC_MARK_LM_BEGIN);
     const bool folded = c->final_norm_pending;         // only the 1/rms factor is still to be applied: the LM head's epilogue does
     c->final_norm_pending = false;
-    const bool in_head = std::is_same<T, float>::value;      // the norm is applied by the LM head's GEMM
-    if (!folded && !in_head)
-        launch_k(rmsnorm_kernel<T>, dim3(n), dim3(NORM_THREADS), 0, st, sd, n, d.d_model, h, src, c->pend, c->final_norm, d.rms_eps, a, a_lo, half_gemm ? 1 : 0, c->err);
+    if constexpr (!in_head) {
+        T* a_lo = half_gemm ? nullptr : reinterpret_cast<T*>(c->ws + c->cv.a_lo);
+        if (!folded)
+            launch_k(rmsnorm_kernel<T>, dim3(n), dim3(NORM_THREADS), 0, st, sd, n, d.d_model, h, src, c->pend, c->final_norm, d.rms_eps,
+                     reinterpret_cast<T*>(c->ws + c->cv.a), a_lo, half_gemm ? 1 : 0, c->err);
+    }
     c->pend = pc::Partials{nullptr, 0, 0, 0};
-    if constexpr (std::is_same<T, float>::value) {
+    if constexpr (in_head) {
         const T* wlm = reinterpret_cast<const T*>(d.tied_embed ? c->embed : c->lm_head);
         launch_gemm_simt(st, c->dep_launch != 0 && c->prof_active_layer < 0, c->num_sms, sd, h, wlm, n, d.vocab, d.d_model, SimtNorm{c->final_norm, d.rms_eps, src},
                             EpiStoreF32{logits, d.vocab, nullptr});
@@ -1625,9 +1627,7 @@ int pc_decode_run(pc_ctx* ctx, void* stream, int n_steps, const pc_step_desc* st
     if (ctx->d.dtype == PC_DTYPE_BF16)
         if (int rc = arena_maps(ctx, prompt_kv, prompt_slots, suffix_kv, suffix_slots)) return rc;
     int32_t* counter = reinterpret_cast<int32_t*>(ctx->ws + ctx->cv.step_counter);
-    pc::StepDesc* sd = reinterpret_cast<pc::StepDesc*>(ctx->ws + ctx->cv.step_desc);
     if (int rc = upload_decode_args(ctx, st, a, steps_dev)) return rc;
-    const pc::DecodeArgsDev* da = reinterpret_cast<const pc::DecodeArgsDev*>(ctx->ws + ctx->cv.dargs);
     cudaError_t e = cudaMemsetAsync(counter, 0, 2 * sizeof(int32_t), st);
     if (e != cudaSuccess) return cuda_fail(e, "reset step counter");
     for (int s = 0; s < n_steps; ++s) {
