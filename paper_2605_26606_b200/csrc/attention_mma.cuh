@@ -552,7 +552,7 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
     SuffixItem* slots = all_slots + team * S_SLOTS;
     uint64_t* all_bars = reinterpret_cast<uint64_t*>(all_slots + S_WARPS / T * S_SLOTS);
     uint64_t* bars = all_bars + warp * S_STAGES;
-    // of the team: a wait ran out, items its first warp has entered in the slots so far, the shared-prefix records are there
+    // of the team: a wait ran out, items entered in the slots so far, the shared-prefix records are there
     volatile int* abort_flag = reinterpret_cast<volatile int*>(all_bars + S_WARPS * S_STAGES) + team * 4;
     volatile int *known = abort_flag + 1, *records_there = abort_flag + 2;
     auto team_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(T * 32) : "memory"); };
@@ -561,15 +561,19 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
         grid_dep_wait();
         return;
     }
-    // A team's first warp claims: lane 0 asks for an item while the last tiles of the one before are requested, and enters it when the ring gets there.
-    int claim = 0;
+    // A team's last warp, which has the fewest tiles, claims: lane 0 asks for the item after the one in hand while that one's last tiles are
+    // requested, and enters it when the ring gets there, between two tiles or behind the last.  (Short items were claimed as far ahead as the
+    // ring reaches, by the warp that has their one tile: the CTAs that start first took four, the others one, and a claim and its look-up, 1.4 us,
+    // stood in front of each tile.  Eight steps of 64 groups with prompts of 16-64: 320 rows x 2 slots 17.9 -> 16.9 ms, 512 x 16 22.3 -> 21.3.)
+    const bool claims = me == T - 1;
+    int claim = 0, asked = 1;                     // asked: claims so far, at most two more than the items done
     auto request = [&]() { if (lane == 0) claim = atomicAdd(wk.next, 1); };
-    if (me == 0) request();
+    if (claims) request();
     const uint32_t tiles_u32 = smem_u32(base + warp * RING_BYTES), full0 = smem_u32(bars);
     const int n_rep = Hq / Hkv, n_items = sd->n_rows * Hkv;
 
     if (threadIdx.x == 32) asm volatile("prefetch.tensormap [%0];" ::"l"(&kv_map) : "memory");
-    if (me == 0 && lane == 0) { *abort_flag = 0; *known = 0; *records_there = part.done == nullptr; }
+    if (claims && lane == 0) { *abort_flag = 0; *known = 0; *records_there = part.done == nullptr; }
     if (lane == 0) {
         for (int s = 0; s < S_STAGES; ++s) mbar_init(full0 + 8 * s, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -593,28 +597,29 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
         }
         __syncwarp();
     };
-    if (me == 0) enter(0);
+    if (claims) enter(0);
     __syncthreads();
 
-    // producer cursor: item p_seq, tile p_tile (tracked identically by every lane; lane 0 issues)
+    // item in hand; producer cursor: item p_seq, tile p_tile (tracked identically by every lane; lane 0 issues)
     const uint64_t policy = policy_evict_first();
-    int p_seq = 0, p_tile = me, p_tiles = 0, issued = 0, consumed = 0;
+    int seq = 0, p_seq = 0, p_tile = me, p_tiles = 0, issued = 0, consumed = 0;
     int64_t p_krow = 0;
-    bool p_asked = false, p_open = false;
-    auto refill = [&]() {
+    bool p_open = false;
+    auto refill = [&](bool may_enter) {           // may_enter: the warp that claims may wait for its claim
         while (issued - consumed < S_STAGES) {
+            if (claims && asked == seq + 1 && (p_seq > seq || (p_open && p_tile + 2 * T >= p_tiles))) { request(); ++asked; }
             if (!p_open) {
+                if (p_seq > seq + 1) return;
                 if (p_seq >= __shfl_sync(0xffffffffu, *known, 0)) {
-                    if (me != 0) return;          // the first warp has not got there: again at the next tile or item
+                    if (!claims || !may_enter) return;       // again at the next tile or item
                     enter(p_seq);
                 }
                 __syncwarp();
                 const SuffixItem s = slots[p_seq % S_SLOTS];
                 if (s.item < 0) return;
                 p_krow = s.krow; p_tiles = (s.n + S_TP - 1) / S_TP; p_tile = me;
-                p_open = true; p_asked = false;
+                p_open = true;
             }
-            if (me == 0 && !p_asked && p_tile + 2 * T >= p_tiles) { request(); p_asked = true; }
             if (p_tile >= p_tiles) { ++p_seq; p_open = false; continue; }
             const int stage = issued % S_STAGES;
             if (lane == 0) {
@@ -738,8 +743,8 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
         }
         q_seq = seq;
     };
-    refill();
-    for (int seq = 0;; ++seq) {
+    refill(false);
+    for (;; ++seq) {
         const SuffixItem it = slots[seq % S_SLOTS];
         if (it.item < 0) break;
         const int row = it.item / Hkv, kvh = it.item - row * Hkv, tiles = (it.n + S_TP - 1) / S_TP;
@@ -747,7 +752,7 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
         uint32_t qb[KS][2];
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks) { qb[ks][0] = qn[ks][0]; qb[ks][1] = qn[ks][1]; }
-        refill();
+        refill(false);
         float o[DT][4];
 #pragma unroll
         for (int t = 0; t < DT; ++t) { o[t][0] = o[t][1] = o[t][2] = o[t][3] = 0.f; }
@@ -760,21 +765,17 @@ attn_suffix_kernel(const __grid_constant__ CUtensorMap kv_map, const StepDesc* _
             suffix_tile<HD>(kb, kb + TILE_BYTES, lane, min(S_TP, it.n - tile * S_TP), scale_log2, qb, o, mh, lh, [&]() {
                 ++consumed;
                 __syncwarp();
-                refill();
+                refill(tile + T < tiles);
             });
         }
-        if (me == 0) {
-            if (ok && p_seq == seq) refill();     // (its last tile was requested, the next item may not have been looked up)
-            if (lane == 0) {
-                if (!ok) *abort_flag = 1;
-                if (*records_there == 0 && *reinterpret_cast<volatile int32_t*>(part.done) >= wk.prefix_ctas) *records_there = 1;
-            }
-        }
+        if (claims && ok) refill(true);           // (the next item may not have been looked up)
+        if (me == 0 && lane == 0 && *records_there == 0 && *reinterpret_cast<volatile int32_t*>(part.done) >= wk.prefix_ctas) *records_there = 1;
         if (!ok) *abort_flag = 1;
         const size_t rh0 = (size_t)row * Hq + (size_t)kvh * n_rep;
         if (waited) fetch_records(rh0, false);    // (they travel while the warps meet)
         team_sync();                              // the item before has been merged; the next is known
         if (*abort_flag) { ok = false; break; }
+        refill(false);
         suffix_finish<HD>(lane, o, mh, lh, ml + me * 16, ml + me * 16 + 8, obuf + me * 8 * HD);
         if (*known > seq + 1) fetch_q(seq + 1);
         const bool now = *records_there != 0;
