@@ -456,12 +456,14 @@ struct AttnPlan {
 bool suffix_teams(const pc_ctx* c, int M) { return M * c->d.n_kv_heads <= 2 * c->num_sms; }
 
 // Warps that share an item of attn_suffix_kernel: two, so that a CTA has two items in hand and one is streamed while the other is merged;
-// four where the items would be one to two rounds of the pairs, the second of them partly empty.  Eight decode steps with pairs / with
-// four, 1.5B shape, 296 CTAs = 592 pairs: 237 rows x 512 (474 items) 19.03 / 19.25 ms, 336 x 900 (672) 29.9 / 29.4, 2,048 x 512 (4,096) 95.1 /
-// 96.7; 8B shape, 64 x 300 (512) 34.7 / 35.3.
+// four where a second round of the pairs would be less than half full, which gains with long suffixes and loses with short ones (their depth only
+// the device knows); beyond half full more is lost than gained.  Eight decode steps with pairs / with four, 296 CTAs = 592 pairs, 1.5B shape:
+// 310 rows x 900 (620 items) 28.0 / 26.9 ms, 336 x 512 (672) 24.3 / 23.8, 336 x 900 29.6 / 28.6, 400 x 64 (800) 21.6 / 22.1, 400 x 512 27.5 / 27.2; 460 x
+// 300 (920) 26.6 / 26.6, 512 x 16 (1,024) 21.7 / 22.7, 512 x 300 27.2 / 27.9, 592 x 512 (1,184) 35.8 / 36.4, 2,048 x 32 66.4 / 70.4; 8B shape, 90 x 300 (720)
+// 37.8 / 38.3, 90 x 700 44.9 / 43.7, 140 x 400 (1,120) 49.3 / 50.8, 500 x 4 77.3 / 82.5.  One round: 237 x 512 (474) 19.0 / 19.3, 8B 64 x 300 (512) 34.7 / 35.3.
 int suffix_team_warps(const pc_ctx* c, int items) {
     const int pairs = c->num_sms * pc::am::S_CTAS * pc::am::S_WARPS / 2;
-    return items > pairs && items <= 2 * pairs ? 4 : 2;
+    return items > pairs && 2 * items <= 3 * pairs ? 4 : 2;
 }
 
 // Whether the teams read the prompt too, once per row instead of once per group, and there is no shared-prefix kernel.  With so few rows

@@ -48,8 +48,9 @@ def test_decode_logits_at_attention_tile_edges(cuda_device, model, prompt, rows,
                                                           (wl.SMALL_BF16, 300, 160, 35, False), (wl.SMALL_BF16, 64, 300, 18, True),
                                                           (wl.TINY_BF16, 130, 160, 34, True)], ids=lambda v: getattr(v, "name", str(v)))
 def test_decode_logits_where_suffix_items_are_claimed(cuda_device, model, prompt, rows, depth, half):
-    """600 to 1,200 (row, KV head) items: up to one, between one and two, and more than two rounds of warp pairs.  Long prompts beside short
-    suffixes: items are finished before the shared-prefix records are there, and some warps have no tile."""
+    """600 to 1,200 (row, KV head) items, where B200 has room for 592 pairs of warps: four to an item up to one and a half rounds of pairs, two beyond.
+    Suffixes of one to five tiles, so some warps have none; long prompts beside short suffixes, so items are finished before the shared-prefix
+    records are there.  (Fewer items, other head counts and ragged caps: below.)"""
     test_decode_logits_at_attention_tile_edges(cuda_device, model, prompt, rows, depth, half)
 
 
