@@ -28,8 +28,8 @@ if ROOT not in sys.path:
 from paper_2605_26606_b200 import dist_util  # noqa: E402
 from paper_2605_26606_b200 import workloads as wl  # noqa: E402
 
-# DRAM traffic of the suffix attention kernel per algorithmic byte, from the ncu captures in profiles/decode_kernels_ncu.md: 146.2 MB
-# moved for 136.1 MB at 256 rollouts x 513 slots (1.045 at 64 x 513, 1.041 at 1,024 x 129).  The kernel streams every (rollout, KV
+# DRAM traffic of the suffix attention kernel per algorithmic byte, from the ncu captures in profiles/decode_kernels_ncu.md: 145.6 MB
+# moved for 136.1 MB at 256 rollouts x 513 slots (1.035 at 1,024 x 129).  The kernel streams every (rollout, KV
 # head) suffix once, so traffic grows in proportion to the algorithmic bytes of a launch.
 SUFFIX_TRAFFIC_PER_ALGORITHMIC_BYTE = 1.07
 METRIC = "generated tokens/s"
